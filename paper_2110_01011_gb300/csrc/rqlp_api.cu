@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "split_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace rqlp {
@@ -53,8 +54,7 @@ class Ops {
     gates = ar.take<int>(kGates);
     cstore_ = ar.take<char>(chol_global_bytes(dcap_, o_.small_fp64 != 0));
     if (with_tc) {
-      tc_.layout(ar, m, n, dcap_, std::max(m, n), false, three_);
-      tc_.set_profiled(true);
+      split_gemm_layout(ar, &sg_, std::max(m, n), std::max(m, n), dcap_, three_ ? 3 : 2);
       // Tall d-column operands of CholeskyQR: the Gram (BF16x3) and the
       // products X R^{-1} (exact mode, six products) on the tensor cores.
       tcs_.layout(ar, std::max(m, n), dcap_, dcap_, dcap_, true, /*three_part=*/true);
@@ -88,10 +88,13 @@ class Ops {
   }
 
   cudaError_t init() {
-    tc_.reset();
     tcs_.reset();
+    CK(begin_products());
     return init_scratch(info_, gates, kGates, scal, kScal, st_);
   }
+
+  // Before the first product of a call.
+  cudaError_t begin_products() { return tc_on_ ? split_gemm_reset(&sg_, st_) : cudaSuccess; }
 
   // transA: out (n x d) = A^T X (X m x d); else out (m x d) = A X (X n x d).
   cudaError_t pass(bool transA, const float* A, int64_t m, int64_t n, int64_t lda, const float* X,
@@ -103,8 +106,8 @@ class Ops {
       if (prof) profile_mark_end(st_, transA ? 1 : 0);
       return e;
     }
-    if (o_.precision == RQLP_PREC_BF16X3)   // the engine brackets its MMA kernel when profiling
-      return tc_.pass(transA, A, m, n, lda, X, ldx, d_, out, ldout, sumsq, info_, st_, three_);
+    if (o_.precision == RQLP_PREC_BF16X3)   // (brackets its kernels itself when profiling)
+      return split_product(transA, transA ? n : m, transA ? m : n, A, lda, X, ldx, out, ldout, sumsq);
     const bool prof = profiling_on();
     if (prof) profile_mark_begin(st_);
     const int64_t M = transA ? n : m, K = transA ? m : n;
@@ -114,15 +117,11 @@ class Ops {
     return e;
   }
   // out (n x d) = A(r0 .. r0 + rows - 1, :)^T X (X: those rows), A m x n on
-  // the device; first: rows start at 0 (the split of A begins). ||A||_F^2 of
-  // the rows rides along into scal[0].
+  // the device. ||A||_F^2 of the rows rides along into scal[0].
   cudaError_t pass_rows(const float* A, int64_t m, int64_t n, int64_t lda, int64_t r0, int64_t rows,
                         const float* X, int64_t ldx, float* out, int64_t ldout) {
-    if (o_.precision == RQLP_PREC_BF16X3) {
-      if (r0 == 0) CK(tc_.begin_split(A, m, n, st_));
-      CK(tc_.split_rows(A + r0 * lda, r0, rows, lda, &scal[0], st_));
-      return tc_.pass_k(true, r0, rows, X, ldx, d_, out, ldout, info_, st_, three_);
-    }
+    if (o_.precision == RQLP_PREC_BF16X3)
+      return split_product(true, n, rows, A + r0 * lda, lda, X, ldx, out, ldout, &scal[0]);
     const bool prof = profiling_on();
     if (prof) profile_mark_begin(st_);
     cudaError_t e = gemm_f32_ex(true, n, d_, rows, A + r0 * lda, lda, X, ldx, out, ldout,
@@ -138,15 +137,15 @@ class Ops {
   cudaError_t power_fused(const float* A, int64_t m, int64_t n, int64_t lda, const float* X, int64_t ldx, float* Y,
                           int64_t ldy, float* Z, float* T) {
     const bool tc = o_.precision == RQLP_PREC_BF16X3;
-    const int64_t h = fused_rows(m, n, tc ? (three_ ? 6 : 4) : 4);
-    for (int64_t r0 = 0; r0 < m; r0 += h) {   // (in the BF16x3 form A's split is current: the sketch made it)
+    const int64_t h = fused_rows(m, n, 4);
+    for (int64_t r0 = 0; r0 < m; r0 += h) {
       const int64_t rows = std::min(h, m - r0);
       float* zb = Z + r0 * ld_;
       float* dst = r0 == 0 ? Y : T;
       const int64_t ldd = r0 == 0 ? ldy : ld_;
       if (tc) {
-        CK(tc_.pass_k(false, 0, n, X, ldx, d_, zb, ld_, info_, st_, three_, r0, rows));
-        CK(tc_.pass_k(true, r0, rows, zb, ld_, d_, dst, ldd, info_, st_, three_));
+        CK(split_product(false, rows, n, A + r0 * lda, lda, X, ldx, zb, ld_, nullptr));
+        CK(split_product(true, n, rows, A + r0 * lda, lda, zb, ld_, dst, ldd, nullptr));
       } else {
         CK(gemm_f32_ex(false, rows, d_, n, A + r0 * lda, lda, X, ldx, zb, ld_, gemm_f32_splits(rows, d_, n), part_,
                        nullptr, nullptr, kGateNone, false, st_));
@@ -156,6 +155,12 @@ class Ops {
       if (r0 > 0) CK(add_matrix(n, d_, T, ld_, Y, ldy, st_));
     }
     return cudaSuccess;
+  }
+  // out (M x d) = op(A) X with X K x d in the BF16x3 form (A M x K, or K x M when transA).
+  cudaError_t split_product(bool transA, int64_t M, int64_t K, const float* A, int64_t lda, const float* X, int64_t ldx,
+                            float* out, int64_t ldout, double* sumsq) {
+    return split_gemm(&sg_, transA, M, d_, K, A, lda, X, ldx, out, ldout, three_ ? kSplitThree : kSplitTwo, sumsq,
+                      nullptr, info_, true, st_);
   }
   // Row-panel height of power_fused: at most ~48 MB of A's pass operands
   // (bpe bytes per element of A), a multiple of 128 rows.
@@ -280,7 +285,8 @@ class Ops {
   int* info_ = nullptr;
   float *G_ = nullptr, *R_[3] = {}, *Ri_[3] = {}, *Ra_ = nullptr, *part_ = nullptr;
   void* cstore_ = nullptr;
-  TcEngine tc_, tcs_;
+  SplitGemmWs sg_;
+  TcEngine tcs_;
   bool tc_on_ = false;
   bool three_ = false;
   const SparseA* sp_ = nullptr;
@@ -740,7 +746,8 @@ rqlp_status rqlp_sketch(int trans, const float* A, int64_t m, int64_t n, int64_t
   ops.set_three_part(three_part_passes(o, m, n, -1));
   ops.layout(ar, Ops::pass_part_floats(m, n, d), o.precision == RQLP_PREC_BF16X3, m, n);
   ops.bind(static_cast<cudaStream_t>(stream), nullptr);
-  cudaError_t e = ops.pass(trans == 1, A, m, n, lda, X, ldx, Y, ldy, nullptr);
+  cudaError_t e = ops.begin_products();
+  if (e == cudaSuccess) e = ops.pass(trans == 1, A, m, n, lda, X, ldx, Y, ldy, nullptr);
   return e == cudaSuccess ? RQLP_OK : RQLP_ERR_CUDA;
 }
 

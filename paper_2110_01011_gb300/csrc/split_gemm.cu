@@ -1,0 +1,1051 @@
+// out = op(A) X (N <= 256 columns) on the tensor cores, with A read once in
+// FP32 and split into BF16 parts inside the kernel.
+//
+// A = A_1 + A_2 [+ A_3] and X likewise, each part the BF16 rounding of what
+// the earlier ones leave. Two parts: A_1 X_1 + A_1 X_2 + A_2 X_1 (the BF16x3
+// form, products above 2^-16). Three parts: the six products above 2^-24;
+// three parts hold all 24 bits of an FP32 value, so the sum is as accurate as
+// FP32 arithmetic.
+//
+// What bounds the product: with A's parts in shared memory the MMAs read A (4
+// KB) and X (up to 8 KB) per product and 16 of K, and the copies into shared
+// memory come on top: ~170 bytes per clock against the 128 that shared memory
+// delivers. Here A never passes through shared memory: four warps load it from
+// global memory into registers, split it there and store the parts to tensor
+// memory, from where the MMA takes its A operand. Shared memory then serves X
+// only, and neither a separate pass over A nor a copy of its parts is needed
+// (4 bytes per element of A and pass instead of 4 or 6 and a 8 or 10 byte
+// split).
+//
+// CG = 2: two CTAs of a cluster share one 256-row tile (cta_group::2): each
+// holds half of X's columns, so X is read from L2 once per 256 rows and each
+// shared memory feeds half of X.
+//
+// X's parts are written by split_x_kernel as the images of the shared-memory
+// stages (32 of K, K-major rows of 64 bytes, 64-byte swizzle), so a stage is
+// one bulk copy.
+//
+// Warps: 0 copies X stages, 1 issues the MMAs, 2 allocates tensor memory; 4-7
+// load and split A; 8-15 drain the accumulators. Chains in tensor memory are
+// cut every `chunk` units of 32 (the accumulation there loses a little of
+// every add in the same direction); the drain warps hold the running sums in
+// registers and add with round-to-nearest. The (tile, unit) pairs are dealt
+// evenly to the CTAs (stream-K); split tiles are summed by the last CTA to
+// arrive, or by split_fixup_kernel when a tile spans more than kMaxSlots of
+// them. Every wait is bounded; a timeout is reported in the status word.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "split_gemm.cuh"
+#include "tc_ptx.cuh"
+
+namespace rqlp {
+namespace {
+
+constexpr int BM = 128;               // rows per CTA (TMEM lanes)
+constexpr int BK = 32;                // K per unit
+constexpr int kThreads = 640;          // 4 + 8 + 8 warps
+constexpr int kGroups = 7;             // 16-column groups of a drain warp: N <= 224
+constexpr int CG = 2;                 // CTAs per tile (cta_group::2)
+constexpr int kMaxStages = 8;
+constexpr int kMaxASlots = 8;
+constexpr int kMaxSlots = 16;
+constexpr uint32_t kABytes = BM * BK * 4;   // FP32 stage of A
+constexpr int kCopyStages = 6;        // FP32 stages when the split warps copy A themselves
+constexpr int kPrefetch = 12;         // units between their L2 prefetch and the copy
+constexpr long long kWaitLimit = 4000000000LL;   // cycles (~2 s)
+// Parts hold a value exactly when its magnitude lies in [2^-96, 2^127) (or is
+// zero): below, the last part would be subnormal; above, the first may round
+// to infinity.
+constexpr uint32_t kRangeHi = 0x7F000000u, kRangeLo = 0x0F800000u;
+
+struct Args {
+  const float* A;
+  long long lda;
+  const uint16_t* img;
+  float* out;
+  long long ldo;
+  float* part;
+  int* cnt;
+  const int* xlo;
+  int* bad;
+  int* next0;               // words of the next product, cleared here
+  int* next1;
+  double* sumsq;
+  int* info;
+  int M, N, K, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole;   // sx, sf, sa: stages of X, of A in FP32, A slots
+  int chunk;                // units per chain of the main accumulator
+  int corr_first;           // chains of one unit, the correction products first
+  int flush;                // units whose sums are held in registers before they are added to global memory
+  int corr;                 // 0: one accumulator; else main chains per chain of the correction accumulator
+  int units;                // tiles x kb
+  uint32_t idesc;
+};
+
+__device__ void post_timeout(int* info) {
+  if (info != nullptr && atomicCAS(info, 0, RQLP_ERR_TIMEOUT) == 0) info[1] = 0;
+}
+
+// First unit of group c: an even share of all units, or of the whole tiles.
+__host__ __device__ inline int first_unit(int c, int units, int G, int whole, int tiles, int kb) {
+  if (whole) return (int)((long long)c * tiles / G) * kb;
+  return (int)((long long)c * units / G);
+}
+// The group whose range holds unit u (stream-K deal).
+__host__ __device__ inline int unit_owner(int u, int units, int G) {
+  return (int)((((long long)u + 1) * G + units - 1) / units) - 1;
+}
+// Tile and unit of K at a position of a range.
+struct Cursor {
+  int t, k;
+  __device__ Cursor(int u, int kb) : t(u / kb), k(u % kb) {}
+  __device__ void next(int kb) {
+    if (++k == kb) {
+      k = 0;
+      ++t;
+    }
+  }
+};
+// Stage of a ring and the parity of its current round.
+struct Ring {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ void next(int n) {
+    if (++s == n) {
+      s = 0;
+      ph ^= 1u;
+    }
+  }
+};
+
+// D[tmem] (+)= A[tmem] B[shared memory] over the CTA pair, issued by its leader.
+__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+               " tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d), "r"(a), "l"(b),
+               "r"(idesc), "r"(acc) : "memory");
+}
+// Arrive on `bar` of both CTAs of the pair once the MMAs issued so far are done.
+__device__ __forceinline__ void commit(uint64_t* bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+               ::"r"(tc::smem_u32(bar)), "h"((uint16_t)3) : "memory");
+}
+// Arrive on the pair leader's barrier. Relaxed: what the arrival hands over
+// lies in tensor memory and is ordered by the tcgen05 waits and fences around
+// it; a releasing arrive at cluster scope takes most of a microsecond (a unit
+// of 256 x 32 took 1.5 us with it and 0.7 us without).
+__device__ __forceinline__ void arrive_leader(uint64_t* bar) {
+  uint32_t remote;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(tc::smem_u32(bar)));
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+}
+__device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.relaxed.cta.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok) : "r"(tc::smem_u32(bar)), "r"(parity) : "memory");
+  return ok != 0;
+}
+// Wait for MMAs, tensor-memory hand-overs or free stages; data that was copied
+// to shared memory is waited for with tc::mbar_wait (acquire).
+__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) {
+  if (try_wait(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!try_wait(bar, parity))
+    if (clock64() - t0 > kWaitLimit) return false;
+  return true;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// True in one lane of a converged warp. The loops that issue copies and MMAs run
+// in the whole warp with the issue itself under elect: their operands then stay
+// in uniform registers (under a divergent branch an MMA took ~75 clocks to
+// issue).
+__device__ __forceinline__ bool elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                   tc::smem_u32(dst)), "l"(src), "r"(bytes), "r"(tc::smem_u32(bar)) : "memory");
+}
+// Eight 32-bit columns of this lane's row.
+__device__ __forceinline__ void st_row8(uint32_t t, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(t), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
+// Sixteen columns of this lane's row; the values are there after ld_wait().
+__device__ __forceinline__ void ld16(uint32_t t, float* v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+      : "r"(t));
+}
+__device__ __forceinline__ void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Keeps the uses of v behind the wait above (no instruction).
+__device__ __forceinline__ void ld_done(float* v) {
+  asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                    "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]),
+                    "+f"(v[15]));
+}
+__device__ __forceinline__ void st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+__device__ __forceinline__ uint32_t pack(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// (x0, x1) -> packed parts; the differences are exact in FP32.
+template <int PARTS>
+__device__ __forceinline__ void split2(float x0, float x1, uint32_t* p) {
+  p[0] = pack(x0, x1);
+  const float r0 = x0 - __uint_as_float(p[0] << 16), r1 = x1 - __uint_as_float(p[0] & 0xFFFF0000u);
+  p[1] = pack(r0, r1);
+  if (PARTS == 3) p[2] = pack(r0 - __uint_as_float(p[1] << 16), r1 - __uint_as_float(p[1] & 0xFFFF0000u));
+}
+
+template <bool TRANS, int PARTS, bool TMA>
+__global__ void __launch_bounds__(kThreads, 1)
+split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int nh = a.npad / CG;                                  // X columns held by this CTA
+  const uint32_t part_bytes = (uint32_t)nh * BK * 2, stage_bytes = PARTS * part_bytes;
+  unsigned char* fstage = smem;                                // FP32 stages of A, then X stages (both 1 KB aligned)
+  unsigned char* xstage = smem + (size_t)a.sf * kABytes;
+  uint64_t* xfull = reinterpret_cast<uint64_t*>(xstage + (size_t)a.sx * stage_bytes);
+  uint64_t* xempty = xfull + kMaxStages;
+  uint64_t* ffull = xempty + kMaxStages;
+  uint64_t* fempty = ffull + kMaxStages;
+  uint64_t* afull = fempty + kMaxStages;
+  uint64_t* aempty = afull + kMaxASlots;
+  uint64_t* accf = aempty + kMaxASlots;
+  uint64_t* acce = accf + 2;
+  uint64_t* corre = acce + 2;
+  uint64_t* done = corre + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+  int* last = reinterpret_cast<int*>(tmem_slot + 1);
+  int* nslots = last + 1;
+  int* slots = nslots + 1;
+
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
+  const int grp = (int)blockIdx.x / CG, rank = (int)blockIdx.x % CG;
+  const int KB = a.kb;
+  const int u0 = first_unit(grp, a.units, a.G, a.whole, a.tiles, KB);
+  const int u1 = first_unit(grp + 1, a.units, a.G, a.whole, a.tiles, KB);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *a.next0 = 0;
+    *a.next1 = 0;
+  }
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < a.sx; ++s) {
+      tc::mbar_init(&xfull[s], 1);
+      tc::mbar_init(&xempty[s], 1);
+    }
+    for (int s = 0; s < a.sf; ++s) {
+      tc::mbar_init(&ffull[s], 1);
+      tc::mbar_init(&fempty[s], 4);
+    }
+    for (int s = 0; s < a.sa; ++s) {
+      tc::mbar_init(&afull[s], 4 * CG);
+      tc::mbar_init(&aempty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&accf[b], 1);
+      tc::mbar_init(&acce[b], 8 * CG);
+    }
+    tc::mbar_init(corre, 8 * CG);
+    tc::mbar_init(done, 1);
+    tc::fence_barrier_init();
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(tc::smem_u32(tmem_slot))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  cluster_sync();   // the peer's barriers are initialised
+  tc::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  // Tensor memory: main accumulator buffers, the correction accumulator, A
+  // slots (slot s, part p: + (s PARTS + p) 16 columns).
+  const uint32_t corr_base = tmem + (uint32_t)(a.nbuf * a.npad);
+  const uint32_t a_base = corr_base + (a.corr ? (uint32_t)a.npad : 0u);
+  const uint32_t smem_x = tc::smem_u32(xstage);
+  const int nx = (*a.xlo) ? PARTS : 1;                          // X may be exact in its first part
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");   // 48 + 2 x 64 + 2 x 152 = 5 x 96
+    if (warp == 0) {
+      // ------------------------------------------------ X stages
+      const size_t img_stage = (size_t)CG * stage_bytes;
+      const unsigned char* img = reinterpret_cast<const unsigned char*>(a.img) + (size_t)rank * stage_bytes;
+      bool ok = true;
+      Ring r;
+      int n = u1 - u0, k = u0 % KB;
+      for (int i = 0; i < n; ++i) {
+        if (!wait(&xempty[r.s], r.ph ^ 1u)) {
+          ok = false;
+          n = i;
+          break;
+        }
+        if (elect()) {
+          tc::mbar_expect_tx(&xfull[r.s], (uint32_t)nx * part_bytes);
+          bulk_copy(xstage + (size_t)r.s * stage_bytes, img + (size_t)k * img_stage, (uint32_t)nx * part_bytes,
+                    &xfull[r.s]);
+        }
+        k = k + 1 == KB ? 0 : k + 1;
+        r.next(a.sx);
+      }
+      if (!ok) post_timeout(a.info);
+      for (int i = max(0, n - a.sx); i < n; ++i)   // no copy in flight at exit
+        if (!tc::mbar_wait(&xfull[i % a.sx], (uint32_t)((i / a.sx) & 1), kWaitLimit)) post_timeout(a.info);
+    } else if (warp == 1) {
+      // ------------------------------------------------ MMAs (the pair's leader)
+      bool ok = true;
+      if (rank == 0) {
+        Ring rx, ra, rb;      // X stages, A slots, main accumulators
+        int k = u0 % KB, left = u1 - u0, chain = 0;   // chain: main chains of this tile part
+        uint32_t cph = 0;     // parity of the correction chains
+        while (left > 0 && ok) {
+          const int n = min(min(left, KB - k), a.chunk);
+          const bool cnew = a.corr != 0 && chain % a.corr == 0;   // a correction chain begins
+          if (!wait(&acce[rb.s], rb.ph ^ 1u) || (cnew && !wait(corre, cph ^ 1u))) {
+            ok = false;
+            break;
+          }
+          tc::tc_fence_after();
+          const uint32_t d = tmem + (uint32_t)(rb.s * a.npad), dc = a.corr ? corr_base : d;
+          uint32_t acc = 0, cacc = cnew ? 0u : 1u;   // (with one accumulator the main product comes first)
+          for (int i = 0; i < n; ++i) {
+            if (!tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit) || !wait(&afull[ra.s], ra.ph)) {
+              ok = false;
+              break;
+            }
+            tc::tc_fence_after();
+            if (elect()) {
+              // Descriptors of the stage's parts; 16 of K are 32 bytes on.
+              uint64_t x[PARTS];
+#pragma unroll
+              for (int p = 0; p < PARTS; ++p)
+                x[p] = tc::smem_desc(smem_x + (uint32_t)rx.s * stage_bytes + p * part_bytes, 16, 512, tc::kSwizzle64);
+              const uint32_t t0 = a_base + (uint32_t)(ra.s * PARTS * 16);
+              if (PARTS == 3 && a.corr_first) {   // a chain of one unit: the small products, then the main ones
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                  const uint32_t t = t0 + ks * 8;
+                  mma_ts(d, t + 32, x[0] + 2 * ks, a.idesc, ks);
+                  if (nx > 1) {
+                    mma_ts(d, t + 16, x[1] + 2 * ks, a.idesc, 1u);
+                    mma_ts(d, t, x[PARTS - 1] + 2 * ks, a.idesc, 1u);
+                    mma_ts(d, t, x[1] + 2 * ks, a.idesc, 1u);
+                  }
+                  mma_ts(d, t + 16, x[0] + 2 * ks, a.idesc, 1u);
+                }
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) mma_ts(d, t0 + ks * 8, x[0] + 2 * ks, a.idesc, 1u);
+              } else {
+#pragma unroll
+                for (int ks = 0; ks < 2; ++ks) {
+                  const uint32_t t = t0 + ks * 8;
+                  mma_ts(d, t, x[0] + 2 * ks, a.idesc, ks ? 1u : acc);
+                  mma_ts(dc, t + 16, x[0] + 2 * ks, a.idesc, ks ? 1u : cacc);
+                  if (nx > 1) mma_ts(dc, t, x[1] + 2 * ks, a.idesc, 1u);
+                  if (PARTS == 3) {
+                    mma_ts(dc, t + 32, x[0] + 2 * ks, a.idesc, 1u);
+                    if (nx > 1) {
+                      mma_ts(dc, t + 16, x[1] + 2 * ks, a.idesc, 1u);
+                      mma_ts(dc, t, x[PARTS - 1] + 2 * ks, a.idesc, 1u);
+                    }
+                  }
+                }
+              }
+              commit(&xempty[rx.s]);
+              commit(&aempty[ra.s]);
+            }
+            acc = cacc = 1;
+            rx.next(a.sx);
+            ra.next(a.sa);
+          }
+          if (!ok) break;
+          if (elect()) commit(&accf[rb.s]);
+          rb.next(a.nbuf);
+          ++chain;
+          k += n;
+          left -= n;
+          if (a.corr && (chain % a.corr == 0 || k == KB || left == 0)) cph ^= 1u;
+          if (k == KB) k = chain = 0;
+        }
+        if (elect()) commit(done);   // no MMA in flight at teardown
+      }
+      if (!ok) post_timeout(a.info);
+      if (!wait(done, 0)) post_timeout(a.info);
+    }
+    else if (TMA && warp == 3) {
+      // ------------------------------------------------ FP32 tiles of A
+      bool ok = true;
+      Ring r;
+      Cursor c(u0, KB);
+      int n = u1 - u0;
+      for (int i = 0; i < n; ++i) {
+        if (!wait(&fempty[r.s], r.ph ^ 1u)) {
+          ok = false;
+          n = i;
+          break;
+        }
+        if (elect()) {
+          tc::mbar_expect_tx(&ffull[r.s], kABytes);
+          const int row = (c.t * CG + rank) * BM, k = c.k * BK;   // both multiples of four floats
+          tc::tma_load_2d(fstage + r.s * kABytes, &tmA, &ffull[r.s], TRANS ? row : k, TRANS ? k : row);
+        }
+        c.next(KB);
+        r.next(a.sf);
+      }
+      if (!ok) post_timeout(a.info);
+      for (int i = max(0, n - a.sf); i < n; ++i)
+        if (!tc::mbar_wait(&ffull[i % a.sf], (uint32_t)((i / a.sf) & 1), kWaitLimit)) post_timeout(a.info);
+    }
+  } else if (warp < 12) {
+    // -------------------------------------------------- A: load, split, store to tensor memory
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    const int w = warp & 3, odd = (warp >> 2) - 1;   // two warpgroups take the units by turns
+    const bool check = PARTS == 3 && a.bad != nullptr, sq = a.sumsq != nullptr;
+    uint32_t umax = 0, umin = 0xFFFFFFFFu;
+    float ss = 0.f, comp = 0.f, acc2 = 0.f;
+    // A stage holds 128 rows of op(A) by 32 of K. TRANS: as in memory, [K][row];
+    // else [row][K] with the 16-byte chunks of a row xored with row % 8 (the
+    // 128-byte swizzle). v[j] = op(A)(this lane's row, 16 half + j): both reads
+    // are free of bank conflicts.
+    auto read = [&](const unsigned char* f, int half, float* v) {
+      if (TRANS) {
+        const float* p = reinterpret_cast<const float*>(f) + (16 * half) * BM + 32 * w + lane;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = p[j * BM];
+      } else {
+        const unsigned char* p = f + (32 * w + lane) * (BK * 4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 q = *reinterpret_cast<const float4*>(p + (((4 * half + i) ^ (lane & 7)) << 4));
+          v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+        }
+      }
+    };
+    // Without TMA (rows of A that are not 16-byte aligned): this warp's 32 rows
+    // of a stage by 4-byte asynchronous copies, 128 consecutive bytes each.
+    auto copy = [&](const Cursor& c, unsigned char* f) {
+      const int k0 = c.k * BK, r0 = (c.t * CG + rank) * BM + 32 * w;
+      float* s = reinterpret_cast<float*>(f);
+      const int last_i = TRANS ? a.K - k0 : a.M - r0;                 // valid rows of memory
+      const bool in = lane < (TRANS ? a.M - r0 : a.K - k0);
+      const float* p = a.A + (TRANS ? (long long)k0 * a.lda + r0 : (long long)r0 * a.lda + k0) + lane;
+#pragma unroll 8
+      for (int i = 0; i < 32; ++i) {
+        float* d = TRANS ? s + i * BM + 32 * w + lane
+                         : s + (32 * w + i) * BK + (((lane >> 2) ^ (i & 7)) << 2) + (lane & 3);
+        const bool ok = in && i < last_i;
+        cp_async4(d, ok ? p + (long long)i * a.lda : a.A, ok ? 4 : 0);
+      }
+    };
+    // One line of A per lane into L2.
+    auto prefetch = [&](const Cursor& c) {
+      const int k0 = c.k * BK, r0 = (c.t * CG + rank) * BM + 32 * w;
+      const int row = TRANS ? k0 + lane : r0 + lane, col = TRANS ? r0 : k0;
+      if (row < (TRANS ? a.K : a.M) && col < (TRANS ? a.M : a.K))
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.A + (long long)row * a.lda + col));
+    };
+    auto split = [&](const float* v, uint32_t (&o)[PARTS][8]) {
+      if (check) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          const uint32_t x = __float_as_uint(v[j]) & 0x7FFFFFFFu;
+          umax = max(umax, x);
+          umin = min(umin, x - 1u);   // zero wraps to the largest value
+        }
+      }
+      if (sq) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc2 = fmaf(v[j], v[j], acc2);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint32_t p[PARTS];
+        split2<PARTS>(v[2 * j], v[2 * j + 1], p);
+#pragma unroll
+        for (int q = 0; q < PARTS; ++q) o[q][j] = p[q];
+      }
+    };
+    const uint32_t lanes = (uint32_t)(32 * w) << 16;
+    bool ok = true;
+    const int n = u1 - u0;
+    Cursor cc(u0, KB), cp(u0, KB);   // next unit to copy, to prefetch (without TMA)
+    Ring ra, rx, rf;                 // A slot, X stage, FP32 stage of the current unit
+    int fc = odd;                    // FP32 stage of the next copy
+    auto two = [&](Cursor& c) {      // this warpgroup's next unit
+      c.next(KB);
+      c.next(KB);
+    };
+    if (odd) {
+      cc.next(KB);
+      cp.next(KB);
+      ra.next(a.sa);
+      rx.next(a.sx);
+      rf.next(a.sf);
+    }
+    constexpr int kAhead = kCopyStages / 2 - 1;   // own units copied ahead
+    if (!TMA) {
+      for (int i = 0; i < kAhead; ++i) {
+        if (odd + 2 * i < n) copy(cc, fstage + fc * kABytes);
+        cp_async_commit();
+        two(cc);
+        fc += 2;
+      }
+      for (int i = odd; i < odd + kPrefetch; i += 2) {
+        if (i >= 2 * kAhead && i < n) prefetch(cp);
+        two(cp);
+      }
+    }
+    for (int i = odd; i < n; i += 2) {
+      const unsigned char* f = fstage + rf.s * kABytes;
+      if (TMA) {
+        if (!tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit)) {
+          ok = false;
+          break;
+        }
+      } else {
+        if (i + kPrefetch < n) prefetch(cp);
+        two(cp);
+        __syncwarp();   // every lane has read the stage that is filled next
+        if (i + 2 * kAhead < n) copy(cc, fstage + fc * kABytes);
+        cp_async_commit();
+        two(cc);
+        fc = fc + 2 >= kCopyStages ? fc + 2 - kCopyStages : fc + 2;
+        cp_async_wait<kAhead>();
+        __syncwarp();
+      }
+      float v[16];
+      uint32_t o[PARTS][8];
+      read(f, 0, v);
+      split(v, o);
+      if (!wait(&aempty[ra.s], ra.ph ^ 1u)) {
+        ok = false;
+        break;
+      }
+      tc::tc_fence_after();
+      const uint32_t ta = a_base + lanes + (uint32_t)(ra.s * PARTS * 16);
+#pragma unroll
+      for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
+      read(f, 1, v);
+      split(v, o);
+#pragma unroll
+      for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
+      if (sq) {
+        const float y = acc2 - comp, t = ss + y;
+        comp = (t - ss) - y;
+        ss = t;
+        acc2 = 0.f;
+      }
+      st_wait();
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (TMA) tc::mbar_arrive(&fempty[rf.s]);
+        // The pair's leader learns of the peer's X stage through the peer's A.
+        if (rank != 0 && !tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit)) ok = false;
+        arrive_leader(&afull[ra.s]);
+      }
+      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      if (!ok) break;
+      ra.next(a.sa);
+      ra.next(a.sa);
+      rx.next(a.sx);
+      rx.next(a.sx);
+      rf.next(a.sf);
+      rf.next(a.sf);
+    }
+    if (!TMA) cp_async_wait_all();
+    if (!ok && lane == 0) post_timeout(a.info);
+    if (check && __any_sync(0xffffffffu, umax >= kRangeHi || umin < kRangeLo - 1u) && lane == 0) atomicOr(a.bad, 1);
+    if (sq) {
+      double v = (double)ss - (double)comp;
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if (lane == 0) atomicAdd(a.sumsq, v);
+    }
+  } else {
+    // -------------------------------------------------- drain: TMEM -> registers -> global
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
+    const int e = warp - 12, half = e >> 2, tid = threadIdx.x - 384;
+    const int row = 32 * (e & 3) + lane;
+    const int groups = a.npad / 16, g0 = half ? (groups + 1) / 2 : 0, ng = half ? groups / 2 : (groups + 1) / 2;
+    float s[kGroups][16];
+    auto clear = [&] {
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g)
+#pragma unroll
+        for (int j = 0; j < 16; ++j) s[g][j] = 0.f;
+    };
+    clear();
+    bool ok = true;   // after a timeout the loop runs on without waiting, so that its barriers stay in step
+    int chain = 0, k = u0 % KB, t = u0 / KB, left = u1 - u0, part0 = k;   // part0: first unit of this tile part
+    int since = 0;
+    bool flushed = false;   // earlier sums of this part are in memory
+    Ring rb;
+    while (left > 0) {
+      const int n = min(min(left, KB - k), a.chunk);
+      const bool part_end = n == left || k + n == KB;
+      if (ok && !wait(&accf[rb.s], rb.ph)) {
+        ok = false;
+        if (lane == 0) post_timeout(a.info);
+      }
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        tc::tc_fence_after();
+        const uint32_t lanes = (uint32_t)(32 * (e & 3)) << 16, cols = (uint32_t)(16 * g0);
+        auto drain = [&](uint32_t ta) {
+#pragma unroll
+          for (int g = 0; g < kGroups; ++g) {
+            if (g < ng) {
+              float v[16];
+              ld16(ta + 16 * g, v);
+              ld_wait();
+              ld_done(v);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) s[g][j] += v[j];
+            }
+          }
+          tc::tc_fence_before();
+          __syncwarp();
+        };
+        drain(tmem + lanes + (uint32_t)(rb.s * a.npad) + cols);
+        if (lane == 0) arrive_leader(&acce[rb.s]);
+        if (a.corr && ((chain + 1) % a.corr == 0 || part_end)) {
+          drain(corr_base + lanes + cols);
+          if (lane == 0) arrive_leader(corre);
+        }
+      }
+      rb.next(a.nbuf);
+      ++chain;
+      k += n;
+      left -= n;
+      since += n;
+      if (!part_end && since < a.flush) continue;
+      // End of this CTA's part of tile t (or a flush on the way).
+      const int rt = t * CG + rank;                   // 128-row tile
+      const long long gm = (long long)rt * BM + row;
+      const bool all = part0 == 0 && (k == KB || left + k >= KB), first_part = t == u0 / KB;
+      float* dst;
+      int ncols, qstep = 4;   // floats from one float4 of the row to the next
+      bool vec;
+      if (all) {
+        dst = a.out + gm * a.ldo;
+        ncols = gm < a.M ? a.N : 0;
+        vec = a.vec_out != 0;
+      } else {
+        const int slot = first_part ? 2 * grp : 2 * grp + 1;   // first or last tile of the range
+        dst = a.part + (long long)(slot * CG + rank) * BM * a.npad + row * 4;   // [npad / 4][128 rows][4]
+        ncols = a.npad;
+        qstep = 4 * BM;
+        vec = true;
+      }
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g) {
+        const int c0 = 16 * (g0 + g);
+        if (g < ng) {
+          if (flushed) {
+            if (vec && c0 + 16 <= ncols) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const float4 o = *reinterpret_cast<const float4*>(dst + (c0 / 4 + q) * qstep);
+                s[g][4 * q] += o.x; s[g][4 * q + 1] += o.y; s[g][4 * q + 2] += o.z; s[g][4 * q + 3] += o.w;
+              }
+            } else {
+#pragma unroll
+              for (int j = 0; j < 16; ++j)
+                if (c0 + j < ncols) s[g][j] += dst[c0 + j];
+            }
+          }
+          if (vec && c0 + 16 <= ncols) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              *reinterpret_cast<float4*>(dst + (c0 / 4 + q) * qstep) =
+                  make_float4(s[g][4 * q], s[g][4 * q + 1], s[g][4 * q + 2], s[g][4 * q + 3]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              if (c0 + j < ncols) dst[c0 + j] = s[g][j];
+          }
+        }
+      }
+      if (part_end && !all && !a.fixup) {
+        // Publish the partial tile; the last CTA to arrive sums them in CTA order.
+        __threadfence();
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (tid == 0) {
+          const int ub = t * KB, ue = ub + KB;
+          const int clo = unit_owner(ub, a.units, a.G), chi = unit_owner(ue - 1, a.units, a.G);
+          int n = 0;
+          for (int c = clo; c <= chi; ++c) {
+            const int cb = first_unit(c, a.units, a.G, 0, a.tiles, KB);
+            if (cb == first_unit(c + 1, a.units, a.G, 0, a.tiles, KB)) continue;
+            if (n < kMaxSlots) slots[n] = ((cb / KB == t) ? 2 * c : 2 * c + 1) * CG + rank;
+            ++n;
+          }
+          const int old = atomicAdd(&a.cnt[rt], 1);
+          *last = old == n - 1 ? 1 : 0;
+          *nslots = min(n, kMaxSlots);
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        if (*last) {
+          __threadfence();
+          // Thread: row lane % 8 of two row groups, float4 lane / 8 of every
+          // four (128-byte reads, 64-byte writes); two slots times eight float4
+          // in flight, as the loads' latency is the time of this step.
+          const int n = *nslots, Q = a.npad / 4;
+          for (int c0 = lane >> 3; c0 < Q; c0 += 16) {
+            float4 acc[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int z = 0; z < n; z += 2) {
+              float4 v[2][8];
+#pragma unroll
+              for (int y = 0; y < 2; ++y)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  const int r = 8 * (2 * e + (j >> 2)) + (lane & 7), c = c0 + 4 * (j & 3);
+                  const bool in = z + y < n && c < Q;
+                  v[y][j] = in ? __ldcg(reinterpret_cast<const float4*>(
+                                     a.part + (long long)slots[z + y] * BM * a.npad + (c * BM + r) * 4))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+              for (int y = 0; y < 2; ++y)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                  acc[j].x += v[y][j].x; acc[j].y += v[y][j].y; acc[j].z += v[y][j].z; acc[j].w += v[y][j].w;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const int r = 8 * (2 * e + (j >> 2)) + (lane & 7), c = 4 * (c0 + 4 * (j & 3));
+              const long long gr = (long long)rt * BM + r;
+              if (gr >= a.M || c >= a.N) continue;
+              float* o = a.out + gr * a.ldo + c;
+              if (a.vec_out && c + 3 < a.N) {
+                *reinterpret_cast<float4*>(o) = acc[j];
+              } else {
+                const float x[4] = {acc[j].x, acc[j].y, acc[j].z, acc[j].w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                  if (c + q < a.N) o[q] = x[q];
+              }
+            }
+          }
+          if (tid == 0) a.cnt[rt] = 0;
+        }
+      }
+      clear();   // (here, so that the sums are not live across the code above)
+      flushed = !part_end;
+      since = 0;
+      if (part_end) {
+        if (k == KB) ++t;
+        chain = k = part0 = 0;
+      }
+      if (part_end) asm volatile("bar.sync 1, 256;" ::: "memory");   // (slots are read no more)
+    }
+  }
+
+  tc::tc_fence_before();
+  __syncthreads();
+  cluster_sync();   // no remote arrival is still on its way
+  tc::tc_fence_after();
+  if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
+}
+
+// Sums the partial tiles of a product whose tiles span many CTAs: thread f
+// takes float4 f of the tiles that were split, slots in CTA order.
+__global__ void split_fixup_kernel(const Args a) {
+  const int Q = a.npad / 4;
+  const long long per = (long long)BM * Q, total = (long long)a.tiles * CG * per;
+  for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < total;
+       f += (long long)gridDim.x * blockDim.x) {
+    const int rt = (int)(f / per), t = rt / CG, e = (int)(f % per), r = e % BM, c = (e / BM) * 4;
+    const long long gr = (long long)rt * BM + r;
+    if (gr >= a.M || c >= a.N) continue;
+    const int ub = t * a.kb, ue = ub + a.kb;
+    const int clo = unit_owner(ub, a.units, a.G), chi = unit_owner(ue - 1, a.units, a.G);
+    if (clo == chi) continue;   // one group had the whole tile
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int z0 = clo; z0 <= chi; z0 += 8) {
+      float4 v[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int z = z0 + j;
+        if (z > chi) continue;
+        const int cb = first_unit(z, a.units, a.G, 0, a.tiles, a.kb);
+        if (cb == first_unit(z + 1, a.units, a.G, 0, a.tiles, a.kb)) continue;
+        const int slot = ((cb / a.kb == t) ? 2 * z : 2 * z + 1) * CG + rt % CG;
+        v[j] = __ldcg(reinterpret_cast<const float4*>(a.part + (long long)slot * BM * a.npad + (c / 4 * BM + r) * 4));
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w;
+      }
+    }
+    float* o = a.out + gr * a.ldo + c;
+    if (a.vec_out && c + 3 < a.N) {
+      *reinterpret_cast<float4*>(o) = acc;
+    } else {
+      const float x[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (c + q < a.N) o[q] = x[q];
+    }
+  }
+}
+
+// X (K x N FP32) -> stage images: for every unit of 32 of K, CTA of a group,
+// and part, npad / CG rows (columns of X) of 32 K entries, 16-byte chunks
+// swizzled over 64-byte rows; zeros past K and N. A block of 256 threads takes
+// 64 of K and 32 columns through shared memory; a thread writes one 16-byte
+// chunk (8 of K) of each part.
+__global__ void __launch_bounds__(256)
+split_x_kernel(const float* __restrict__ X, long long K, int N, long long ldx, uint16_t* __restrict__ img, int npad,
+               int parts, int kb, int* xlo, int* bad) {
+  __shared__ float tile[64][33];
+  const long long k0 = (long long)blockIdx.x * 64;
+  const int n0 = blockIdx.y * 32;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int kk = (threadIdx.x >> 5) + 8 * i, nn = threadIdx.x & 31;
+    const long long k = k0 + kk;
+    tile[kk][nn] = (k < K && n0 + nn < N) ? X[k * ldx + n0 + nn] : 0.f;
+  }
+  __syncthreads();
+  const int nn = threadIdx.x >> 3, ch = threadIdx.x & 7;   // column, chunk of 8 of K
+  const int n = n0 + nn;
+  const long long unit = (k0 >> 5) + (ch >> 2);
+  bool any = false, out_of_range = false;
+  if (n < npad && unit < kb) {
+    uint32_t p[3][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint32_t q[3];
+      const float x0 = tile[ch * 8 + 2 * j][nn], x1 = tile[ch * 8 + 2 * j + 1][nn];
+      split2<3>(x0, x1, q);
+      p[0][j] = q[0]; p[1][j] = q[1]; p[2][j] = q[2];
+      any |= (q[1] & 0x7FFF7FFFu) != 0;
+      const uint32_t m0 = __float_as_uint(x0) & 0x7FFFFFFFu, m1 = __float_as_uint(x1) & 0x7FFFFFFFu;
+      out_of_range |= max(m0, m1) >= kRangeHi || min(m0 - 1u, m1 - 1u) < kRangeLo - 1u;
+    }
+    const int nh = npad / CG, r = n % nh;
+    const size_t stage = ((size_t)unit * CG + n / nh) * parts * nh * 32;
+    const size_t at = stage + (size_t)r * 32 + (size_t)(((ch & 3) ^ ((r >> 1) & 3)) * 8);
+    for (int q = 0; q < parts; ++q)
+      *reinterpret_cast<uint4*>(img + at + (size_t)q * nh * 32) = make_uint4(p[q][0], p[q][1], p[q][2], p[q][3]);
+  }
+  if (__syncthreads_or(any) && threadIdx.x == 0 && *(volatile int*)xlo == 0) atomicOr(xlo, 1);
+  if (bad != nullptr && __syncthreads_or(out_of_range) && threadIdx.x == 0) atomicOr(bad, 1);
+}
+
+int npad_of(int n) { return (int)round_up(n, 16); }   // N of the MMA; each CTA holds half of it, a multiple of 8
+
+size_t smem_optin() {
+  static size_t v = 0;
+  if (v == 0) {
+    int dev = 0, x = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&x, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess && x > 0)
+      v = (size_t)x;
+    else
+      v = 227 * 1024;
+  }
+  return v;
+}
+constexpr size_t kSmemExtra = 1024 + 1024;   // alignment, barriers
+
+template <bool TRANS, int PARTS, bool TMA>
+cudaError_t launch(const CUtensorMap& map, Args& a, int cap, size_t smem, cudaStream_t st) {
+  static int resident = 0;   // pairs that run at the same time
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CG;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (resident == 0) {
+    CK(cudaFuncSetAttribute(split_gemm_kernel<TRANS, PARTS, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)smem_optin()));
+    int n = 0;
+    cfg.gridDim = dim3((unsigned)(sm_count() / CG * CG));
+    cfg.dynamicSmemBytes = smem_optin();
+    CK(cudaOccupancyMaxActiveClusters(&n, split_gemm_kernel<TRANS, PARTS, TMA>, &cfg));
+    resident = std::max(1, std::min(n, sm_count() / CG));
+  }
+  a.G = std::min(resident, cap);
+  a.fixup = (!a.whole && a.G / a.tiles + 2 > kMaxSlots) ? 1 : 0;
+  cfg.gridDim = dim3((unsigned)(a.G * CG));
+  cfg.dynamicSmemBytes = smem;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, split_gemm_kernel<TRANS, PARTS, TMA>, map, a);
+  note_launch();
+  return e;
+}
+
+using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeFn encode_fn() {
+  static const EncodeFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<EncodeFn>(p);
+  }();
+  return fn;
+}
+// FP32 map over A (rows x cols, row stride lda): boxes of 128 columns x 32 rows
+// (op(A) = A^T), or 32 columns x 128 rows with the 128-byte swizzle. False when
+// the rows are not 16-byte aligned (or the encoder is missing): the kernel
+// variant without TMA takes those.
+bool map_a(CUtensorMap* map, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans) {
+  EncodeFn fn = encode_fn();
+  if (fn == nullptr || reinterpret_cast<uintptr_t>(A) % 16 != 0 || lda % 4 != 0) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)(lda * 4)};
+  cuuint32_t box[2] = {trans ? (cuuint32_t)BM : (cuuint32_t)BK, trans ? (cuuint32_t)BK : (cuuint32_t)BM};
+  cuuint32_t es[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(A), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, trans ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, int64_t K, const float* A, int64_t lda,
+                    const float* X, int64_t ldx, float* out, int64_t ldo, SplitMode mode, double* sumsq, int* bad,
+                    int* info, cudaStream_t st) {
+  const int parts = mode == kSplitTwo ? 2 : 3;
+  const int npad = npad_of(N), kb = (int)cdiv(K, BK);
+  int* w = ws->words;
+  split_x_kernel<<<dim3((unsigned)cdiv(kb, 2), (unsigned)cdiv(npad, 32)), 256, 0, st>>>(
+      X, K, N, ldx, ws->img, npad, parts, kb, w + turn, bad);
+  note_launch();
+  CK(cudaGetLastError());
+
+  Args a = {};
+  a.A = A; a.lda = lda;
+  a.img = ws->img;
+  a.out = out; a.ldo = ldo;
+  a.part = ws->part;
+  a.cnt = ws->cnt;
+  a.xlo = w + turn;
+  a.bad = bad;
+  a.next0 = w + (turn ^ 1);
+  a.next1 = w + 2 + (turn ^ 1);
+  a.sumsq = sumsq;
+  a.info = info;
+  a.M = (int)M; a.N = N; a.K = (int)K; a.npad = npad;
+  a.kb = kb;
+  a.tiles = (int)cdiv(M, (int64_t)BM * CG);
+  if ((long long)a.tiles * kb > (1LL << 30)) return cudaErrorInvalidValue;
+  a.units = a.tiles * kb;
+  // Short K: a split tile would cost more than it saves; whole tiles per CTA.
+  a.whole = kb <= 32 ? 1 : 0;
+  const int cap = a.whole ? a.tiles : a.units;
+  a.vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0 && ldo % 4 == 0) ? 1 : 0;
+  // Chains. An MMA loses about half a unit in the last place of the sum that
+  // it adds to, always toward zero. FP32: one chain per unit, the correction
+  // products (2^-8 of the main ones) first, so that only two MMAs add to a
+  // sum of full size; 64 units are summed in registers, then in memory.
+  // BF16x3: K = 4096, the corrections apart where tensor memory has room (npad
+  // <= 128) or there are three parts.
+  if (mode == kSplitFp32) {
+    a.chunk = 1;
+    a.corr = 0;
+    a.corr_first = 1;
+    a.flush = 64;
+  } else {
+    a.chunk = 4096 / BK;
+    a.corr = parts == 3 || npad <= 128 ? 1 : 0;
+    a.flush = 1 << 30;
+  }
+  // Tensor memory: two main buffers where at least two A slots still fit.
+  const int cc = a.corr != 0 ? npad : 0;
+  a.nbuf = 2 * npad + cc + 2 * parts * 16 <= 512 ? 2 : 1;
+  a.sa = std::min(kMaxASlots, (512 - a.nbuf * npad - cc) / (parts * 16));
+  const size_t stage = (size_t)(npad / CG) * BK * 2 * parts;
+  CUtensorMap map = {};
+  const bool tma = map_a(&map, A, transA ? K : M, transA ? M : K, lda, transA);
+  // Shared memory: four X stages first, then FP32 stages of A, then X again.
+  const size_t avail = smem_optin() - kSmemExtra;
+  a.sf = tma ? (int)std::min<size_t>(kMaxStages, (avail - 4 * stage) / kABytes) : kCopyStages;
+  a.sx = (int)std::min<size_t>(kMaxStages, (avail - a.sf * kABytes) / stage);
+  a.idesc = tc::idesc_bf16(BM * CG, npad, false, false);
+  const size_t smem = a.sf * kABytes + a.sx * stage + kSmemExtra;
+#define RQLP_SPLIT(T, P) (tma ? launch<T, P, true>(map, a, cap, smem, st) : launch<T, P, false>(map, a, cap, smem, st))
+  cudaError_t e = transA ? (parts == 3 ? RQLP_SPLIT(true, 3) : RQLP_SPLIT(true, 2))
+                         : (parts == 3 ? RQLP_SPLIT(false, 3) : RQLP_SPLIT(false, 2));
+#undef RQLP_SPLIT
+  if (e == cudaSuccess && a.fixup) {
+    const long long total = (long long)a.tiles * CG * BM * (npad / 4);
+    const int blocks = (int)std::min<long long>(cdiv(total, 256), (long long)sm_count() * 8);
+    split_fixup_kernel<<<blocks, 256, 0, st>>>(a);
+    note_launch();
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+}  // namespace
+
+void split_gemm_layout(Arena& ar, SplitGemmWs* ws, int64_t m_cap, int64_t k_cap, int n_cap, int parts) {
+  const int npad = npad_of(n_cap);
+  ws->img = ar.take<uint16_t>((size_t)cdiv(k_cap, BK) * BK * npad * parts);
+  ws->slots = 2 * sm_count();
+  ws->part = ar.take<float>((size_t)ws->slots * BM * npad);
+  const size_t words = 4 + (size_t)cdiv(m_cap, 2 * BM) * 2;
+  ws->words_bytes = words * sizeof(int);
+  ws->words = ar.take<int>(words);
+  ws->cnt = ar.dry ? nullptr : ws->words + 4;
+  ws->turn = 0;
+}
+
+cudaError_t split_gemm_reset(SplitGemmWs* ws, cudaStream_t st) {
+  ws->turn = 0;
+  return cudaMemsetAsync(ws->words, 0, ws->words_bytes, st);
+}
+
+cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K, const float* A, int64_t lda,
+                       const float* X, int64_t ldx, float* out, int64_t ldo, SplitMode mode, double* sumsq,
+                       const int** range_word, int* info, bool profiled, cudaStream_t st) {
+  if (M <= 0 || N <= 0 || N > 256 || K <= 0 || M > (int64_t(1) << 30) || K > (int64_t(1) << 30))
+    return cudaErrorInvalidValue;
+  const int turn = ws->turn & 1;
+  ws->turn ^= 1;
+  int* bad = mode == kSplitFp32 ? ws->words + 2 + turn : nullptr;
+  if (range_word != nullptr) *range_word = bad;
+  const int parts = mode == kSplitTwo ? 2 : 3;
+  // Three parts need two accumulators and two A slots (96 columns) of tensor
+  // memory: above 208 columns the product runs as two column halves.
+  const int n0 = npad_of(N) > (parts == 3 ? 208 : 16 * 2 * kGroups) ? npad_of((int)cdiv(N, 2)) : N;
+  const bool prof = profiled && profiling_on();
+  if (prof) profile_mark_begin(st);
+  cudaError_t e = product(ws, turn, transA, M, n0, K, A, lda, X, ldx, out, ldo, mode, sumsq, bad, info, st);
+  if (e == cudaSuccess && n0 < N)
+    e = product(ws, turn, transA, M, N - n0, K, A, lda, X + n0, ldx, out + n0, ldo, mode, nullptr, bad, info, st);
+  if (prof) profile_mark_end(st, transA ? 1 : 0);
+  return e;
+}
+
+}  // namespace rqlp

@@ -1,0 +1,41 @@
+// out = op(A) X on the tensor cores with A read in FP32 and split into BF16
+// parts on its way to tensor memory (see split_gemm.cu).
+#pragma once
+
+#include "common.cuh"
+
+namespace rqlp {
+
+// Scratch of split_gemm for products with K <= k_cap and N <= n_cap, laid out
+// once in the caller's workspace. The words at `words` and the tile counters
+// must be zero before the first product (split_gemm_reset).
+struct SplitGemmWs {
+  uint16_t* img = nullptr;   // X's parts as shared-memory stage images
+  float* part = nullptr;     // partial tiles of split K ranges
+  int* words = nullptr;      // [0..1] X low part nonzero, [2..3] values outside the split's range, by turn
+  int* cnt = nullptr;        // tile arrival counters
+  size_t words_bytes = 0;    // words and counters, one block
+  int slots = 0;             // 128-row partial slots that fit in part
+  int turn = 0;
+};
+// m_cap: largest number of output rows, k_cap: largest K, n_cap: largest N;
+// parts: 2 or 3 (the largest used).
+void split_gemm_layout(Arena& ar, SplitGemmWs* ws, int64_t m_cap, int64_t k_cap, int n_cap, int parts);
+cudaError_t split_gemm_reset(SplitGemmWs* ws, cudaStream_t st);
+
+// kSplitTwo: two parts, three products (BF16x3 form); kSplitThree: three parts,
+// six products, chains as in the BF16x3 form; kSplitFp32: three parts, short
+// chains, FP32 accuracy.
+enum SplitMode { kSplitTwo = 2, kSplitThree = 3, kSplitFp32 = 4 };
+
+// transA: out (M x N) = A^T X with A K x M; else out = A X with A M x K; X is
+// K x N (N <= 256), all row-major FP32. sumsq (optional) += sum of squares of
+// A. *range_word (optional) receives the device word that a kSplitFp32 product
+// raises when a value of A or X lies outside the range that the parts
+// represent: the result then has to be recomputed in FP32, gated on that word
+// (before the next product but one clears it). Null in the other modes.
+cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K, const float* A, int64_t lda,
+                       const float* X, int64_t ldx, float* out, int64_t ldo, SplitMode mode, double* sumsq,
+                       const int** range_word, int* info, bool profiled, cudaStream_t st);
+
+}  // namespace rqlp
