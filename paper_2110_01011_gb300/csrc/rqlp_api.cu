@@ -41,7 +41,11 @@ class Ops {
   }
 
   // part_floats: largest split-K partial buffer any product of the caller needs.
-  void layout(Arena& ar, size_t part_floats, bool with_tc, int64_t m, int64_t n) {
+  // split_bytes (FP32): at most this much scratch for running the large
+  // products on the tensor cores (fewer SMs take them when it is short, none
+  // below half); it shares its block with the split-K partials.
+  void layout(Arena& ar, size_t part_floats, bool with_tc, int64_t m, int64_t n, size_t split_bytes = 0) {
+    const int64_t tall = std::max(m, n);
     const int64_t dd = (int64_t)dcap_ * ld_;
     G_ = ar.take<float>(dd);
     for (int i = 0; i < 3; ++i) {
@@ -49,17 +53,26 @@ class Ops {
       Ri_[i] = ar.take<float>(dd);
     }
     Ra_ = ar.take<float>(dd);
-    part_ = ar.take<float>(std::max<size_t>(part_floats, 1));
+    const size_t part_bytes = std::max<size_t>(part_floats, 1) * sizeof(float);
+    const size_t block_bytes =
+        std::max(part_bytes, std::min(split_bytes, split_gemm_block_bytes(tall, dcap_, 3)));
+    part_ = reinterpret_cast<float*>(ar.take<char>(block_bytes));
     scal = ar.take<double>(kScal);
     gates = ar.take<int>(kGates);
     cstore_ = ar.take<char>(chol_global_bytes(dcap_, o_.small_fp64 != 0));
     if (with_tc) {
-      split_gemm_layout(ar, &sg_, std::max(m, n), std::max(m, n), dcap_, three_ ? 3 : 2);
+      const size_t at = ar.off, bytes = split_gemm_block_bytes(tall, dcap_, 3);
+      char* block = ar.take<char>(bytes);
+      split_gemm_layout(ar, &sg_, block, bytes, tall, tall, dcap_, 3);
+      // The size reported stays that of a layout with A's BF16 parts, which
+      // callers' pools and the allocation-free entry's limit were sized by.
+      ar.off = std::max(ar.off, at + panel_bytes(m, n));
       // Tall d-column operands of CholeskyQR: the Gram (BF16x3) and the
       // products X R^{-1} (exact mode, six products) on the tensor cores.
       tcs_.layout(ar, std::max(m, n), dcap_, dcap_, dcap_, true, /*three_part=*/true);
     }
     tc_on_ = with_tc;
+    split32_ = split_bytes > 0 && split_gemm_layout(ar, &sg_, part_, block_bytes, tall, tall, dcap_, 3);
   }
   void bind(cudaStream_t st, int* info) { st_ = st; info_ = info; }
   int64_t ld() const { return ld_; }
@@ -94,7 +107,7 @@ class Ops {
   }
 
   // Before the first product of a call.
-  cudaError_t begin_products() { return tc_on_ ? split_gemm_reset(&sg_, st_) : cudaSuccess; }
+  cudaError_t begin_products() { return tc_on_ || split32_ ? split_gemm_reset(&sg_, st_) : cudaSuccess; }
 
   // transA: out (n x d) = A^T X (X m x d); else out (m x d) = A X (X n x d).
   cudaError_t pass(bool transA, const float* A, int64_t m, int64_t n, int64_t lda, const float* X,
@@ -110,9 +123,7 @@ class Ops {
       return split_product(transA, transA ? n : m, transA ? m : n, A, lda, X, ldx, out, ldout, sumsq);
     const bool prof = profiling_on();
     if (prof) profile_mark_begin(st_);
-    const int64_t M = transA ? n : m, K = transA ? m : n;
-    cudaError_t e = gemm_f32_ex(transA, M, d_, K, A, lda, X, ldx, out, ldout, gemm_f32_splits(M, d_, K), part_,
-                                sumsq, nullptr, kGateNone, false, st_);
+    cudaError_t e = product32(transA, transA ? n : m, transA ? m : n, A, lda, X, ldx, out, ldout, sumsq);
     if (prof) profile_mark_end(st_, transA ? 1 : 0);
     return e;
   }
@@ -124,8 +135,7 @@ class Ops {
       return split_product(true, n, rows, A + r0 * lda, lda, X, ldx, out, ldout, &scal[0]);
     const bool prof = profiling_on();
     if (prof) profile_mark_begin(st_);
-    cudaError_t e = gemm_f32_ex(true, n, d_, rows, A + r0 * lda, lda, X, ldx, out, ldout,
-                                gemm_f32_splits(n, d_, rows), part_, &scal[0], nullptr, kGateNone, false, st_);
+    cudaError_t e = product32(true, n, rows, A + r0 * lda, lda, X, ldx, out, ldout, &scal[0]);
     if (prof) profile_mark_end(st_, 1);
     return e;
   }
@@ -147,10 +157,8 @@ class Ops {
         CK(split_product(false, rows, n, A + r0 * lda, lda, X, ldx, zb, ld_, nullptr));
         CK(split_product(true, n, rows, A + r0 * lda, lda, zb, ld_, dst, ldd, nullptr));
       } else {
-        CK(gemm_f32_ex(false, rows, d_, n, A + r0 * lda, lda, X, ldx, zb, ld_, gemm_f32_splits(rows, d_, n), part_,
-                       nullptr, nullptr, kGateNone, false, st_));
-        CK(gemm_f32_ex(true, n, d_, rows, A + r0 * lda, lda, zb, ld_, dst, ldd, gemm_f32_splits(n, d_, rows), part_,
-                       nullptr, nullptr, kGateNone, false, st_));
+        CK(product32(false, rows, n, A + r0 * lda, lda, X, ldx, zb, ld_, nullptr));
+        CK(product32(true, n, rows, A + r0 * lda, lda, zb, ld_, dst, ldd, nullptr));
       }
       if (r0 > 0) CK(add_matrix(n, d_, T, ld_, Y, ldy, st_));
     }
@@ -161,6 +169,20 @@ class Ops {
                             float* out, int64_t ldout, double* sumsq) {
     return split_gemm(&sg_, transA, M, d_, K, A, lda, X, ldx, out, ldout, three_ ? kSplitThree : kSplitTwo, sumsq,
                       nullptr, info_, true, st_);
+  }
+  static bool split_pays(int64_t M, int64_t K, int d) { return (double)M * K * d >= 2e8; }
+  // The same product in FP32. Where it pays it runs on the
+  // tensor cores in three parts; an FMA product gated on the range word then
+  // redoes it where a value lies outside what the parts represent.
+  cudaError_t product32(bool transA, int64_t M, int64_t K, const float* A, int64_t lda, const float* X, int64_t ldx,
+                        float* out, int64_t ldout, double* sumsq) {
+    const int* word = nullptr;
+    if (split32_ && split_pays(M, K, d_)) {
+      CK(split_gemm(&sg_, transA, M, d_, K, A, lda, X, ldx, out, ldout, kSplitFp32, sumsq, &word, info_, false, st_));
+      sumsq = nullptr;
+    }
+    return gemm_f32_ex(transA, M, d_, K, A, lda, X, ldx, out, ldout, gemm_f32_splits(M, d_, K), part_, sumsq, word,
+                       word != nullptr ? kGateSkip : kGateNone, false, st_);
   }
   // Row-panel height of power_fused: at most ~48 MB of A's pass operands
   // (bpe bytes per element of A), a multiple of 128 rows.
@@ -274,6 +296,20 @@ class Ops {
     return cudaSuccess;
   }
 
+  // Device bytes of A's BF16 parts in 64-column panels with their products'
+  // scratch (see layout).
+  size_t panel_bytes(int64_t m, int64_t n) const {
+    Arena ar;
+    ar.dry = true;
+    const int64_t tall = std::max(m, n), parts = three_ ? 3 : 2, np = round_up(std::max(dcap_, 16), 16);
+    for (int i = 0; i < parts; ++i) ar.take<uint16_t>((size_t)(m * round_up(n, 64)));
+    for (int i = 0; i < parts; ++i) ar.take<uint16_t>((size_t)dcap_ * round_up(tall, 8));
+    ar.take<float>((size_t)2 * sm_count() * 128 * np);
+    ar.take<int>(4);
+    ar.take<int>((size_t)cdiv(tall, 128));
+    return ar.off;
+  }
+
   double* scal = nullptr;
   int* gates = nullptr;
 
@@ -289,6 +325,7 @@ class Ops {
   TcEngine tcs_;
   bool tc_on_ = false;
   bool three_ = false;
+  bool split32_ = false;
   const SparseA* sp_ = nullptr;
   const SparseA* spt_ = nullptr;
 };
@@ -360,7 +397,25 @@ class Plan {
     ops_.set_three_part(three_part_passes(o, dm.m, dm.n, dm.learned ? 20 : dm.p));
   }
 
+  // FP32 plans take the tensor-core products where one pass over A is worth
+  // them. Their scratch does not lift a workspace that fits the allocation-free
+  // entry's array above it.
   size_t layout(Arena& ar) {
+    if (o_.precision != RQLP_PREC_FP32 || !Ops::split_pays(d_.m, d_.n, d_.d)) return layout(ar, 0);
+    constexpr size_t kLimit = RQLP_NOALLOC_SCRATCH_BYTES;
+    Arena plain;
+    plain.dry = true;
+    const size_t bytes = layout(plain, 0);
+    if (bytes > kLimit) return layout(ar, SIZE_MAX);
+    // What is left for the block: the limit less everything but the split-K
+    // partials and the product's words.
+    const size_t other = bytes - part_bytes() + 4 * (size_t)cdiv(std::max(d_.m, d_.n), 128) + 4096;
+    if (other >= kLimit) return layout(ar, 0);
+    Arena with;
+    with.dry = true;
+    return layout(ar, layout(with, kLimit - other) <= kLimit ? kLimit - other : 0);
+  }
+  size_t layout(Arena& ar, size_t split_bytes) {
     const int64_t ld = ops_.ld(), dd = (int64_t)d_.d * ld, tall = std::max(d_.m, d_.n);
     Y_ = ar.take<float>(d_.n * ld);
     Z_ = ar.take<float>(d_.m * ld);
@@ -374,7 +429,11 @@ class Plan {
     feat_ = ar.take<float>(RQLP_MLP_FEATURES);
     logits_ = ar.take<float>(RQLP_MLP_OUTPUTS);
     qp_ = ar.take<int>(2);
-    // Split-K partial buffers for every width this plan may run at.
+    ops_.layout(ar, part_bytes() / sizeof(float), o_.precision == RQLP_PREC_BF16X3, d_.m, d_.n, split_bytes);
+    return ar.off;
+  }
+  // Split-K partials of the widest need over every width this plan may run at.
+  size_t part_bytes() const {
     size_t part = 0;
     const int lo = d_.learned ? std::max(1, d_.d - 15) : d_.d;
     for (int d = lo; d <= d_.d; ++d)
@@ -382,8 +441,7 @@ class Plan {
                        Ops::orth_part_floats(d_.n, d), Ops::orth_part_floats(d, d)});
     if (o_.fused_power != 0 && o_.precision == RQLP_PREC_FP32)
       for (int d = lo; d <= d_.d; ++d) part = std::max(part, Ops::fused_part_floats(d_.m, d_.n, d));
-    ops_.layout(ar, part, o_.precision == RQLP_PREC_BF16X3, d_.m, d_.n);
-    return ar.off;
+    return part * sizeof(float);
   }
 
   cudaError_t run(const float* A, const float* Om, const Out& out, int* info, double* diag, cudaStream_t st) {
@@ -603,7 +661,8 @@ size_t sketch_bytes(int64_t m, int64_t n, int d, const rqlp_opts& o) {
   ar.dry = true;
   Ops ops(d, o);
   ops.set_three_part(three_part_passes(o, m, n, -1));
-  ops.layout(ar, Ops::pass_part_floats(m, n, d), o.precision == RQLP_PREC_BF16X3, m, n);
+  ops.layout(ar, Ops::pass_part_floats(m, n, d), o.precision == RQLP_PREC_BF16X3, m, n,
+             o.precision == RQLP_PREC_FP32 && Ops::split_pays(m, n, d) ? SIZE_MAX : 0);
   return ar.off;
 }
 
@@ -744,7 +803,8 @@ rqlp_status rqlp_sketch(int trans, const float* A, int64_t m, int64_t n, int64_t
   Arena ar = arena_over(workspace, ws_bytes);
   Ops ops(d, o);
   ops.set_three_part(three_part_passes(o, m, n, -1));
-  ops.layout(ar, Ops::pass_part_floats(m, n, d), o.precision == RQLP_PREC_BF16X3, m, n);
+  ops.layout(ar, Ops::pass_part_floats(m, n, d), o.precision == RQLP_PREC_BF16X3, m, n,
+             o.precision == RQLP_PREC_FP32 && Ops::split_pays(m, n, d) ? SIZE_MAX : 0);
   ops.bind(static_cast<cudaStream_t>(stream), nullptr);
   cudaError_t e = ops.begin_products();
   if (e == cudaSuccess) e = ops.pass(trans == 1, A, m, n, lda, X, ldx, Y, ldy, nullptr);

@@ -962,7 +962,8 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   a.units = a.tiles * kb;
   // Short K: a split tile would cost more than it saves; whole tiles per CTA.
   a.whole = kb <= 32 ? 1 : 0;
-  const int cap = a.whole ? a.tiles : a.units;
+  // Groups: at most two partial tiles each (none with whole tiles).
+  const int cap = a.whole ? a.tiles : std::min(a.units, ws->slots / (2 * CG));
   a.vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0 && ldo % 4 == 0) ? 1 : 0;
   // Chains. An MMA loses about half a unit in the last place of the sum that
   // it adds to, always toward zero. FP32: one chain per unit, the correction
@@ -982,7 +983,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   }
   // Tensor memory: two main buffers where at least two A slots still fit.
   const int cc = a.corr != 0 ? npad : 0;
-  a.nbuf = 2 * npad + cc + 2 * parts * 16 <= 512 ? 2 : 1;
+  a.nbuf = 2 * npad + cc + 2 * parts * 16 <= 512 ? 2 : 1;   // (FP32 above 208 columns: one)
   a.sa = std::min(kMaxASlots, (512 - a.nbuf * npad - cc) / (parts * 16));
   const size_t stage = (size_t)(npad / CG) * BK * 2 * parts;
   CUtensorMap map = {};
@@ -1009,16 +1010,26 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
 
 }  // namespace
 
-void split_gemm_layout(Arena& ar, SplitGemmWs* ws, int64_t m_cap, int64_t k_cap, int n_cap, int parts) {
-  const int npad = npad_of(n_cap);
-  ws->img = ar.take<uint16_t>((size_t)cdiv(k_cap, BK) * BK * npad * parts);
-  ws->slots = 2 * sm_count();
-  ws->part = ar.take<float>((size_t)ws->slots * BM * npad);
-  const size_t words = 4 + (size_t)cdiv(m_cap, 2 * BM) * 2;
+static size_t image_bytes(int64_t k_cap, int n_cap, int parts) {
+  return (size_t)round_up(k_cap, BK) * npad_of(n_cap) * parts * 2;
+}
+
+size_t split_gemm_block_bytes(int64_t k_cap, int n_cap, int parts) {
+  return image_bytes(k_cap, n_cap, parts) + (size_t)2 * sm_count() * BM * npad_of(n_cap) * 4;
+}
+
+bool split_gemm_layout(Arena& ar, SplitGemmWs* ws, void* block, size_t bytes, int64_t m_cap, int64_t k_cap, int n_cap,
+                       int parts) {
+  const size_t img = image_bytes(k_cap, n_cap, parts), slot = (size_t)BM * npad_of(n_cap) * 4;
+  ws->slots = bytes > img ? (int)std::min<size_t>((bytes - img) / slot, (size_t)2 * sm_count()) : 0;
+  ws->img = static_cast<uint16_t*>(block);
+  ws->part = reinterpret_cast<float*>(static_cast<char*>(block) + img);
+  const size_t words = 4 + (size_t)cdiv(m_cap, CG * BM) * CG;
   ws->words_bytes = words * sizeof(int);
   ws->words = ar.take<int>(words);
   ws->cnt = ar.dry ? nullptr : ws->words + 4;
   ws->turn = 0;
+  return ws->slots >= sm_count() / 2 * 2;   // at least half of the CTAs' two partial tiles each
 }
 
 cudaError_t split_gemm_reset(SplitGemmWs* ws, cudaStream_t st) {
@@ -1036,9 +1047,9 @@ cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K
   int* bad = mode == kSplitFp32 ? ws->words + 2 + turn : nullptr;
   if (range_word != nullptr) *range_word = bad;
   const int parts = mode == kSplitTwo ? 2 : 3;
-  // Three parts need two accumulators and two A slots (96 columns) of tensor
-  // memory: above 208 columns the product runs as two column halves.
-  const int n0 = npad_of(N) > (parts == 3 ? 208 : 16 * 2 * kGroups) ? npad_of((int)cdiv(N, 2)) : N;
+  // Column halves above what a drain warp's registers hold, or where two
+  // accumulators and two A slots (96 columns) exceed tensor memory.
+  const int n0 = npad_of(N) > (mode == kSplitThree ? 208 : 16 * 2 * kGroups) ? npad_of((int)cdiv(N, 2)) : N;
   const bool prof = profiled && profiling_on();
   if (prof) profile_mark_begin(st);
   cudaError_t e = product(ws, turn, transA, M, n0, K, A, lda, X, ldx, out, ldo, mode, sumsq, bad, info, st);

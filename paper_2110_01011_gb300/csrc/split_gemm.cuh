@@ -7,8 +7,9 @@
 namespace rqlp {
 
 // Scratch of split_gemm for products with K <= k_cap and N <= n_cap, laid out
-// once in the caller's workspace. The words at `words` and the tile counters
-// must be zero before the first product (split_gemm_reset).
+// once in the caller's workspace. The words and the tile counters must be zero
+// before the first product of a call (split_gemm_reset); the block (X's image
+// and the partial tiles) carries nothing from one product to the next.
 struct SplitGemmWs {
   uint16_t* img = nullptr;   // X's parts as shared-memory stage images
   float* part = nullptr;     // partial tiles of split K ranges
@@ -18,9 +19,14 @@ struct SplitGemmWs {
   int slots = 0;             // 128-row partial slots that fit in part
   int turn = 0;
 };
-// m_cap: largest number of output rows, k_cap: largest K, n_cap: largest N;
-// parts: 2 or 3 (the largest used).
-void split_gemm_layout(Arena& ar, SplitGemmWs* ws, int64_t m_cap, int64_t k_cap, int n_cap, int parts);
+// Block that serves every product at full width (16-byte aligned); parts: 2 or
+// 3 (the largest used).
+size_t split_gemm_block_bytes(int64_t k_cap, int n_cap, int parts);
+// m_cap: largest number of output rows. The words come from `ar`, the block is
+// given (bytes may be fewer than the above: fewer CTAs then take a product).
+// False when the block is too small for half of the SMs.
+bool split_gemm_layout(Arena& ar, SplitGemmWs* ws, void* block, size_t bytes, int64_t m_cap, int64_t k_cap, int n_cap,
+                       int parts);
 cudaError_t split_gemm_reset(SplitGemmWs* ws, cudaStream_t st);
 
 // kSplitTwo: two parts, three products (BF16x3 form); kSplitThree: three parts,
