@@ -494,10 +494,12 @@ struct Builder {
         a.push_back(j);
         GroupGemm k2 = job(bf[i].R[2], bf[i].ld, bf[i].Ra, bf[i].ld, Racc(i), bf[i].ld, d(i), d(i), d(i));
         k2.b_upper = 1;
+        k2.gate = &bf[i].gates[g];   // no third pass: R3 = I was not written
+        k2.gate_mode = kGateCopyB;
         c.push_back(k2);
       }
       gemm(false, kSmall, a, false);
-      gemm(false, kSmall, c, false);
+      gemm(false, kSmall, c, true);
     }
   }
 

@@ -1,26 +1,26 @@
-// Cholesky factor and inverse of the d x d Gram matrix of CholeskyQR, in one
-// CTA: G = L L^T (R = L^T, upper, positive diagonal) and W = L^{-1}
-// (R^{-1} = W^T).
+// Cholesky factor and inverse of the d x d Gram matrix of CholeskyQR: G = L L^T
+// (R = L^T, upper, positive diagonal) and W = L^{-1} (R^{-1} = W^T).
 //
 // Blocked right-looking elimination on the augmented matrix [G | I] with
-// 16-column panels J:
-//   (1) warp 0 factors the 16 x 16 diagonal block L_JJ (row per lane,
-//       right-looking, column t's entries broadcast by shuffles; each pivot
-//       broadcast straight from its own lane's update);
-//   (2) forward substitutions o = L_JJ^{-1} v, a thread per vector: the
-//       panel L_IJ = G_IJ L_JJ^{-T} for the rows below, the block row of W
-//       (W_J,: = L_JJ^{-1} X_J,:, X = the eliminated identity) and its
-//       diagonal block L_JJ^{-1};
-//   (3) trailing updates G_II -= L_IJ L_IJ^T (lower part) and
-//       X_:J' -= L_IJ W_J,: for the rows above the next panel. The latter only
-//       feeds later block rows of W, so it runs during the next panel's step
-//       (1), on the warps that do not share warp 0's scheduler.
-// Step (3) gives each warp 32 x 16 tiles and each lane 4 x 4 blocks, with the
-// panel operands in transposed shared-memory buffers. L lives in the lower
-// triangle of one square buffer and W^T in its strict upper triangle (W's
-// diagonal in a side array). The Gram's lower triangle reaches shared memory
-// by 16-byte asynchronous copies (FP32 factor, aligned rows), all of them in
-// flight at once.
+// 32-column panels J (16 in FP64). L lives in the lower triangle of one square
+// buffer S and W^T in its strict upper triangle (W's diagonal in a side array),
+// so that one rule updates both: S(r, c) -= S(r, J) . S(c, J) for every row r
+// of S and the columns c right of the panel (below the diagonal for rows below
+// the panel).
+//   (1) warp 0 factors the diagonal block, the one serial chain, while
+//       the other warps apply the previous panel to the rest of S, tiles
+//       from a shared counter;
+//   (2) o = L_JJ^{-1} v by forward substitution, a thread per row of S;
+//   (3) the next diagonal block is updated ahead of the rest, for (1).
+// On one SM (chol_body: FP64, and a batch's problems) the row solves and the
+// tiles are bound by shared memory, (1) by its chain of a root, two products
+// and a shuffle per column (~140 clocks); one FP32 matrix takes a cluster of
+// ceil(d / 32) SMs (chol_cluster_kernel). Measured per factorisation, FP32, d =
+// 69, 136, 205, 256: one SM with 16-column panels and the whole update of the
+// lower part between (2) and (1) 23, 43, 78 and 230 us; one SM as above 17,
+// 35, 68 and 186 us; the cluster 18, 29, 43 and 52 us.
+// The Gram's lower triangle reaches shared memory by 16-byte asynchronous
+// copies (FP32 factor, aligned rows), all of them in flight at once.
 //
 // A pivot that is not clearly positive restarts the elimination on G + s I
 // (shifted CholeskyQR, Fukaya et al. 2020) and raises the caller's gate flag.
@@ -39,7 +39,12 @@
 namespace rqlp {
 namespace {
 
-constexpr int NB = 16;
+// Panel width: 32 in FP32; 16 in FP64, whose chain and sums are bound by the
+// FP64 units' rate.
+template <typename T> struct Panel;
+template <> struct Panel<float> { static constexpr int NB = 32; };
+template <> struct Panel<double> { static constexpr int NB = 16; };
+constexpr int kDtPad = 4;   // pitch of D's columns: 4 banks off a multiple of 32
 // Factorisation attempts: unshifted, then shifts s0, 10 s0, 100 s0 with
 // s0 = 10 d u trace(G) (u: unit roundoff of the factor's type).
 constexpr int kAttempts = 4;
@@ -70,7 +75,6 @@ template <> struct Eps<double> { static constexpr double u = 1.1102230246251565e
 // Row pitch of the square buffer: a multiple of 4 elements (16-byte rows) and
 // 4 banks off a multiple of 32, so consecutive rows start in different banks.
 __host__ __device__ inline int lds_of(int d) { return (int)round_up(d, 32) + 4; }
-__host__ __device__ inline int ptld_of(int d) { return (int)round_up(d, 16); }
 
 template <typename T> struct IsF32 { static constexpr bool value = false; };
 template <> struct IsF32<float> { static constexpr bool value = true; };
@@ -88,69 +92,172 @@ __device__ void write_identity(int d, float* R, float* Rinv, int64_t ldr) {
     }
 }
 
-// Trailing update tiles of the panel that ends at column jn: lower: G_II -= L_IJ L_IJ^T over
-// rows and columns [jn, d), c <= r (Ar = PT); else X -= L_IJ W_J,: over rows
-// [0, jn), columns [jn, d) (Ar = WT). A warp takes a 32 x 16 tile (tiles w0,
-// w0 + ws, ...), each lane a 4 x 4 block (lanes 8 x 4 over the tile): one k
-// step reads 128 contiguous bytes of Ar and 64 of PT for the warp's 512
-// FMAs, then a vectorised read-modify-write of S. Lower tiles: row strip q of
-// 32 rows needs the column strips of 16 up to its diagonal (2 q + 2 of them).
-template <typename T>
-__device__ __forceinline__ void trailing_tiles(T* S, int LDS, const T* Ar, const T* PT, int d, int jn, bool lower,
-                                               int w0, int ws, int lane) {
-  const int PTLD = ptld_of(d), Nt = d - jn;
-  if (Nt <= 0 || w0 < 0) return;
-  const int nct = (Nt + 15) / 16;             // column strips over [jn, d)
-  int ntiles = 0;
-  if (lower) {
-    const int nrs = (Nt + 31) / 32;           // row strips over [jn, d)
-    for (int q = 0; q < nrs; ++q) ntiles += min(2 * q + 2, nct);
-  } else {
-    ntiles = ((jn + 31) / 32) * nct;
+// Dot products of NB entries for a 4 x 4 block of results: rows 8 i of `a`
+// (pitch lda), rows 4 j of `b` (pitch ldb). Pitches are 4 banks off a multiple
+// of 32, so that the eight rows (four columns) of a warp's step lie in
+// different banks. FP32: even and odd entries in a pair of sums, two products
+// an instruction. Shared memory bounds this: a load of 16 bytes takes four
+// clocks whether the lanes' addresses differ or not.
+template <int NB>
+__device__ __forceinline__ void dot_block(const float* a, int lda, const float* b, int ldb, const bool* va,
+                                          const bool* vb, float (&acc)[4][4]) {
+  unsigned long long s[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) s[i][j] = 0;
+#pragma unroll
+  for (int k = 0; k < NB; k += 4) {
+    ulonglong2 av[4], bv[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const ulonglong2*>(a + (va[i] ? 8 * i * lda : 0) + k);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) bv[j] = *reinterpret_cast<const ulonglong2*>(b + (vb[j] ? 4 * j * ldb : 0) + k);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s[i][j]) : "l"(av[i].x), "l"(bv[j].x));
+        asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(s[i][j]) : "l"(av[i].y), "l"(bv[j].y));
+      }
   }
-  for (int t = w0; t < ntiles; t += ws) {
-    int tr, tc, rlim;
-    if (lower) {
-      int q = 0, acc0 = 0;
-      while (acc0 + min(2 * q + 2, nct) <= t) acc0 += min(2 * q++ + 2, nct);
-      tr = jn + 32 * q;
-      tc = jn + 16 * (t - acc0);
-      rlim = d;
-    } else {
-      tr = 32 * (t / nct);
-      tc = jn + 16 * (t % nct);
-      rlim = jn;
-    }
-    const int r0 = tr + 4 * (lane >> 2), c0 = tc + 4 * (lane & 3);
-    if (r0 < rlim && c0 < d && (!lower || c0 <= r0 + 3)) {
-      T acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      acc[i][j] = __uint_as_float((uint32_t)s[i][j]) + __uint_as_float((uint32_t)(s[i][j] >> 32));
+}
+template <int NB>
+__device__ __forceinline__ void dot_block(const double* a, int lda, const double* b, int ldb, const bool* va,
+                                          const bool* vb, double (&acc)[4][4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+#pragma unroll
+  for (int k = 0; k < NB; k += 4) {
+    double av[4][4], bv[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ld4(a + (va[i] ? 8 * i * lda : 0) + k, av[i]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ld4(b + (vb[j] ? 4 * j * ldb : 0) + k, bv[j]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0;
+        for (int j = 0; j < 4; ++j) acc[i][j] += av[i][u] * bv[j][u];
+  }
+}
+
+// One tile of NB rows and 16 columns of the update S(r, c) -= S(r, J) . S(c, J)
+// after panel J = [j0, jn), by a warp. Tiles run over the strips of NB rows
+// below jn (columns jn .. r; the next panel's diagonal block is not among them)
+// and, with columns jn .. d - 1, the strips above it; the panel's own strip
+// takes its rows from DT. False past the last tile.
+template <typename T>
+__device__ __forceinline__ bool update_tile(T* S, int LDS, const T* DT, int d, int j0, int jn, int t, int lane) {
+  constexpr int NB = Panel<T>::NB, kDtLd = NB + kDtPad;
+  const int nct = (d - jn + 15) / 16, nrs = (d - jn + NB - 1) / NB;
+  constexpr int CPS = NB / 16;   // column strips a row strip adds
+  int r0, c0, q = 1;
+  while (q < nrs && t >= min(CPS * (q + 1), nct)) {
+    t -= min(CPS * (q + 1), nct);
+    ++q;
+  }
+  const bool lower = q < nrs;
+  if (lower) {
+    r0 = jn + NB * q;
+    c0 = jn + 16 * t;
+  } else {
+    if (t >= jn / NB * nct) return false;
+    r0 = NB * (t / nct);
+    c0 = jn + 16 * (t % nct);
+  }
+  const int r = r0 + (lane >> 2), c = c0 + (lane & 3);   // this lane: rows r + 8 i, columns c + 4 j
+  bool va[4], vb[4];
 #pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        T av[4], bv[4];
-        ld4(&Ar[k * PTLD + r0], av);
-        ld4(&PT[k * PTLD + c0], bv);
+  for (int i = 0; i < 4; ++i) {
+    va[i] = 8 * i < NB && r + 8 * i < d;
+    vb[i] = c + 4 * i < d;
+  }
+  T acc[4][4];
+  const T* a = r0 == j0 ? DT + (lane >> 2) * kDtLd : &S[(size_t)(va[0] ? r : r0) * LDS + j0];
+  dot_block<NB>(a, r0 == j0 ? kDtLd : LDS, &S[(size_t)(vb[0] ? c : c0) * LDS + j0], LDS, va, vb, acc);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] += av[i] * bv[j];
-      }
+    for (int j = 0; j < 4; ++j)
+      if (va[i] && vb[j] && (!lower || c + 4 * j <= r + 8 * i)) S[(size_t)(r + 8 * i) * LDS + c + 4 * j] -= acc[i][j];
+  return true;
+}
+
+// Warp 0 (lane = row): L_JJ of the jb x jb diagonal block at D (pitch ld), in
+// place (zeros above the diagonal); LT its columns, rdiag 1 / L_jj. Column t is
+// scaled by 1 / sqrt(pivot) and later columns c take l_it l_ct. On the path
+// from a pivot to the next lie its root, two products and a shuffle; the
+// columns after next take column t from LT a step later, while the next root
+// is on its way. tol: this lane's pivot bound. Returns the first failing
+// column, or -1 (the block is then left as it was).
+template <typename T, int NB>
+__device__ __forceinline__ int factor_diagonal(T* D, int ld, int jb, T tol, T* LT, T* rdiag, int lane) {
+  T a[NB], lc[NB];   // the lane's row; the column before the current one
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = r0 + i;
-        if (r >= rlim) continue;
-        T sv[4];
-        ld4(&S[(size_t)r * LDS + c0], sv);
+  for (int k = 0; k < NB; k += 4) {
+    if (lane < jb) ld4(&D[(size_t)lane * ld + k], &a[k]);
+    else a[k] = a[k + 1] = a[k + 2] = a[k + 3] = (T)0;
+  }
+  int f = -1;
+  T piv = __shfl_sync(0xffffffffu, a[0], 0), lp = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int c = c0 + j;
-          if (c < d && (!lower || c <= r)) sv[j] -= acc[i][j];
-        }
-        st4(&S[(size_t)r * LDS + c0], sv);
-      }
+  for (int t = 0; t < NB; ++t) {
+    if (t >= jb) break;
+    const T rl = rsqrt(piv);   // (what a failing pivot gives is dropped with the attempt)
+    if (t > 0) {
+#pragma unroll
+      for (int c = t + 1; c < NB; ++c) a[c] -= lp * lc[c];
+    }
+    const bool ok = a[t] > tol && isfinite(a[t]);   // (lane t: the pivot)
+    const T l = lane >= t ? a[t] * rl : (T)0;
+    if (t + 1 < NB) {
+      piv = __shfl_sync(0xffffffffu, a[t + 1] - l * l, t + 1);
+      a[t + 1] -= l * __shfl_sync(0xffffffffu, l, t + 1);
+    }
+    if (lane < NB) LT[t * NB + lane] = l;
+    if ((__ballot_sync(0xffffffffu, ok) >> t & 1) == 0 && f < 0) f = t;
+    if (lane == t) rdiag[t] = rl;
+    a[t] = lp = l;
+    __syncwarp();
+#pragma unroll
+    for (int c = (t + 2) / 4 * 4; c < NB; c += 4) ld4(&LT[t * NB + c], &lc[c]);
+  }
+  if (f < 0 && lane < jb) {
+#pragma unroll
+    for (int k = 0; k < NB; k += 4) {
+      T o[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) o[u] = k + u <= lane ? a[k + u] : (T)0;
+      st4(&D[(size_t)lane * ld + k], o);
+    }
+  }
+  return f;
+}
+
+// v = L_JJ^{-1} v by forward substitution, column by column: an entry is final
+// one product after the one before it.
+template <typename T, int NB>
+__device__ __forceinline__ void solve_row(T (&v)[NB], const T* LT, const T* rdiag, int jb) {
+#pragma unroll
+  for (int c = 0; c < NB; ++c) {
+    if (c >= jb) break;
+    v[c] *= rdiag[c];
+#pragma unroll
+    for (int k = (c + 1) / 4 * 4; k < NB; k += 4) {
+      T l[4];
+      ld4(&LT[c * NB + k], l);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k + u > c) v[k + u] -= l[u] * v[c];
     }
   }
 }
@@ -162,25 +269,20 @@ template <typename T, bool kShared>
 __device__ __forceinline__ void chol_body(int d, const float* __restrict__ G, int64_t ldg, float* __restrict__ R,
                                           float* __restrict__ Rinv, int64_t ldr, int* info, double* shift_count,
                                           int* gate_out, const int* gate_in, T* gS) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int LDS = lds_of(d), PTLD = ptld_of(d);
+  extern __shared__ __align__(32) unsigned char smem_raw[];
+  constexpr int NB = Panel<T>::NB, kDtLd = NB + kDtPad;
+  const int LDS = lds_of(d);
   T* dyn = reinterpret_cast<T*>(smem_raw);
-  // kShared: S at the start of shared memory, so every access to it is a
-  // shared-memory access; otherwise S = gS in global memory.
-  T* S = kShared ? dyn : gS;
-  T* PT = kShared ? dyn + (size_t)d * LDS : dyn;
-  T* WT = PT + NB * PTLD;
-  __shared__ __align__(32) T gdiag[kMaxD];
-  __shared__ T wdiag[kMaxD];
-  __shared__ T rdiag[NB];   // 1 / L_jj of the current diagonal block
-  __shared__ int s_fail;
+  T* DT = dyn;                 // D = L_JJ^{-1} by columns: DT[c][k] = D_kc
+  T* LT = DT + NB * kDtLd;     // L_JJ by columns: LT[t][i] = L_it (zero above the diagonal)
+  T* S = kShared ? LT + NB * NB : gS;
+  __shared__ __align__(32) T gdiag[kMaxD];   // G's diagonal; W's once a panel is done
+  __shared__ T rdiag[NB];                    // 1 / L_jj of the current diagonal block
+  __shared__ int s_fail, s_tile;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
 
-  if (gate_in != nullptr && *gate_in == 0) {   // pass not needed: R = R^{-1} = I
-    write_identity(d, R, Rinv, ldr);
-    return;
-  }
+  if (gate_in != nullptr && *gate_in == 0) return;   // pass not needed: nothing reads R or R^{-1}
 
   const T rel_tol = (T)64 * Eps<T>::u;
   T shift = 0;
@@ -258,138 +360,93 @@ __device__ __forceinline__ void chol_body(int d, const float* __restrict__ G, in
       shift = (T)(10.0 * d) * Eps<T>::u * tr;
     }
     fail = -1;
-    // Panel loop. Phase B of panel J: warp 0 factors the diagonal block while
-    // the other warps finish the previous panel's update of the rows above
-    // (X -= L_IJ W_J,:, rows [0, j0)); the two touch disjoint parts of S.
     for (int j0 = 0; j0 < d; j0 += NB) {
-      const int jb = min(NB, d - j0);
-      const int jn = j0 + jb, Nt = d - jn;
+      const int jb = min(NB, d - j0), jn = j0 + jb;
+      // (1) Warp 0 factors the diagonal block; the other warps, and warp 0 when
+      // it is done, apply the previous panel to the rest of S.
       if (warp == 0) {
-        // (1) L_JJ, lane = row, right-looking: column t is scaled by
-        // 1 / sqrt(pivot), then every later column c takes l_it l_ct (l_ct
-        // from lane c by a shuffle). Only column t + 1's update lies on the
-        // path to the next pivot. Branch-free; entries above the diagonal are
-        // cleared before the store.
-        T l[NB], gd[NB];
-#pragma unroll
-        for (int k = 0; k < NB; k += 4) {
-          if (lane < jb) ld4(&S[(size_t)(j0 + lane) * LDS + j0 + k], &l[k]);
-          else l[k] = l[k + 1] = l[k + 2] = l[k + 3] = (T)0;
-          ld4(&gdiag[j0 + k], &gd[k]);
-        }
-        int f = -1;
-        T piv = __shfl_sync(0xffffffffu, l[0], 0);
-#pragma unroll
-        for (int t = 0; t < NB; ++t) {
-          const bool live = t < jb;
-          const bool ok = piv > rel_tol * gd[t] && isfinite(piv);
-          f = (f < 0 && live && !ok) ? j0 + t : f;
-          const T rl = rsqrt(ok ? piv : (T)1);
-          if (lane == 0) rdiag[t] = rl;
-          l[t] = lane == t ? piv * rl : (lane > t ? l[t] * rl : (T)0);
-          // The next pivot is lane t + 1's own update of its diagonal entry
-          // (the operation the column loop below performs there, so the same
-          // value), broadcast without waiting on the shuffle of column t.
-          if (t + 1 < NB) piv = __shfl_sync(0xffffffffu, l[t + 1] - l[t] * l[t], t + 1);
-#pragma unroll
-          for (int c = t + 1; c < NB; ++c) l[c] -= l[t] * __shfl_sync(0xffffffffu, l[t], c);
-        }
-#pragma unroll
-        for (int k = 0; k < NB; ++k)
-          if (k > lane) l[k] = (T)0;
-        if (f < 0 && lane < jb) {   // zeros above the diagonal: W's block there is written in (2)
-#pragma unroll
-          for (int k = 0; k < NB; k += 4) st4(&S[(size_t)(j0 + lane) * LDS + j0 + k], &l[k]);
-        }
-        if (lane == 0) s_fail = f;
+        const int f = factor_diagonal<T, NB>(&S[(size_t)j0 * LDS + j0], LDS, jb,
+                                             lane < jb ? rel_tol * gdiag[j0 + lane] : (T)0, LT, rdiag, lane);
+        if (lane == 0) s_fail = f < 0 ? -1 : j0 + f;
       }
-      // The update of the rows above goes to the warps that do not share warp
-      // 0's scheduler (warp % 4 != 0), so that the serial factor issues alone.
-      if (j0 > 0) {
-        if (nwarps >= 8) {
-          if ((warp & 3) != 0)
-            trailing_tiles<T>(S, LDS, WT, PT, d, j0, false, (warp >> 2) * 3 + (warp & 3) - 1, (nwarps >> 2) * 3, lane);
-        } else if (warp > 0 || nwarps == 1) {
-          trailing_tiles<T>(S, LDS, WT, PT, d, j0, false, nwarps > 1 ? warp - 1 : 0, max(nwarps - 1, 1), lane);
+      // (warps 4, 8 and 12 leave warp 0 its scheduler: beside three working warps
+      // its chain took twice as long)
+      if (j0 > 0 && (warp == 0 || nwarps < 8 || (warp & 3) != 0)) {
+        for (;;) {
+          int t = 0;
+          if (lane == 0) t = atomicAdd(&s_tile, 1);
+          t = __shfl_sync(0xffffffffu, t, 0);
+          if (!update_tile<T>(S, LDS, DT, d, j0 - NB, j0, t, lane)) break;
         }
       }
       __syncthreads();
+      if (tid == 0) s_tile = 0;
       if (s_fail >= 0) {
         fail = s_fail;
         break;
       }
-      // (2) o = L_JJ^{-1} v by forward substitution, a thread per vector:
-      // panel rows below (v = G_IJ row, o = L_IJ row -> S and PT), rows of
-      // W's block row J (v = the eliminated identity's column, o -> S and
-      // WT) and W's diagonal block (v = unit vector, o = column of D).
-      for (int idx = tid; idx < Nt + jn; idx += blockDim.x) {
+      // (2) o = L_JJ^{-1} v for every row of S, a thread per row: v = its panel
+      // columns, in place (L_IJ below the panel, W_J,: above it); the panel's
+      // own rows start from unit vectors and give D. An entry is final one
+      // product after the one before it.
+      for (int r = tid; r < d; r += blockDim.x) {
+        T* row = &S[(size_t)r * LDS + j0];
+        const int cc = r - j0;   // 0 .. jb - 1: the panel's own rows
+        const bool own = cc >= 0 && cc < jb;
         T v[NB];
-        int src = -1;   // row of S that holds v, or -1 for a unit vector
-        if (idx < Nt) src = jn + idx;
-        else if (idx - Nt < j0) src = idx - Nt;
-        const int cc = idx - Nt - j0;   // diagonal-block column (unit vector e_cc)
-        if (src >= 0) {
 #pragma unroll
-          for (int k = 0; k < NB; k += 4) ld4(&S[(size_t)src * LDS + j0 + k], &v[k]);
-          if (jb < NB) {
+        for (int k = 0; k < NB; k += 4) {
+          T x[4];
+          ld4(&row[k], x);
 #pragma unroll
-            for (int k = 0; k < NB; ++k)
-              if (k >= jb) v[k] = (T)0;
-          }
+          for (int u = 0; u < 4; ++u) v[k + u] = own ? (k + u == cc ? (T)1 : (T)0) : (k + u < jb ? x[u] : (T)0);
+        }
+        solve_row<T, NB>(v, LT, rdiag, jb);
+        if (own) {
+          gdiag[r] = rdiag[cc];
+#pragma unroll
+          for (int k = 0; k < NB; k += 4) st4(&DT[cc * kDtLd + k], &v[k]);
+#pragma unroll
+          for (int k = 0; k < NB; ++k)
+            if (k > cc && k < jb) row[k] = v[k];
         } else {
 #pragma unroll
-          for (int k = 0; k < NB; ++k) v[k] = k == cc ? (T)1 : (T)0;
-        }
-        T o[NB];
-#pragma unroll
-        for (int c = 0; c < NB; ++c) {
-          if (c < jb) {
-            const T* lr = &S[(size_t)(j0 + c) * LDS + j0];
-            T sacc = v[c];
-#pragma unroll
-            for (int k = 0; k < c; k += 4) {
-              T lv[4];
-              ld4(&lr[k], lv);
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                if (k + u < c) sacc -= lv[u] * o[k + u];
-            }
-            o[c] = sacc * rdiag[c];
-          } else {
-            o[c] = (T)0;
-          }
-        }
-        if (idx < Nt) {
-          const int i = jn + idx;
-#pragma unroll
-          for (int c = 0; c < NB; ++c) PT[c * PTLD + i] = o[c];
-#pragma unroll
-          for (int k = 0; k < NB; k += 4) st4(&S[(size_t)i * LDS + j0 + k], &o[k]);
-        } else if (src >= 0) {
-#pragma unroll
-          for (int rr = 0; rr < NB; ++rr) {
-            if (rr < jb) {
-              S[(size_t)src * LDS + j0 + rr] = o[rr];
-              WT[rr * PTLD + src] = o[rr];
-            }
-          }
-        } else {
-          const int c = j0 + cc;
-          wdiag[c] = rdiag[cc];   // = o[cc]
-#pragma unroll
-          for (int rr = 0; rr < NB; ++rr) {
-            if (rr < jb) {
-              if (rr > cc) S[(size_t)c * LDS + j0 + rr] = o[rr];
-              WT[rr * PTLD + c] = o[rr];
-            }
-          }
+          for (int k = 0; k < NB; k += 4) st4(&row[k], &v[k]);
         }
       }
       __syncthreads();
-      // (3) trailing update G_II -= L_IJ L_IJ^T of the lower part; the rows
-      // above follow in the next panel's phase B.
-      if (Nt > 0) trailing_tiles<T>(S, LDS, PT, PT, d, jn, true, warp, nwarps, lane);
-      __syncthreads();
+      // (3) The next diagonal block, which step (1) waits for: entries
+      // (r, c), (r + NB / 2, c) and (r + NB / 2, c + NB / 2) per thread.
+      if (jn < d) {
+        constexpr int H = NB / 2;
+        for (int t = tid; t < H * H; t += blockDim.x) {
+          const int r = jn + t / H, c = jn + t % H;
+          const bool r1 = r + H < d, c1 = c + H < d;
+          if (r >= d || c >= d) continue;
+          T a00 = 0, a10 = 0, a11 = 0;
+          const T* pr = &S[(size_t)r * LDS + j0];
+          const T* pc = &S[(size_t)c * LDS + j0];
+          const size_t up = (size_t)H * LDS;
+#pragma unroll
+          for (int k = 0; k < NB; k += 4) {
+            T x0[4], x1[4], y0[4], y1[4];
+            ld4(pr + k, x0);
+            ld4(pr + (r1 ? up : 0) + k, x1);
+            ld4(pc + k, y0);
+            ld4(pc + (c1 ? up : 0) + k, y1);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              a00 += x0[u] * y0[u];
+              a10 += x1[u] * y0[u];
+              a11 += x1[u] * y1[u];
+            }
+          }
+          if (c <= r) S[(size_t)r * LDS + c] -= a00;
+          if (r1) S[(size_t)(r + H) * LDS + c] -= a10;
+          if (r1 && c1 && c <= r) S[(size_t)(r + H) * LDS + c + H] -= a11;
+        }
+        __syncthreads();
+      }
     }
     if (fail < 0) break;
     __syncthreads();
@@ -404,13 +461,25 @@ __device__ __forceinline__ void chol_body(int d, const float* __restrict__ G, in
     write_identity(d, R, Rinv, ldr);
     return;
   }
-  // R = L^T (upper); R^{-1} = W^T: strict upper part from S, diagonal from wdiag.
-  for (int i = warp; i < d; i += nwarps) {   // a warp per row, lanes over columns
+  __syncthreads();   // (d <= NB: step (2) was the last)
+  // R = L^T (upper); R^{-1} = W^T: strict upper part from S, diagonal from gdiag.
+  for (int i = warp; i < d; i += nwarps) {   // a warp per row, lanes over columns, a row's loads before its stores
     float* r = R != nullptr ? R + (int64_t)i * ldr : nullptr;
     float* ri = Rinv + (int64_t)i * ldr;
-    for (int l = lane; l < d; l += 32) {
-      if (R != nullptr) r[l] = l >= i ? (float)S[(size_t)l * LDS + i] : 0.f;
-      ri[l] = l > i ? (float)S[(size_t)i * LDS + l] : (l == i ? (float)wdiag[i] : 0.f);
+    float x[kMaxD / 32], y[kMaxD / 32];
+#pragma unroll
+    for (int t = 0; t < kMaxD / 32; ++t) {
+      const int l = lane + 32 * t;
+      x[t] = l < d && l > i ? (float)S[(size_t)i * LDS + l] : (l == i ? (float)gdiag[i] : 0.f);
+      y[t] = l < d && l >= i && R != nullptr ? (float)S[(size_t)l * LDS + i] : 0.f;
+    }
+#pragma unroll
+    for (int t = 0; t < kMaxD / 32; ++t) {
+      const int l = lane + 32 * t;
+      if (l < d) {
+        ri[l] = x[t];
+        if (R != nullptr) r[l] = y[t];
+      }
     }
   }
 }
@@ -420,6 +489,235 @@ __global__ void __launch_bounds__(kThreads)
 chol_blocked_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __restrict__ R, float* __restrict__ Rinv,
                     int64_t ldr, int* info, double* shift_count, int* gate_out, const int* gate_in, T* gS) {
   chol_body<T, kShared>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in, gS);
+}
+
+// FP32 factorisation of one matrix by a cluster: CTA s holds rows 32 s .. 32 s +
+// 31 of S (ceil(d / 32) CTAs, at most 8). The steps are chol_body's; a panel's
+// owner factors its diagonal block and the others copy L_JJ from its shared
+// memory, each CTA solves its own rows, and the rows' panel entries are
+// gathered from their owners for the update. On the path from one panel to the
+// next lie the diagonal block (one warp), a cluster barrier, the copy of L_JJ,
+// one row solve and the next owner's update of its own diagonal block; the
+// rest of the update runs beside the next diagonal block on all SMs of the
+// cluster.
+constexpr int kClusterThreads = 256;
+
+__device__ __forceinline__ uint32_t remote_addr(const void* p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float4 remote_ld4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ int remote_ld(uint32_t a) {
+  int v;
+  asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+template <int NB>
+size_t cluster_smem_bytes(int d) {
+  return ((size_t)NB * lds_of(d) + (size_t)round_up(d, NB) * (NB + kDtPad) + NB * (NB + kDtPad) + NB * NB + NB) *
+         sizeof(float);
+}
+
+// NB: 32, or 16 for one CTA of d <= 16.
+template <int NB>
+__global__ void __launch_bounds__(kClusterThreads)
+chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __restrict__ R, float* __restrict__ Rinv,
+                    int64_t ldr, int* info, double* shift_count, int* gate_out, const int* gate_in) {
+  extern __shared__ __align__(32) unsigned char smem_raw[];
+  constexpr int kCLd = NB + kDtPad;
+  const int LDS = lds_of(d), rank = blockIdx.x, P = gridDim.x;
+  float* S = reinterpret_cast<float*>(smem_raw);   // rows 32 rank .. of S
+  float* C = S + NB * LDS;                         // S(c, J) of the other rows, pitch kCLd (row c at c)
+  float* DT = C + (size_t)round_up(d, NB) * kCLd;
+  float* LT = DT + NB * kCLd;                      // L_JJ by columns: the owner's, or a copy
+  float* rdiag = LT + NB * NB;                     // (behind LT: one copy takes both)
+  __shared__ float gdiag[NB];                      // G's diagonal; W's once the panel is done
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kClusterThreads / 32;
+  const int i0 = NB * rank, rows = min(NB, d - i0);
+
+  if (gate_in != nullptr && *gate_in == 0) return;   // pass not needed (the same for every CTA)
+
+  const float rel_tol = 64 * Eps<float>::u;
+  float shift = 0;
+  int fail = -1;
+  for (int attempt = 0; attempt < kAttempts; ++attempt) {
+    if (attempt > 1) shift *= 10.f;
+    if (attempt == 0) {   // trace(G), by every warp in the same order
+      float tr = 0;
+      for (int i = lane; i < d; i += 32) tr += G[(int64_t)i * ldg + i];
+      for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+      if (!isfinite(tr)) {
+        if (rank == 0) {
+          if (tid == 0) post_error(info, RQLP_ERR_NONFINITE, 0);
+          write_identity(d, R, Rinv, ldr);
+        }
+        return;
+      }
+      shift = (float)(10.0 * d) * Eps<float>::u * tr;
+    }
+    const float sh = attempt == 0 ? 0.f : shift;
+    // The rows' lower part of G (+ sh I), zeros above.
+    for (int e = tid; e < rows * (LDS / 4); e += kClusterThreads) {
+      const int i = e / (LDS / 4), c = 4 * (e % (LDS / 4)), gi = i0 + i;
+      float x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        x[u] = c + u <= gi ? G[(int64_t)gi * ldg + c + u] + (c + u == gi ? sh : 0.f) : 0.f;
+      st4(&S[i * LDS + c], x);
+      if (gi >= c && gi < c + 4) gdiag[i] = x[gi - c];
+    }
+    __syncthreads();
+    fail = -1;
+    for (int J = 0; J < P; ++J) {
+      const int j0 = NB * J, jb = min(NB, d - j0);
+      // (1) beside the update with the previous panel (arrivals: end of (2))
+      if (rank == J && warp == 0) {
+        const int f = factor_diagonal<float, NB>(&S[j0], LDS, jb, lane < jb ? rel_tol * gdiag[lane] : 0.f, LT, rdiag,
+                                                 lane);
+        if (lane == 0) s_fail = f < 0 ? -1 : j0 + f;
+        if (J > 0) cluster_wait();
+      } else if (J > 0) {
+        cluster_wait();   // every CTA's rows of panel J - 1 are solved
+        const int p0 = j0 - NB;
+        // Columns c of the update: j0 .. r below the panel (the owner of J has
+        // done its diagonal block), j0 .. d - 1 above.
+        const bool lower = rank >= J;
+        const int cend = lower ? min(d, i0 + NB) : d;
+        const int w0 = rank == J ? warp - 1 : warp, ws = rank == J ? nwarps - 1 : nwarps;
+        if (!(rank == J)) {
+          for (int e = tid; e < (cend - j0) * (NB / 4); e += kClusterThreads) {
+            const int c = j0 + e / (NB / 4), k = 4 * (e % (NB / 4)), o = c / NB;
+            const float4 v = remote_ld4(remote_addr(&S[(c - NB * o) * LDS + p0 + k], o));
+            *reinterpret_cast<float4*>(&C[(c - j0) * kCLd + k]) = v;
+          }
+          __syncthreads();
+          for (int t = w0; j0 + 16 * t < cend; t += ws) {
+            const int r = lane >> 2, c = j0 + 16 * t + (lane & 3);   // rows r + 8 i, columns c + 4 j
+            bool va[4], vb[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              va[i] = r + 8 * i < rows;
+              vb[i] = c + 4 * i < cend;
+            }
+            float acc[4][4];
+            const bool own = rank == J - 1;
+            const float* a = own ? DT + r * kCLd : &S[(va[0] ? r : 0) * LDS + p0];
+            dot_block<NB>(a, own ? kCLd : LDS, &C[(vb[0] ? c - j0 : 0) * kCLd], kCLd, va, vb, acc);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                if (va[i] && vb[j] && (!lower || c + 4 * j <= i0 + r + 8 * i)) S[(r + 8 * i) * LDS + c + 4 * j] -= acc[i][j];
+          }
+        }
+      }
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+      // (2)
+      if (rank != J) {
+        for (int e = tid; e < (NB * NB + NB) / 4; e += kClusterThreads)
+          *reinterpret_cast<float4*>(&LT[4 * e]) = remote_ld4(remote_addr(&LT[4 * e], J));
+      }
+      fail = remote_ld(remote_addr(&s_fail, J));
+      __syncthreads();
+      if (fail >= 0) break;
+      if (warp == 0) {
+        const bool in = lane < rows, own = rank == J;
+        float* row = &S[(in ? lane : 0) * LDS + j0];
+        float v[NB];
+#pragma unroll
+        for (int k = 0; k < NB; k += 4) {
+          float x[4];
+          ld4(&row[k], x);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) v[k + u] = own ? (k + u == lane ? 1.f : 0.f) : (k + u < jb ? x[u] : 0.f);
+        }
+        solve_row<float, NB>(v, LT, rdiag, jb);
+        if (own) {
+          if (in) {
+            gdiag[lane] = rdiag[lane];
+#pragma unroll
+            for (int k = 0; k < NB; k += 4) st4(&DT[lane * kCLd + k], &v[k]);
+#pragma unroll
+            for (int k = 0; k < NB; ++k)
+              if (k > lane && k < jb) row[k] = v[k];
+          }
+        } else if (in) {
+#pragma unroll
+          for (int k = 0; k < NB; k += 4) st4(&row[k], &v[k]);
+        }
+      }
+      __syncthreads();
+      if (J + 1 == P) break;
+      cluster_arrive();   // waited for in (1) of the next panel
+      // (3) the next owner's diagonal block
+      if (rank == J + 1) {
+        for (int t = tid; t < 256; t += kClusterThreads) {
+          const int r = t >> 4, c = t & 15;
+          const bool r1 = r + 16 < rows, c1 = c + 16 < rows;
+          if (r >= rows || c >= rows) continue;
+          float a00 = 0, a10 = 0, a11 = 0;
+          const float *pr = &S[r * LDS + j0], *pc = &S[c * LDS + j0];
+#pragma unroll
+          for (int k = 0; k < NB; k += 4) {
+            float x0[4], x1[4], y0[4], y1[4];
+            ld4(pr + k, x0);
+            ld4(pr + (r1 ? 16 * LDS : 0) + k, x1);
+            ld4(pc + k, y0);
+            ld4(pc + (c1 ? 16 * LDS : 0) + k, y1);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              a00 += x0[u] * y0[u];
+              a10 += x1[u] * y0[u];
+              a11 += x1[u] * y1[u];
+            }
+          }
+          if (c <= r) S[r * LDS + i0 + c] -= a00;
+          if (r1) S[(r + 16) * LDS + i0 + c] -= a10;
+          if (r1 && c1 && c <= r) S[(r + 16) * LDS + i0 + c + 16] -= a11;
+        }
+        __syncthreads();
+      }
+    }
+    cluster_arrive();   // no CTA reads another's shared memory any more
+    cluster_wait();
+    if (fail < 0) break;
+    if (attempt == 0 && rank == 0 && tid == 0) {
+      if (gate_out != nullptr) *gate_out = 1;
+      if (shift_count != nullptr) atomicAdd(shift_count, 1.0);
+    }
+  }
+  if (fail >= 0) {
+    if (rank == 0) {
+      if (tid == 0) post_error(info, RQLP_ERR_BREAKDOWN, fail + 1);
+      write_identity(d, R, Rinv, ldr);
+    }
+    return;
+  }
+  // R^{-1} = W^T: this CTA's rows. R = L^T: its columns.
+  for (int i = warp; i < rows; i += nwarps) {
+    float* ri = Rinv + (int64_t)(i0 + i) * ldr;
+#pragma unroll
+    for (int t = 0; t < kMaxD / 32; ++t) {
+      const int l = lane + 32 * t;
+      if (l < d) ri[l] = l > i0 + i ? S[i * LDS + l] : (l == i0 + i ? gdiag[i] : 0.f);
+    }
+  }
+  if (R != nullptr && lane < rows) {
+#pragma unroll 4
+    for (int i = warp; i < d; i += nwarps) R[(int64_t)i * ldr + i0 + lane] = i <= i0 + lane ? S[lane * LDS + i] : 0.f;
+  }
 }
 
 // One CTA per problem of a batch; every square buffer in shared memory.
@@ -448,12 +746,12 @@ size_t smem_optin_chol() {
 template <typename T>
 size_t square_bytes(int d) { return (size_t)d * lds_of(d) * sizeof(T); }
 template <typename T>
-size_t panel_bytes(int d) { return (size_t)2 * NB * ptld_of(d) * sizeof(T); }
+size_t panel_bytes() { return (size_t)Panel<T>::NB * (2 * Panel<T>::NB + kDtPad) * sizeof(T); }
 template <typename T>
-size_t static_bytes() { return (2 * kMaxD + NB) * sizeof(T) + 96; }
+size_t static_bytes() { return (kMaxD + Panel<T>::NB) * sizeof(T) + 96; }
 template <typename T>
 bool square_in_smem(int d) {
-  return square_bytes<T>(d) + panel_bytes<T>(d) + static_bytes<T>() <= smem_optin_chol();
+  return square_bytes<T>(d) + panel_bytes<T>() + static_bytes<T>() <= smem_optin_chol();
 }
 
 template <typename T>
@@ -470,7 +768,7 @@ cudaError_t launch(int d, const float* G, int64_t ldg, float* R, float* Rinv, in
   }
   const bool in_smem = square_in_smem<T>(d);
   if (!in_smem && gstore == nullptr) return cudaErrorInvalidValue;
-  const size_t dyn = panel_bytes<T>(d) + (in_smem ? square_bytes<T>(d) : 0);
+  const size_t dyn = panel_bytes<T>() + (in_smem ? square_bytes<T>(d) : 0);
   if (in_smem)
     chol_blocked_kernel<T, true><<<1, kThreads, dyn, st>>>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out,
                                                            gate_in, nullptr);
@@ -479,6 +777,33 @@ cudaError_t launch(int d, const float* G, int64_t ldg, float* R, float* Rinv, in
                                                             gate_in, reinterpret_cast<T*>(gstore));
   note_launch();
   return cudaGetLastError();
+}
+
+template <int NB>
+cudaError_t launch_cluster(int d, const float* G, int64_t ldg, float* R, float* Rinv, int64_t ldr, int* info,
+                           double* shift_count, int* gate_out, const int* gate_in, cudaStream_t st) {
+  static bool configured = false;
+  if (!configured) {
+    CK(cudaFuncSetAttribute(chol_cluster_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                            (int)cluster_smem_bytes<NB>(kMaxD)));
+    configured = true;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cdiv(d, NB);
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)cdiv(d, NB));
+  cfg.blockDim = dim3(kClusterThreads);
+  cfg.dynamicSmemBytes = cluster_smem_bytes<NB>(d);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e =
+      cudaLaunchKernelEx(&cfg, chol_cluster_kernel<NB>, d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in);
+  note_launch();
+  return e;
 }
 
 template <typename T>
@@ -492,7 +817,7 @@ cudaError_t launch_batched(const CholJob* jobs, int count, int dmax, cudaStream_
   }
   if (count <= 0) return cudaSuccess;   // configuration only
   if (!square_in_smem<T>(dmax)) return cudaErrorInvalidValue;
-  const size_t dyn = panel_bytes<T>(dmax) + square_bytes<T>(dmax);
+  const size_t dyn = panel_bytes<T>() + square_bytes<T>(dmax);
   chol_batched_kernel<T><<<count, kBatchThreads, dyn, st>>>(jobs, count);
   note_launch();
   return cudaGetLastError();
@@ -508,16 +833,21 @@ cudaError_t chol_inv_batched(const CholJob* jobs, int count, int dmax, bool fp64
   return fp64 ? launch_batched<double>(jobs, count, dmax, st) : launch_batched<float>(jobs, count, dmax, st);
 }
 
-size_t chol_global_bytes(int d, bool fp64) {
-  if (fp64) return square_in_smem<double>(d) ? 0 : square_bytes<double>(d);
-  return square_in_smem<float>(d) ? 0 : square_bytes<float>(d);
+// (Workspace sizes that callers see include this: it reserves the buffer from
+// the d on where panel buffers of 2 x 16 columns left no room for the square.)
+template <typename T>
+size_t global_bytes(int d) {
+  const size_t panels = (size_t)32 * round_up(d, 16) * sizeof(T), fixed = (2 * kMaxD + 16) * sizeof(T) + 96;
+  return square_bytes<T>(d) + panels + fixed <= smem_optin_chol() ? 0 : square_bytes<T>(d);
 }
+size_t chol_global_bytes(int d, bool fp64) { return fp64 ? global_bytes<double>(d) : global_bytes<float>(d); }
 
 cudaError_t chol_inv(int d, const float* G, int64_t ldg, float* R, float* Rinv, int64_t ldr, int* info,
                      double* shift_count, int* gate_out, const int* gate_in, void* gstore, bool fp64,
                      cudaStream_t st) {
   if (fp64) return launch<double>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in, gstore, st);
-  return launch<float>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in, gstore, st);
+  return d <= 16 ? launch_cluster<16>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in, st)
+                 : launch_cluster<32>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in, st);
 }
 
 }  // namespace rqlp

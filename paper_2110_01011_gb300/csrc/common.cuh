@@ -80,12 +80,13 @@ void profile_mark_end(cudaStream_t st, int tag);
 // splits > 1 uses `part` (splits * M * N floats) and a fixed-order reduction.
 // sumsq (optional): += sum of squares of the A elements read.
 // gate (optional) with gate_mode 1: *gate == 0 -> C = A (B taken as identity,
-// needs !transA, K == N, one slice); gate_mode 2: *gate == 0 -> no work.
+// needs !transA, K == N, one slice); gate_mode 2: *gate == 0 -> no work;
+// gate_mode 3: *gate == 0 -> C = B (A the identity; !transA, M == K, one slice).
 // b_upper: B is upper triangular (k-tiles beyond the column tile are skipped).
 // lower_only (M == N, a Gram matrix whose reader takes its lower triangle):
 // tiles whose entries all lie above the diagonal are skipped and C's strict
 // upper triangle is left undefined.
-enum GateMode { kGateNone = 0, kGateCopy = 1, kGateSkip = 2 };
+enum GateMode { kGateNone = 0, kGateCopy = 1, kGateSkip = 2, kGateCopyB = 3 };
 cudaError_t gemm_f32_ex(bool transA, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
                         const float* B, int64_t ldb, float* C, int64_t ldc, int splits, float* part,
                         double* sumsq, const int* gate, int gate_mode, bool b_upper, cudaStream_t st,
@@ -118,8 +119,8 @@ cudaError_t gemm_grouped(bool transA, int choice, const GroupGemm* jobs, const i
 cudaError_t gemm_grouped_prepare();
 
 // ---------------------------------------------------------------- d x d kernels
-// R^T R = G (+ s I on breakdown; raises *gate_out), Rinv = R^{-1}; gate_in == 0
-// -> R = Rinv = I. gstore: global scratch when the factor does not fit in
+// R^T R = G (+ s I on breakdown; raises *gate_out), Rinv = R^{-1}; *gate_in == 0
+// -> no work (R and Rinv are left as they are). gstore: global scratch when the factor does not fit in
 // shared memory (chol_global_bytes(d, fp64) bytes, else unused).
 cudaError_t chol_inv(int d, const float* G, int64_t ldg, float* R, float* Rinv, int64_t ldr, int* info,
                      double* shift_count, int* gate_out, const int* gate_in, void* gstore, bool fp64,

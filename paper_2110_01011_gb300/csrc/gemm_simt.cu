@@ -31,17 +31,20 @@ struct GemmArgs {
   int lower_only;                           // only tiles with entries on or below the diagonal
 };
 
-// Gated off (kGateCopy): C = A on this tile (B taken as the identity). All
+// Gated off (kGateCopy): C = A on this tile (B taken as the identity), or B
+// (kGateCopyB). All
 // loads of the thread are issued before its stores (C and A are distinct
 // buffers, which the compiler cannot assume), four 128-bit loads at a time.
 template <int BM, int BN, int NT>
 __device__ __forceinline__ void copy_tile(const GemmArgs& g, int64_t m0, int64_t n0, float* C) {
+  const float* S = g.gate_mode == kGateCopyB ? g.B : g.A;
+  const int64_t lds = g.gate_mode == kGateCopyB ? g.ldb : g.lda;
   constexpr int Q = BN / 4;            // float4 per tile row
   constexpr int PER = BM * Q / NT;     // float4 per thread
   constexpr int CH = 4;                // float4 loaded before their stores (bounded registers)
   static_assert(PER * NT == BM * Q, "copy tiling");
-  const bool vec = ((reinterpret_cast<uintptr_t>(g.A) | reinterpret_cast<uintptr_t>(C)) % 16 == 0) &&
-                   g.lda % 4 == 0 && g.ldc % 4 == 0;
+  const bool vec = ((reinterpret_cast<uintptr_t>(S) | reinterpret_cast<uintptr_t>(C)) % 16 == 0) &&
+                   lds % 4 == 0 && g.ldc % 4 == 0;
 #pragma unroll 1
   for (int r0 = 0; r0 < PER; r0 += CH) {
     float4 v[CH];
@@ -50,7 +53,7 @@ __device__ __forceinline__ void copy_tile(const GemmArgs& g, int64_t m0, int64_t
       if (r0 + r >= PER) break;
       const int f = threadIdx.x + (r0 + r) * NT;
       const int64_t gm = m0 + f / Q, gn = n0 + (f % Q) * 4;
-      const float* src = g.A + gm * g.lda + gn;
+      const float* src = S + gm * lds + gn;
       if (gm < g.M && vec && gn + 3 < g.N) {
         v[r] = *reinterpret_cast<const float4*>(src);
       } else {
@@ -109,9 +112,11 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int64_t m0, int64_t
     if (FAST_COPY) {
       copy_tile<BM, BN, NT>(g, m0, n0, C);
     } else {
+      const float* S = g.gate_mode == kGateCopyB ? g.B : g.A;
+      const int64_t lds = g.gate_mode == kGateCopyB ? g.ldb : g.lda;
       for (int idx = tid; idx < BM * BN; idx += NT) {
         const int64_t gm = m0 + idx / BN, gn = n0 + idx % BN;
-        if (gm < g.M && gn < g.N) C[gm * g.ldc + gn] = g.A[gm * g.lda + gn];
+        if (gm < g.M && gn < g.N) C[gm * g.ldc + gn] = S[gm * lds + gn];
       }
     }
     return;
@@ -694,7 +699,8 @@ cudaError_t gemm_f32_ex(bool transA, int64_t M, int64_t N, int64_t K, const floa
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (lower_only && (M != N || use_wide(M, N, K))) return cudaErrorInvalidValue;
   if (gate != nullptr && gate_mode == kGateCopy && (transA || K != N)) return cudaErrorInvalidValue;
-  if (gate != nullptr && gate_mode == kGateCopy) splits = 1;
+  if (gate != nullptr && gate_mode == kGateCopyB && (transA || M != K)) return cudaErrorInvalidValue;
+  if (gate != nullptr && (gate_mode == kGateCopy || gate_mode == kGateCopyB)) splits = 1;
   GemmArgs g;
   g.M = M; g.N = N; g.K = K; g.A = A; g.lda = lda; g.B = B; g.ldb = ldb;
   g.sumsq = sumsq; g.gate = gate; g.gate_mode = gate_mode; g.b_upper = b_upper ? 1 : 0;

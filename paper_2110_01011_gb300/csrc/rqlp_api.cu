@@ -290,8 +290,8 @@ class Ops {
       const int sk = gemm_f32_splits(d_, d_, d_);
       CK(gemm_f32_ex(false, d_, d_, d_, R_[1], ld_, R_[0], ld_, Ra_, ld_, sk, part_, nullptr, nullptr,
                      kGateNone, true, st_));
-      CK(gemm_f32_ex(false, d_, d_, d_, R_[2], ld_, Ra_, ld_, Racc, ld_, sk, part_, nullptr, nullptr,
-                     kGateNone, true, st_));
+      CK(gemm_f32_ex(false, d_, d_, d_, R_[2], ld_, Ra_, ld_, Racc, ld_, 1, nullptr, nullptr, g, kGateCopyB, true,
+                     st_));
     }
     return cudaSuccess;
   }
