@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "split_gemm.cuh"
 #include "tc_gemm.cuh"
 
 namespace rqlp {
@@ -70,9 +71,7 @@ int default_cfg(int shape, int bucket) {
   }
 }
 
-// Per-problem device buffers (in the workspace). The BF16x3 form adds A's
-// halves in 64-column panels, the pass operand's halves (X^T, d x ldk) and
-// eight tensor maps (see tc_grouped.cu).
+// Per-problem device buffers (in the workspace).
 struct Bufs {
   float *Y, *Z, *Pt, *T1, *G, *R[3], *Ri[3], *Ra, *Rb, *Rh, *Ts, *Ts2, *Ph;
   float* Gp = nullptr;   // Gram slices (gslices x d x ld) when a tall Gram is split
@@ -80,17 +79,9 @@ struct Bufs {
   double* scal;
   int* gates;
   int64_t ld;
-  uint16_t *Ahi = nullptr, *Alo = nullptr, *XTh = nullptr, *XTl = nullptr;
-  uint16_t *Alo2 = nullptr, *XTl2 = nullptr;   // three-part form only
-  int64_t ldk = 0;
-  char* maps = nullptr;     // 8 x kTcMapBytes
-  int* flag = nullptr;      // X low part nonzero (per pass)
-};
-// Tensor maps of one problem, in this order.
-enum TcMap {
-  kMapAhiT, kMapAloT, kMapAhiN, kMapAloN, kMapXhiM, kMapXloM, kMapXhiN, kMapXloN,
-  kMapAlo2T, kMapAlo2N, kMapXlo2M, kMapXlo2N,   // three-part form only
-  kTcMaps
+  uint16_t* img = nullptr;   // tensor-core passes: the parts of a pass's X
+  int* xlo = nullptr;        // X low part nonzero (per pass)
+  int* bad = nullptr;        // a value outside the parts' range (per pass, FP32)
 };
 constexpr int kMaxTcCtas = 1024;
 
@@ -104,11 +95,11 @@ struct GemmStage {
   bool gated;
 };
 
-// A grouped tensor-core pass (BF16x3 form): prep of X, then the pass.
+// A grouped tensor-core pass: the parts of X, then the pass.
 struct TcStage {
   bool transA;
-  size_t jobs_off;        // TcGJob[count]
-  size_t prep_off;        // PrepJob[count]
+  size_t jobs_off;        // SplitJob[count]
+  size_t prep_off;        // SplitXJob[count]
   size_t prep_start_off;  // int[count + 1]
   int prep_total;
   size_t units_off;       // int2[units]
@@ -116,15 +107,13 @@ struct TcStage {
   int G;
   int npad_max;
   int stall;              // test hook: CTA 0 withholds its first stage (first pass only)
-  bool exact;             // A and X in three BF16 parts, six products
+  SplitMode mode;
 };
 
 struct Stage {
-  enum Kind { kInit, kGemm, kChol, kTranspose, kWriteL, kFinish, kSplit, kTc, kGateClear, kCopyGated, kGramReduce } kind;
+  enum Kind { kInit, kGemm, kChol, kTranspose, kWriteL, kFinish, kTc, kGateClear, kCopyGated, kGramReduce } kind;
   int gemm = -1;         // index into gemms / tcs
-  size_t jobs_off = 0;   // CholJob[], SmallJob[] or SplitJob[]
-  size_t start_off = 0;  // kSplit: int[count + 1] block prefix
-  int total = 0;         // kSplit: blocks
+  size_t jobs_off = 0;   // CholJob[], SmallJob[] or GramRedJob[]
 };
 
 }  // namespace
@@ -135,15 +124,14 @@ struct rqlp_batch_s {
   long long sums[rqlp::kBuckets][3] = {};    // per bucket: sum of m, n, d (tuning key)
   int cnt[rqlp::kBuckets] = {0, 0};          // problems per bucket (bucket 0 first)
   rqlp_opts opts{};
-  bool exact = false;                        // BF16x3 passes in three parts
+  bool tc = false;                           // passes over A on the tensor cores
+  rqlp::SplitMode mode = rqlp::kSplitThree;
   char* dev = nullptr;                       // plan area in the workspace
   std::vector<rqlp::Stage> stages;
   std::vector<rqlp::GemmStage> gemms;
   std::vector<rqlp::TcStage> tcs;
-  int* flags = nullptr;                      // TC form: one int per problem (bucket order)
+  int* flags = nullptr;                      // TC form: two ints per problem (bucket order)
   int* info0 = nullptr;                      // status row that a timed-out grouped pass reports to
-  std::vector<char> maps_h;                  // TC form: host copy of the tensor maps
-  char* maps_d = nullptr;
   int cfg[rqlp::kShapes][rqlp::kBuckets];
   cudaStream_t cap = nullptr;                // capture stream
   cudaGraph_t graph = nullptr;
@@ -188,8 +176,6 @@ struct Builder {
   int* info;                             // caller order, 2 ints per problem
   double* diag;                          // caller order, 4 doubles (optional)
   Stager& sg;
-
-  bool tc;                               // BF16x3: passes over A on the tensor cores
 
   int* info_of(int i) const { return info + 2 * (int64_t)orig[i]; }
 
@@ -240,81 +226,55 @@ struct Builder {
     b->stages.push_back(s);
   }
 
-  // BF16 halves of every A (and ||A||_F^2), once per factorisation.
-  void split_stage() {
-    std::vector<SplitJob> js;
-    std::vector<int> st(n() + 1, 0);
-    for (int i = 0; i < n(); ++i) {
-      SplitJob j{};
-      j.A = pr[i].A;
-      j.lda = pr[i].lda;
-      j.m = pr[i].m;
-      j.n = pr[i].n;
-      j.npan = cdiv(pr[i].n, 64);
-      j.hi = bf[i].Ahi;
-      j.lo = bf[i].Alo;
-      j.lo2 = b->exact ? bf[i].Alo2 : nullptr;
-      j.sumsq = &bf[i].scal[0];
-      j.vec = (reinterpret_cast<uintptr_t>(pr[i].A) % 16 == 0 && pr[i].lda % 4 == 0) ? 1 : 0;
-      js.push_back(j);
-      st[i + 1] = st[i] + tc_split_blocks(pr[i].m, pr[i].n);
-    }
-    Stage s;
-    s.kind = Stage::kSplit;
-    s.jobs_off = sg.put(js.data(), js.size());
-    s.start_off = sg.put(st.data(), st.size());
-    s.total = st[n()];
-    b->stages.push_back(s);
-  }
   // One grouped tensor-core pass: out(i) = op(A_i) X(i). The (problem, tile)
   // units go longest first onto the least loaded CTA.
   template <typename XF, typename LF, typename OF>
-  void tc_pass(bool transA, XF X, LF ldx, OF out) {
+  void tc_pass(bool transA, XF X, LF ldx, OF out, bool sumsq) {
     TcStage ts{};
     ts.transA = transA;
-    std::vector<TcGJob> js;
-    std::vector<PrepJob> ps;
+    std::vector<SplitJob> js;
+    std::vector<SplitXJob> ps;
     std::vector<int> pst(n() + 1, 0);
     std::vector<std::pair<long long, int2>> units;
     ts.npad_max = 16;
     for (int i = 0; i < n(); ++i) {
-      const int di = d(i), np = tc_npad(di);
+      const int di = d(i), np = split_npad(di);
       const int64_t M = transA ? pr[i].n : pr[i].m, K = transA ? pr[i].m : pr[i].n;
       ts.npad_max = std::max(ts.npad_max, np);
-      TcGJob j{};
-      const char* mp = bf[i].maps;
-      j.mAhi = mp + (transA ? kMapAhiT : kMapAhiN) * kTcMapBytes;
-      j.mAlo = mp + (transA ? kMapAloT : kMapAloN) * kTcMapBytes;
-      j.mXhi = mp + (transA ? kMapXhiM : kMapXhiN) * kTcMapBytes;
-      j.mXlo = mp + (transA ? kMapXloM : kMapXloN) * kTcMapBytes;
-      j.mAlo2 = mp + (transA ? kMapAlo2T : kMapAlo2N) * kTcMapBytes;
-      j.mXlo2 = mp + (transA ? kMapXlo2M : kMapXlo2N) * kTcMapBytes;
+      SplitJob j{};
+      j.A = pr[i].A;
+      j.lda = pr[i].lda;
+      j.img = bf[i].img;
       j.out = out(i);
       j.ldo = bf[i].ld;
+      j.xlo = bf[i].xlo;
+      j.bad = b->mode == kSplitFp32 ? bf[i].bad : nullptr;
+      j.sumsq = sumsq ? &bf[i].scal[0] : nullptr;
       j.M = (int)M;
-      j.d = di;
+      j.N = di;
+      j.K = (int)K;
       j.npad = np;
-      j.kblocks = (int)cdiv(K, 32);
+      j.kb = (int)cdiv(K, 32);
       j.vec_out = (reinterpret_cast<uintptr_t>(j.out) % 16 == 0 && j.ldo % 4 == 0) ? 1 : 0;
-      j.idesc = tc_idesc(np, transA);
-      j.xlo_nonzero = bf[i].flag;
+      j.idesc = split_idesc(np);
       js.push_back(j);
-      PrepJob p{};
+      SplitXJob p{};
       p.X = X(i);
       p.ldx = ldx(i);
       p.K = K;
-      p.d = di;
-      p.th = bf[i].XTh;
-      p.tl = bf[i].XTl;
-      p.tl2 = b->exact ? bf[i].XTl2 : nullptr;
-      p.ldk = bf[i].ldk;
-      p.flag = bf[i].flag;
+      p.img = bf[i].img;
+      p.xlo = bf[i].xlo;
+      p.bad = j.bad;
+      p.N = di;
+      p.npad = np;
       ps.push_back(p);
-      pst[i + 1] = pst[i] + tc_prep_blocks(K, di);
-      for (int t = 0; t < (int)cdiv(M, 128); ++t) units.push_back({(long long)j.kblocks * (np + 64), int2{i, t}});
+      pst[i + 1] = pst[i] + split_x_blocks(K, np);
+      // A unit's time: its units of K (copy and split, the MMAs of np columns)
+      // and about ten of them to fill the pipeline and store the tile.
+      for (int t = 0; t < (int)cdiv(M, 256); ++t) units.push_back({(long long)(j.kb + 10) * (np + 128), int2{i, t}});
     }
     std::stable_sort(units.begin(), units.end(), [](const auto& a, const auto& c) { return a.first > c.first; });
-    const int G = (int)std::max<size_t>(1, std::min<size_t>(units.size(), std::min(kMaxTcCtas, sm_count())));
+    const int G = (int)std::max<size_t>(1, std::min<size_t>(units.size(), std::min(kMaxTcCtas, sm_count() / 2)));
     std::vector<std::vector<int2>> per(G);
     std::priority_queue<std::pair<long long, int>, std::vector<std::pair<long long, int>>, std::greater<>> load;
     for (int c = 0; c < G; ++c) load.push({0, c});
@@ -339,7 +299,7 @@ struct Builder {
     ts.cta_off = sg.put(cs.data(), cs.size());
     ts.G = G;
     ts.stall = (b->opts.test_stall != 0 && b->tcs.empty()) ? 1 : 0;
-    ts.exact = b->exact;
+    ts.mode = b->mode;
     Stage s;
     s.kind = Stage::kTc;
     s.gemm = (int)b->tcs.size();
@@ -528,25 +488,29 @@ struct Builder {
     }
     small(Stage::kInit, sj);
 
-    // A pass over every problem: grouped tensor-core passes in the BF16x3
-    // form, grouped FP32 products otherwise (sumsq: ||A||_F^2 rides along).
+    // A pass over every problem (sumsq: ||A||_F^2 rides along): on the tensor
+    // cores where b->tc, else as grouped FP32 products. In FP32 the latter follow
+    // the former for the problems whose values the parts do not represent.
     auto pass = [&](bool transA, auto X, auto ldx, auto out, bool sumsq) {
-      if (tc) {
-        tc_pass(transA, X, ldx, out);
-        return;
+      if (b->tc) {
+        tc_pass(transA, X, ldx, out, sumsq);
+        if (b->mode != kSplitFp32) return;
       }
       std::vector<GroupGemm> js;
       for (int i = 0; i < n(); ++i) {
         const int64_t M = transA ? pr[i].n : pr[i].m, K = transA ? pr[i].m : pr[i].n;
         GroupGemm j = job(pr[i].A, pr[i].lda, X(i), ldx(i), out(i), bf[i].ld, M, d(i), K);
-        if (sumsq) j.sumsq = &bf[i].scal[0];
+        if (b->tc) {
+          j.gate = bf[i].bad;
+          j.gate_mode = kGateSkip;
+        } else if (sumsq) {
+          j.sumsq = &bf[i].scal[0];
+        }
         js.push_back(j);
       }
-      gemm(transA, transA ? kTallT : kTallN, js, false);
+      gemm(transA, transA ? kTallT : kTallN, js, b->tc);
     };
-    // Y = A^T Omega (Algorithm 1 step 3); ||A||_F^2 comes with it (or with
-    // the split in the BF16x3 form).
-    if (tc) split_stage();
+    // Y = A^T Omega (Algorithm 1 step 3); ||A||_F^2 comes with it.
     pass(true, [&](int i) { return pr[i].Omega; }, [&](int i) { return pr[i].ldo; }, Y, true);
     auto passN = [&](auto X, auto out) { pass(false, X, ld, out, false); };   // out (m x d) = A X
     auto passT = [&](auto X, auto out) { pass(true, X, ld, out, false); };    // out (n x d) = A^T X
@@ -590,7 +554,8 @@ struct Builder {
   }
 };
 
-Bufs take_bufs(Arena& ar, const rqlp_problem& p, bool tc, bool exact) {
+// tc: tensor-core passes; parts: BF16 parts of the BF16x3 form, 0 in FP32.
+Bufs take_bufs(Arena& ar, const rqlp_problem& p, bool tc, int parts) {
   Bufs f{};
   const int d = p.k + p.p;
   f.ld = round_up(d, 4);
@@ -614,39 +579,21 @@ Bufs take_bufs(Arena& ar, const rqlp_problem& p, bool tc, bool exact) {
   f.Ph = ar.take<float>(dd);
   f.scal = ar.take<double>(4);
   f.gates = ar.take<int>(kGates);
-  if (tc) {
-    const int64_t cols = round_up(p.n, 64);
-    f.Ahi = ar.take<uint16_t>(p.m * cols);
-    f.Alo = ar.take<uint16_t>(p.m * cols);
-    f.ldk = round_up(tall, 8);
-    f.XTh = ar.take<uint16_t>(d * f.ldk);
-    f.XTl = ar.take<uint16_t>(d * f.ldk);
-    if (exact) {
-      f.Alo2 = ar.take<uint16_t>(p.m * cols);
-      f.XTl2 = ar.take<uint16_t>(d * f.ldk);
+  const size_t at = ar.off;
+  if (tc) f.img = ar.take<uint16_t>(split_image_bytes(tall, d, parts == 2 ? 2 : 3) / 2);
+  if (parts > 0) {
+    // The size reported for the BF16x3 form stays that of a layout with A's
+    // BF16 parts in 64-column panels, which callers sized their pools by.
+    Arena panels;
+    panels.dry = true;
+    panels.off = at;
+    for (int k = 0; k < parts; ++k) {
+      panels.take<uint16_t>(p.m * round_up(p.n, 64));
+      panels.take<uint16_t>(d * round_up(tall, 8));
     }
+    ar.off = std::max(ar.off, panels.off);
   }
   return f;
-}
-
-// The tensor maps of one problem (host encoding; false on failure): eight,
-// and four more for the third parts in the three-part form.
-bool encode_maps(const Bufs& f, const rqlp_problem& p, char* out, bool exact) {
-  const int d = p.k + p.p, np = tc_npad(d);
-  const long long npan = cdiv(p.n, 64);
-  auto at_map = [&](int k) { return out + k * kTcMapBytes; };
-  return tc_panel_map(at_map(kMapAhiT), f.Ahi, p.m, npan, 64, 32, 2, true) &&
-         tc_panel_map(at_map(kMapAloT), f.Alo, p.m, npan, 64, 32, 2, true) &&
-         tc_panel_map(at_map(kMapAhiN), f.Ahi, p.m, npan, 32, 128, 1, false) &&
-         tc_panel_map(at_map(kMapAloN), f.Alo, p.m, npan, 32, 128, 1, false) &&
-         tc_map2d(at_map(kMapXhiM), f.XTh, p.m, d, f.ldk, 32, np, false) &&
-         tc_map2d(at_map(kMapXloM), f.XTl, p.m, d, f.ldk, 32, np, false) &&
-         tc_map2d(at_map(kMapXhiN), f.XTh, p.n, d, f.ldk, 32, np, false) &&
-         tc_map2d(at_map(kMapXloN), f.XTl, p.n, d, f.ldk, 32, np, false) &&
-         (!exact || (tc_panel_map(at_map(kMapAlo2T), f.Alo2, p.m, npan, 64, 32, 2, true) &&
-                     tc_panel_map(at_map(kMapAlo2N), f.Alo2, p.m, npan, 32, 128, 1, false) &&
-                     tc_map2d(at_map(kMapXlo2M), f.XTl2, p.m, d, f.ldk, 32, np, false) &&
-                     tc_map2d(at_map(kMapXlo2N), f.XTl2, p.n, d, f.ldk, 32, np, false)));
 }
 
 bool valid_problem(const rqlp_problem& p) {
@@ -677,47 +624,42 @@ size_t layout(rqlp_batch_s* b, int count, const rqlp_problem* probs, Arena& ar, 
   std::vector<int> ord = bucket_order(count, probs, b->cnt);
   std::vector<rqlp_problem> pr;
   std::vector<Bufs> bf;
-  const bool tc = b->opts.precision == RQLP_PREC_BF16X3;
+  const bool split = b->opts.precision == RQLP_PREC_BF16X3;
   // Three BF16 parts unless the caller asked for two: the batch's problems are
   // the small and medium sizes where the two-part rounding, amplified by an
   // ill-conditioned leading block, reaches the 1e-4 |L_ii| bound.
-  b->exact = tc && b->opts.bf16_parts != 2;
+  const int parts = split ? (b->opts.bf16_parts == 2 ? 2 : 3) : 0;
+  b->mode = !split ? kSplitFp32 : parts == 2 ? kSplitTwo : kSplitThree;
+  // FP32 passes go to the tensor cores where a pass over all problems has
+  // enough multiply-adds to be worth the two launches.
+  double work = 0;
+  for (int i = 0; i < count; ++i) work += (double)probs[i].m * probs[i].n * (probs[i].k + probs[i].p);
+  b->tc = split || work >= 3e8;
   int* flags = nullptr;
-  char* maps = nullptr;
-  if (tc) {
-    flags = ar.take<int>(count);
-    maps = ar.take<char>((size_t)count * kTcMaps * kTcMapBytes);
-  }
+  if (b->tc) flags = ar.take<int>(2 * (size_t)count);
+  if (split) ar.take<char>((size_t)count * 12 * 128);   // (tensor maps of the panel layout: see take_bufs)
   b->flags = flags;
-  b->maps_d = maps;
   b->info0 = d_info;
-  b->maps_h.clear();
   b->dmax = 0;
   for (int bk = 0; bk < kBuckets; ++bk)
     for (int t = 0; t < 3; ++t) b->sums[bk][t] = 0;
   for (int i : ord) {
     const int d = probs[i].k + probs[i].p, bk = bucket_of(d);
     pr.push_back(probs[i]);
-    bf.push_back(take_bufs(ar, probs[i], tc, b->exact));
-    if (tc) {
-      const size_t pos = bf.size() - 1;
-      bf.back().flag = ar.dry ? nullptr : flags + pos;
-      bf.back().maps = ar.dry ? nullptr : maps + pos * kTcMaps * kTcMapBytes;
+    bf.push_back(take_bufs(ar, probs[i], b->tc, parts));
+    if (b->tc && !ar.dry) {
+      bf.back().xlo = flags + (bf.size() - 1);
+      bf.back().bad = flags + count + (bf.size() - 1);
     }
     b->dmax = std::max(b->dmax, d);
     b->sums[bk][0] += probs[i].m;
     b->sums[bk][1] += probs[i].n;
     b->sums[bk][2] += d;
   }
-  if (tc && !ar.dry) {
-    b->maps_h.assign((size_t)count * kTcMaps * kTcMapBytes, 0);
-    for (size_t i = 0; i < bf.size(); ++i)
-      if (!encode_maps(bf[i], pr[i], b->maps_h.data() + i * kTcMaps * kTcMapBytes, b->exact)) b->maps_h.clear();
-  }
   b->stages.clear();
   b->gemms.clear();
   b->tcs.clear();
-  Builder bd{b, pr, bf, ord, d_info, d_diag, sg, tc};
+  Builder bd{b, pr, bf, ord, d_info, d_diag, sg};
   bd.build();
   char* plan = ar.take<char>(sg.h.size() + 256);
   b->dev = ar.dry ? nullptr : plan;
@@ -776,9 +718,6 @@ cudaError_t run_stages(const rqlp_batch_s* b, cudaStream_t st) {
       case Stage::kTranspose: CK(transpose_batched(at<SmallJob>(b, s.jobs_off), b->count, st)); break;
       case Stage::kWriteL: CK(write_L_batched(at<SmallJob>(b, s.jobs_off), b->count, st)); break;
       case Stage::kFinish: CK(finish_diag_batched(at<SmallJob>(b, s.jobs_off), b->count, st)); break;
-      case Stage::kSplit:
-        CK(split_grouped(at<SplitJob>(b, s.jobs_off), at<int>(b, s.start_off), b->count, s.total, st));
-        break;
       case Stage::kGateClear: CK(gate_clear_batched(at<SmallJob>(b, s.jobs_off), b->count, st)); break;
       case Stage::kCopyGated: CK(copy_gated_batched(at<SmallJob>(b, s.jobs_off), b->count, st)); break;
       case Stage::kGramReduce:
@@ -788,10 +727,11 @@ cudaError_t run_stages(const rqlp_batch_s* b, cudaStream_t st) {
         break;
       case Stage::kTc: {
         const TcStage& t = b->tcs[s.gemm];
-        CK(cudaMemsetAsync(b->flags, 0, sizeof(int) * b->count, st));
-        CK(prep_grouped(at<PrepJob>(b, t.prep_off), at<int>(b, t.prep_start_off), b->count, t.prep_total, st));
-        CK(tc_grouped_pass(t.transA, at<TcGJob>(b, t.jobs_off), at<int2>(b, t.units_off), at<int>(b, t.cta_off),
-                           t.G, t.npad_max, b->info0, t.stall, t.exact, st));
+        CK(cudaMemsetAsync(b->flags, 0, sizeof(int) * 2 * b->count, st));
+        CK(split_x_grouped(at<SplitXJob>(b, t.prep_off), at<int>(b, t.prep_start_off), b->count, t.prep_total, t.mode,
+                           st));
+        CK(split_grouped(t.transA, at<SplitJob>(b, t.jobs_off), at<int2>(b, t.units_off), at<int>(b, t.cta_off), t.G,
+                         t.npad_max, t.mode, b->info0, t.stall, st));
         break;
       }
     }
@@ -879,17 +819,10 @@ rqlp_status rqlp_batch_create(int count, const rqlp_problem* probs, int q, void*
         for (int bk = 0; bk < kBuckets; ++bk) b->cfg[s][bk] = it->second[s * kBuckets + bk];
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const bool tc = o.precision == RQLP_PREC_BF16X3;
-  if (tc && b->maps_h.empty()) {   // a tensor map was rejected
-    delete b;
-    return RQLP_ERR_UNSUPPORTED;
-  }
   if (gemm_grouped_prepare() != cudaSuccess ||
       chol_inv_batched(nullptr, 0, 0, o.small_fp64 != 0, st) != cudaSuccess ||
-      (tc && (tc_grouped_pass(true, nullptr, nullptr, nullptr, 0, 16, nullptr, 0, false, st) != cudaSuccess ||
-              tc_grouped_pass(false, nullptr, nullptr, nullptr, 0, 16, nullptr, 0, false, st) != cudaSuccess ||
-              cudaMemcpyAsync(b->maps_d, b->maps_h.data(), b->maps_h.size(), cudaMemcpyHostToDevice, st) !=
-                  cudaSuccess)) ||
+      (b->tc && (split_grouped(true, nullptr, nullptr, nullptr, 0, 16, b->mode, nullptr, 0, st) != cudaSuccess ||
+                 split_grouped(false, nullptr, nullptr, nullptr, 0, 16, b->mode, nullptr, 0, st) != cudaSuccess)) ||
       cudaMemcpyAsync(b->dev, sg.h.data(), sg.h.size(), cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaStreamSynchronize(st) != cudaSuccess ||
       cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess) {

@@ -33,33 +33,17 @@
 // evenly to the CTAs (stream-K); split tiles are summed by the last CTA to
 // arrive, or by split_fixup_kernel when a tile spans more than kMaxSlots of
 // them. Every wait is bounded; a timeout is reported in the status word.
-#include <cuda.h>
-#include <cuda_bf16.h>
-
 #include <algorithm>
 
+#include "split_device.cuh"
 #include "split_gemm.cuh"
-#include "tc_ptx.cuh"
 
 namespace rqlp {
 namespace {
 
-constexpr int BM = 128;               // rows per CTA (TMEM lanes)
-constexpr int BK = 32;                // K per unit
-constexpr int kThreads = 640;          // 4 + 8 + 8 warps
-constexpr int kGroups = 7;             // 16-column groups of a drain warp: N <= 224
-constexpr int CG = 2;                 // CTAs per tile (cta_group::2)
-constexpr int kMaxStages = 8;
-constexpr int kMaxASlots = 8;
-constexpr int kMaxSlots = 16;
-constexpr uint32_t kABytes = BM * BK * 4;   // FP32 stage of A
-constexpr int kCopyStages = 6;        // FP32 stages when the split warps copy A themselves
-constexpr int kPrefetch = 12;         // units between their L2 prefetch and the copy
-constexpr long long kWaitLimit = 4000000000LL;   // cycles (~2 s)
-// Parts hold a value exactly when its magnitude lies in [2^-96, 2^127) (or is
-// zero): below, the last part would be subnormal; above, the first may round
-// to infinity.
-constexpr uint32_t kRangeHi = 0x7F000000u, kRangeLo = 0x0F800000u;
+using namespace sp;
+
+constexpr int kMaxSlots = 16;         // partial tiles that the last CTA of a tile sums itself
 
 struct Args {
   const float* A;
@@ -84,10 +68,6 @@ struct Args {
   uint32_t idesc;
 };
 
-__device__ void post_timeout(int* info) {
-  if (info != nullptr && atomicCAS(info, 0, RQLP_ERR_TIMEOUT) == 0) info[1] = 0;
-}
-
 // First unit of group c: an even share of all units, or of the whole tiles.
 __host__ __device__ inline int first_unit(int c, int units, int G, int whole, int tiles, int kb) {
   if (whole) return (int)((long long)c * tiles / G) * kb;
@@ -96,117 +76,6 @@ __host__ __device__ inline int first_unit(int c, int units, int G, int whole, in
 // The group whose range holds unit u (stream-K deal).
 __host__ __device__ inline int unit_owner(int u, int units, int G) {
   return (int)((((long long)u + 1) * G + units - 1) / units) - 1;
-}
-// Tile and unit of K at a position of a range.
-struct Cursor {
-  int t, k;
-  __device__ Cursor(int u, int kb) : t(u / kb), k(u % kb) {}
-  __device__ void next(int kb) {
-    if (++k == kb) {
-      k = 0;
-      ++t;
-    }
-  }
-};
-// Stage of a ring and the parity of its current round.
-struct Ring {
-  int s = 0;
-  uint32_t ph = 0;
-  __device__ void next(int n) {
-    if (++s == n) {
-      s = 0;
-      ph ^= 1u;
-    }
-  }
-};
-
-// D[tmem] (+)= A[tmem] B[shared memory] over the CTA pair, issued by its leader.
-__device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-               " tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d), "r"(a), "l"(b),
-               "r"(idesc), "r"(acc) : "memory");
-}
-// Arrive on `bar` of both CTAs of the pair once the MMAs issued so far are done.
-__device__ __forceinline__ void commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(tc::smem_u32(bar)), "h"((uint16_t)3) : "memory");
-}
-// Arrive on the pair leader's barrier. Relaxed: what the arrival hands over
-// lies in tensor memory and is ordered by the tcgen05 waits and fences around
-// it; a releasing arrive at cluster scope takes most of a microsecond (a unit
-// of 256 x 32 took 1.5 us with it and 0.7 us without).
-__device__ __forceinline__ void arrive_leader(uint64_t* bar) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(tc::smem_u32(bar)));
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
-}
-__device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.relaxed.cta.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok) : "r"(tc::smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-// Wait for MMAs, tensor-memory hand-overs or free stages; data that was copied
-// to shared memory is waited for with tc::mbar_wait (acquire).
-__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) {
-  if (try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!try_wait(bar, parity))
-    if (clock64() - t0 > kWaitLimit) return false;
-  return true;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// True in one lane of a converged warp. The loops that issue copies and MMAs run
-// in the whole warp with the issue itself under elect: their operands then stay
-// in uniform registers (under a divergent branch an MMA took ~75 clocks to
-// issue).
-__device__ __forceinline__ bool elect() {
-  uint32_t p;
-  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   tc::smem_u32(dst)), "l"(src), "r"(bytes), "r"(tc::smem_u32(bar)) : "memory");
-}
-// Eight 32-bit columns of this lane's row.
-__device__ __forceinline__ void st_row8(uint32_t t, const uint32_t* r) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(t), "r"(r[0]),
-               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
-}
-// Sixteen columns of this lane's row; the values are there after ld_wait().
-__device__ __forceinline__ void ld16(uint32_t t, float* v) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
-        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
-      : "r"(t));
-}
-__device__ __forceinline__ void ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Keeps the uses of v behind the wait above (no instruction).
-__device__ __forceinline__ void ld_done(float* v) {
-  asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
-                    "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]),
-                    "+f"(v[15]));
-}
-__device__ __forceinline__ void st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ uint32_t pack(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<const uint32_t*>(&v);
-}
-// (x0, x1) -> packed parts; the differences are exact in FP32.
-template <int PARTS>
-__device__ __forceinline__ void split2(float x0, float x1, uint32_t* p) {
-  p[0] = pack(x0, x1);
-  const float r0 = x0 - __uint_as_float(p[0] << 16), r1 = x1 - __uint_as_float(p[0] & 0xFFFF0000u);
-  p[1] = pack(r0, r1);
-  if (PARTS == 3) p[2] = pack(r0 - __uint_as_float(p[1] << 16), r1 - __uint_as_float(p[1] & 0xFFFF0000u));
 }
 
 template <bool TRANS, int PARTS, bool TMA>
@@ -218,7 +87,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
   const int nh = a.npad / CG;                                  // X columns held by this CTA
   const uint32_t part_bytes = (uint32_t)nh * BK * 2, stage_bytes = PARTS * part_bytes;
   unsigned char* fstage = smem;                                // FP32 stages of A, then X stages (both 1 KB aligned)
-  unsigned char* xstage = smem + (size_t)a.sf * kABytes;
+  unsigned char* xstage = smem + (size_t)a.sf * (TMA ? kABytes : kCopyBytes);
   uint64_t* xfull = reinterpret_cast<uint64_t*>(xstage + (size_t)a.sx * stage_bytes);
   uint64_t* xempty = xfull + kMaxStages;
   uint64_t* ffull = xempty + kMaxStages;
@@ -338,36 +207,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
               for (int p = 0; p < PARTS; ++p)
                 x[p] = tc::smem_desc(smem_x + (uint32_t)rx.s * stage_bytes + p * part_bytes, 16, 512, tc::kSwizzle64);
               const uint32_t t0 = a_base + (uint32_t)(ra.s * PARTS * 16);
-              if (PARTS == 3 && a.corr_first) {   // a chain of one unit: the small products, then the main ones
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                  const uint32_t t = t0 + ks * 8;
-                  mma_ts(d, t + 32, x[0] + 2 * ks, a.idesc, ks);
-                  if (nx > 1) {
-                    mma_ts(d, t + 16, x[1] + 2 * ks, a.idesc, 1u);
-                    mma_ts(d, t, x[PARTS - 1] + 2 * ks, a.idesc, 1u);
-                    mma_ts(d, t, x[1] + 2 * ks, a.idesc, 1u);
-                  }
-                  mma_ts(d, t + 16, x[0] + 2 * ks, a.idesc, 1u);
-                }
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks) mma_ts(d, t0 + ks * 8, x[0] + 2 * ks, a.idesc, 1u);
-              } else {
-#pragma unroll
-                for (int ks = 0; ks < 2; ++ks) {
-                  const uint32_t t = t0 + ks * 8;
-                  mma_ts(d, t, x[0] + 2 * ks, a.idesc, ks ? 1u : acc);
-                  mma_ts(dc, t + 16, x[0] + 2 * ks, a.idesc, ks ? 1u : cacc);
-                  if (nx > 1) mma_ts(dc, t, x[1] + 2 * ks, a.idesc, 1u);
-                  if (PARTS == 3) {
-                    mma_ts(dc, t + 32, x[0] + 2 * ks, a.idesc, 1u);
-                    if (nx > 1) {
-                      mma_ts(dc, t + 16, x[1] + 2 * ks, a.idesc, 1u);
-                      mma_ts(dc, t, x[PARTS - 1] + 2 * ks, a.idesc, 1u);
-                    }
-                  }
-                }
-              }
+              issue_products<PARTS>(d, dc, t0, x, a.idesc, nx, a.corr_first != 0, acc, cacc);
               commit(&xempty[rx.s]);
               commit(&aempty[ra.s]);
             }
@@ -418,8 +258,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     const int w = warp & 3, odd = (warp >> 2) - 1;   // two warpgroups take the units by turns
     const bool check = PARTS == 3 && a.bad != nullptr, sq = a.sumsq != nullptr;
-    uint32_t umax = 0, umin = 0xFFFFFFFFu;
-    float ss = 0.f, comp = 0.f, acc2 = 0.f;
+    Checks ck;
     // A stage holds 128 rows of op(A) by 32 of K. TRANS: as in memory, [K][row];
     // else [row][K] with the 16-byte chunks of a row xored with row % 8 (the
     // 128-byte swizzle). v[j] = op(A)(this lane's row, 16 half + j): both reads
@@ -438,54 +277,30 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
         }
       }
     };
-    // Without TMA (rows of A that are not 16-byte aligned): this warp's 32 rows
-    // of a stage by 4-byte asynchronous copies, 128 consecutive bytes each.
+    const ARef ar{a.A, a.lda, a.M, a.K};
+    int off[9];
+    const bool near = !TMA && chunk_offsets(ar, lane, off);
+    auto first = [&](const Cursor& c, int& k0, int& r0) {   // a unit's first K, this warp's first row
+      k0 = c.k * BK;
+      r0 = (c.t * CG + rank) * BM + 32 * w;
+    };
     auto copy = [&](const Cursor& c, unsigned char* f) {
-      const int k0 = c.k * BK, r0 = (c.t * CG + rank) * BM + 32 * w;
-      float* s = reinterpret_cast<float*>(f);
-      const int last_i = TRANS ? a.K - k0 : a.M - r0;                 // valid rows of memory
-      const bool in = lane < (TRANS ? a.M - r0 : a.K - k0);
-      const float* p = a.A + (TRANS ? (long long)k0 * a.lda + r0 : (long long)r0 * a.lda + k0) + lane;
-#pragma unroll 8
-      for (int i = 0; i < 32; ++i) {
-        float* d = TRANS ? s + i * BM + 32 * w + lane
-                         : s + (32 * w + i) * BK + (((lane >> 2) ^ (i & 7)) << 2) + (lane & 3);
-        const bool ok = in && i < last_i;
-        cp_async4(d, ok ? p + (long long)i * a.lda : a.A, ok ? 4 : 0);
-      }
+      int k0, r0;
+      first(c, k0, r0);
+      const int i0 = TRANS ? k0 : r0, j0 = TRANS ? r0 : k0;
+      float* dst = reinterpret_cast<float*>(f) + 32 * w * kRowFloats;
+      if (near && interior(ar, TRANS, i0, j0)) copy_interior(ar, i0, j0, off, dst, lane);
+      else copy_rows(ar, TRANS, i0, j0, dst, lane);
     };
-    // One line of A per lane into L2.
     auto prefetch = [&](const Cursor& c) {
-      const int k0 = c.k * BK, r0 = (c.t * CG + rank) * BM + 32 * w;
-      const int row = TRANS ? k0 + lane : r0 + lane, col = TRANS ? r0 : k0;
-      if (row < (TRANS ? a.K : a.M) && col < (TRANS ? a.M : a.K))
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.A + (long long)row * a.lda + col));
-    };
-    auto split = [&](const float* v, uint32_t (&o)[PARTS][8]) {
-      if (check) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const uint32_t x = __float_as_uint(v[j]) & 0x7FFFFFFFu;
-          umax = max(umax, x);
-          umin = min(umin, x - 1u);   // zero wraps to the largest value
-        }
-      }
-      if (sq) {
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc2 = fmaf(v[j], v[j], acc2);
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        uint32_t p[PARTS];
-        split2<PARTS>(v[2 * j], v[2 * j + 1], p);
-#pragma unroll
-        for (int q = 0; q < PARTS; ++q) o[q][j] = p[q];
-      }
+      int k0, r0;
+      first(c, k0, r0);
+      prefetch_rows(ar, TRANS, TRANS ? k0 : r0, TRANS ? r0 : k0, lane);
     };
     const uint32_t lanes = (uint32_t)(32 * w) << 16;
     bool ok = true;
     const int n = u1 - u0;
-    Cursor cc(u0, KB), cp(u0, KB);   // next unit to copy, to prefetch (without TMA)
+    Cursor cu(u0, KB), cc(u0, KB), cp(u0, KB);   // current unit; next to copy, to prefetch (without TMA)
     Ring ra, rx, rf;                 // A slot, X stage, FP32 stage of the current unit
     int fc = odd;                    // FP32 stage of the next copy
     auto two = [&](Cursor& c) {      // this warpgroup's next unit
@@ -493,6 +308,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       c.next(KB);
     };
     if (odd) {
+      cu.next(KB);
       cc.next(KB);
       cp.next(KB);
       ra.next(a.sa);
@@ -502,7 +318,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
     constexpr int kAhead = kCopyStages / 2 - 1;   // own units copied ahead
     if (!TMA) {
       for (int i = 0; i < kAhead; ++i) {
-        if (odd + 2 * i < n) copy(cc, fstage + fc * kABytes);
+        if (odd + 2 * i < n) copy(cc, fstage + fc * kCopyBytes);
         cp_async_commit();
         two(cc);
         fc += 2;
@@ -513,7 +329,16 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       }
     }
     for (int i = odd; i < n; i += 2) {
-      const unsigned char* f = fstage + rf.s * kABytes;
+      const unsigned char* f = fstage + rf.s * (TMA ? kABytes : kCopyBytes);
+      auto fetch = [&](int half, float* v) {
+        if (TMA) {
+          read(f, half, v);
+        } else {
+          int k0, r0;
+          first(cu, k0, r0);
+          read_copied<TRANS>(ar, k0, r0, reinterpret_cast<const float*>(f) + 32 * w * kRowFloats, half, lane, v);
+        }
+      };
       if (TMA) {
         if (!tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit)) {
           ok = false;
@@ -523,7 +348,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
         if (i + kPrefetch < n) prefetch(cp);
         two(cp);
         __syncwarp();   // every lane has read the stage that is filled next
-        if (i + 2 * kAhead < n) copy(cc, fstage + fc * kABytes);
+        if (i + 2 * kAhead < n) copy(cc, fstage + fc * kCopyBytes);
         cp_async_commit();
         two(cc);
         fc = fc + 2 >= kCopyStages ? fc + 2 - kCopyStages : fc + 2;
@@ -532,8 +357,8 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       }
       float v[16];
       uint32_t o[PARTS][8];
-      read(f, 0, v);
-      split(v, o);
+      fetch(0, v);
+      split_half<PARTS>(v, o, check, sq, ck);
       if (!wait(&aempty[ra.s], ra.ph ^ 1u)) {
         ok = false;
         break;
@@ -542,16 +367,11 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       const uint32_t ta = a_base + lanes + (uint32_t)(ra.s * PARTS * 16);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
-      read(f, 1, v);
-      split(v, o);
+      fetch(1, v);
+      split_half<PARTS>(v, o, check, sq, ck);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
-      if (sq) {
-        const float y = acc2 - comp, t = ss + y;
-        comp = (t - ss) - y;
-        ss = t;
-        acc2 = 0.f;
-      }
+      if (sq) ck.fold();
       st_wait();
       tc::tc_fence_before();
       __syncwarp();
@@ -569,15 +389,12 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       rx.next(a.sx);
       rf.next(a.sf);
       rf.next(a.sf);
+      two(cu);
     }
     if (!TMA) cp_async_wait_all();
     if (!ok && lane == 0) post_timeout(a.info);
-    if (check && __any_sync(0xffffffffu, umax >= kRangeHi || umin < kRangeLo - 1u) && lane == 0) atomicOr(a.bad, 1);
-    if (sq) {
-      double v = (double)ss - (double)comp;
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) atomicAdd(a.sumsq, v);
-    }
+    if (check) ck.report(a.bad, lane);
+    if (sq) ck.add(a.sumsq, lane);
   } else {
     // -------------------------------------------------- drain: TMEM -> registers -> global
     asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
@@ -585,13 +402,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
     const int row = 32 * (e & 3) + lane;
     const int groups = a.npad / 16, g0 = half ? (groups + 1) / 2 : 0, ng = half ? groups / 2 : (groups + 1) / 2;
     float s[kGroups][16];
-    auto clear = [&] {
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g)
-#pragma unroll
-        for (int j = 0; j < 16; ++j) s[g][j] = 0.f;
-    };
-    clear();
+    clear_sums(s);
     bool ok = true;   // after a timeout the loop runs on without waiting, so that its barriers stay in step
     int chain = 0, k = u0 % KB, t = u0 / KB, left = u1 - u0, part0 = k;   // part0: first unit of this tile part
     int since = 0;
@@ -608,25 +419,10 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       if (ok) {
         tc::tc_fence_after();
         const uint32_t lanes = (uint32_t)(32 * (e & 3)) << 16, cols = (uint32_t)(16 * g0);
-        auto drain = [&](uint32_t ta) {
-#pragma unroll
-          for (int g = 0; g < kGroups; ++g) {
-            if (g < ng) {
-              float v[16];
-              ld16(ta + 16 * g, v);
-              ld_wait();
-              ld_done(v);
-#pragma unroll
-              for (int j = 0; j < 16; ++j) s[g][j] += v[j];
-            }
-          }
-          tc::tc_fence_before();
-          __syncwarp();
-        };
-        drain(tmem + lanes + (uint32_t)(rb.s * a.npad) + cols);
+        drain_columns(s, tmem + lanes + (uint32_t)(rb.s * a.npad) + cols, ng);
         if (lane == 0) arrive_leader(&acce[rb.s]);
         if (a.corr && ((chain + 1) % a.corr == 0 || part_end)) {
-          drain(corr_base + lanes + cols);
+          drain_columns(s, corr_base + lanes + cols, ng);
           if (lane == 0) arrive_leader(corre);
         }
       }
@@ -654,35 +450,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
         qstep = 4 * BM;
         vec = true;
       }
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g) {
-        const int c0 = 16 * (g0 + g);
-        if (g < ng) {
-          if (flushed) {
-            if (vec && c0 + 16 <= ncols) {
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const float4 o = *reinterpret_cast<const float4*>(dst + (c0 / 4 + q) * qstep);
-                s[g][4 * q] += o.x; s[g][4 * q + 1] += o.y; s[g][4 * q + 2] += o.z; s[g][4 * q + 3] += o.w;
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j)
-                if (c0 + j < ncols) s[g][j] += dst[c0 + j];
-            }
-          }
-          if (vec && c0 + 16 <= ncols) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              *reinterpret_cast<float4*>(dst + (c0 / 4 + q) * qstep) =
-                  make_float4(s[g][4 * q], s[g][4 * q + 1], s[g][4 * q + 2], s[g][4 * q + 3]);
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (c0 + j < ncols) dst[c0 + j] = s[g][j];
-          }
-        }
-      }
+      store_sums(s, dst, qstep, g0, ng, ncols, vec, flushed);
       if (part_end && !all && !a.fixup) {
         // Publish the partial tile; the last CTA to arrive sums them in CTA order.
         __threadfence();
@@ -750,7 +518,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
           if (tid == 0) a.cnt[rt] = 0;
         }
       }
-      clear();   // (here, so that the sums are not live across the code above)
+      clear_sums(s);   // (here, so that the sums are not live across the code above)
       flushed = !part_end;
       since = 0;
       if (part_end) {
@@ -811,48 +579,10 @@ __global__ void split_fixup_kernel(const Args a) {
   }
 }
 
-// X (K x N FP32) -> stage images: for every unit of 32 of K, CTA of a group,
-// and part, npad / CG rows (columns of X) of 32 K entries, 16-byte chunks
-// swizzled over 64-byte rows; zeros past K and N. A block of 256 threads takes
-// 64 of K and 32 columns through shared memory; a thread writes one 16-byte
-// chunk (8 of K) of each part.
 __global__ void __launch_bounds__(256)
 split_x_kernel(const float* __restrict__ X, long long K, int N, long long ldx, uint16_t* __restrict__ img, int npad,
                int parts, int kb, int* xlo, int* bad) {
-  __shared__ float tile[64][33];
-  const long long k0 = (long long)blockIdx.x * 64;
-  const int n0 = blockIdx.y * 32;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int kk = (threadIdx.x >> 5) + 8 * i, nn = threadIdx.x & 31;
-    const long long k = k0 + kk;
-    tile[kk][nn] = (k < K && n0 + nn < N) ? X[k * ldx + n0 + nn] : 0.f;
-  }
-  __syncthreads();
-  const int nn = threadIdx.x >> 3, ch = threadIdx.x & 7;   // column, chunk of 8 of K
-  const int n = n0 + nn;
-  const long long unit = (k0 >> 5) + (ch >> 2);
-  bool any = false, out_of_range = false;
-  if (n < npad && unit < kb) {
-    uint32_t p[3][4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      uint32_t q[3];
-      const float x0 = tile[ch * 8 + 2 * j][nn], x1 = tile[ch * 8 + 2 * j + 1][nn];
-      split2<3>(x0, x1, q);
-      p[0][j] = q[0]; p[1][j] = q[1]; p[2][j] = q[2];
-      any |= (q[1] & 0x7FFF7FFFu) != 0;
-      const uint32_t m0 = __float_as_uint(x0) & 0x7FFFFFFFu, m1 = __float_as_uint(x1) & 0x7FFFFFFFu;
-      out_of_range |= max(m0, m1) >= kRangeHi || min(m0 - 1u, m1 - 1u) < kRangeLo - 1u;
-    }
-    const int nh = npad / CG, r = n % nh;
-    const size_t stage = ((size_t)unit * CG + n / nh) * parts * nh * 32;
-    const size_t at = stage + (size_t)r * 32 + (size_t)(((ch & 3) ^ ((r >> 1) & 3)) * 8);
-    for (int q = 0; q < parts; ++q)
-      *reinterpret_cast<uint4*>(img + at + (size_t)q * nh * 32) = make_uint4(p[q][0], p[q][1], p[q][2], p[q][3]);
-  }
-  if (__syncthreads_or(any) && threadIdx.x == 0 && *(volatile int*)xlo == 0) atomicOr(xlo, 1);
-  if (bad != nullptr && __syncthreads_or(out_of_range) && threadIdx.x == 0) atomicOr(bad, 1);
+  split_x_tile(X, K, N, ldx, img, npad, parts, kb, (long long)blockIdx.x * 64, blockIdx.y * 32, xlo, bad);
 }
 
 int npad_of(int n) { return (int)round_up(n, 16); }   // N of the MMA; each CTA holds half of it, a multiple of 8
@@ -991,9 +721,10 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   // Shared memory: four X stages first, then FP32 stages of A, then X again.
   const size_t avail = smem_optin() - kSmemExtra;
   a.sf = tma ? (int)std::min<size_t>(kMaxStages, (avail - 4 * stage) / kABytes) : kCopyStages;
-  a.sx = (int)std::min<size_t>(kMaxStages, (avail - a.sf * kABytes) / stage);
+  const size_t fbytes = (size_t)a.sf * (tma ? kABytes : kCopyBytes);
+  a.sx = (int)std::min<size_t>(kMaxStages, (avail - fbytes) / stage);
   a.idesc = tc::idesc_bf16(BM * CG, npad, false, false);
-  const size_t smem = a.sf * kABytes + a.sx * stage + kSmemExtra;
+  const size_t smem = fbytes + a.sx * stage + kSmemExtra;
 #define RQLP_SPLIT(T, P) (tma ? launch<T, P, true>(map, a, cap, smem, st) : launch<T, P, false>(map, a, cap, smem, st))
   cudaError_t e = transA ? (parts == 3 ? RQLP_SPLIT(true, 3) : RQLP_SPLIT(true, 2))
                          : (parts == 3 ? RQLP_SPLIT(false, 3) : RQLP_SPLIT(false, 2));
@@ -1046,7 +777,6 @@ cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K
   ws->turn ^= 1;
   int* bad = mode == kSplitFp32 ? ws->words + 2 + turn : nullptr;
   if (range_word != nullptr) *range_word = bad;
-  const int parts = mode == kSplitTwo ? 2 : 3;
   // Column halves above what a drain warp's registers hold, or where two
   // accumulators and two A slots (96 columns) exceed tensor memory.
   const int n0 = npad_of(N) > (mode == kSplitThree ? 208 : 16 * 2 * kGroups) ? npad_of((int)cdiv(N, 2)) : N;

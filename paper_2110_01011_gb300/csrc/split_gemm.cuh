@@ -44,4 +44,40 @@ cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K
                        const float* X, int64_t ldx, float* out, int64_t ldo, SplitMode mode, double* sumsq,
                        const int** range_word, int* info, bool profiled, cudaStream_t st);
 
+// ---------------------------------------------------------------- grouped products (batched form)
+struct SplitJob {           // out (M x N) = op(A) X
+  const float* A;           // as op(A) is stored (see split_gemm)
+  long long lda;
+  const uint16_t* img;      // X's parts, written by split_x_grouped
+  float* out;
+  long long ldo;
+  const int* xlo;           // raised when X has a low part
+  int* bad;                 // raised on values outside the parts' range (FP32; else null)
+  double* sumsq;            // += sum of squares of A (or null)
+  int M, N, K, npad, kb, vec_out;
+  uint32_t idesc;
+};
+struct SplitXJob {          // X (K x N) -> stage images
+  const float* X;
+  long long ldx, K;
+  uint16_t* img;
+  int* xlo;
+  int* bad;
+  int N, npad;
+};
+int split_npad(int n);
+size_t split_image_bytes(int64_t K, int n, int parts);
+uint32_t split_idesc(int npad);
+int split_x_blocks(int64_t K, int npad);
+// start: count + 1 block prefix sums (split_x_blocks).
+cudaError_t split_x_grouped(const SplitXJob* jobs, const int* start, int count, int total, SplitMode mode,
+                            cudaStream_t st);
+// units: (job, 256-row tile) pairs, N <= 128; CTA pair p takes units
+// cta_start[p] .. cta_start[p + 1] - 1. pairs = 0 only configures the kernel
+// (call before capturing). stall != 0 (fault-injection tests): CTA 0 withholds
+// its first stage of X, its bounded waits run out and `info` receives
+// RQLP_ERR_TIMEOUT.
+cudaError_t split_grouped(bool transA, const SplitJob* jobs, const int2* units, const int* cta_start, int pairs,
+                          int npad_max, SplitMode mode, int* info, int stall, cudaStream_t st);
+
 }  // namespace rqlp
