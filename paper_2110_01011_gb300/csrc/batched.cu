@@ -125,6 +125,7 @@ struct rqlp_batch_s {
   int cnt[rqlp::kBuckets] = {0, 0};          // problems per bucket (bucket 0 first)
   rqlp_opts opts{};
   bool tc = false;                           // passes over A on the tensor cores
+  bool maps_ok = true;                       // their tensor maps were encoded
   rqlp::SplitMode mode = rqlp::kSplitThree;
   char* dev = nullptr;                       // plan area in the workspace
   std::vector<rqlp::Stage> stages;
@@ -234,6 +235,7 @@ struct Builder {
     ts.transA = transA;
     std::vector<SplitJob> js;
     std::vector<SplitXJob> ps;
+    std::vector<char> ts_maps;
     std::vector<int> pst(n() + 1, 0);
     std::vector<std::pair<long long, int2>> units;
     ts.npad_max = 16;
@@ -242,8 +244,9 @@ struct Builder {
       const int64_t M = transA ? pr[i].n : pr[i].m, K = transA ? pr[i].m : pr[i].n;
       ts.npad_max = std::max(ts.npad_max, np);
       SplitJob j{};
-      j.A = pr[i].A;
-      j.lda = pr[i].lda;
+      alignas(64) char maps[kSplitMapBytes];
+      if (bf[i].img != nullptr && !split_job_maps(maps, &j, pr[i].A, pr[i].m, pr[i].n, pr[i].lda, transA)) b->maps_ok = false;
+      ts_maps.insert(ts_maps.end(), maps, maps + kSplitMapBytes);
       j.img = bf[i].img;
       j.out = out(i);
       j.ldo = bf[i].ld;
@@ -252,7 +255,6 @@ struct Builder {
       j.sumsq = sumsq ? &bf[i].scal[0] : nullptr;
       j.M = (int)M;
       j.N = di;
-      j.K = (int)K;
       j.npad = np;
       j.kb = (int)cdiv(K, 32);
       j.vec_out = (reinterpret_cast<uintptr_t>(j.out) % 16 == 0 && j.ldo % 4 == 0) ? 1 : 0;
@@ -291,6 +293,8 @@ struct Builder {
       flat.insert(flat.end(), per[c].begin(), per[c].end());
     }
     for (int c = G; c <= kMaxTcCtas; ++c) cs[c] = (int)flat.size();
+    const size_t maps_off = sg.put(ts_maps.data(), ts_maps.size());
+    for (int i = 0; i < n(); ++i) js[i].maps = b->dev + maps_off + i * kSplitMapBytes;
     ts.jobs_off = sg.put(js.data(), js.size());
     ts.prep_off = sg.put(ps.data(), ps.size());
     ts.prep_start_off = sg.put(pst.data(), pst.size());
@@ -659,10 +663,10 @@ size_t layout(rqlp_batch_s* b, int count, const rqlp_problem* probs, Arena& ar, 
   b->stages.clear();
   b->gemms.clear();
   b->tcs.clear();
+  b->dev = ar.take<char>(0);   // the plan area (null when only measuring): its tables point into it
   Builder bd{b, pr, bf, ord, d_info, d_diag, sg};
   bd.build();
-  char* plan = ar.take<char>(sg.h.size() + 256);
-  b->dev = ar.dry ? nullptr : plan;
+  ar.take<char>(sg.h.size() + 256);
   return ar.off;
 }
 
@@ -819,6 +823,10 @@ rqlp_status rqlp_batch_create(int count, const rqlp_problem* probs, int q, void*
         for (int bk = 0; bk < kBuckets; ++bk) b->cfg[s][bk] = it->second[s * kBuckets + bk];
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (!b->maps_ok) {   // a tensor map was rejected
+    delete b;
+    return RQLP_ERR_UNSUPPORTED;
+  }
   if (gemm_grouped_prepare() != cudaSuccess ||
       chol_inv_batched(nullptr, 0, 0, o.small_fp64 != 0, st) != cudaSuccess ||
       (b->tc && (split_grouped(true, nullptr, nullptr, nullptr, 0, 16, b->mode, nullptr, 0, st) != cudaSuccess ||

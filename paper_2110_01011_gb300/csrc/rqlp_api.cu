@@ -177,7 +177,7 @@ class Ops {
   cudaError_t product32(bool transA, int64_t M, int64_t K, const float* A, int64_t lda, const float* X, int64_t ldx,
                         float* out, int64_t ldout, double* sumsq) {
     const int* word = nullptr;
-    if (split32_ && split_pays(M, K, d_)) {
+    if (split32_ && split_pays(M, K, d_) && tc_supported(A, lda, X, ldx)) {
       CK(split_gemm(&sg_, transA, M, d_, K, A, lda, X, ldx, out, ldout, kSplitFp32, sumsq, &word, info_, false, st_));
       sumsq = nullptr;
     }

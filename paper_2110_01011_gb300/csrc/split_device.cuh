@@ -20,10 +20,6 @@ constexpr int kGroups = 7;            // 16-column groups of a drain warp: N <= 
 constexpr int kMaxStages = 8;
 constexpr int kMaxASlots = 8;
 constexpr uint32_t kABytes = BM * BK * 4;        // FP32 stage of A by TMA
-constexpr int kRowFloats = BK + 4;               // a row of a stage copied by the split warps: nine 16-byte chunks
-constexpr uint32_t kCopyBytes = BM * kRowFloats * 4;   // such a stage (18 KB)
-constexpr int kCopyStages = 6;
-constexpr int kPrefetch = 12;         // units between the L2 prefetch and the copy
 constexpr long long kWaitLimit = 4000000000LL;   // cycles (~2 s)
 // Parts hold a value exactly when its magnitude lies in [2^-96, 2^127) (or is
 // zero): below, the last part would be subnormal; above, the first may round
@@ -72,10 +68,18 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
 // lies in tensor memory and is ordered by the tcgen05 waits and fences around
 // it; a releasing arrive at cluster scope takes most of a microsecond (a unit
 // of 256 x 32 took 1.5 us with it and 0.7 us without).
-__device__ __forceinline__ void arrive_leader(uint64_t* bar) {
+__device__ __forceinline__ uint32_t leader_addr(const void* p) {   // p's place in the leader's shared memory
   uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(tc::smem_u32(bar)));
-  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(tc::smem_u32(p)));
+  return remote;
+}
+__device__ __forceinline__ void arrive_remote(uint32_t bar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void arrive_leader(uint64_t* bar) { arrive_remote(leader_addr(bar)); }
+// Hands back a stage whose values this warp holds in registers.
+__device__ __forceinline__ void arrive_read(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
@@ -183,10 +187,11 @@ __device__ __forceinline__ void issue_products(uint32_t d, uint32_t dc, uint32_t
   }
 }
 
-// What the split warps collect beside the parts: the extremes of |A| (zero
-// counts as large) and the sum of squares, Kahan-compensated per unit.
+// What the split warps collect beside the parts: the smallest nonzero |A| and
+// the sum of squares, Kahan-compensated per unit. (Values too large for the
+// parts give sums that are not finite: the drain warps look for those.)
 struct Checks {
-  uint32_t umax = 0, umin = 0xFFFFFFFFu;
+  uint32_t umin = 0xFFFFFFFFu;   // of 2 |bits| - 1: zero wraps to the largest value
   float ss = 0.f, comp = 0.f, part = 0.f;
   __device__ void fold() {
     const float y = part - comp, t = ss + y;
@@ -195,7 +200,7 @@ struct Checks {
     part = 0.f;
   }
   __device__ void report(int* bad, int lane) const {
-    if (__any_sync(0xffffffffu, umax >= kRangeHi || umin < kRangeLo - 1u) && lane == 0) atomicOr(bad, 1);
+    if (__any_sync(0xffffffffu, umin < 2u * kRangeLo - 1u) && lane == 0) atomicOr(bad, 1);
   }
   __device__ void add(double* sumsq, int lane) const {
     double v = (double)ss - (double)comp;
@@ -208,11 +213,8 @@ template <int PARTS>
 __device__ __forceinline__ void split_half(const float* v, uint32_t (&o)[PARTS][8], bool check, bool sq, Checks& ck) {
   if (check) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const uint32_t x = __float_as_uint(v[j]) & 0x7FFFFFFFu;
-      ck.umax = max(ck.umax, x);
-      ck.umin = min(ck.umin, x - 1u);   // zero wraps to the largest value
-    }
+    for (int j = 0; j < 16; j += 2)
+      ck.umin = __vimin3_u32(ck.umin, 2u * __float_as_uint(v[j]) - 1u, 2u * __float_as_uint(v[j + 1]) - 1u);
   }
   if (sq) {
 #pragma unroll
@@ -251,6 +253,17 @@ __device__ __forceinline__ void drain_columns(float (&s)[NG][16], uint32_t ta, i
   }
   tc::tc_fence_before();
   __syncwarp();
+}
+// Raises *bad where one of the ncols sums of the lane's row is not finite.
+template <int NG>
+__device__ __forceinline__ void check_sums(const float (&s)[NG][16], int g0, int ng, int ncols, int* bad) {
+  bool fine = true;
+#pragma unroll
+  for (int g = 0; g < NG; ++g)
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (g < ng && 16 * (g0 + g) + j < ncols) fine = fine && fabsf(s[g][j]) <= 3.402823466e38f;
+  if (!fine) atomicOr(bad, 1);
 }
 // s -> ncols columns of the lane's row at dst (float4 q of it at q qstep; vec:
 // 16-byte aligned), added to what an earlier flush left there.
@@ -331,109 +344,60 @@ __device__ __forceinline__ void split_x_tile(const float* __restrict__ X, long l
   if (bad != nullptr && __syncthreads_or(out_of_range) && threadIdx.x == 0) atomicOr(bad, 1);
 }
 
-// ---------------------------------------------------------------- copies of A by the split warps
-// Without TMA (rows of A that are not 16-byte aligned, or many problems): a
-// warp copies its 32 rows of a stage by 16-byte asynchronous copies. The 32
-// values of a row start at any 4-byte address, so nine aligned chunks cover
-// them, shift() words ahead of the first. (By 4-byte copies, 32 instead of nine
-// instructions a unit, a unit took twice as long.) TRANS: stage rows are rows of
-// memory, this warp's 32 columns each; else this warp's rows, 32 of K each.
-struct ARef {
-  const float* A;
-  long long lda;
-  int M, K;                // op(A) is M x K
+// ---------------------------------------------------------------- A with rows at any 4-byte address
+// TMA wants 16-byte aligned rows. Four rows apart, rows of any FP32 matrix have
+// the same alignment and a stride that is a multiple of 16 bytes: so one map
+// takes the rows of one class r % 4, from the aligned address at or before the
+// class's first value, and the values lie `shift` floats behind where the map
+// puts them. A stage is four boxes, four floats wider than the tile; what lies
+// past A is zero. op(A) = A: box c holds 32 rows (4 i + c) of 36 floats, read by
+// split warp c, so that TMEM lane 32 c + i is row 4 i + c of the tile. op(A) =
+// A^T: box c holds 8 rows (K = 4 i + c) of 132 floats. (Copies by the split
+// warps themselves, nine 16-byte chunks per row, took 1.3 to 1.7 times as long
+// per unit.)
+constexpr uint32_t kBoxN = 32 * 36 * 4, kBoxT = 8 * 132 * 4;   // bytes of a box
+constexpr uint32_t kClassBytes = 4 * kBoxN;                    // a stage
+struct Classes {
+  int shift[4];
+  int past[4];             // 1: no row in the class (its box starts past the map's end)
 };
-// Byte offsets of this lane's nine chunks (chunk lane + 32 i: row r = e / 9) from
-// a warp's first value in a unit. They are the same for every unit, as first
-// rows and columns are multiples of 32. False when a row stride is too long
-// for them.
-__device__ __forceinline__ bool chunk_offsets(const ARef& a, int lane, int (&off)[9]) {
-  const int b = (int)(reinterpret_cast<uintptr_t>(a.A) & 15);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const int e = lane + 32 * i, r = e / 9, c = e - 9 * r;
-    off[i] = (int)((((long long)r * a.lda * 4 + b) & ~15LL) + 16 * c - b);
-  }
-  return a.lda < (1 << 24);
-}
-// The same copy as copy_rows for a unit whose chunks all lie inside A.
-__device__ __forceinline__ void copy_interior(const ARef& a, long long i0, long long j0, const int (&off)[9], float* dst,
-                                              int lane) {
-  const char* p = reinterpret_cast<const char*>(a.A + i0 * a.lda + j0);
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst) + 16 * lane;   // chunk e at 16 e: rows are nine chunks
-#pragma unroll
-  for (int i = 0; i < 9; ++i)
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 512 * i), "l"(p + off[i]) : "memory");
-}
-__device__ __forceinline__ bool interior(const ARef& a, bool trans, long long i0, long long j0) {
-  return i0 + 32 <= (trans ? a.K : a.M) && j0 + kRowFloats <= (trans ? a.M : a.K) &&
-         (i0 > 0 || j0 > 0 || (reinterpret_cast<uintptr_t>(a.A) & 15) == 0);
-}
-// Copies rows r = 0 .. 31 of this warp (first row / column of memory: i0, j0)
-// to dst; rows past the end of memory are zeros, chunks outside A are clipped.
-__device__ __forceinline__ void copy_rows(const ARef& a, bool trans, long long i0, long long j0, float* dst, int lane) {
-  const long long rows = trans ? a.K : a.M, cols = trans ? a.M : a.K;
-  const char* lo = reinterpret_cast<const char*>(a.A);
-  const char* hi = reinterpret_cast<const char*>(a.A + (rows - 1) * a.lda + cols);   // end of A
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const int e = lane + 32 * i, r = e / 9, c = e - 9 * r;
-    const char* p = reinterpret_cast<const char*>(a.A + (i0 + r) * a.lda + j0);
-    p = reinterpret_cast<const char*>(reinterpret_cast<uintptr_t>(p) & ~uintptr_t(15)) + 16 * c;
-    float* d = dst + r * kRowFloats + 4 * c;
-    const long long left = hi - p;
-    if (i0 + r >= rows || left <= 0) {
-      cp_async16(d, reinterpret_cast<const void*>(reinterpret_cast<uintptr_t>(lo) & ~uintptr_t(15)), 0);
-    } else if (p < lo) {   // the chunk that A's first value lies in
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const char* q = p + 4 * u;
-        cp_async4(d + u, q >= lo && q < hi ? q : lo, q >= lo && q < hi ? 4 : 0);
-      }
-    } else {
-      cp_async16(d, p, left < 16 ? (int)left : 16);
-    }
-  }
-}
-__device__ __forceinline__ int shift(const float* p) { return (int)((reinterpret_cast<uintptr_t>(p) >> 2) & 3); }
-
-// v[j] = op(A)(this lane's row, k0 + 16 half + j) from such a stage (this
-// warp's part of it), zero past M and K (what lies there in memory is not A's).
+// The four maps (rows x cols, row stride lda); false when the encoder is missing.
+bool class_maps(CUtensorMap* m, Classes* cl, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans);
 template <bool TRANS>
-__device__ __forceinline__ void read_copied(const ARef& a, int k0, int r0, const float* f, int half, int lane, float* v) {
+__device__ __forceinline__ void load_classes(unsigned char* f, const CUtensorMap* m0, const CUtensorMap* m1,
+                                             const CUtensorMap* m2, const CUtensorMap* m3, const Classes& cl,
+                                             uint64_t* bar, int k, int row) {
+  const CUtensorMap* m[4] = {m0, m1, m2, m3};
+  tc::mbar_expect_tx(bar, 4 * (TRANS ? kBoxT : kBoxN));
+#pragma unroll
+  for (int c = 0; c < 4; ++c)   // first columns are multiples of 32 floats
+    tc::tma_load_2d(f + c * (TRANS ? kBoxT : kBoxN), m[c], bar, TRANS ? row : k, (TRANS ? k : row) / 4 + cl.past[c]);
+}
+// v[j] = op(A)(this lane's row, 16 half + j) of split warp w.
+template <bool TRANS>
+__device__ __forceinline__ void read_classes(const unsigned char* f, const Classes& cl, int w, int half, int lane,
+                                             float* v) {
   if (TRANS) {
-    // row k of the stage is shifted by (s + k lda) % 4
-    const int s = shift(a.A + (long long)k0 * a.lda + r0), l3 = (int)(a.lda & 3);
     const float* p[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) p[j] = f + (16 * half + j) * kRowFloats + ((s + j * l3) & 3) + lane;
+    for (int c = 0; c < 4; ++c)
+      p[c] = reinterpret_cast<const float*>(f + c * kBoxT) + 4 * half * 132 + cl.shift[c] + 32 * w + lane;
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = p[j & 3][(j & ~3) * kRowFloats];
+    for (int j = 0; j < 16; ++j) v[j] = p[j & 3][(j >> 2) * 132];
   } else {
-    const int s = shift(a.A + (long long)(r0 + lane) * a.lda + k0);
-    const float* p = f + lane * kRowFloats + 16 * half;
-    float w[20];
+    const int s = w < 2 ? (w == 0 ? cl.shift[0] : cl.shift[1]) : (w == 2 ? cl.shift[2] : cl.shift[3]);
+    const float* p = reinterpret_cast<const float*>(f + w * kBoxN) + lane * 36 + 16 * half;
+    float x[20];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
       const float4 q = *reinterpret_cast<const float4*>(p + 4 * i);
-      w[4 * i] = q.x; w[4 * i + 1] = q.y; w[4 * i + 2] = q.z; w[4 * i + 3] = q.w;
+      x[4 * i] = q.x; x[4 * i + 1] = q.y; x[4 * i + 2] = q.z; x[4 * i + 3] = q.w;
     }
 #pragma unroll
-    for (int i = 0; i < 18; ++i) w[i] = s & 1 ? w[i + 1] : w[i];
+    for (int i = 0; i < 18; ++i) x[i] = s & 1 ? x[i + 1] : x[i];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = s & 2 ? w[i + 2] : w[i];
+    for (int i = 0; i < 16; ++i) v[i] = s & 2 ? x[i + 2] : x[i];
   }
-  if (k0 + 16 * half + 16 > a.K || r0 + 32 > a.M) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (k0 + 16 * half + j >= a.K || r0 + lane >= a.M) v[j] = 0.f;
-  }
-}
-// One line of A per lane into L2.
-__device__ __forceinline__ void prefetch_rows(const ARef& a, bool trans, long long i0, long long j0, int lane) {
-  const long long rows = trans ? a.K : a.M, cols = trans ? a.M : a.K;
-  if (i0 + lane < rows && j0 < cols)
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.A + (i0 + lane) * a.lda + j0));
 }
 
 }  // namespace sp

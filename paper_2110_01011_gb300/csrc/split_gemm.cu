@@ -39,6 +39,61 @@
 #include "split_gemm.cuh"
 
 namespace rqlp {
+namespace sp {
+
+using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+static EncodeFn encode_fn() {
+  static const EncodeFn fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<EncodeFn>(p);
+  }();
+  return fn;
+}
+static bool encode(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint64_t stride, uint32_t bc,
+                   uint32_t br, CUtensorMapSwizzle sw) {
+  EncodeFn fn = encode_fn();
+  if (fn == nullptr) return false;
+  cuuint64_t dims[2] = {cols, rows}, strides[1] = {stride};
+  cuuint32_t box[2] = {bc, br}, es[2] = {1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+bool class_maps(CUtensorMap* m, Classes* cl, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans) {
+  for (int c = 0; c < 4; ++c) {
+    const bool empty = c >= rows;
+    const uintptr_t p = reinterpret_cast<uintptr_t>(A + (empty ? 0 : c) * lda);
+    cl->shift[c] = (int)((p & 15) / 4);
+    cl->past[c] = empty ? 1 : 0;
+    if (!encode(&m[c], reinterpret_cast<const void*>(p & ~uintptr_t(15)), (uint64_t)(cols + cl->shift[c]),
+                empty ? 1 : (uint64_t)((rows - c + 3) / 4), (uint64_t)lda * 16, trans ? 132 : 36, trans ? 8 : 32,
+                CU_TENSOR_MAP_SWIZZLE_NONE))
+      return false;
+  }
+  return true;
+}
+
+// Maps over A (rows x cols, row stride lda): one of boxes of 128 columns x 32
+// rows (op(A) = A^T), or 32 columns x 128 rows with the 128-byte swizzle, where
+// its rows are 16-byte aligned; else one per class of rows. False when the
+// encoder is missing.
+static bool split_maps(CUtensorMap* m, Classes* cl, bool* aligned, const float* A, int64_t rows, int64_t cols,
+                       int64_t lda, bool trans) {
+  *aligned = reinterpret_cast<uintptr_t>(A) % 16 == 0 && lda % 4 == 0;
+  if (!*aligned) return class_maps(m, cl, A, rows, cols, lda, trans);
+  return encode(m, A, (uint64_t)cols, (uint64_t)rows, (uint64_t)lda * 4, trans ? BM : BK, trans ? BK : BM,
+                trans ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+}  // namespace sp
+
 namespace {
 
 using namespace sp;
@@ -46,8 +101,6 @@ using namespace sp;
 constexpr int kMaxSlots = 16;         // partial tiles that the last CTA of a tile sums itself
 
 struct Args {
-  const float* A;
-  long long lda;
   const uint16_t* img;
   float* out;
   long long ldo;
@@ -59,13 +112,14 @@ struct Args {
   int* next1;
   double* sumsq;
   int* info;
-  int M, N, K, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole;   // sx, sf, sa: stages of X, of A in FP32, A slots
+  int M, N, K, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole, perm;   // sx, sf, sa: stages of X, of A in FP32, A slots
   int chunk;                // units per chain of the main accumulator
   int corr_first;           // chains of one unit, the correction products first
   int flush;                // units whose sums are held in registers before they are added to global memory
   int corr;                 // 0: one accumulator; else main chains per chain of the correction accumulator
   int units;                // tiles x kb
   uint32_t idesc;
+  Classes cl;
 };
 
 // First unit of group c: an even share of all units, or of the whole tiles.
@@ -78,16 +132,23 @@ __host__ __device__ inline int unit_owner(int u, int units, int G) {
   return (int)((((long long)u + 1) * G + units - 1) / units) - 1;
 }
 
-template <bool TRANS, int PARTS, bool TMA>
+// Maps over A: one, or one per class of rows.
+struct MapsA {
+  CUtensorMap m[4];
+};
+
+// ALIGNED: A's rows are 16-byte aligned, one box a stage; else four.
+template <bool TRANS, int PARTS, bool ALIGNED>
 __global__ void __launch_bounds__(kThreads, 1)
-split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
+split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int nh = a.npad / CG;                                  // X columns held by this CTA
   const uint32_t part_bytes = (uint32_t)nh * BK * 2, stage_bytes = PARTS * part_bytes;
   unsigned char* fstage = smem;                                // FP32 stages of A, then X stages (both 1 KB aligned)
-  unsigned char* xstage = smem + (size_t)a.sf * (TMA ? kABytes : kCopyBytes);
+  constexpr uint32_t kStage = ALIGNED ? kABytes : kClassBytes;
+  unsigned char* xstage = smem + (size_t)a.sf * kStage;
   uint64_t* xfull = reinterpret_cast<uint64_t*>(xstage + (size_t)a.sx * stage_bytes);
   uint64_t* xempty = xfull + kMaxStages;
   uint64_t* ffull = xempty + kMaxStages;
@@ -152,7 +213,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
   const int nx = (*a.xlo) ? PARTS : 1;                          // X may be exact in its first part
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");   // 48 + 2 x 64 + 2 x 152 = 5 x 96
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");   // 40 + 2 x 64 + 2 x 152 <= 5 x 96
     if (warp == 0) {
       // ------------------------------------------------ X stages
       const size_t img_stage = (size_t)CG * stage_bytes;
@@ -229,7 +290,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       if (!ok) post_timeout(a.info);
       if (!wait(done, 0)) post_timeout(a.info);
     }
-    else if (TMA && warp == 3) {
+    else if (warp == 3) {
       // ------------------------------------------------ FP32 tiles of A
       bool ok = true;
       Ring r;
@@ -242,9 +303,14 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
           break;
         }
         if (elect()) {
-          tc::mbar_expect_tx(&ffull[r.s], kABytes);
           const int row = (c.t * CG + rank) * BM, k = c.k * BK;   // both multiples of four floats
-          tc::tma_load_2d(fstage + r.s * kABytes, &tmA, &ffull[r.s], TRANS ? row : k, TRANS ? k : row);
+          if (ALIGNED) {
+            tc::mbar_expect_tx(&ffull[r.s], kABytes);
+            tc::tma_load_2d(fstage + r.s * kABytes, &tm.m[0], &ffull[r.s], TRANS ? row : k, TRANS ? k : row);
+          } else {
+            load_classes<TRANS>(fstage + r.s * kClassBytes, &tm.m[0], &tm.m[1], &tm.m[2], &tm.m[3], a.cl, &ffull[r.s], k,
+                                row);
+          }
         }
         c.next(KB);
         r.next(a.sf);
@@ -277,121 +343,66 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
         }
       }
     };
-    const ARef ar{a.A, a.lda, a.M, a.K};
-    int off[9];
-    const bool near = !TMA && chunk_offsets(ar, lane, off);
-    auto first = [&](const Cursor& c, int& k0, int& r0) {   // a unit's first K, this warp's first row
-      k0 = c.k * BK;
-      r0 = (c.t * CG + rank) * BM + 32 * w;
-    };
-    auto copy = [&](const Cursor& c, unsigned char* f) {
-      int k0, r0;
-      first(c, k0, r0);
-      const int i0 = TRANS ? k0 : r0, j0 = TRANS ? r0 : k0;
-      float* dst = reinterpret_cast<float*>(f) + 32 * w * kRowFloats;
-      if (near && interior(ar, TRANS, i0, j0)) copy_interior(ar, i0, j0, off, dst, lane);
-      else copy_rows(ar, TRANS, i0, j0, dst, lane);
-    };
-    auto prefetch = [&](const Cursor& c) {
-      int k0, r0;
-      first(c, k0, r0);
-      prefetch_rows(ar, TRANS, TRANS ? k0 : r0, TRANS ? r0 : k0, lane);
-    };
     const uint32_t lanes = (uint32_t)(32 * w) << 16;
     bool ok = true;
     const int n = u1 - u0;
-    Cursor cu(u0, KB), cc(u0, KB), cp(u0, KB);   // current unit; next to copy, to prefetch (without TMA)
     Ring ra, rx, rf;                 // A slot, X stage, FP32 stage of the current unit
-    int fc = odd;                    // FP32 stage of the next copy
-    auto two = [&](Cursor& c) {      // this warpgroup's next unit
-      c.next(KB);
-      c.next(KB);
-    };
     if (odd) {
-      cu.next(KB);
-      cc.next(KB);
-      cp.next(KB);
       ra.next(a.sa);
       rx.next(a.sx);
       rf.next(a.sf);
     }
-    constexpr int kAhead = kCopyStages / 2 - 1;   // own units copied ahead
-    if (!TMA) {
-      for (int i = 0; i < kAhead; ++i) {
-        if (odd + 2 * i < n) copy(cc, fstage + fc * kCopyBytes);
-        cp_async_commit();
-        two(cc);
-        fc += 2;
-      }
-      for (int i = odd; i < odd + kPrefetch; i += 2) {
-        if (i >= 2 * kAhead && i < n) prefetch(cp);
-        two(cp);
-      }
-    }
+    const uint32_t afull0 = leader_addr(afull);
     for (int i = odd; i < n; i += 2) {
-      const unsigned char* f = fstage + rf.s * (TMA ? kABytes : kCopyBytes);
+      const unsigned char* f = fstage + rf.s * kStage;
       auto fetch = [&](int half, float* v) {
-        if (TMA) {
-          read(f, half, v);
-        } else {
-          int k0, r0;
-          first(cu, k0, r0);
-          read_copied<TRANS>(ar, k0, r0, reinterpret_cast<const float*>(f) + 32 * w * kRowFloats, half, lane, v);
-        }
+        if (ALIGNED) read(f, half, v);
+        else read_classes<TRANS>(f, a.cl, w, half, lane, v);
       };
-      if (TMA) {
-        if (!tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit)) {
-          ok = false;
-          break;
-        }
-      } else {
-        if (i + kPrefetch < n) prefetch(cp);
-        two(cp);
-        __syncwarp();   // every lane has read the stage that is filled next
-        if (i + 2 * kAhead < n) copy(cc, fstage + fc * kCopyBytes);
-        cp_async_commit();
-        two(cc);
-        fc = fc + 2 >= kCopyStages ? fc + 2 - kCopyStages : fc + 2;
-        cp_async_wait<kAhead>();
-        __syncwarp();
+      ok = tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit);
+      if (!__all_sync(0xffffffffu, ok)) {
+        ok = false;
+        break;
       }
       float v[16];
       uint32_t o[PARTS][8];
       fetch(0, v);
-      split_half<PARTS>(v, o, check, sq, ck);
-      if (!wait(&aempty[ra.s], ra.ph ^ 1u)) {
+      // (the slot is waited for while the values are on their way)
+      ok = wait(&aempty[ra.s], ra.ph ^ 1u);
+      if (!__all_sync(0xffffffffu, ok)) {
         ok = false;
         break;
       }
       tc::tc_fence_after();
+      split_half<PARTS>(v, o, check, sq, ck);
+      fetch(1, v);
       const uint32_t ta = a_base + lanes + (uint32_t)(ra.s * PARTS * 16);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
-      fetch(1, v);
       split_half<PARTS>(v, o, check, sq, ck);
+      __syncwarp();
+      if (lane == 0) arrive_read(&fempty[rf.s]);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
       if (sq) ck.fold();
+      if (rank != 0) {   // the pair's leader learns of the peer's X stage through the peer's A
+        ok = tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit);
+        if (!__all_sync(0xffffffffu, ok)) {
+          ok = false;
+          break;
+        }
+      }
       st_wait();
       tc::tc_fence_before();
       __syncwarp();
-      if (lane == 0) {
-        if (TMA) tc::mbar_arrive(&fempty[rf.s]);
-        // The pair's leader learns of the peer's X stage through the peer's A.
-        if (rank != 0 && !tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit)) ok = false;
-        arrive_leader(&afull[ra.s]);
-      }
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) break;
+      if (lane == 0) arrive_remote(afull0 + 8 * ra.s);
       ra.next(a.sa);
       ra.next(a.sa);
       rx.next(a.sx);
       rx.next(a.sx);
       rf.next(a.sf);
       rf.next(a.sf);
-      two(cu);
     }
-    if (!TMA) cp_async_wait_all();
     if (!ok && lane == 0) post_timeout(a.info);
     if (check) ck.report(a.bad, lane);
     if (sq) ck.add(a.sumsq, lane);
@@ -399,6 +410,8 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
     // -------------------------------------------------- drain: TMEM -> registers -> global
     asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
     const int e = warp - 12, half = e >> 2, tid = threadIdx.x - 384;
+    // TMEM lane -> row of the tile (see read_classes)
+    auto tile_row = [&](int l) { return ALIGNED || TRANS ? l : 4 * (l & 31) + (l >> 5); };
     const int row = 32 * (e & 3) + lane;
     const int groups = a.npad / 16, g0 = half ? (groups + 1) / 2 : 0, ng = half ? groups / 2 : (groups + 1) / 2;
     float s[kGroups][16];
@@ -434,7 +447,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
       if (!part_end && since < a.flush) continue;
       // End of this CTA's part of tile t (or a flush on the way).
       const int rt = t * CG + rank;                   // 128-row tile
-      const long long gm = (long long)rt * BM + row;
+      const long long gm = (long long)rt * BM + tile_row(row);
       const bool all = part0 == 0 && (k == KB || left + k >= KB), first_part = t == u0 / KB;
       float* dst;
       int ncols, qstep = 4;   // floats from one float4 of the row to the next
@@ -450,6 +463,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
         qstep = 4 * BM;
         vec = true;
       }
+      if (PARTS == 3 && a.bad != nullptr) check_sums(s, g0, ng, gm < a.M ? a.N : 0, a.bad);
       store_sums(s, dst, qstep, g0, ng, ncols, vec, flushed);
       if (part_end && !all && !a.fixup) {
         // Publish the partial tile; the last CTA to arrive sums them in CTA order.
@@ -502,7 +516,7 @@ split_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const Args a) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const int r = 8 * (2 * e + (j >> 2)) + (lane & 7), c = 4 * (c0 + 4 * (j & 3));
-              const long long gr = (long long)rt * BM + r;
+              const long long gr = (long long)rt * BM + tile_row(r);
               if (gr >= a.M || c >= a.N) continue;
               float* o = a.out + gr * a.ldo + c;
               if (a.vec_out && c + 3 < a.N) {
@@ -544,7 +558,7 @@ __global__ void split_fixup_kernel(const Args a) {
   for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < total;
        f += (long long)gridDim.x * blockDim.x) {
     const int rt = (int)(f / per), t = rt / CG, e = (int)(f % per), r = e % BM, c = (e / BM) * 4;
-    const long long gr = (long long)rt * BM + r;
+    const long long gr = (long long)rt * BM + (a.perm ? 4 * (r & 31) + (r >> 5) : r);
     if (gr >= a.M || c >= a.N) continue;
     const int ub = t * a.kb, ue = ub + a.kb;
     const int clo = unit_owner(ub, a.units, a.G), chi = unit_owner(ue - 1, a.units, a.G);
@@ -601,8 +615,8 @@ size_t smem_optin() {
 }
 constexpr size_t kSmemExtra = 1024 + 1024;   // alignment, barriers
 
-template <bool TRANS, int PARTS, bool TMA>
-cudaError_t launch(const CUtensorMap& map, Args& a, int cap, size_t smem, cudaStream_t st) {
+template <bool TRANS, int PARTS, bool ALIGNED>
+cudaError_t launch(const MapsA& map, Args& a, int cap, size_t smem, cudaStream_t st) {
   static int resident = 0;   // pairs that run at the same time
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -615,51 +629,21 @@ cudaError_t launch(const CUtensorMap& map, Args& a, int cap, size_t smem, cudaSt
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (resident == 0) {
-    CK(cudaFuncSetAttribute(split_gemm_kernel<TRANS, PARTS, TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    CK(cudaFuncSetAttribute(split_gemm_kernel<TRANS, PARTS, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)smem_optin()));
     int n = 0;
     cfg.gridDim = dim3((unsigned)(sm_count() / CG * CG));
     cfg.dynamicSmemBytes = smem_optin();
-    CK(cudaOccupancyMaxActiveClusters(&n, split_gemm_kernel<TRANS, PARTS, TMA>, &cfg));
+    CK(cudaOccupancyMaxActiveClusters(&n, split_gemm_kernel<TRANS, PARTS, ALIGNED>, &cfg));
     resident = std::max(1, std::min(n, sm_count() / CG));
   }
   a.G = std::min(resident, cap);
   a.fixup = (!a.whole && a.G / a.tiles + 2 > kMaxSlots) ? 1 : 0;
   cfg.gridDim = dim3((unsigned)(a.G * CG));
   cfg.dynamicSmemBytes = smem;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, split_gemm_kernel<TRANS, PARTS, TMA>, map, a);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, split_gemm_kernel<TRANS, PARTS, ALIGNED>, map, a);
   note_launch();
   return e;
-}
-
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeFn encode_fn() {
-  static const EncodeFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeFn>(p);
-  }();
-  return fn;
-}
-// FP32 map over A (rows x cols, row stride lda): boxes of 128 columns x 32 rows
-// (op(A) = A^T), or 32 columns x 128 rows with the 128-byte swizzle. False when
-// the rows are not 16-byte aligned (or the encoder is missing): the kernel
-// variant without TMA takes those.
-bool map_a(CUtensorMap* map, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans) {
-  EncodeFn fn = encode_fn();
-  if (fn == nullptr || reinterpret_cast<uintptr_t>(A) % 16 != 0 || lda % 4 != 0) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)(lda * 4)};
-  cuuint32_t box[2] = {trans ? (cuuint32_t)BM : (cuuint32_t)BK, trans ? (cuuint32_t)BK : (cuuint32_t)BM};
-  cuuint32_t es[2] = {1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(A), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, trans ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, int64_t K, const float* A, int64_t lda,
@@ -674,7 +658,6 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   CK(cudaGetLastError());
 
   Args a = {};
-  a.A = A; a.lda = lda;
   a.img = ws->img;
   a.out = out; a.ldo = ldo;
   a.part = ws->part;
@@ -716,16 +699,19 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   a.nbuf = 2 * npad + cc + 2 * parts * 16 <= 512 ? 2 : 1;   // (FP32 above 208 columns: one)
   a.sa = std::min(kMaxASlots, (512 - a.nbuf * npad - cc) / (parts * 16));
   const size_t stage = (size_t)(npad / CG) * BK * 2 * parts;
-  CUtensorMap map = {};
-  const bool tma = map_a(&map, A, transA ? K : M, transA ? M : K, lda, transA);
+  MapsA map = {};
+  bool aligned = false;
+  if (!split_maps(map.m, &a.cl, &aligned, A, transA ? K : M, transA ? M : K, lda, transA)) return cudaErrorNotSupported;
+  a.perm = !aligned && !transA ? 1 : 0;
   // Shared memory: four X stages first, then FP32 stages of A, then X again.
   const size_t avail = smem_optin() - kSmemExtra;
-  a.sf = tma ? (int)std::min<size_t>(kMaxStages, (avail - 4 * stage) / kABytes) : kCopyStages;
-  const size_t fbytes = (size_t)a.sf * (tma ? kABytes : kCopyBytes);
+  const size_t fstage = aligned ? kABytes : kClassBytes;
+  a.sf = (int)std::min<size_t>(kMaxStages, (avail - 4 * stage) / fstage);
+  const size_t fbytes = a.sf * fstage;
   a.sx = (int)std::min<size_t>(kMaxStages, (avail - fbytes) / stage);
   a.idesc = tc::idesc_bf16(BM * CG, npad, false, false);
   const size_t smem = fbytes + a.sx * stage + kSmemExtra;
-#define RQLP_SPLIT(T, P) (tma ? launch<T, P, true>(map, a, cap, smem, st) : launch<T, P, false>(map, a, cap, smem, st))
+#define RQLP_SPLIT(T, P) (aligned ? launch<T, P, true>(map, a, cap, smem, st) : launch<T, P, false>(map, a, cap, smem, st))
   cudaError_t e = transA ? (parts == 3 ? RQLP_SPLIT(true, 3) : RQLP_SPLIT(true, 2))
                          : (parts == 3 ? RQLP_SPLIT(false, 3) : RQLP_SPLIT(false, 2));
 #undef RQLP_SPLIT

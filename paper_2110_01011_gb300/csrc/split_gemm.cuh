@@ -46,16 +46,16 @@ cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K
 
 // ---------------------------------------------------------------- grouped products (batched form)
 struct SplitJob {           // out (M x N) = op(A) X
-  const float* A;           // as op(A) is stored (see split_gemm)
-  long long lda;
+  const void* maps;         // four tensor maps over A, on the device (split_job_maps)
   const uint16_t* img;      // X's parts, written by split_x_grouped
   float* out;
   long long ldo;
   const int* xlo;           // raised when X has a low part
   int* bad;                 // raised on values outside the parts' range (FP32; else null)
   double* sumsq;            // += sum of squares of A (or null)
-  int M, N, K, npad, kb, vec_out;
+  int M, N, npad, kb, vec_out;
   uint32_t idesc;
+  int shift[4], past[4];
 };
 struct SplitXJob {          // X (K x N) -> stage images
   const float* X;
@@ -65,6 +65,10 @@ struct SplitXJob {          // X (K x N) -> stage images
   int* bad;
   int N, npad;
 };
+constexpr size_t kSplitMapBytes = 4 * 128;   // four tensor maps
+// Encodes the maps of A (rows x cols, row stride lda; A K x M when trans) into
+// host memory (128-byte entries) and sets the job's shifts.
+bool split_job_maps(void* maps, SplitJob* j, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans);
 int split_npad(int n);
 size_t split_image_bytes(int64_t K, int n, int parts);
 uint32_t split_idesc(int npad);

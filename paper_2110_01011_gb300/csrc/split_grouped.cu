@@ -5,8 +5,8 @@
 // A work unit is one 256-row tile of one problem's output over that problem's
 // whole K; the host balances the units over the CTA pairs (longest first, onto
 // the least loaded pair), so no tile is split and no pair waits for another.
-// A's FP32 rows are copied by the warps that split them (a problem's rows may
-// start at any 4-byte address), X's parts come as stage images that
+// A's FP32 tiles come by TMA through four maps per problem (its rows may start at
+// any 4-byte address), X's parts come as stage images that
 // split_x_grouped_kernel writes before the pass. The earlier form kept A's
 // parts in memory (a split of every A first, then 4 or 6 bytes per element and
 // pass); reading A in FP32 takes 4 and no split. Every wait is bounded.
@@ -28,7 +28,7 @@ struct GroupArgs {
   const int* cta_start;     // pair p takes units cta_start[p] .. cta_start[p + 1] - 1
   int* info;
   int npm;                  // largest npad: the layout of shared and tensor memory
-  int sx, sa, nbuf, corr, corr_first, chunk, flush, stall;
+  int sx, sf, sa, nbuf, corr, corr_first, chunk, flush, stall;
 };
 
 template <bool TRANS, int PARTS>
@@ -38,10 +38,12 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const uint32_t stage_bytes = (uint32_t)PARTS * (a.npm / CG) * BK * 2;
   unsigned char* fstage = smem;
-  unsigned char* xstage = smem + kCopyStages * kCopyBytes;
+  unsigned char* xstage = smem + a.sf * kClassBytes;
   uint64_t* xfull = reinterpret_cast<uint64_t*>(xstage + (size_t)a.sx * stage_bytes);
   uint64_t* xempty = xfull + kMaxStages;
-  uint64_t* afull = xempty + kMaxStages;
+  uint64_t* ffull = xempty + kMaxStages;
+  uint64_t* fempty = ffull + kMaxStages;
+  uint64_t* afull = fempty + kMaxStages;
   uint64_t* aempty = afull + kMaxASlots;
   uint64_t* accf = aempty + kMaxASlots;
   uint64_t* acce = accf + 2;
@@ -58,6 +60,10 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
     for (int s = 0; s < a.sx; ++s) {
       tc::mbar_init(&xfull[s], 1);
       tc::mbar_init(&xempty[s], 1);
+    }
+    for (int s = 0; s < a.sf; ++s) {
+      tc::mbar_init(&ffull[s], 1);
+      tc::mbar_init(&fempty[s], 4);
     }
     for (int s = 0; s < a.sa; ++s) {
       tc::mbar_init(&afull[s], 4 * CG);
@@ -86,7 +92,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
   const uint32_t smem_x = tc::smem_u32(xstage);
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");   // 48 + 2 x 96 + 2 x 112 <= 5 x 96
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");   // 40 + 2 x 112 + 2 x 104 <= 5 x 96
     if (warp == 0) {
       // ------------------------------------------------ X stages
       bool ok = true;
@@ -166,95 +172,108 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       }
       if (!ok) post_timeout(a.info);
       if (!wait(done, 0)) post_timeout(a.info);
+    } else if (warp == 3) {
+      // ------------------------------------------------ FP32 tiles of A
+      bool ok = true;
+      Ring r;
+      int i = 0;
+      for (int ui = ub; ui < ue && ok; ++ui) {
+        const int2 un = a.units[ui];
+        const SplitJob& j = a.jobs[un.x];
+        const CUtensorMap* m = static_cast<const CUtensorMap*>(j.maps);
+        Classes cl;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) cl.past[c] = j.past[c];
+        const int n = j.kb, row = (un.y * CG + rank) * BM;
+        for (int k = 0; k < n; ++k, ++i) {
+          if (!wait(&fempty[r.s], r.ph ^ 1u)) {
+            ok = false;
+            break;
+          }
+          if (elect())
+            load_classes<TRANS>(fstage + r.s * kClassBytes, m, m + 1, m + 2, m + 3, cl, &ffull[r.s], k * BK, row);
+          r.next(a.sf);
+        }
+      }
+      if (!ok) post_timeout(a.info);
+      for (int s = max(0, i - a.sf); s < i; ++s)
+        if (!tc::mbar_wait(&ffull[s % a.sf], (uint32_t)((s / a.sf) & 1), kWaitLimit)) post_timeout(a.info);
     }
   } else if (warp < 12) {
-    // -------------------------------------------------- A: copy, split, store to tensor memory
+    // -------------------------------------------------- A: split, store to tensor memory
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     const int w = warp & 3, odd = (warp >> 2) - 1;   // two warpgroups take the units of K by turns
     const uint32_t lanes = (uint32_t)(32 * w) << 16;
     bool ok = true;
-    Ring ra, rx;
+    Ring ra, rx, rf;
     if (odd) {
       ra.next(a.sa);
       rx.next(a.sx);
+      rf.next(a.sf);
     }
+    const uint32_t afull0 = leader_addr(afull);
     int turn = odd;   // this warpgroup's first unit of K within the tile
     for (int ui = ub; ui < ue && ok; ++ui) {
-      const int2 un = a.units[ui];
-      const SplitJob& j = a.jobs[un.x];
-      const ARef ar{j.A, j.lda, j.M, j.K};
+      const SplitJob& j = a.jobs[a.units[ui].x];
       const bool check = PARTS == 3 && j.bad != nullptr, sq = j.sumsq != nullptr;
       Checks ck;
-      const int n = j.kb, r0 = (un.y * CG + rank) * BM + 32 * w;
-      int off[9];
-      const bool near = chunk_offsets(ar, lane, off);
-      auto copy = [&](int k, float* dst) {   // unit k of K
-        const int i0 = TRANS ? k * BK : r0, j0 = TRANS ? r0 : k * BK;
-        if (near && interior(ar, TRANS, i0, j0)) copy_interior(ar, i0, j0, off, dst, lane);
-        else copy_rows(ar, TRANS, i0, j0, dst, lane);
-      };
-      constexpr int kAhead = kCopyStages / 2 - 1;   // own units copied ahead
-      // Own stages: odd, odd + 2, odd + 4, by turns from each tile's start.
-      float* own = reinterpret_cast<float*>(fstage + odd * kCopyBytes) + 32 * w * kRowFloats;
-      constexpr int kOwn = 2 * (int)(kCopyBytes / 4);   // floats from one own stage to the next
-      __syncwarp();   // every lane has read the stages of the tile before
+      Classes cl;
 #pragma unroll
-      for (int i = 0; i < kAhead; ++i) {
-        if (turn + 2 * i < n) copy(turn + 2 * i, own + i * kOwn);
-        cp_async_commit();
-      }
-      int fc = kAhead, fr = 0;   // own stage of the next copy, of the current unit
+      for (int c = 0; c < 4; ++c) cl.shift[c] = j.shift[c];
+      const int n = j.kb;
       for (int k = turn; k < n; k += 2) {
-        if (k + kPrefetch < n)
-          prefetch_rows(ar, TRANS, TRANS ? (k + kPrefetch) * BK : r0, TRANS ? r0 : (k + kPrefetch) * BK, lane);
-        __syncwarp();   // every lane has read the stage that is filled next
-        if (k + 2 * kAhead < n) copy(k + 2 * kAhead, own + fc * kOwn);
-        cp_async_commit();
-        fc = fc == kAhead ? 0 : fc + 1;
-        cp_async_wait<kAhead>();
-        __syncwarp();
-        const float* f = own + fr * kOwn;
-        fr = fr == kAhead ? 0 : fr + 1;
+        const unsigned char* f = fstage + rf.s * kClassBytes;
+        ok = tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit);
+        if (!__all_sync(0xffffffffu, ok)) {
+          ok = false;
+          break;
+        }
         float v[16];
         uint32_t o[PARTS][8];
-        read_copied<TRANS>(ar, k * BK, r0, f, 0, lane, v);
-        split_half<PARTS>(v, o, check, sq, ck);
-        if (!wait(&aempty[ra.s], ra.ph ^ 1u)) {
+        read_classes<TRANS>(f, cl, w, 0, lane, v);
+        ok = wait(&aempty[ra.s], ra.ph ^ 1u);
+        if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
           break;
         }
         tc::tc_fence_after();
+        split_half<PARTS>(v, o, check, sq, ck);
+        read_classes<TRANS>(f, cl, w, 1, lane, v);
         const uint32_t ta = a_base + lanes + (uint32_t)(ra.s * PARTS * 16);
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
-        read_copied<TRANS>(ar, k * BK, r0, f, 1, lane, v);
         split_half<PARTS>(v, o, check, sq, ck);
+        __syncwarp();
+        if (lane == 0) arrive_read(&fempty[rf.s]);
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
         if (sq) ck.fold();
+        if (rank != 0) {   // the pair's leader learns of the peer's X stage through the peer's A
+          ok = tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit);
+          if (!__all_sync(0xffffffffu, ok)) {
+            ok = false;
+            break;
+          }
+        }
         st_wait();
         tc::tc_fence_before();
         __syncwarp();
-        if (lane == 0) {
-          // The pair's leader learns of the peer's X stage through the peer's A.
-          if (rank != 0 && !tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit)) ok = false;
-          arrive_leader(&afull[ra.s]);
-        }
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        if (!ok) break;
+        if (lane == 0) arrive_remote(afull0 + 8 * ra.s);
         ra.next(a.sa);
         ra.next(a.sa);
         rx.next(a.sx);
         rx.next(a.sx);
+        rf.next(a.sf);
+        rf.next(a.sf);
       }
       if (n & 1) turn ^= 1;   // the other warpgroup begins the next tile
-      cp_async_wait_all();
       if (check) ck.report(j.bad, lane);
       if (sq) ck.add(j.sumsq, lane);
     }
     if (!ok && lane == 0) post_timeout(a.info);
   } else {
     // -------------------------------------------------- drain: TMEM -> registers -> global
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
     const int e = warp - 12, half = e >> 2;
     const uint32_t lanes = (uint32_t)(32 * (e & 3)) << 16;
     float s[kGroupedCols][16];
@@ -264,7 +283,8 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       const int2 un = a.units[ui];
       const SplitJob& j = a.jobs[un.x];
       const int groups = j.npad / 16, g0 = half ? (groups + 1) / 2 : 0, ng = half ? groups / 2 : (groups + 1) / 2;
-      const long long gm = (long long)(un.y * CG + rank) * BM + 32 * (e & 3) + lane;
+      // (TMEM lane -> row: see read_classes)
+      const long long gm = (long long)(un.y * CG + rank) * BM + (TRANS ? 32 * (e & 3) + lane : 4 * lane + (e & 3));
       float* dst = j.out + gm * j.ldo;
       const int ncols = gm < j.M ? j.N : 0;
       clear_sums(s);
@@ -290,6 +310,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         left -= n;
         since += n;
         if (left > 0 && since < a.flush) continue;
+        if (PARTS == 3 && j.bad != nullptr) check_sums(s, g0, ng, ncols, j.bad);
         store_sums(s, dst, 4, g0, ng, ncols, j.vec_out != 0, flushed);
         clear_sums(s);
         flushed = true;
@@ -369,6 +390,15 @@ cudaError_t launch(const GroupArgs& a, int pairs, size_t smem, cudaStream_t st) 
 int split_npad(int n) { return (int)round_up(n, 16); }
 size_t split_image_bytes(int64_t K, int n, int parts) { return (size_t)round_up(K, BK) * split_npad(n) * parts * 2; }
 uint32_t split_idesc(int npad) { return tc::idesc_bf16(BM * CG, npad, false, false); }
+bool split_job_maps(void* maps, SplitJob* j, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans) {
+  Classes cl;
+  if (!class_maps(static_cast<CUtensorMap*>(maps), &cl, A, rows, cols, lda, trans)) return false;
+  for (int c = 0; c < 4; ++c) {
+    j->shift[c] = cl.shift[c];
+    j->past[c] = cl.past[c];
+  }
+  return true;
+}
 int split_x_blocks(int64_t K, int npad) { return (int)(cdiv(K, 64) * cdiv(npad, 32)); }
 
 cudaError_t split_x_grouped(const SplitXJob* jobs, const int* start, int count, int total, SplitMode mode,
@@ -397,9 +427,11 @@ cudaError_t split_grouped(bool transA, const SplitJob* jobs, const int2* units, 
   a.nbuf = 2 * a.npm + cc + 2 * parts * 16 <= 512 ? 2 : 1;
   a.sa = std::min(kMaxASlots, (512 - a.nbuf * a.npm - cc) / (parts * 16));
   const size_t stage = (size_t)parts * (a.npm / CG) * BK * 2, extra = 2048;
-  a.sx = (int)std::min<size_t>(kMaxStages, (smem_optin_grouped() - extra - kCopyStages * kCopyBytes) / stage);
-  if (a.sa < 2 || a.sx < 2) return cudaErrorInvalidValue;
-  const size_t smem = kCopyStages * kCopyBytes + a.sx * stage + extra;
+  const size_t avail = smem_optin_grouped() - extra;
+  a.sf = (int)std::min<size_t>(kMaxStages, (avail - 4 * stage) / kClassBytes);
+  a.sx = (int)std::min<size_t>(kMaxStages, (avail - a.sf * kClassBytes) / stage);
+  if (a.sa < 2) return cudaErrorInvalidValue;
+  const size_t smem = a.sf * kClassBytes + a.sx * stage + extra;
   if (transA) return parts == 3 ? launch<true, 3>(a, pairs, smem, st) : launch<true, 2>(a, pairs, smem, st);
   return parts == 3 ? launch<false, 3>(a, pairs, smem, st) : launch<false, 2>(a, pairs, smem, st);
 }
