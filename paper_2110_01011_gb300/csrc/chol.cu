@@ -488,6 +488,7 @@ template <typename T, bool kShared>
 __global__ void __launch_bounds__(kThreads)
 chol_blocked_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __restrict__ R, float* __restrict__ Rinv,
                     int64_t ldr, int* info, double* shift_count, int* gate_out, const int* gate_in, T* gS) {
+  grid_wait();
   chol_body<T, kShared>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in, gS);
 }
 
@@ -532,6 +533,7 @@ template <int NB>
 __global__ void __launch_bounds__(kClusterThreads)
 chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __restrict__ R, float* __restrict__ Rinv,
                     int64_t ldr, int* info, double* shift_count, int* gate_out, const int* gate_in) {
+  grid_wait();
   extern __shared__ __align__(32) unsigned char smem_raw[];
   constexpr int kCLd = NB + kDtPad;
   const int LDS = lds_of(d), rank = blockIdx.x, P = gridDim.x;
@@ -770,11 +772,11 @@ cudaError_t launch(int d, const float* G, int64_t ldg, float* R, float* Rinv, in
   if (!in_smem && gstore == nullptr) return cudaErrorInvalidValue;
   const size_t dyn = panel_bytes<T>() + (in_smem ? square_bytes<T>(d) : 0);
   if (in_smem)
-    chol_blocked_kernel<T, true><<<1, kThreads, dyn, st>>>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out,
-                                                           gate_in, nullptr);
+    launch_pdl(chol_blocked_kernel<T, true>, 1, kThreads, dyn, st, d, G, ldg, R, Rinv, ldr, info, shift_count,
+               gate_out, gate_in, nullptr);
   else
-    chol_blocked_kernel<T, false><<<1, kThreads, dyn, st>>>(d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out,
-                                                            gate_in, reinterpret_cast<T*>(gstore));
+    launch_pdl(chol_blocked_kernel<T, false>, 1, kThreads, dyn, st, d, G, ldg, R, Rinv, ldr, info, shift_count,
+               gate_out, gate_in, reinterpret_cast<T*>(gstore));
   note_launch();
   return cudaGetLastError();
 }
@@ -789,17 +791,19 @@ cudaError_t launch_cluster(int d, const float* G, int64_t ldg, float* R, float* 
     configured = true;
   }
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)cdiv(d, NB);
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // (see launch_pdl)
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3((unsigned)cdiv(d, NB));
   cfg.blockDim = dim3(kClusterThreads);
   cfg.dynamicSmemBytes = cluster_smem_bytes<NB>(d);
   cfg.stream = st;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   const cudaError_t e =
       cudaLaunchKernelEx(&cfg, chol_cluster_kernel<NB>, d, G, ldg, R, Rinv, ldr, info, shift_count, gate_out, gate_in);
   note_launch();

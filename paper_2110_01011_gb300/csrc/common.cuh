@@ -69,6 +69,37 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // (reported by rqlp_kernel_launches). Every launch site calls note_launch().
 void note_launch(int n = 1);
 
+// Kernels of a chain follow one another on a stream and each needs its predecessor's
+// results. Programmatic dependent launch lets a kernel's CTAs be placed while
+// the predecessor's last CTAs still run: launch_pdl sets the attribute, and the
+// kernel starts with grid_wait(), which returns once the predecessor has
+// completed with its writes visible. The wait comes before anything else,
+// allocations of tensor memory included (a waiting CTA must hold nothing that
+// the predecessor may ask for), in every kernel launched this way and by every
+// thread, so that completion of a kernel implies that of all before it. Errors
+// are left to cudaGetLastError. Measured: 1000 x 1000 FP32 (68 launches) 362 ->
+// 206 us, 4097 x 2999 882 -> 678 us. The batched kernels are launched plainly:
+// they run from a CUDA graph, whose launches are as close already (64 problems
+// 2.10 ms plainly, 2.18 ms with the attribute).
+template <typename... P, typename... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Optional per-pass timing: when enabled, every pass over A is bracketed by a
 // CUDA event pair recorded on the launching stream.
 bool profiling_on();

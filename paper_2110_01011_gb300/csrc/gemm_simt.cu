@@ -298,6 +298,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int64_t m0, int64_t
 template <int BM, int BN, int BK, int TM, int TN, bool TRANS_A>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), 512 / ((BM / TM) * (BN / TN)))
 gemm_f32_kernel(GemmArgs g) {
+  grid_wait();
   gemm_tile<BM, BN, BK, TM, TN, TRANS_A>(g, (int64_t)blockIdx.y * BM, (int64_t)blockIdx.x * BN, blockIdx.z);
 }
 
@@ -355,6 +356,7 @@ constexpr size_t wide_tot_bytes() { return (size_t)8 * (4 + (BN - 64) / 16) * kW
 
 template <bool TRANS_A, bool VEC, int BN>
 __global__ void __launch_bounds__(kWideThreads, kWidePerSm) gemm_f32_wide_kernel(GemmArgs g) {
+  grid_wait();
   constexpr int BM = kWideBM, BK = kWideBK, NT = kWideThreads;
   constexpr int TN2 = (BN - 64) / 16, TN = 4 + TN2;
   constexpr int QB = BN / 4;                 // float4 per row of a B tile
@@ -548,6 +550,7 @@ __global__ void __launch_bounds__(kWideThreads, kWidePerSm) gemm_f32_wide_kernel
 // with kGateSkip wrote no partial tiles, and nothing is summed.
 __global__ void splitk_reduce_kernel(int64_t M, int64_t N, int splits, const float* __restrict__ part,
                                      float* __restrict__ C, int64_t ldc, int lower_only, const int* skip_gate) {
+  grid_wait();
   if (skip_gate != nullptr && *skip_gate == 0) return;
   const int64_t total = M * N;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
@@ -662,7 +665,7 @@ static cudaError_t launch_gemm(bool transA, const GemmArgs& g, int splits, cudaS
       if (e_ != cudaSuccess) return e_;                                                                 \
       set_ = true;                                                                                      \
     }                                                                                                   \
-    gemm_f32_wide_kernel<T, V, W><<<grid, kWideThreads, wide_tot_bytes<W>(), st>>>(g);                 \
+    launch_pdl(gemm_f32_wide_kernel<T, V, W>, grid, kWideThreads, wide_tot_bytes<W>(), st, g);                 \
   } while (0)
     if (bn == 112) {
       if (transA) { if (vec) RQLP_WIDE(true, true, 112); else RQLP_WIDE(true, false, 112); }
@@ -675,18 +678,18 @@ static cudaError_t launch_gemm(bool transA, const GemmArgs& g, int splits, cudaS
     note_launch();
   } else if (big && big_bn(g.N, g.K) == 32) {
     dim3 grid((unsigned)cdiv(g.N, 32), (unsigned)cdiv(g.M, 128), (unsigned)splits);
-    if (transA) gemm_f32_kernel<128, 32, 16, 8, 4, true><<<grid, 128, 0, st>>>(g);
-    else        gemm_f32_kernel<128, 32, 16, 8, 4, false><<<grid, 128, 0, st>>>(g);
+    if (transA) launch_pdl(gemm_f32_kernel<128, 32, 16, 8, 4, true>, grid, 128, 0, st, g);
+    else        launch_pdl(gemm_f32_kernel<128, 32, 16, 8, 4, false>, grid, 128, 0, st, g);
     note_launch();
   } else if (big) {
     dim3 grid((unsigned)cdiv(g.N, 64), (unsigned)cdiv(g.M, 128), (unsigned)splits);
-    if (transA) gemm_f32_kernel<128, 64, 16, 8, 4, true><<<grid, 256, 0, st>>>(g);
-    else        gemm_f32_kernel<128, 64, 16, 8, 4, false><<<grid, 256, 0, st>>>(g);
+    if (transA) launch_pdl(gemm_f32_kernel<128, 64, 16, 8, 4, true>, grid, 256, 0, st, g);
+    else        launch_pdl(gemm_f32_kernel<128, 64, 16, 8, 4, false>, grid, 256, 0, st, g);
     note_launch();
   } else {
     dim3 grid((unsigned)cdiv(g.N, 32), (unsigned)cdiv(g.M, 32), (unsigned)splits);
-    if (transA) gemm_f32_kernel<32, 32, 16, 4, 4, true><<<grid, 64, 0, st>>>(g);
-    else        gemm_f32_kernel<32, 32, 16, 4, 4, false><<<grid, 64, 0, st>>>(g);
+    if (transA) launch_pdl(gemm_f32_kernel<32, 32, 16, 4, 4, true>, grid, 64, 0, st, g);
+    else        launch_pdl(gemm_f32_kernel<32, 32, 16, 4, 4, false>, grid, 64, 0, st, g);
     note_launch();
   }
   return cudaGetLastError();
@@ -716,8 +719,8 @@ cudaError_t gemm_f32_ex(bool transA, int64_t M, int64_t N, int64_t K, const floa
   if (e != cudaSuccess) return e;
   int64_t total = M * N;
   int blocks = (int)std::min<int64_t>(cdiv(total, 256), (int64_t)sm_count() * 8);
-  splitk_reduce_kernel<<<blocks, 256, 0, st>>>(M, N, used, part, C, ldc, lower_only ? 1 : 0,
-                                                 gate_mode == kGateSkip ? gate : nullptr);
+  launch_pdl(splitk_reduce_kernel, blocks, 256, 0, st, M, N, used, part, C, ldc, lower_only ? 1 : 0,
+             gate_mode == kGateSkip ? gate : nullptr);
   note_launch();
   return cudaGetLastError();
 }

@@ -40,6 +40,7 @@ template <bool BACKWARD>
 __global__ void __launch_bounds__(H)
 mlp_sample_kernel(const float* __restrict__ prm, const float* __restrict__ X, int B, const float* __restrict__ Y,
                   float* __restrict__ est, SampleBufs sb) {
+  grid_wait();
   __shared__ float x[F], h1[H], h2[H], d3[NO], dz2[H], sq[NO];
   const int t = threadIdx.x;
   for (int b = blockIdx.x; b < B; b += gridDim.x) {
@@ -93,6 +94,7 @@ mlp_sample_kernel(const float* __restrict__ prm, const float* __restrict__ X, in
 // grad[i] = sum over samples b (in order) of the per-sample term of parameter i.
 __global__ void mlp_grad_reduce_kernel(const float* __restrict__ X, int B, SampleBufs sb, float* __restrict__ grad,
                                        float* __restrict__ loss) {
+  grid_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == NPARAM && loss != nullptr) {
     float s = 0.f;
@@ -126,6 +128,7 @@ __global__ void mlp_grad_reduce_kernel(const float* __restrict__ X, int B, Sampl
 __global__ void adam_kernel(float* __restrict__ prm, const float* __restrict__ g, float* __restrict__ m1,
                             float* __restrict__ m2, int n, float lr, float beta1, float beta2, float eps, float c1,
                             float c2) {
+  grid_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float gi = g[i];
@@ -140,6 +143,7 @@ __global__ void adam_kernel(float* __restrict__ prm, const float* __restrict__ g
 // in the FP64 reference. One warp.
 __global__ void probe_features_kernel(const float* __restrict__ R, int64_t ldr, int w, int k, int64_t mn,
                                       float* __restrict__ feat) {
+  grid_wait();
   __shared__ float lr[RQLP_MAX_D];
   const int t = threadIdx.x;
   const float r0 = R[0];
@@ -186,6 +190,7 @@ __global__ void probe_features_kernel(const float* __restrict__ R, int64_t ldr, 
 // or delta is not finite.
 __global__ void predict_kernel(const float* __restrict__ est, const float* __restrict__ prm, const int* __restrict__ info,
                                float log_target, int k, int* __restrict__ qp) {
+  grid_wait();
   const float delta = prm[OFF_DELTA];
   bool ok = (info == nullptr || info[0] == 0) && isfinite(delta);
   for (int o = 0; o < NO; ++o) ok = ok && isfinite(est[o]);
@@ -228,7 +233,7 @@ size_t mlp_workspace_floats(int B) { return (size_t)B * (4 * H + NO + 1); }
 
 cudaError_t mlp_forward(const float* prm, const float* X, int B, float* est, cudaStream_t st) {
   const int blocks = std::min(B, sm_count() * 8);
-  mlp_sample_kernel<false><<<blocks, H, 0, st>>>(prm, X, B, nullptr, est, SampleBufs{});
+  launch_pdl(mlp_sample_kernel<false>, blocks, H, 0, st, prm, X, B, nullptr, est, SampleBufs{});
   note_launch();
   return cudaGetLastError();
 }
@@ -237,11 +242,11 @@ cudaError_t mlp_grad(const float* prm, const float* X, const float* Y, int B, fl
                      cudaStream_t st) {
   SampleBufs sb = carve(ws, B);
   const int blocks = std::min(B, sm_count() * 8);
-  mlp_sample_kernel<true><<<blocks, H, 0, st>>>(prm, X, B, Y, nullptr, sb);
+  launch_pdl(mlp_sample_kernel<true>, blocks, H, 0, st, prm, X, B, Y, nullptr, sb);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  mlp_grad_reduce_kernel<<<(NPARAM + 1 + 127) / 128, 128, 0, st>>>(X, B, sb, grad, loss);
+  launch_pdl(mlp_grad_reduce_kernel, (NPARAM + 1 + 127) / 128, 128, 0, st, X, B, sb, grad, loss);
   note_launch();
   return cudaGetLastError();
 }
@@ -249,20 +254,20 @@ cudaError_t mlp_grad(const float* prm, const float* X, const float* Y, int B, fl
 cudaError_t mlp_adam(float* prm, const float* g, float* m1, float* m2, int n, float lr, float beta1, float beta2,
                      float eps, int step, cudaStream_t st) {
   const float c1 = 1.f - powf(beta1, (float)step), c2 = 1.f - powf(beta2, (float)step);
-  adam_kernel<<<(n + 255) / 256, 256, 0, st>>>(prm, g, m1, m2, n, lr, beta1, beta2, eps, c1, c2);
+  launch_pdl(adam_kernel, (n + 255) / 256, 256, 0, st, prm, g, m1, m2, n, lr, beta1, beta2, eps, c1, c2);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t probe_features(const float* R, int64_t ldr, int w, int k, int64_t mn, float* feat, cudaStream_t st) {
-  probe_features_kernel<<<1, 32, 0, st>>>(R, ldr, w, k, mn, feat);
+  launch_pdl(probe_features_kernel, 1, 32, 0, st, R, ldr, w, k, mn, feat);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t predict_qp(const float* est, const float* prm, const int* info, double target, int k, int* qp,
                        cudaStream_t st) {
-  predict_kernel<<<1, 1, 0, st>>>(est, prm, info, (float)std::log10(target), k, qp);
+  launch_pdl(predict_kernel, 1, 1, 0, st, est, prm, info, (float)std::log10(target), k, qp);
   note_launch();
   return cudaGetLastError();
 }

@@ -23,7 +23,7 @@
 namespace rqlp {
 namespace {
 
-constexpr int kGates = 8;   // gate words: one per final orthonormalisation, [3] intermediate ones
+constexpr int kGates = 64;   // gate words: one per final orthonormalisation, the rest intermediate ones in turn
 constexpr int kInterGate = 3;
 constexpr int kScal = 4;    // [0] ||A||^2, [1] ||L||^2, [2] shifted Cholesky count, [3] spare
 
@@ -103,6 +103,7 @@ class Ops {
   cudaError_t init() {
     tcs_.reset();
     CK(begin_products());
+    inter_ = kInterGate;
     return init_scratch(info_, gates, kGates, scal, kScal, st_);
   }
 
@@ -242,11 +243,14 @@ class Ops {
   // product). have_r0: the R factor is already in slot 0 (the probe) and the
   // probe's shift flag in gates[kInterGate].
   cudaError_t orth_inter(float* X, int64_t ldx, int64_t rows, float* out, int64_t ldout, bool have_r0 = false) {
-    int* g = &gates[kInterGate];
+    // A cleared gate word of its own; past the last one, that one is cleared
+    // again (a launch and a break in the chain of dependent launches).
+    const bool fresh = inter_ < kGates;
+    int* g = &gates[fresh ? inter_++ : kGates - 1];
     if (have_r0) {
       CK(apply_r0(X, ldx, rows, out, ldout));
     } else {
-      CK(cudaMemsetAsync(g, 0, sizeof(int), st_));
+      if (!fresh) CK(cudaMemsetAsync(g, 0, sizeof(int), st_));
       if (tc_on_ && rows > (int64_t)d_) {
         CK(tc_cqr(X, ldx, rows, out, ldout, 0, g, false));
       } else {
@@ -326,6 +330,7 @@ class Ops {
   bool tc_on_ = false;
   bool three_ = false;
   bool split32_ = false;
+  int inter_ = kInterGate;   // next intermediate gate word
   const SparseA* sp_ = nullptr;
   const SparseA* spt_ = nullptr;
 };

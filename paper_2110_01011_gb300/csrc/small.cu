@@ -16,6 +16,7 @@ __device__ void post_error(int* info, int code, int detail) {
 // Y = X^T for a d x d matrix.
 __global__ void transpose_kernel(int d, const float* __restrict__ X, int64_t ldx, float* __restrict__ Y,
                                  int64_t ldy) {
+  grid_wait();
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * d; e += gridDim.x * blockDim.x) {
     int i = e / d, l = e % d;
     Y[(int64_t)l * ldy + i] = X[(int64_t)i * ldx + l];
@@ -26,6 +27,7 @@ __global__ void transpose_kernel(int d, const float* __restrict__ X, int64_t ldx
 // ||L||_F^2 accumulated into *l2 (double, one atomic per CTA).
 __global__ void write_L_kernel(int d, const float* __restrict__ Rh, int64_t ldrh, float* __restrict__ L,
                                int64_t ldl, double* l2) {
+  grid_wait();
   __shared__ double red[32];
   double acc = 0.0;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * d; e += gridDim.x * blockDim.x) {
@@ -46,6 +48,7 @@ __global__ void write_L_kernel(int d, const float* __restrict__ Rh, int64_t ldrh
 
 // info <- 0, scratch scalars <- 0.
 __global__ void init_kernel(int* info, int* gates, int ngates, double* scal, int nscal) {
+  grid_wait();
   int t = threadIdx.x;
   if (t < 2) info[t] = 0;
   if (t < ngates) gates[t] = 0;
@@ -54,6 +57,7 @@ __global__ void init_kernel(int* info, int* gates, int ngates, double* scal, int
 
 // diag = [||A||^2, ||L||^2, ||A||^2 - ||L||^2, shifts]; flags non-finite A.
 __global__ void finish_diag_kernel(const double* scal, double* diag, int* info) {
+  grid_wait();
   if (threadIdx.x != 0) return;
   double a2 = scal[0], l2 = scal[1];
   if (!isfinite(a2)) post_error(info, RQLP_ERR_NONFINITE, 0);
@@ -67,6 +71,7 @@ __global__ void finish_diag_kernel(const double* scal, double* diag, int* info) 
 
 __global__ void copy_kernel(int64_t rows, int64_t cols, const float* __restrict__ X, int64_t ldx,
                             float* __restrict__ Y, int64_t ldy, const int* __restrict__ gate) {
+  grid_wait();
   if (gate != nullptr && *gate == 0) return;
   const int64_t total = rows * cols;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
@@ -165,7 +170,7 @@ cudaError_t finish_diag_batched(const SmallJob* jobs, int count, cudaStream_t st
 
 cudaError_t transpose_small(int d, const float* X, int64_t ldx, float* Y, int64_t ldy, cudaStream_t st) {
   int blocks = std::max(1, std::min(64, (d * d + 255) / 256));
-  transpose_kernel<<<blocks, 256, 0, st>>>(d, X, ldx, Y, ldy);
+  launch_pdl(transpose_kernel, blocks, 256, 0, st, d, X, ldx, Y, ldy);
   note_launch();
   return cudaGetLastError();
 }
@@ -173,19 +178,19 @@ cudaError_t transpose_small(int d, const float* X, int64_t ldx, float* Y, int64_
 cudaError_t write_L(int d, const float* Rh, int64_t ldrh, float* L, int64_t ldl, double* l2,
                     cudaStream_t st) {
   int blocks = std::max(1, std::min(64, (d * d + 255) / 256));
-  write_L_kernel<<<blocks, 256, 0, st>>>(d, Rh, ldrh, L, ldl, l2);
+  launch_pdl(write_L_kernel, blocks, 256, 0, st, d, Rh, ldrh, L, ldl, l2);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t init_scratch(int* info, int* gates, int ngates, double* scal, int nscal, cudaStream_t st) {
-  init_kernel<<<1, 64, 0, st>>>(info, gates, ngates, scal, nscal);
+  launch_pdl(init_kernel, 1, 64, 0, st, info, gates, ngates, scal, nscal);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t finish_diag(const double* scal, double* diag, int* info, cudaStream_t st) {
-  finish_diag_kernel<<<1, 32, 0, st>>>(scal, diag, info);
+  launch_pdl(finish_diag_kernel, 1, 32, 0, st, scal, diag, info);
   note_launch();
   return cudaGetLastError();
 }
@@ -223,6 +228,7 @@ cudaError_t copy_gated_batched(const SmallJob* jobs, int count, cudaStream_t st)
 
 __global__ void add_kernel(int64_t rows, int64_t cols, const float* __restrict__ X, int64_t ldx,
                            float* __restrict__ Y, int64_t ldy) {
+  grid_wait();
   const int64_t total = rows * cols;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
@@ -236,7 +242,7 @@ cudaError_t add_matrix(int64_t rows, int64_t cols, const float* X, int64_t ldx, 
   const int64_t total = rows * cols;
   if (total <= 0) return cudaSuccess;
   const int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sm_count() * 8);
-  add_kernel<<<blocks, 256, 0, st>>>(rows, cols, X, ldx, Y, ldy);
+  launch_pdl(add_kernel, blocks, 256, 0, st, rows, cols, X, ldx, Y, ldy);
   note_launch();
   return cudaGetLastError();
 }
@@ -246,7 +252,7 @@ cudaError_t copy_matrix(int64_t rows, int64_t cols, const float* X, int64_t ldx,
   int64_t total = rows * cols;
   if (total <= 0) return cudaSuccess;
   int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)sm_count() * 8);
-  copy_kernel<<<blocks, 256, 0, st>>>(rows, cols, X, ldx, Y, ldy, gate);
+  launch_pdl(copy_kernel, blocks, 256, 0, st, rows, cols, X, ldx, Y, ldy, gate);
   note_launch();
   return cudaGetLastError();
 }

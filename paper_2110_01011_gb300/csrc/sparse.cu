@@ -29,6 +29,7 @@ __global__ void __launch_bounds__(256)
 csr_spmm_kernel(const int64_t* __restrict__ ptr, const int* __restrict__ idx, const float* __restrict__ val,
                 int64_t rows, int64_t K, const float* __restrict__ X, int64_t ldx, int d, float* __restrict__ Y,
                 int64_t ldy, double* sumsq, int* info) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -69,6 +70,7 @@ csr_spmm_kernel(const int64_t* __restrict__ ptr, const int* __restrict__ idx, co
 
 // counts[j] = number of entries in column j (valid indices only).
 __global__ void csc_count_kernel(const int* __restrict__ idx, int64_t nnz, int64_t n, int* __restrict__ counts) {
+  grid_wait();
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz; p += (int64_t)gridDim.x * blockDim.x) {
     const int j = idx[p];
     if (j >= 0 && j < n) atomicAdd(&counts[j], 1);
@@ -78,6 +80,7 @@ __global__ void csc_count_kernel(const int* __restrict__ idx, int64_t nnz, int64
 // col_ptr = exclusive prefix sum of counts (n + 1 entries); one CTA.
 __global__ void __launch_bounds__(1024) csc_scan_kernel(const int* __restrict__ counts, int64_t n,
                                                         int64_t* __restrict__ col_ptr) {
+  grid_wait();
   __shared__ int64_t part[1024];
   const int t = threadIdx.x;
   const int64_t chunk = (n + blockDim.x - 1) / blockDim.x;
@@ -108,6 +111,7 @@ __global__ void __launch_bounds__(256)
 csc_fill_kernel(const int64_t* __restrict__ ptr, const int* __restrict__ idx, const float* __restrict__ val,
                 int64_t rows, int64_t n, const int64_t* __restrict__ col_ptr, int* __restrict__ fill,
                 int* __restrict__ ridx, float* __restrict__ rval) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -127,6 +131,7 @@ csc_fill_kernel(const int64_t* __restrict__ ptr, const int* __restrict__ idx, co
 // per column): the scatter's order depends on the atomics.
 __global__ void csc_sort_kernel(const int64_t* __restrict__ col_ptr, int64_t n, int* __restrict__ ridx,
                                 float* __restrict__ rval) {
+  grid_wait();
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
     const int64_t s = col_ptr[j], e = col_ptr[j + 1];
     for (int64_t p = s + 1; p < e; ++p) {
@@ -171,15 +176,15 @@ cudaError_t sparse_build_csc(const SparseA& a, void* ws, SparseA* t, int* info, 
   CK(cudaMemsetAsync(counts, 0, sizeof(int) * a.n, st));
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(a.nnz, 256), (int64_t)sm_count() * 8));
   if (a.nnz > 0) {
-    csc_count_kernel<<<blocks, 256, 0, st>>>(a.col_idx, a.nnz, a.n, counts);
+    launch_pdl(csc_count_kernel, blocks, 256, 0, st, a.col_idx, a.nnz, a.n, counts);
     note_launch();
   }
-  csc_scan_kernel<<<1, 1024, 0, st>>>(counts, a.n, col_ptr);
+  launch_pdl(csc_scan_kernel, 1, 1024, 0, st, counts, a.n, col_ptr);
   CK(cudaMemsetAsync(counts, 0, sizeof(int) * a.n, st));   // reused as the fill cursor
-  csc_fill_kernel<<<spmm_blocks(a.m), 256, 0, st>>>(a.row_ptr, a.col_idx, a.vals, a.m, a.n, col_ptr, counts, ridx,
-                                                    rval);
-  csc_sort_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>(cdiv(a.n, 128), (int64_t)sm_count() * 4)), 128, 0,
-                    st>>>(col_ptr, a.n, ridx, rval);
+  launch_pdl(csc_fill_kernel, spmm_blocks(a.m), 256, 0, st, a.row_ptr, a.col_idx, a.vals, a.m, a.n, col_ptr, counts,
+             ridx, rval);
+  launch_pdl(csc_sort_kernel, (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(a.n, 128), (int64_t)sm_count() * 4)),
+             128, 0, st, col_ptr, a.n, ridx, rval);
   note_launch(3);
   t->m = a.n;
   t->n = a.m;
@@ -194,8 +199,8 @@ cudaError_t sparse_build_csc(const SparseA& a, void* ws, SparseA* t, int* info, 
 cudaError_t sparse_spmm(const SparseA& s, const float* X, int64_t ldx, int d, float* Y, int64_t ldy, double* sumsq,
                         int* info, cudaStream_t st) {
   if (d > RQLP_MAX_D) return cudaErrorInvalidValue;
-  csr_spmm_kernel<<<spmm_blocks(s.m), 256, 0, st>>>(s.row_ptr, s.col_idx, s.vals, s.m, s.n, X, ldx, d, Y, ldy, sumsq,
-                                                    info);
+  launch_pdl(csr_spmm_kernel, spmm_blocks(s.m), 256, 0, st, s.row_ptr, s.col_idx, s.vals, s.m, s.n, X, ldx, d, Y, ldy,
+             sumsq, info);
   note_launch();
   return cudaGetLastError();
 }

@@ -114,6 +114,7 @@ struct Args {
   int* info;
   int M, N, K, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole, perm;   // sx, sf, sa: stages of X, of A in FP32, A slots
   int chunk;                // units per chain of the main accumulator
+  int stagger;              // 128-row tiles over SMs that the cuts of the chains are staggered by (0: chains from the range's start)
   int corr_first;           // chains of one unit, the correction products first
   int flush;                // units whose sums are held in registers before they are added to global memory
   int corr;                 // 0: one accumulator; else main chains per chain of the correction accumulator
@@ -132,6 +133,23 @@ __host__ __device__ inline int unit_owner(int u, int units, int G) {
   return (int)((((long long)u + 1) * G + units - 1) / units) - 1;
 }
 
+// Units of the chain that starts at unit k of tile t, of which `left` are to do.
+// Truncation makes every chain lose a little toward zero; chains that start at
+// the same K in all rows make that a coherent change of A, which moves the
+// subspaces (P of the 20000^2 learned factorisation: 3.8e-5 off with cuts at
+// multiples of 4096 everywhere, 2.7e-5 with cuts that differ from tile to tile).
+// So each tile has a cut of its own, where even shares of 128-row tiles per SM
+// would split it, and the chains before and after it count from 0 and from the
+// cut, wherever the tile is split among CTAs.
+__device__ inline int chain_units(const Args& a, int t, int k, int left) {
+  if (a.stagger == 0) return min(left, a.chunk);
+  const long long tiles = cdiv(a.M, (int64_t)BM), g = a.stagger, u = 2 * t;
+  const long long c = (u * g + tiles - 1) / tiles;   // first share that starts in tile u
+  const int cut = (int)((2 * (tiles * c - u * g) + tiles - g) * a.kb / (2 * g));
+  if (k < cut) return min(min(left, cut - k), a.chunk - k % a.chunk);
+  return min(left, a.chunk - (k - cut) % a.chunk);
+}
+
 // Maps over A: one, or one per class of rows.
 struct MapsA {
   CUtensorMap m[4];
@@ -141,6 +159,7 @@ struct MapsA {
 template <bool TRANS, int PARTS, bool ALIGNED>
 __global__ void __launch_bounds__(kThreads, 1)
 split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
+  grid_wait();
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -243,10 +262,10 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
       bool ok = true;
       if (rank == 0) {
         Ring rx, ra, rb;      // X stages, A slots, main accumulators
-        int k = u0 % KB, left = u1 - u0, chain = 0;   // chain: main chains of this tile part
+        int k = u0 % KB, t = u0 / KB, left = u1 - u0, chain = 0;   // chain: main chains of this tile part
         uint32_t cph = 0;     // parity of the correction chains
         while (left > 0 && ok) {
-          const int n = min(min(left, KB - k), a.chunk);
+          const int n = chain_units(a, t, k, min(left, KB - k));
           const bool cnew = a.corr != 0 && chain % a.corr == 0;   // a correction chain begins
           if (!wait(&acce[rb.s], rb.ph ^ 1u) || (cnew && !wait(corre, cph ^ 1u))) {
             ok = false;
@@ -283,7 +302,10 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
           k += n;
           left -= n;
           if (a.corr && (chain % a.corr == 0 || k == KB || left == 0)) cph ^= 1u;
-          if (k == KB) k = chain = 0;
+          if (k == KB) {
+            k = chain = 0;
+            ++t;
+          }
         }
         if (elect()) commit(done);   // no MMA in flight at teardown
       }
@@ -422,7 +444,7 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
     bool flushed = false;   // earlier sums of this part are in memory
     Ring rb;
     while (left > 0) {
-      const int n = min(min(left, KB - k), a.chunk);
+      const int n = chain_units(a, t, k, min(left, KB - k));
       const bool part_end = n == left || k + n == KB;
       if (ok && !wait(&accf[rb.s], rb.ph)) {
         ok = false;
@@ -553,6 +575,7 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
 // Sums the partial tiles of a product whose tiles span many CTAs: thread f
 // takes float4 f of the tiles that were split, slots in CTA order.
 __global__ void split_fixup_kernel(const Args a) {
+  grid_wait();
   const int Q = a.npad / 4;
   const long long per = (long long)BM * Q, total = (long long)a.tiles * CG * per;
   for (long long f = (long long)blockIdx.x * blockDim.x + threadIdx.x; f < total;
@@ -596,6 +619,7 @@ __global__ void split_fixup_kernel(const Args a) {
 __global__ void __launch_bounds__(256)
 split_x_kernel(const float* __restrict__ X, long long K, int N, long long ldx, uint16_t* __restrict__ img, int npad,
                int parts, int kb, int* xlo, int* bad) {
+  grid_wait();
   split_x_tile(X, K, N, ldx, img, npad, parts, kb, (long long)blockIdx.x * 64, blockIdx.y * 32, xlo, bad);
 }
 
@@ -619,15 +643,17 @@ template <bool TRANS, int PARTS, bool ALIGNED>
 cudaError_t launch(const MapsA& map, Args& a, int cap, size_t smem, cudaStream_t st) {
   static int resident = 0;   // pairs that run at the same time
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   cfg.blockDim = dim3(kThreads);
   cfg.stream = st;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = CG;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // (see launch_pdl)
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   if (resident == 0) {
     CK(cudaFuncSetAttribute(split_gemm_kernel<TRANS, PARTS, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)smem_optin()));
@@ -652,8 +678,8 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   const int parts = mode == kSplitTwo ? 2 : 3;
   const int npad = npad_of(N), kb = (int)cdiv(K, BK);
   int* w = ws->words;
-  split_x_kernel<<<dim3((unsigned)cdiv(kb, 2), (unsigned)cdiv(npad, 32)), 256, 0, st>>>(
-      X, K, N, ldx, ws->img, npad, parts, kb, w + turn, bad);
+  launch_pdl(split_x_kernel, dim3((unsigned)cdiv(kb, 2), (unsigned)cdiv(npad, 32)), 256, 0, st, X, K, N, ldx, ws->img,
+             npad, parts, kb, w + turn, bad);
   note_launch();
   CK(cudaGetLastError());
 
@@ -678,6 +704,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   // Groups: at most two partial tiles each (none with whole tiles).
   const int cap = a.whole ? a.tiles : std::min(a.units, ws->slots / (2 * CG));
   a.vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0 && ldo % 4 == 0) ? 1 : 0;
+  a.stagger = mode != kSplitFp32 && !a.whole && cdiv(M, BM) > sm_count() ? sm_count() : 0;
   // Chains. An MMA loses about half a unit in the last place of the sum that
   // it adds to, always toward zero. FP32: one chain per unit, the correction
   // products (2^-8 of the main ones) first, so that only two MMAs add to a
@@ -718,7 +745,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   if (e == cudaSuccess && a.fixup) {
     const long long total = (long long)a.tiles * CG * BM * (npad / 4);
     const int blocks = (int)std::min<long long>(cdiv(total, 256), (long long)sm_count() * 8);
-    split_fixup_kernel<<<blocks, 256, 0, st>>>(a);
+    launch_pdl(split_fixup_kernel, blocks, 256, 0, st, a);
     note_launch();
     e = cudaGetLastError();
   }

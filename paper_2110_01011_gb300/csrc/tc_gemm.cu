@@ -123,6 +123,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
                const __grid_constant__ CUtensorMap tmXhi, const __grid_constant__ CUtensorMap tmXlo,
                const __grid_constant__ CUtensorMap tmAlo2, const __grid_constant__ CUtensorMap tmXlo2,
                const TcArgs a) {
+  grid_wait();
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -483,6 +484,7 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
 // output per thread, over the tile's contributors in CTA order (the order
 // and the values of the last-arriver reduction).
 __global__ void tc_fixup_kernel(const TcArgs a) {
+  grid_wait();
   const int Q = a.npad / 4, KB = a.kblocks;
   const long long total = (long long)a.tiles * BM * Q;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -533,6 +535,7 @@ struct GramArgs {
 __global__ void __launch_bounds__(kThreads, 1)
 tc_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUtensorMap tmLo,
                const GramArgs a) {
+  grid_wait();
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -648,6 +651,7 @@ tc_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__
 // to L2 instead of G.
 __global__ void tc_gram_reduce_kernel(const float* __restrict__ part, int G, int mtiles, int npad, int cols,
                                       float* __restrict__ out, long long ldo) {
+  grid_wait();
   const long long slot = (long long)mtiles * BM * npad;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < cols * cols; e += gridDim.x * blockDim.x) {
     const int i = e / cols, j = e % cols;
@@ -682,6 +686,7 @@ __global__ void tc_gram_reduce_kernel(const float* __restrict__ part, int G, int
 __global__ void split_a_kernel(const float* __restrict__ A, long long m, long long n, long long lda, bool vec,
                                bf16* __restrict__ hi, bf16* __restrict__ lo, bf16* __restrict__ lo2, long long npan,
                                double* sumsq, long long mstride, long long row0) {
+  grid_wait();
   const long long cpr = npan * 8, total = m * cpr;
   float s = 0.f, comp = 0.f;
   for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
@@ -739,6 +744,7 @@ constexpr int kPrepRows = 64;
 __global__ void prep_x_kernel(const float* __restrict__ X, long long rows, int d, long long ldx,
                               bf16* __restrict__ th, bf16* __restrict__ tl, bf16* __restrict__ tl2, long long ldk,
                               int* nonzero_lo) {
+  grid_wait();
   __shared__ float tile[kPrepRows][33];
   const long long r0 = (long long)blockIdx.x * kPrepRows;
   const int c0 = blockIdx.y * 32;
@@ -865,7 +871,7 @@ cudaError_t launch_pass(const CUtensorMap& ah, const CUtensorMap& al, const CUte
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  tc_pass_kernel<MN_A, BKP><<<a.G, kThreads, smem, st>>>(ah, al, xh, xl, al2, xl2, a);
+  launch_pdl(tc_pass_kernel<MN_A, BKP>, a.G, kThreads, smem, st, ah, al, xh, xl, al2, xl2, a);
   note_launch();
   return cudaGetLastError();
 }
@@ -915,9 +921,8 @@ cudaError_t TcEngine::split(const float* A, int64_t rows, int64_t cols, int64_t 
   const long long npan = cdiv(cols, 64);
   const long long total = rows * npan * 8;
   const int blocks = (int)std::min<long long>(cdiv(total, 256), (long long)G_ * 8);
-  split_a_kernel<<<blocks, 256, 0, st>>>(A, rows, cols, lda, vec, reinterpret_cast<bf16*>(Ahi_),
-                                         reinterpret_cast<bf16*>(Alo_), reinterpret_cast<bf16*>(Alo2_), npan,
-                                         sumsq, rows, 0);
+  launch_pdl(split_a_kernel, blocks, 256, 0, st, A, rows, cols, lda, vec, reinterpret_cast<bf16*>(Ahi_),
+             reinterpret_cast<bf16*>(Alo_), reinterpret_cast<bf16*>(Alo2_), npan, sumsq, rows, 0);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -943,9 +948,8 @@ cudaError_t TcEngine::split_rows(const float* Ablock, int64_t row0, int64_t rows
   const long long npan = cdiv(n_, 64);
   const long long total = rows * npan * 8;
   const int blocks = (int)std::max<long long>(1, std::min<long long>(cdiv(total, 256), (long long)G_ * 8));
-  split_a_kernel<<<blocks, 256, 0, st>>>(Ablock, rows, n_, lda, vec, reinterpret_cast<bf16*>(Ahi_),
-                                         reinterpret_cast<bf16*>(Alo_), reinterpret_cast<bf16*>(Alo2_), npan,
-                                         sumsq, m_, row0);
+  launch_pdl(split_a_kernel, blocks, 256, 0, st, Ablock, rows, n_, lda, vec, reinterpret_cast<bf16*>(Ahi_),
+             reinterpret_cast<bf16*>(Alo_), reinterpret_cast<bf16*>(Alo2_), npan, sumsq, m_, row0);
   note_launch();
   return cudaGetLastError();
 }
@@ -977,10 +981,9 @@ cudaError_t TcEngine::pass_k(bool transA, int64_t k0, int64_t K, const float* X,
   if ((e = cudaMemsetAsync(flag_, 0, sizeof(int), st)) != cudaSuccess) return e;
   {
     dim3 grid((unsigned)cdiv(round_up(K, 8), kPrepRows), (unsigned)cdiv(d, 32));
-    prep_x_kernel<<<grid, dim3(32, 8), 0, st>>>(X, K, d, ldx, reinterpret_cast<bf16*>(Xhi_),
-                                                 reinterpret_cast<bf16*>(Xlo_),
-                                                 exact ? reinterpret_cast<bf16*>(Xlo2_) : nullptr, round_up(K, 8),
-                                                 flag_);
+    launch_pdl(prep_x_kernel, grid, dim3(32, 8), 0, st, X, K, d, ldx, reinterpret_cast<bf16*>(Xhi_),
+               reinterpret_cast<bf16*>(Xlo_), exact ? reinterpret_cast<bf16*>(Xlo2_) : nullptr, round_up(K, 8),
+               flag_);
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -1060,7 +1063,7 @@ cudaError_t TcEngine::pass_k(bool transA, int64_t k0, int64_t K, const float* X,
   if (e == cudaSuccess && a.fixup) {
     const long long total = (long long)a.tiles * BM * (npad_ / 4);
     const int blocks = (int)std::min<long long>(cdiv(total, 256), (long long)G_ * 8);
-    tc_fixup_kernel<<<blocks, 256, 0, st>>>(a);
+    launch_pdl(tc_fixup_kernel, blocks, 256, 0, st, a);
     note_launch();
     e = cudaGetLastError();
   }
@@ -1103,12 +1106,12 @@ cudaError_t TcEngine::gram(float* Gout, int64_t ldg, int* info, cudaStream_t st)
     configured = true;
   }
   const size_t smem = (size_t)a.stages * a.stage_bytes + 1024 + 512;
-  tc_gram_kernel<<<a.G, kThreads, smem, st>>>(hi, lo, a);
+  launch_pdl(tc_gram_kernel, a.G, kThreads, smem, st, hi, lo, a);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int blocks = std::max(1, std::min(G_ * 2, (cols * cols + 255) / 256));
-  tc_gram_reduce_kernel<<<blocks, 256, 0, st>>>(gpart_, a.G, mtiles, npad, cols, Gout, ldg);
+  launch_pdl(tc_gram_reduce_kernel, blocks, 256, 0, st, gpart_, a.G, mtiles, npad, cols, Gout, ldg);
   note_launch();
   return cudaGetLastError();
 }
