@@ -114,7 +114,7 @@ struct Args {
   int* info;
   int M, N, K, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole, perm;   // sx, sf, sa: stages of X, of A in FP32, A slots
   int chunk;                // units per chain of the main accumulator
-  int stagger;              // 128-row tiles over SMs that the cuts of the chains are staggered by (0: chains from the range's start)
+  int shares;               // SMs whose even shares bound the chains (0: the chunk alone)
   int corr_first;           // chains of one unit, the correction products first
   int flush;                // units whose sums are held in registers before they are added to global memory
   int corr;                 // 0: one accumulator; else main chains per chain of the correction accumulator
@@ -133,21 +133,21 @@ __host__ __device__ inline int unit_owner(int u, int units, int G) {
   return (int)((((long long)u + 1) * G + units - 1) / units) - 1;
 }
 
-// Units of the chain that starts at unit k of tile t, of which `left` are to do.
-// Truncation makes every chain lose a little toward zero; chains that start at
-// the same K in all rows make that a coherent change of A, which moves the
-// subspaces (P of the 20000^2 learned factorisation: 3.8e-5 off with cuts at
-// multiples of 4096 everywhere, 2.7e-5 with cuts that differ from tile to tile).
-// So each tile has a cut of its own, where even shares of 128-row tiles per SM
-// would split it, and the chains before and after it count from 0 and from the
-// cut, wherever the tile is split among CTAs.
+// Units of the chain that starts at unit k of tile t, of which `left` are to do:
+// to the end of an even share of the 128-row tiles per SM, at most `chunk` from
+// its start. Truncation makes every chain lose a little toward zero, so the
+// lengths and places of the chains are what the result's rounding consists of.
+// They follow from the product's shape alone, not from how its tiles are paired
+// and dealt: a pair's range can be twice a share where one of its CTAs has no
+// rows (156512 x 336: L 8e-6 off with chains as long as the ranges, 2e-6 with
+// shares), and chains cut at the same K in all rows add up to a coherent change
+// of A (P of the 20000^2 learned factorisation 3.8e-5 off, else 2.7e-5).
 __device__ inline int chain_units(const Args& a, int t, int k, int left) {
-  if (a.stagger == 0) return min(left, a.chunk);
-  const long long tiles = cdiv(a.M, (int64_t)BM), g = a.stagger, u = 2 * t;
-  const long long c = (u * g + tiles - 1) / tiles;   // first share that starts in tile u
-  const int cut = (int)((2 * (tiles * c - u * g) + tiles - g) * a.kb / (2 * g));
-  if (k < cut) return min(min(left, cut - k), a.chunk - k % a.chunk);
-  return min(left, a.chunk - (k - cut) % a.chunk);
+  if (a.shares == 0) return min(left, a.chunk);
+  const long long units = (long long)cdiv(a.M, (int64_t)BM) * a.kb, u0 = (long long)CG * t * a.kb, u = u0 + k;
+  const long long c = ((u + 1) * a.shares + units - 1) / units - 1;   // the share that holds u
+  const long long b = max(c * units / a.shares, u0), e = (c + 1) * units / a.shares;
+  return (int)min(min((long long)left, e - u), a.chunk - (u - b) % a.chunk);
 }
 
 // Maps over A: one, or one per class of rows.
@@ -704,7 +704,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   // Groups: at most two partial tiles each (none with whole tiles).
   const int cap = a.whole ? a.tiles : std::min(a.units, ws->slots / (2 * CG));
   a.vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0 && ldo % 4 == 0) ? 1 : 0;
-  a.stagger = mode != kSplitFp32 && !a.whole && cdiv(M, BM) > sm_count() ? sm_count() : 0;
+  a.shares = mode != kSplitFp32 ? (int)std::min<int64_t>(sm_count(), cdiv(M, BM) * kb) : 0;
   // Chains. An MMA loses about half a unit in the last place of the sum that
   // it adds to, always toward zero. FP32: one chain per unit, the correction
   // products (2^-8 of the main ones) first, so that only two MMAs add to a
@@ -717,7 +717,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
     a.corr_first = 1;
     a.flush = 64;
   } else {
-    a.chunk = 4096 / BK;
+    a.chunk = (parts == 3 ? 2048 : 4096) / BK;
     a.corr = parts == 3 || npad <= 128 ? 1 : 0;
     a.flush = 1 << 30;
   }
