@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "gram.cuh"
 #include "split_gemm.cuh"
 #include "tc_gemm.cuh"
 
@@ -57,6 +58,7 @@ class Ops {
     const size_t block_bytes =
         std::max(part_bytes, std::min(split_bytes, split_gemm_block_bytes(tall, dcap_, 3)));
     part_ = reinterpret_cast<float*>(ar.take<char>(block_bytes));
+    part_floats_ = block_bytes / sizeof(float);
     scal = ar.take<double>(kScal);
     gates = ar.take<int>(kGates);
     cstore_ = ar.take<char>(chol_global_bytes(dcap_, o_.small_fp64 != 0));
@@ -205,6 +207,7 @@ class Ops {
 
   // G = X^T X, lower triangle (the Cholesky kernel reads G(i, j) for j <= i).
   cudaError_t gram(const float* X, int64_t ldx, int64_t rows, const int* gate) {
+    if (gram_pays(rows, d_, part_floats_)) return gram_f32({X, ldx, rows, G_, ld_, gate, d_}, part_, part_floats_, st_);
     return gemm_f32_ex(true, d_, d_, rows, X, ldx, X, ldx, G_, ld_, gemm_f32_splits(d_, d_, rows), part_,
                        nullptr, gate, kGateSkip, false, st_, /*lower_only=*/true);
   }
@@ -324,6 +327,7 @@ class Ops {
   cudaStream_t st_ = nullptr;
   int* info_ = nullptr;
   float *G_ = nullptr, *R_[3] = {}, *Ri_[3] = {}, *Ra_ = nullptr, *part_ = nullptr;
+  size_t part_floats_ = 0;
   void* cstore_ = nullptr;
   SplitGemmWs sg_;
   TcEngine tcs_;
