@@ -379,17 +379,16 @@ struct Builder {
     }
     chol(js);
   }
-  // out = X R_slot^{-1}; gate_slot >= 0: when that gate is 0, out = X
-  // (kGateCopy) or no work (kGateSkip).
+  // out = X R_slot^{-1}; gate_slot >= 0: no work when that gate is 0.
   template <typename XF, typename OF, typename LF, typename RF>
-  void trmm(XF X, OF out, LF ldout, RF rows, int slot, int shape, int gate_slot, int gate_mode = kGateCopy) {
+  void trmm(XF X, OF out, LF ldout, RF rows, int slot, int shape, int gate_slot) {
     std::vector<GroupGemm> js;
     for (int i = 0; i < n(); ++i) {
       GroupGemm j = job(X(i), bf[i].ld, bf[i].Ri[slot], bf[i].ld, out(i), ldout(i), rows(i), d(i), d(i));
       j.b_upper = 1;
       if (gate_slot >= 0) {
         j.gate = &bf[i].gates[gate_slot];
-        j.gate_mode = gate_mode;
+        j.gate_mode = kGateSkip;
       }
       js.push_back(j);
     }
@@ -432,7 +431,7 @@ struct Builder {
     trmm(X, out, ld, rows, 0, ts, -1);
     gram(out, rows, gs, kInterGate);
     cholesky(1, -1, kInterGate);
-    trmm(out, X, ld, rows, 1, ts, kInterGate, kGateSkip);
+    trmm(out, X, ld, rows, 1, ts, kInterGate);
     copy_gated(X, out, rows, kInterGate);
   }
   // CholeskyQR2 plus a third pass gated on a shifted Cholesky; X is
@@ -446,7 +445,10 @@ struct Builder {
     trmm(X, tmp, ld, rows, 0, ts, -1);
     gram(tmp, rows, gs, -1);
     cholesky(1, g, -1);
-    trmm(tmp, X, ld, rows, 1, ts, -1);
+    trmm(tmp, out, ldout, rows, 1, ts, -1);
+    // The third pass, for the problems that need it, starts over from tmp: the
+    // others' results are in place without another copy.
+    trmm(tmp, X, ld, rows, 1, ts, g);
     gram(X, rows, gs, g);
     cholesky(2, -1, g);
     trmm(X, out, ldout, rows, 2, ts, g);

@@ -110,14 +110,13 @@ void profile_mark_end(cudaStream_t st, int tag);
 // C[M x N] = op(A)[M x K] * B[K x N], op(A) = A^T when transA, row-major.
 // splits > 1 uses `part` (splits * M * N floats) and a fixed-order reduction.
 // sumsq (optional): += sum of squares of the A elements read.
-// gate (optional) with gate_mode 1: *gate == 0 -> C = A (B taken as identity,
-// needs !transA, K == N, one slice); gate_mode 2: *gate == 0 -> no work;
-// gate_mode 3: *gate == 0 -> C = B (A the identity; !transA, M == K, one slice).
+// gate (optional), when *gate == 0: kGateSkip does no work; kGateCopyB gives C = B
+// (A the identity; !transA, M == K, one slice).
 // b_upper: B is upper triangular (k-tiles beyond the column tile are skipped).
 // lower_only (M == N, a Gram matrix whose reader takes its lower triangle):
 // tiles whose entries all lie above the diagonal are skipped and C's strict
 // upper triangle is left undefined.
-enum GateMode { kGateNone = 0, kGateCopy = 1, kGateSkip = 2, kGateCopyB = 3 };
+enum GateMode { kGateNone, kGateSkip, kGateCopyB };
 cudaError_t gemm_f32_ex(bool transA, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
                         const float* B, int64_t ldb, float* C, int64_t ldc, int splits, float* part,
                         double* sumsq, const int* gate, int gate_mode, bool b_upper, cudaStream_t st,

@@ -31,63 +31,9 @@ struct GemmArgs {
   int lower_only;                           // only tiles with entries on or below the diagonal
 };
 
-// Gated off (kGateCopy): C = A on this tile (B taken as the identity), or B
-// (kGateCopyB). All
-// loads of the thread are issued before its stores (C and A are distinct
-// buffers, which the compiler cannot assume), four 128-bit loads at a time.
-template <int BM, int BN, int NT>
-__device__ __forceinline__ void copy_tile(const GemmArgs& g, int64_t m0, int64_t n0, float* C) {
-  const float* S = g.gate_mode == kGateCopyB ? g.B : g.A;
-  const int64_t lds = g.gate_mode == kGateCopyB ? g.ldb : g.lda;
-  constexpr int Q = BN / 4;            // float4 per tile row
-  constexpr int PER = BM * Q / NT;     // float4 per thread
-  constexpr int CH = 4;                // float4 loaded before their stores (bounded registers)
-  static_assert(PER * NT == BM * Q, "copy tiling");
-  const bool vec = ((reinterpret_cast<uintptr_t>(S) | reinterpret_cast<uintptr_t>(C)) % 16 == 0) &&
-                   lds % 4 == 0 && g.ldc % 4 == 0;
-#pragma unroll 1
-  for (int r0 = 0; r0 < PER; r0 += CH) {
-    float4 v[CH];
-#pragma unroll
-    for (int r = 0; r < CH; ++r) {
-      if (r0 + r >= PER) break;
-      const int f = threadIdx.x + (r0 + r) * NT;
-      const int64_t gm = m0 + f / Q, gn = n0 + (f % Q) * 4;
-      const float* src = S + gm * lds + gn;
-      if (gm < g.M && vec && gn + 3 < g.N) {
-        v[r] = *reinterpret_cast<const float4*>(src);
-      } else {
-        float t[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) t[i] = (gm < g.M && gn + i < g.N) ? src[i] : 0.f;
-        v[r] = make_float4(t[0], t[1], t[2], t[3]);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < CH; ++r) {
-      if (r0 + r >= PER) break;
-      const int f = threadIdx.x + (r0 + r) * NT;
-      const int64_t gm = m0 + f / Q, gn = n0 + (f % Q) * 4;
-      if (gm >= g.M) continue;
-      float* dst = C + gm * g.ldc + gn;
-      if (vec && gn + 3 < g.N) {
-        *reinterpret_cast<float4*>(dst) = v[r];
-      } else {
-        const float t[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (gn + i < g.N) dst[i] = t[i];
-      }
-    }
-  }
-}
-
 // One BM x BN tile of C (rows m0.., columns n0..) over K-slice `slice`, by the
 // whole CTA.
-// FAST_COPY: the gated copy by copy_tile (single-matrix kernels); the
-// grouped kernels keep a plain per-element loop, which holds no registers
-// beyond the main loop's (copy_tile raises their spills at 128 registers).
-template <int BM, int BN, int BK, int TM, int TN, bool TRANS_A, bool FAST_COPY = true>
+template <int BM, int BN, int BK, int TM, int TN, bool TRANS_A>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int64_t m0, int64_t n0, int slice) {
   constexpr int NT = (BM / TM) * (BN / TN);
   constexpr int TX = BN / TN;
@@ -108,16 +54,10 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int64_t m0, int64_t
 
   if (g.gate != nullptr && *g.gate == 0) {
     if (g.gate_mode == kGateSkip) return;
-    // Gated off: B is taken as the identity (requires !TRANS_A, K == N, one slice).
-    if (FAST_COPY) {
-      copy_tile<BM, BN, NT>(g, m0, n0, C);
-    } else {
-      const float* S = g.gate_mode == kGateCopyB ? g.B : g.A;
-      const int64_t lds = g.gate_mode == kGateCopyB ? g.ldb : g.lda;
-      for (int idx = tid; idx < BM * BN; idx += NT) {
-        const int64_t gm = m0 + idx / BN, gn = n0 + idx % BN;
-        if (gm < g.M && gn < g.N) C[gm * g.ldc + gn] = S[gm * lds + gn];
-      }
+    // kGateCopyB: A is taken as the identity (requires !TRANS_A, M == K, one slice).
+    for (int idx = tid; idx < BM * BN; idx += NT) {
+      const int64_t gm = m0 + idx / BN, gn = n0 + idx % BN;
+      if (gm < g.M && gn < g.N) C[gm * g.ldc + gn] = g.B[gm * g.ldb + gn];
     }
     return;
   }
@@ -334,7 +274,7 @@ gemm_grouped_kernel(const GroupGemm* __restrict__ jobs, const int* __restrict__ 
     g.b_upper = j.b_upper;
     g.lower_only = j.lower_only;
     __syncthreads();   // the previous tile's shared-memory reads are done
-    gemm_tile<BM, BN, BK, TM, TN, TRANS_A, false>(g, (int64_t)(local / tn) * BM, (int64_t)(local % tn) * BN, 0);
+    gemm_tile<BM, BN, BK, TM, TN, TRANS_A>(g, (int64_t)(local / tn) * BM, (int64_t)(local % tn) * BN, 0);
   }
 }
 
@@ -369,11 +309,7 @@ __global__ void __launch_bounds__(kWideThreads, kWidePerSm) gemm_f32_wide_kernel
   const int slice = blockIdx.z;
   float* C = g.C + (int64_t)slice * g.c_slice;
 
-  if (g.gate != nullptr && *g.gate == 0) {
-    if (g.gate_mode == kGateSkip) return;
-    copy_tile<BM, BN, NT>(g, m0, n0, C);   // B taken as the identity (see gemm_tile)
-    return;
-  }
+  if (g.gate != nullptr && *g.gate == 0) return;   // kGateSkip (kGateCopyB has K <= 256)
 
   const int64_t kbeg = (int64_t)slice * g.kchunk;
   int64_t kend = kbeg + g.kchunk < g.K ? kbeg + g.kchunk : g.K;
@@ -701,9 +637,8 @@ cudaError_t gemm_f32_ex(bool transA, int64_t M, int64_t N, int64_t K, const floa
                         bool lower_only) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (lower_only && (M != N || use_wide(M, N, K))) return cudaErrorInvalidValue;
-  if (gate != nullptr && gate_mode == kGateCopy && (transA || K != N)) return cudaErrorInvalidValue;
-  if (gate != nullptr && gate_mode == kGateCopyB && (transA || M != K)) return cudaErrorInvalidValue;
-  if (gate != nullptr && (gate_mode == kGateCopy || gate_mode == kGateCopyB)) splits = 1;
+  if (gate != nullptr && gate_mode == kGateCopyB && (transA || M != K || use_wide(M, N, K))) return cudaErrorInvalidValue;
+  if (gate != nullptr && gate_mode == kGateCopyB) splits = 1;
   GemmArgs g;
   g.M = M; g.N = N; g.K = K; g.A = A; g.lda = lda; g.B = B; g.ldb = ldb;
   g.sumsq = sumsq; g.gate = gate; g.gate_mode = gate_mode; g.b_upper = b_upper ? 1 : 0;
