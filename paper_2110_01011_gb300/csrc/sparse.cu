@@ -77,33 +77,41 @@ __global__ void csc_count_kernel(const int* __restrict__ idx, int64_t nnz, int64
   }
 }
 
-// col_ptr = exclusive prefix sum of counts (n + 1 entries); one CTA.
-__global__ void __launch_bounds__(1024) csc_scan_kernel(const int* __restrict__ counts, int64_t n,
+// col_ptr = exclusive prefix sum of counts (n + 1 entries), counts back to 0
+// (the scatter's cursor); one CTA, the threads' sums by shuffles.
+__global__ void __launch_bounds__(1024) csc_scan_kernel(int* __restrict__ counts, int64_t n,
                                                         int64_t* __restrict__ col_ptr) {
   grid_wait();
-  __shared__ int64_t part[1024];
-  const int t = threadIdx.x;
+  __shared__ int64_t part[32];
+  const int t = threadIdx.x, lane = t & 31;
   const int64_t chunk = (n + blockDim.x - 1) / blockDim.x;
   const int64_t b = (int64_t)t * chunk, e = std::min<int64_t>(n, b + chunk);
-  int64_t s = 0;
-  for (int64_t i = b; i < e; ++i) s += counts[i];
-  part[t] = s;
+  int64_t own = 0;
+  for (int64_t i = b; i < e; ++i) own += counts[i];
+  int64_t s = own;   // inclusive over the warp, then over the warps
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  if (lane == 31) part[t >> 5] = s;
   __syncthreads();
-  if (t == 0) {
-    int64_t run = 0;
-    for (int i = 0; i < (int)blockDim.x; ++i) {
-      const int64_t v = part[i];
-      part[i] = run;
-      run += v;
+  if (t < 32) {
+    int64_t w = part[t];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t v = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += v;
     }
-    col_ptr[n] = run;
+    part[t] = w;
   }
   __syncthreads();
-  int64_t run = part[t];
+  int64_t run = s - own + (t >= 32 ? part[(t >> 5) - 1] : 0);
   for (int64_t i = b; i < e; ++i) {
+    const int c = counts[i];
     col_ptr[i] = run;
-    run += counts[i];
+    counts[i] = 0;
+    run += c;
   }
+  if (t == (int)blockDim.x - 1) col_ptr[n] = run;
 }
 
 // Scatter every entry (r, j, v) to column j's segment (fill: n zeroed ints).
@@ -127,25 +135,95 @@ csc_fill_kernel(const int64_t* __restrict__ ptr, const int* __restrict__ idx, co
   }
 }
 
-// Each column's entries in increasing row order (insertion sort, a thread
-// per column): the scatter's order depends on the atomics.
-__global__ void csc_sort_kernel(const int64_t* __restrict__ col_ptr, int64_t n, int* __restrict__ ridx,
-                                float* __restrict__ rval) {
-  grid_wait();
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t s = col_ptr[j], e = col_ptr[j + 1];
-    for (int64_t p = s + 1; p < e; ++p) {
-      const int r = ridx[p];
-      const float v = rval[p];
-      int64_t q = p - 1;
-      while (q >= s && ridx[q] > r) {
-        ridx[q + 1] = ridx[q];
-        rval[q + 1] = rval[q];
-        --q;
+// (row, value bits) in order: entries of one place go by value, so that their
+// sum does not depend on the scatter either.
+__device__ __forceinline__ bool after(int ra, float va, int rb, float vb) {
+  return ra > rb || (ra == rb && __float_as_uint(va) > __float_as_uint(vb));
+}
+
+// A column of L entries in place, by the CTA: bitonic merges whose first step
+// mirrors (every exchange puts the larger entry higher, so that any L does).
+template <typename I, typename V>
+__device__ __forceinline__ void sort_column(I ri, V rv, int64_t L) {
+  for (int64_t k = 2; k < 2 * L; k <<= 1) {
+    for (int64_t j = k >> 1; j > 0; j >>= 1) {
+      const bool mirror = j == k >> 1;
+      for (int64_t i = threadIdx.x; i < L; i += blockDim.x) {
+        const int64_t o = mirror ? i ^ (k - 1) : i ^ j;
+        if (o <= i || o >= L) continue;
+        const int a = ri[i], b = ri[o];
+        const float va = rv[i], vb = rv[o];
+        if (after(a, va, b, vb)) {
+          ri[i] = b; rv[i] = vb;
+          ri[o] = a; rv[o] = va;
+        }
       }
-      ridx[q + 1] = r;
-      rval[q + 1] = v;
+      __syncthreads();
     }
+  }
+}
+
+// Each column's entries in increasing row order (the scatter's order depends on
+// the atomics). CTA b takes columns b, b + G, ..: those of up to 32 entries by a
+// warp (every lane counts the entries before its own), longer ones by the CTA, in
+// shared memory up to kSortShared. Serial chains bound it: a thread per column with
+// insertion sort took 38 us at 7320 columns of ~14, and most of a 10 ms call at
+// 55000 x 2000 with columns of ~500.
+constexpr int kSortShared = 2048;
+__global__ void __launch_bounds__(256)
+csc_sort_kernel(const int64_t* __restrict__ col_ptr, int64_t n, int* __restrict__ ridx, float* __restrict__ rval) {
+  grid_wait();
+  __shared__ int sr[kSortShared];
+  __shared__ float sv[kSortShared];
+  __shared__ int cols[2][256];   // slots of short and long columns of this round
+  __shared__ int found[2];
+  const int t = threadIdx.x, lane = t & 31;
+  const int64_t G = gridDim.x, per = G * blockDim.x;
+  for (int64_t base = blockIdx.x; base < n; base += per) {
+    if (t < 2) found[t] = 0;
+    __syncthreads();
+    const int64_t j = base + t * G;
+    if (j < n) {
+      const int64_t L = col_ptr[j + 1] - col_ptr[j];
+      if (L > 1) cols[L > 32][atomicAdd(&found[L > 32], 1)] = t;
+    }
+    __syncthreads();
+    for (int f = t >> 5; f < found[0]; f += blockDim.x / 32) {
+      const int64_t c = base + cols[0][f] * G, s = col_ptr[c];
+      const int L = (int)(col_ptr[c + 1] - s);
+      const int r = lane < L ? ridx[s + lane] : 0;
+      const float v = lane < L ? rval[s + lane] : 0.f;
+      int at = 0;
+      for (int i = 0; i < L; ++i) {
+        const int ro = __shfl_sync(0xffffffffu, r, i);
+        const float vo = __shfl_sync(0xffffffffu, v, i);
+        if (after(r, v, ro, vo) || (i < lane && ro == r && __float_as_uint(vo) == __float_as_uint(v))) ++at;
+      }
+      __syncwarp();
+      if (lane < L) {
+        ridx[s + at] = r;
+        rval[s + at] = v;
+      }
+    }
+    for (int f = 0; f < found[1]; ++f) {
+      const int64_t c = base + cols[1][f] * G, s = col_ptr[c], L = col_ptr[c + 1] - s;
+      if (L <= kSortShared) {
+        for (int64_t i = t; i < L; i += blockDim.x) {
+          sr[i] = ridx[s + i];
+          sv[i] = rval[s + i];
+        }
+        __syncthreads();
+        sort_column(sr, sv, L);
+        for (int64_t i = t; i < L; i += blockDim.x) {
+          ridx[s + i] = sr[i];
+          rval[s + i] = sv[i];
+        }
+        __syncthreads();
+      } else {
+        sort_column(ridx + s, rval + s, L);
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -180,11 +258,10 @@ cudaError_t sparse_build_csc(const SparseA& a, void* ws, SparseA* t, int* info, 
     note_launch();
   }
   launch_pdl(csc_scan_kernel, 1, 1024, 0, st, counts, a.n, col_ptr);
-  CK(cudaMemsetAsync(counts, 0, sizeof(int) * a.n, st));   // reused as the fill cursor
   launch_pdl(csc_fill_kernel, spmm_blocks(a.m), 256, 0, st, a.row_ptr, a.col_idx, a.vals, a.m, a.n, col_ptr, counts,
              ridx, rval);
-  launch_pdl(csc_sort_kernel, (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(a.n, 128), (int64_t)sm_count() * 4)),
-             128, 0, st, col_ptr, a.n, ridx, rval);
+  launch_pdl(csc_sort_kernel, (int)std::max<int64_t>(1, std::min<int64_t>(a.n, (int64_t)sm_count() * 8)), 256, 0, st,
+             col_ptr, a.n, ridx, rval);
   note_launch(3);
   t->m = a.n;
   t->n = a.m;
