@@ -97,7 +97,7 @@ class Ops {
     if (tc_on_ && rows > (int64_t)d_) {
       tcs_.reset();
       CK(tcs_.split(X, rows, d_, ldx, nullptr, st_));
-      return tcs_.pass(false, X, rows, d_, ldx, Ri_[0], ld_, d_, out, ldout, nullptr, info_, st_, true);
+      return tcs_.product(Ri_[0], ld_, d_, out, ldout, info_, st_);
     }
     return trmm(X, ldx, rows, Ri_[0], out, ldout);
   }
@@ -235,7 +235,7 @@ class Ops {
     CK(tcs_.split(X, rows, d_, ldx, nullptr, st_));
     CK(tcs_.gram(G_, ld_, info_, st_));
     CK(chol(slot, gate_out, nullptr, want_r));
-    return tcs_.pass(false, X, rows, d_, ldx, Ri_[slot], ld_, d_, out, ldout, nullptr, info_, st_, true);
+    return tcs_.product(Ri_[slot], ld_, d_, out, ldout, info_, st_);
   }
   // One CholeskyQR pass: out = X R^{-1}, and a second pass when the first
   // Cholesky had to shift (gated on a device flag, so the launch sequence

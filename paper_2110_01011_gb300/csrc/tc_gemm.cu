@@ -1,39 +1,22 @@
-// Tensor-core passes over A in BF16 split precision (tcgen05 / TMEM / TMA).
+// Products of the first CholeskyQR pass in the BF16x3 form (tcgen05 / TMEM / TMA):
+// the Gram X^T X of a tall X and X R^{-1}, X split into BF16 parts in memory once
+// for both.
 //
-// Each pass computes out = op(A) X with op(A) = A^T (Y = A^T X, the sketch
-// and the A^T-half of a power pass) or A (Z = A X, the projection). A and X
-// are split into BF16 high and low parts, A = A_hi + A_lo, X = X_hi + X_lo,
-// and the product is accumulated in FP32 in tensor memory as
-//     A_hi X_hi + A_hi X_lo + A_lo X_hi
-// (the dropped A_lo X_lo term is below 2^-16 relative). When X has no low
-// part (a BF16-exact Omega) the middle product is skipped.
+// The Gram takes two parts, X = X_hi + X_lo, and the products hi hi + hi lo + lo hi
+// (its factor only preconditions). X R^{-1} takes three of each operand and
+// every product above 2^-27, A_hi X_hi + A_hi X_lo + A_lo X_hi + A_lo2 X_hi + A_hi
+// X_lo2 + A_lo X_lo (six): R^{-1} spreads its entries over orders of magnitude, so
+// the two-part form's error, relative to |X| |R^{-1}|, would be kappa(X) times
+// larger relative to the result.
 //
-// Exact mode (the products X R^{-1} of CholeskyQR, K = d): A and X in three
-// parts each, A = A_hi + A_lo + A_lo2 (error 2^-27), and every product above
-// 2^-27, A_hi X_hi + A_hi X_lo + A_lo X_hi + A_lo2 X_hi + A_hi X_lo2 +
-// A_lo X_lo (six). R^{-1} spreads its entries over orders of magnitude, so
-// the two-part form's error, relative to |X| |R^{-1}|, would be kappa(X)
-// times larger relative to the result.
-//
-// Data flow per factorisation: split_a_kernel writes A_hi, A_lo once (and
-// ||A||_F^2) in 64-column panels: panel c / 64 holds rows 0..m-1 of those
-// 64 columns, 128 bytes per row, so that each part of an A tile is one TMA
-// box (A^T X: 32 rows of two panels; A X: 128 rows of one panel);
-// prep_x_kernel writes X_hi^T, X_lo^T (d x K, K-major) before
-// every pass; tc_pass_kernel streams A tiles through shared memory with TMA
-// and issues tcgen05.mma from one thread. A tile whose K range is split over
-// several CTAs (stream-K) is finished by the CTA that arrives last on the
-// tile's counter: it adds the published partial tiles in CTA order
-// (deterministic) and resets the counter; no CTA ever waits for another.
-//
-// tc_pass_kernel is persistent: one CTA per SM, the (tile, k-block) units of
-// the whole pass split evenly over the CTAs (stream-K), so the 157 M-tiles of
-// a 20000-row pass load all 152 SMs equally. Warp roles: warps 0-3 drain the
-// accumulator from TMEM (each warp its 32 lanes), warp 4 issues TMA loads,
-// warp 5 allocates TMEM and issues the MMAs. Two accumulator buffers let the
-// next segment's MMAs run while the epilogue drains the previous one. Every
-// wait is bounded; a timeout is reported in the status word and the kernel
-// drains what it started and frees its TMEM before returning.
+// split_a_kernel writes the parts in 64-column panels: panel c / 64 holds rows 0
+// .. m - 1 of those 64 columns, 128 bytes per row, so that 128 rows of one panel are
+// one TMA box; prep_x_kernel writes the other operand's parts transposed
+// (d x K, K-major). tc_pass_kernel is persistent, a CTA taking whole 128-row
+// tiles: warps 0-3 drain the accumulator from TMEM (each warp its 32 lanes),
+// warp 4 issues TMA loads, warp 5 allocates TMEM and issues the MMAs. Every wait
+// is bounded; a timeout is reported in the status word and the kernel drains what
+// it started and frees its TMEM before returning.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -58,7 +41,6 @@ constexpr long long kWaitLimit = 4000000000LL;   // cycles (~2 s) before a wait 
 // swizzle). Larger TMA boxes stream A faster (measured: 7.1 vs 5.2 TB/s of
 // A_hi + A_lo in the A^T X order at d = 64), but the pipeline needs stages in
 // flight: at d = 224 only two K = 64 stages fit, and K = 32 with five is as fast.
-constexpr int kMaxSlots = 16;                    // partial tiles summed from a cached slot list
 // The FP32 accumulation of tcgen05.mma in TMEM loses a little of every add in
 // the same direction: over K = 20000 a pass shrinks by ~1.5e-6 relative to
 // its partial sums, which the cancelling small-singular-value columns of
@@ -72,15 +54,10 @@ constexpr int kChunkK = 4096;
 
 struct TcArgs {
   int M, K, d, npad, kblocks, tiles, G, stages;
-  int k0;                    // A^T X over A's rows k0 .. k0 + K - 1 (X holds those rows); 0 otherwise
-  int m0;                    // A X over A's rows m0 .. m0 + M - 1 (out row 0 = A's row m0); 0 otherwise
-  int tpc;                   // > 0: whole tiles per CTA (no split tiles); 0: stream-K
+  int tpc;                   // whole tiles per CTA
   int vec_out;               // out rows are 16-byte aligned (float4 stores)
-  long long units;
   float* out;
   long long ldo;
-  float* part;               // 2 * G slots of BM x npad floats
-  int* tile_cnt;             // per-tile arrival counters (zero between passes)
   const int* xlo_nonzero;    // 1 when X has a nonzero low part
   int exact;                 // 1: A and X in three parts, six products
   int chunk;                 // k-blocks per accumulation chain in TMEM
@@ -89,22 +66,11 @@ struct TcArgs {
   int bufcols;               // TMEM columns of one buffer (npad, or 2 npad when split_acc)
   int* info;                 // status word (may be null)
   uint32_t idesc, stage_bytes, tmem_cols;
-  int fixup;                 // 1: split tiles are summed by tc_fixup_kernel after the pass
 };
 
-__host__ __device__ inline long long unit_begin(int c, long long units, int G) {
-  return (long long)c * units / G;
-}
-// First unit of CTA c: stream-K (even split of all units) or, with tpc > 0,
-// whole tiles (tpc tiles of kblocks units each per CTA).
-__device__ inline long long cta_begin(const int c, const long long units, const int G, const int tpc,
-                                      const int tiles, const int kblocks) {
-  if (tpc > 0) return (long long)min(c * tpc, tiles) * kblocks;
-  return unit_begin(c, units, G);
-}
-// The CTA whose unit range holds unit u (empty ranges never match).
-__host__ __device__ inline int unit_owner(long long u, long long units, int G) {
-  return (int)(((u + 1) * G + units - 1) / units) - 1;
+// First unit of CTA c: tpc whole tiles of kblocks units each.
+__device__ inline long long cta_begin(int c, int tpc, int tiles, int kblocks) {
+  return (long long)min(c * tpc, tiles) * kblocks;
 }
 
 // End of the accumulation chunk that starts at unit u (a CTA's range [.., u1)).
@@ -117,7 +83,7 @@ __device__ void post_timeout(int* info) {
   if (info != nullptr && atomicCAS(info, 0, RQLP_ERR_TIMEOUT) == 0) info[1] = 0;
 }
 
-template <bool MN_A, int BKP>
+template <int BKP>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmAlo,
                const __grid_constant__ CUtensorMap tmXhi, const __grid_constant__ CUtensorMap tmXlo,
@@ -134,16 +100,12 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
   uint64_t* acce = accf + 2;
   uint64_t* done = acce + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
-  int* last_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  int* last_lo = last_flag + 1;
-  int* epi_ok = last_lo + 2;
-  int* nslots = epi_ok + 1;
-  int* slots = nslots + 1;   // kMaxSlots entries
+  int* epi_ok = reinterpret_cast<int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cta = blockIdx.x;
-  const long long u0 = cta_begin(cta, a.units, a.G, a.tpc, a.tiles, a.kblocks);
-  const long long u1 = cta_begin(cta + 1, a.units, a.G, a.tpc, a.tiles, a.kblocks);
+  const long long u0 = cta_begin(cta, a.tpc, a.tiles, a.kblocks);
+  const long long u1 = cta_begin(cta + 1, a.tpc, a.tiles, a.kblocks);
   if (u0 >= u1) return;   // no work for this CTA (uniform)
   const int KB = a.kblocks;
 
@@ -198,17 +160,11 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
       unsigned char* base = smem + (size_t)stage * a.stage_bytes;
       tc::mbar_expect_tx(&full[stage], xoff + (uint32_t)nx * xbytes);
       // A maps are 3-D over the panel layout: {column in panel, row, panel}.
-      if (MN_A) {   // 64 rows (K) of panels 2t and 2t + 1 (M), one box
-        const int kr = a.k0 + kb * BKP;
-        tc::tma_load_3d(base, &tmAhi, &full[stage], 0, kr, 2 * t);
-        tc::tma_load_3d(base + kAP, &tmAlo, &full[stage], 0, kr, 2 * t);
-        if (ex) tc::tma_load_3d(base + 2 * kAP, &tmAlo2, &full[stage], 0, kr, 2 * t);
-      } else {      // 128 rows (M) x BKP columns (K) of panel kb BKP / 64
-        const int kx = (kb * BKP) & 63, kp = (kb * BKP) >> 6, mr = a.m0 + t * BM;
-        tc::tma_load_3d(base, &tmAhi, &full[stage], kx, mr, kp);
-        tc::tma_load_3d(base + kAP, &tmAlo, &full[stage], kx, mr, kp);
-        if (ex) tc::tma_load_3d(base + 2 * kAP, &tmAlo2, &full[stage], kx, mr, kp);
-      }
+      // 128 rows (M) x BKP columns (K) of panel kb BKP / 64
+      const int kx = (kb * BKP) & 63, kp = (kb * BKP) >> 6, mr = t * BM;
+      tc::tma_load_3d(base, &tmAhi, &full[stage], kx, mr, kp);
+      tc::tma_load_3d(base + kAP, &tmAlo, &full[stage], kx, mr, kp);
+      if (ex) tc::tma_load_3d(base + 2 * kAP, &tmAlo2, &full[stage], kx, mr, kp);
       tc::tma_load_2d(base + xoff, &tmXhi, &full[stage], kb * BKP, 0);
       if (nx >= 2) tc::tma_load_2d(base + xoff + xbytes, &tmXlo, &full[stage], kb * BKP, 0);
       if (nx == 3) tc::tma_load_2d(base + xoff + 2 * xbytes, &tmXlo2, &full[stage], kb * BKP, 0);
@@ -244,15 +200,10 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
 #pragma unroll
         for (int ks = 0; ks < BKP / 16; ++ks) {
           uint64_t dah, dal, dal2;
-          if (MN_A) {   // MN-major, 128B swizzle: 16 k-rows = two 1024-byte atoms; panels kAP / 2 apart
-            dah = tc::smem_desc(ahi + ks * 2048, kAP / 2, 1024, tc::kSwizzle128);
-            dal = tc::smem_desc(alo + ks * 2048, kAP / 2, 1024, tc::kSwizzle128);
-            dal2 = tc::smem_desc(alo2 + ks * 2048, kAP / 2, 1024, tc::kSwizzle128);
-          } else {      // K-major: 16 k-columns = 32 bytes into the row
-            dah = tc::smem_desc(ahi + ks * 32, 16, kSbo, kSw);
-            dal = tc::smem_desc(alo + ks * 32, 16, kSbo, kSw);
-            dal2 = tc::smem_desc(alo2 + ks * 32, 16, kSbo, kSw);
-          }
+          // K-major: 16 k-columns = 32 bytes into the row
+          dah = tc::smem_desc(ahi + ks * 32, 16, kSbo, kSw);
+          dal = tc::smem_desc(alo + ks * 32, 16, kSbo, kSw);
+          dal2 = tc::smem_desc(alo2 + ks * 32, 16, kSbo, kSw);
           const uint64_t dxh = tc::smem_desc(xhi + ks * 32, 16, kSbo, kSw);
           const uint64_t dxl = tc::smem_desc(xlo + ks * 32, 16, kSbo, kSw);
           const uint64_t dxl2 = tc::smem_desc(xlo2 + ks * 32, 16, kSbo, kSw);
@@ -289,10 +240,8 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
     while (u < u1) {
       const int t = (int)(u / KB);
       const long long seg_begin = u, seg_end = chunk_end(u, u1, KB, kChunk);
-      // This CTA's part of tile t, and where the chunk sits in it.
-      const long long tb = std::max(u0, (long long)t * KB), te = std::min(u1, (long long)(t + 1) * KB);
-      const bool whole = tb == (long long)t * KB && te == (long long)(t + 1) * KB;
-      const bool first_chunk = seg_begin == tb, last_chunk = seg_end == te;
+      const long long tb = (long long)t * KB;
+      const bool first_chunk = seg_begin == tb;
       const int ab = seg % a.nbuf;
       // One thread waits; the verdict is shared so the four warps stay in step.
       if (threadIdx.x == 0) *epi_ok = tc::mbar_wait(&accf[ab], (uint32_t)((seg / a.nbuf) & 1), kWaitLimit) ? 1 : 0;
@@ -306,15 +255,9 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
       const long long gm = (long long)t * BM + row;
       float* dst;
       int ncols;
-      if (whole) {
-        dst = a.out + gm * a.ldo;
-        ncols = gm < a.M ? a.d : 0;
-      } else {
-        const int slot = (tb == u0) ? 2 * cta : 2 * cta + 1;   // first or last tile of the range
-        dst = a.part + ((long long)slot * BM + row) * a.npad;
-        ncols = a.npad;
-      }
-      const bool vec = whole ? (a.vec_out != 0) : true;   // partial slots are 64-byte aligned
+      dst = a.out + gm * a.ldo;
+      ncols = gm < a.M ? a.d : 0;
+      const bool vec = a.vec_out != 0;
       // 32 columns per step: the row's earlier sums (this thread wrote them)
       // are all loaded before the step's stores, so the loads of a step
       // overlap instead of queueing behind stores to the same array.
@@ -372,101 +315,6 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
       }
       tc::tc_fence_before();
       tc::mbar_arrive(&acce[ab]);
-      if (!whole && last_chunk && !a.fixup) {
-        // Publish the partial tile; the last CTA to arrive on the tile sums them.
-        __threadfence();
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (threadIdx.x == 0) {
-          // Slots of this tile's contributors in CTA order (the fixed summation order).
-          const long long ub = (long long)t * KB, ue = ub + KB;
-          const int clo = unit_owner(ub, a.units, a.G), chi = unit_owner(ue - 1, a.units, a.G);
-          int n = 0;
-          for (int c = clo; c <= chi; ++c) {
-            const long long cb = unit_begin(c, a.units, a.G);
-            if (cb == unit_begin(c + 1, a.units, a.G)) continue;
-            if (n < kMaxSlots) slots[n] = (cb / KB == t) ? 2 * c : 2 * c + 1;
-            ++n;
-          }
-          const int old = atomicAdd(&a.tile_cnt[t], 1);
-          *last_flag = (old == n - 1) ? 1 : 0;
-          *nslots = n;
-          last_lo[0] = clo;
-          last_lo[1] = chi;
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        if (*last_flag && *nslots <= kMaxSlots) {
-          // Sum the slots in CTA order, the four warps over consecutive
-          // float4 of the tile (coalesced), eight float4 per thread in flight.
-          __threadfence();
-          const int n = *nslots;
-          const int Q = a.npad / 4, total = BM * Q;
-          for (int f0 = threadIdx.x; f0 < total; f0 += 128 * 8) {
-            float4 acc[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int s2 = 0; s2 < n; ++s2) {
-              const float4* src = reinterpret_cast<const float4*>(a.part + (long long)slots[s2] * BM * a.npad);
-              float4 v[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const int f = f0 + 128 * j;
-                v[j] = f < total ? __ldcg(src + f) : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                acc[j].x += v[j].x; acc[j].y += v[j].y; acc[j].z += v[j].z; acc[j].w += v[j].w;
-              }
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const int f = f0 + 128 * j;
-              if (f >= total) continue;
-              const int r = f / Q, c = (f % Q) * 4;
-              const long long gr = (long long)t * BM + r;
-              if (gr >= a.M || c >= a.d) continue;
-              float* o = a.out + gr * a.ldo + c;
-              if (a.vec_out && c + 3 < a.d) {
-                *reinterpret_cast<float4*>(o) = acc[j];
-              } else {
-                const float w[4] = {acc[j].x, acc[j].y, acc[j].z, acc[j].w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                  if (c + i < a.d) o[i] = w[i];
-              }
-            }
-          }
-          if (threadIdx.x == 0) a.tile_cnt[t] = 0;
-        } else if (*last_flag) {
-          __threadfence();
-          if (gm < a.M) {
-            float* o = a.out + gm * a.ldo;
-            for (int c0 = 0; c0 < a.d; c0 += 16) {
-              float acc[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-              {   // many contributors (tiny problems): recompute the slots
-                for (int c = last_lo[0]; c <= last_lo[1]; ++c) {
-                  const long long cb = unit_begin(c, a.units, a.G);
-                  if (cb == unit_begin(c + 1, a.units, a.G)) continue;
-                  const int slot = (cb / KB == t) ? 2 * c : 2 * c + 1;
-                  const float4* src =
-                      reinterpret_cast<const float4*>(a.part + ((long long)slot * BM + row) * a.npad + c0);
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const float4 v = __ldcg(src + q);
-                    acc[4 * q] += v.x; acc[4 * q + 1] += v.y; acc[4 * q + 2] += v.z; acc[4 * q + 3] += v.w;
-                  }
-                }
-              }
-#pragma unroll
-              for (int i = 0; i < 16; ++i)
-                if (c0 + i < a.d) o[c0 + i] = acc[i];
-            }
-          }
-          if (threadIdx.x == 0) a.tile_cnt[t] = 0;
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-      }
       u = seg_end;
       ++seg;
     }
@@ -476,45 +324,6 @@ tc_pass_kernel(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant_
   __syncthreads();
   tc::tc_fence_after();
   if (warp == 5) tc::tmem_dealloc(tmem_base, a.tmem_cols);
-}
-
-// Sums of the split tiles when a tile has more contributors than the last
-// arriver's slot list holds (few output tiles, e.g. A^T X with n <= ~1300):
-// every split tile's partials are summed here by all SMs, one float4 of the
-// output per thread, over the tile's contributors in CTA order (the order
-// and the values of the last-arriver reduction).
-__global__ void tc_fixup_kernel(const TcArgs a) {
-  grid_wait();
-  const int Q = a.npad / 4, KB = a.kblocks;
-  const long long total = (long long)a.tiles * BM * Q;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(idx / ((long long)BM * Q));
-    const int rem = (int)(idx % ((long long)BM * Q));
-    const int r = rem / Q, c = (rem % Q) * 4;
-    const long long gr = (long long)t * BM + r;
-    if (gr >= a.M || c >= a.d) continue;
-    const long long ub = (long long)t * KB, ue = ub + KB;
-    const int clo = unit_owner(ub, a.units, a.G), chi = unit_owner(ue - 1, a.units, a.G);
-    if (clo == chi) continue;   // one contributor: the tile was written whole
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int cc = clo; cc <= chi; ++cc) {
-      const long long cb = unit_begin(cc, a.units, a.G);
-      if (cb == unit_begin(cc + 1, a.units, a.G)) continue;
-      const int slot = (cb / KB == t) ? 2 * cc : 2 * cc + 1;
-      const float4 v = __ldcg(reinterpret_cast<const float4*>(a.part + ((long long)slot * BM + r) * a.npad + c));
-      acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
-    }
-    float* o = a.out + gr * a.ldo + c;
-    if (a.vec_out && c + 3 < a.d) {
-      *reinterpret_cast<float4*>(o) = acc;
-    } else {
-      const float w[4] = {acc.x, acc.y, acc.z, acc.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (c + i < a.d) o[i] = w[i];
-    }
-  }
 }
 
 // Gram matrix of a split tall matrix on the tensor cores: G = X^T X for
@@ -549,7 +358,7 @@ tc_gram_kernel(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cta = blockIdx.x;
-  const long long kb0 = unit_begin(cta, a.kblocks, a.G), kb1 = unit_begin(cta + 1, a.kblocks, a.G);
+  const long long kb0 = (long long)cta * a.kblocks / a.G, kb1 = (long long)(cta + 1) * a.kblocks / a.G;
   const uint32_t half = (uint32_t)a.nbox * 4096u;   // bytes of one (hi or lo) chunk
 
   if (threadIdx.x == 0) {
@@ -859,19 +668,19 @@ int stages_of(int npad, bool exact, int bkp) {
 }
 int pass_bk(int npad, bool exact) { return stages_of(npad, exact, 64) >= 3 ? 64 : 32; }
 
-template <bool MN_A, int BKP>
+template <int BKP>
 cudaError_t launch_pass(const CUtensorMap& ah, const CUtensorMap& al, const CUtensorMap& xh,
                         const CUtensorMap& xl, const CUtensorMap& al2, const CUtensorMap& xl2, const TcArgs& a,
                         cudaStream_t st) {
   const size_t smem = (size_t)a.stages * a.stage_bytes + 1024 + 512;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tc_pass_kernel<MN_A, BKP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(tc_pass_kernel<BKP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(smem_optin_tc()));
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  launch_pdl(tc_pass_kernel<MN_A, BKP>, a.G, kThreads, smem, st, ah, al, xh, xl, al2, xl2, a);
+  launch_pdl(tc_pass_kernel<BKP>, a.G, kThreads, smem, st, ah, al, xh, xl, al2, xl2, a);
   note_launch();
   return cudaGetLastError();
 }
@@ -905,9 +714,9 @@ void TcEngine::layout(Arena& ar, int64_t rows_cap, int64_t cols_cap, int d_cap, 
   Xhi_ = ar.take<uint16_t>((size_t)d_cap * round_up(k_cap, 8));
   Xlo_ = ar.take<uint16_t>((size_t)d_cap * round_up(k_cap, 8));
   Xlo2_ = three_part ? ar.take<uint16_t>((size_t)d_cap * round_up(k_cap, 8)) : nullptr;
-  part_ = ar.take<float>((size_t)2 * G_ * BM * npad);
+  ar.take<float>((size_t)2 * G_ * BM * npad);   // (partial tiles and their counters once: the reported size stays)
   flag_ = ar.take<int>(4);
-  cnt_ = ar.take<int>((size_t)cdiv(std::max(rows_cap, cols_cap), BM));
+  ar.take<int>((size_t)cdiv(std::max(rows_cap, cols_cap), BM));
   if (gram) {
     const int gp = npad_of((int)cols_cap);
     gpart_ = ar.take<float>((size_t)kGramMaxCtas * cdiv(cols_cap, BM) * BM * gp);
@@ -929,146 +738,68 @@ cudaError_t TcEngine::split(const float* A, int64_t rows, int64_t cols, int64_t 
   split_of_ = A;
   m_ = rows;
   n_ = cols;
-  // Tile counters start at zero; each pass's last arrivals reset them.
-  return cudaMemsetAsync(cnt_, 0, sizeof(int) * cdiv(std::max(rows_cap_, cols_cap_), BM), st);
+  return cudaSuccess;
 }
 
-cudaError_t TcEngine::begin_split(const float* A, int64_t rows, int64_t cols, cudaStream_t st) {
-  if (rows > rows_cap_ || cols > cols_cap_) return cudaErrorInvalidValue;
-  split_of_ = A;
-  m_ = rows;
-  n_ = cols;
-  return cudaMemsetAsync(cnt_, 0, sizeof(int) * cdiv(std::max(rows_cap_, cols_cap_), BM), st);
-}
-
-cudaError_t TcEngine::split_rows(const float* Ablock, int64_t row0, int64_t rows, int64_t lda, double* sumsq,
-                                 cudaStream_t st) {
-  if (split_of_ == nullptr || row0 < 0 || row0 + rows > m_) return cudaErrorInvalidValue;
-  const bool vec = (reinterpret_cast<uintptr_t>(Ablock) % 16 == 0) && (lda % 4 == 0);
-  const long long npan = cdiv(n_, 64);
-  const long long total = rows * npan * 8;
-  const int blocks = (int)std::max<long long>(1, std::min<long long>(cdiv(total, 256), (long long)G_ * 8));
-  launch_pdl(split_a_kernel, blocks, 256, 0, st, Ablock, rows, n_, lda, vec, reinterpret_cast<bf16*>(Ahi_),
-             reinterpret_cast<bf16*>(Alo_), reinterpret_cast<bf16*>(Alo2_), npan, sumsq, m_, row0);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t TcEngine::pass(bool transA, const float* A, int64_t m, int64_t n, int64_t lda, const float* X,
-                           int64_t ldx, int d, float* out, int64_t ldout, double* sumsq, int* info,
-                           cudaStream_t st, bool exact) {
-  if (split_of_ != A || m != m_ || n != n_) {
-    cudaError_t e = split(A, m, n, lda, sumsq, st);
-    if (e != cudaSuccess) return e;
-  } else if (sumsq != nullptr) {
-    return cudaErrorInvalidValue;   // ||A||^2 comes with the split only
-  }
-  return pass_k(transA, 0, transA ? m : n, X, ldx, d, out, ldout, info, st, exact);
-}
-
-cudaError_t TcEngine::pass_k(bool transA, int64_t k0, int64_t K, const float* X, int64_t ldx, int d, float* out,
-                             int64_t ldout, int* info, cudaStream_t st, bool exact, int64_t m0, int64_t Mrows) {
-  if (d > d_cap_ || split_of_ == nullptr) return cudaErrorInvalidValue;
-  if (exact && (Alo2_ == nullptr || Xlo2_ == nullptr)) return cudaErrorInvalidValue;
-  if (k0 < 0 || (!transA && k0 != 0) || k0 + K > (transA ? m_ : n_) || K <= 0) return cudaErrorInvalidValue;
-  if (m0 < 0 || (transA && (m0 != 0 || Mrows >= 0)) || (!transA && Mrows >= 0 && m0 + Mrows > m_))
-    return cudaErrorInvalidValue;
+cudaError_t TcEngine::product(const float* X, int64_t ldx, int d, float* out, int64_t ldout, int* info,
+                              cudaStream_t st) {
+  const int64_t m = m_, n = n_, K = n_;
+  if (d > d_cap_ || split_of_ == nullptr || Alo2_ == nullptr || K <= 0 || K > k_cap_) return cudaErrorInvalidValue;
   cudaError_t e;
-  const int64_t m = m_, n = n_;
   const int npad_ = npad_of(d);
-  const long long M = transA ? n : (Mrows >= 0 ? Mrows : m);
-  if (K > k_cap_) return cudaErrorInvalidValue;
   if ((e = cudaMemsetAsync(flag_, 0, sizeof(int), st)) != cudaSuccess) return e;
   {
     dim3 grid((unsigned)cdiv(round_up(K, 8), kPrepRows), (unsigned)cdiv(d, 32));
     launch_pdl(prep_x_kernel, grid, dim3(32, 8), 0, st, X, K, d, ldx, reinterpret_cast<bf16*>(Xhi_),
-               reinterpret_cast<bf16*>(Xlo_), exact ? reinterpret_cast<bf16*>(Xlo2_) : nullptr, round_up(K, 8),
-               flag_);
+               reinterpret_cast<bf16*>(Xlo_), reinterpret_cast<bf16*>(Xlo2_), round_up(K, 8), flag_);
     note_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   CUtensorMap ah, al, xh, xl, al2, xl2;
   const long long ldk = round_up(K, 8);
   bool ok;
-  // The third parts are read in exact mode only; otherwise their maps repeat
-  // the low parts'.
-  const uint16_t* A3 = exact ? Alo2_ : Alo_;
-  const uint16_t* X3 = exact ? Xlo2_ : Xlo_;
   const long long npan = cdiv(n, 64);
-  const int bkp = pass_bk(npad_, exact);
+  const int bkp = pass_bk(npad_, true);
   const CUtensorMapSwizzle ksw = bkp == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
-  if (transA) {   // op(A) = A^T: MN-major tiles, box 64 (j) x 32 (i) x 2 panels, 128B swizzle
-    ok = make_panel_map(&ah, Ahi_, m, npan, 64, bkp, 2, CU_TENSOR_MAP_SWIZZLE_128B) &&
-         make_panel_map(&al, Alo_, m, npan, 64, bkp, 2, CU_TENSOR_MAP_SWIZZLE_128B) &&
-         make_panel_map(&al2, A3, m, npan, 64, bkp, 2, CU_TENSOR_MAP_SWIZZLE_128B);
-  } else {        // op(A) = A: K-major tiles, box bkp (j) x 128 (i), swizzle = the row
-    ok = make_panel_map(&ah, Ahi_, m, npan, bkp, BM, 1, ksw) &&
-         make_panel_map(&al, Alo_, m, npan, bkp, BM, 1, ksw) &&
-         make_panel_map(&al2, A3, m, npan, bkp, BM, 1, ksw);
-  }
+  // K-major tiles, box bkp (j) x 128 (i), swizzle = the row
+  ok = make_panel_map(&ah, Ahi_, m, npan, bkp, BM, 1, ksw) && make_panel_map(&al, Alo_, m, npan, bkp, BM, 1, ksw) &&
+       make_panel_map(&al2, Alo2_, m, npan, bkp, BM, 1, ksw);
   ok = ok && make_map(&xh, Xhi_, K, d, ldk, bkp, npad_, ksw) &&
        make_map(&xl, Xlo_, K, d, ldk, bkp, npad_, ksw) &&
-       make_map(&xl2, X3, K, d, ldk, bkp, npad_, ksw);
+       make_map(&xl2, Xlo2_, K, d, ldk, bkp, npad_, ksw);
   if (!ok) return cudaErrorInvalidValue;
 
   TcArgs a;
-  a.M = (int)M;
+  a.M = (int)m;
   a.K = (int)K;
-  a.k0 = (int)k0;
-  a.m0 = (int)m0;
   a.d = d;
   a.npad = npad_;
   a.kblocks = (int)cdiv(K, bkp);
-  a.tiles = (int)cdiv(M, BM);
-  a.units = (long long)a.tiles * a.kblocks;
-  a.G = (int)std::min<long long>(G_, a.units);
-  // Short K (e.g. X R^{-1} with K = d): split tiles would cost more in the
-  // epilogue than they save, so give each CTA whole tiles.
-  a.tpc = 0;
-  if (a.kblocks <= 1024 / bkp) {
-    a.tpc = (int)cdiv(a.tiles, G_);
-    a.G = (int)cdiv(a.tiles, a.tpc);
-  }
-  // A tile spans at most G / tiles + 2 CTAs; past the last arriver's slot
-  // list the split tiles are summed by tc_fixup_kernel instead.
-  a.fixup = (a.tpc == 0 && (long long)a.G / a.tiles + 2 > kMaxSlots) ? 1 : 0;
+  a.tiles = (int)cdiv(m, BM);
+  // K = d: split tiles would cost more in the epilogue than they save, so
+  // each CTA takes whole tiles.
+  a.tpc = (int)cdiv(a.tiles, G_);
+  a.G = (int)cdiv(a.tiles, a.tpc);
   a.vec_out = ((reinterpret_cast<uintptr_t>(out) % 16) == 0 && ldout % 4 == 0) ? 1 : 0;
-  a.exact = exact ? 1 : 0;
+  a.exact = 1;
   a.chunk = kChunkK / bkp;
   // Correction products get their own accumulator where two such buffer
   // pairs fit in TMEM's 512 columns (npad <= 128), and always in exact mode
   // (single-buffered above npad = 128: the epilogue then holds the MMAs for
   // the drain of each chain).
-  a.split_acc = (exact || 4 * npad_ <= 512) ? 1 : 0;
+  a.split_acc = 1;
   a.bufcols = (a.split_acc ? 2 : 1) * npad_;
   a.nbuf = 2 * a.bufcols <= 512 ? 2 : 1;
-  a.stages = stages_of(npad_, exact, bkp);
+  a.stages = stages_of(npad_, true, bkp);
   a.out = out;
   a.ldo = ldout;
-  a.part = part_;
-  a.tile_cnt = cnt_;
   a.xlo_nonzero = flag_;
   a.info = info;
-  a.idesc = tc::idesc_bf16(BM, npad_, transA, false);
-  a.stage_bytes = stage_bytes_of(npad_, exact, bkp);
+  a.idesc = tc::idesc_bf16(BM, npad_, false, false);
+  a.stage_bytes = stage_bytes_of(npad_, true, bkp);
   a.tmem_cols = tmem_cols_of(a.nbuf * a.bufcols);
-  const bool prof = profiled_ && profiling_on();
-  if (prof) profile_mark_begin(st);
-  if (bkp == 64)
-    e = transA ? launch_pass<true, 64>(ah, al, xh, xl, al2, xl2, a, st)
-               : launch_pass<false, 64>(ah, al, xh, xl, al2, xl2, a, st);
-  else
-    e = transA ? launch_pass<true, 32>(ah, al, xh, xl, al2, xl2, a, st)
-               : launch_pass<false, 32>(ah, al, xh, xl, al2, xl2, a, st);
-  if (e == cudaSuccess && a.fixup) {
-    const long long total = (long long)a.tiles * BM * (npad_ / 4);
-    const int blocks = (int)std::min<long long>(cdiv(total, 256), (long long)G_ * 8);
-    launch_pdl(tc_fixup_kernel, blocks, 256, 0, st, a);
-    note_launch();
-    e = cudaGetLastError();
-  }
-  if (prof) profile_mark_end(st, transA ? 1 : 0);
-  return e;
+  return bkp == 64 ? launch_pass<64>(ah, al, xh, xl, al2, xl2, a, st)
+                   : launch_pass<32>(ah, al, xh, xl, al2, xl2, a, st);
 }
 
 cudaError_t TcEngine::gram(float* Gout, int64_t ldg, int* info, cudaStream_t st) {
