@@ -247,9 +247,8 @@ def run_reference(a):
 # ------------------------------------------------------------------ our arm
 
 def kernel_sha(prec):
-    """Hash of the source file that holds the dominant kernel of this precision."""
-    f = "gemm_simt.cu" if prec == 0 else "tc_gemm.cu"   # 0: FP32 form
-    p = os.path.join(ROOT, "paper_2110_01011_gb300", "csrc", f)
+    """Hash of the source file that holds the dominant kernel (of both precisions)."""
+    p = os.path.join(ROOT, "paper_2110_01011_gb300", "csrc", "split_gemm.cu")
     return hashlib.sha256(open(p, "rb").read()).hexdigest()[:12]
 
 
@@ -342,11 +341,10 @@ def learned_runner(a, A, Om, params, target, prec, dev):
 
 
 def pass_products(prec, three_part, x_has_low=True):
-    """BF16 MMA products per element pair of a split-form pass: six with three
-    parts; with two, three (two when X is BF16-exact, e.g. a rounded Omega)."""
-    if prec == 0:
-        return 1
-    if three_part:
+    """BF16 MMA products per element pair of a pass: six with three parts (FP32
+    on the tensor cores among them); with two, three (two when X is BF16-exact,
+    e.g. a rounded Omega)."""
+    if prec == 0 or three_part:
         return 6
     return 3 if x_has_low else 2
 
@@ -378,7 +376,9 @@ def roofline(a, recs, d, prec, peaks, dev, three_part, q, ms_step):
     hbm = peaks.get("hbm_gbs", 6761.6)
     burst = peaks.get("bf16_tflops", 1889.1)
     sust = peaks.get("bf16_tflops_sustained", 1683.0)
-    if prec == rqlp.PREC_FP32:
+    # FP32 passes of fewer multiply-adds run on the FMA units.
+    on_alu = prec == rqlp.PREC_FP32 and a.m * a.n * d < 2e8
+    if on_alu:
         peak = nsm * FP32_LANES_PER_SM * 2 * sm_max * 1e6 / 1e12
         roof = {"bound": "alu", "achieved": flops / (pass_ms * 1e-3) / 1e12, "peak": peak, "unit": "TFLOP/s",
                 "peak_source": f"derived: {nsm} SMs x 128 FP32 lanes x 2 x {sm_max:.0f} MHz",
@@ -395,13 +395,13 @@ def roofline(a, recs, d, prec, peaks, dev, three_part, q, ms_step):
     roof["kernel"] = kname
     roof["launch_ms"] = pass_ms
     roof["launches_timed"] = len(by_tag[dom])
-    part_bytes = 4 if prec == 0 else (6 if three_part else 4)
+    part_bytes = 4   # A is read in FP32
     roof["hbm_gbs"] = a.m * a.n * part_bytes / (pass_ms * 1e-3) / 1e9
     roof["hbm_frac_of_measured"] = roof["hbm_gbs"] / hbm
     # the chain: 2q + 2 passes over A
     npass = 2 * q + 2
     chain_bytes = npass * a.m * a.n * part_bytes
-    if prec == rqlp.PREC_FP32:
+    if on_alu:
         chain_flops = npass * flops
         t_flops = chain_flops / (roof["peak"] * 1e12)
         peak_name = "derived FP32"

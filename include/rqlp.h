@@ -76,7 +76,7 @@ typedef struct {
                    /* three products, error ~2^-16 |A| |X| per pass; 3: a    */
                    /* third part each (A_lo2 = bf16(A - A_hi - A_lo)), the   */
                    /* six products above 2^-24, FP32-level error at twice    */
-                   /* the MMA work and 1.5x the bytes of the split A;        */
+                   /* the MMA work (A is read in FP32 either way);           */
                    /* 0: automatic: three parts when p < 5 or m n <= 2^27,  */
                    /* else two (the batched form: three parts)               */
   int literal_step5; /* 0: step 5 on the d x d R, (P^, R^) = qr(R^T),         */
@@ -90,9 +90,9 @@ typedef struct {
                    /* small enough to stay in L2, Z = A P~ not              */
                    /* orthonormalised (its span is all the next product     */
                    /* needs): one pass over A from HBM per power pass       */
-                   /* instead of two. Measured slower than the two passes   */
-                   /* at every shape tried (200000 x 500: 6.2 vs 5.8 ms;    */
-                   /* 20000 x 20000: 12.8 vs 5.3 ms): an L2-sized panel     */
+                   /* instead of two. Slower than the two passes when last  */
+                   /* measured, at every shape (200000 x 500: 6.2, 5.8 ms;  */
+                   /* 20000 x 20000: 9.4, 3.3 ms): an L2-sized panel        */
                    /* holds few 128-row tiles, and each panel writes a      */
                    /* full n x d partial of Y.                              */
                    /* 0: the two passes with qf(Z) between (default).       */

@@ -1,7 +1,10 @@
 // Batched Rand-QLP: many independent problems, each with its own sizes,
 // k, p and buffers (one q for the batch), factored by the same chain as
 // rqlp_factor (Algorithm 1 steps 3-5 with q power passes, truncated to
-// d = k + p columns, CholeskyQR orthonormalisations) in plain FP32.
+// d = k + p columns, CholeskyQR orthonormalisations). The passes over A take the
+// grouped split product in BF16x3, and in FP32 where the batch has 3e8
+// multiply-adds (with an FMA product behind it for problems with values that
+// the parts do not represent); everything else is FP32.
 //
 // Every step of the chain is one grouped launch over all problems: the
 // products are persistent grouped GEMMs over a flattened tile list, the

@@ -1,6 +1,7 @@
-// FP32 SIMT GEMM engine: the plain-FP32 passes over A (Y = A^T X, Z = A X,
-// Algorithm 1 steps 3-4 and the power passes) and the tall-skinny products of
-// CholeskyQR (Gram X^T X, X R^{-1}).
+// FP32 SIMT GEMM engine: the FP32 passes over A (Y = A^T X, Z = A X, Algorithm 1
+// steps 3-4 and the power passes) that are too small for the tensor cores or
+// hold values outside what BF16 parts represent, and the tall-skinny products
+// of CholeskyQR (Gram X^T X, X R^{-1}).
 //
 // C = op(A) B with op(A) = A^T (transA) or A, row-major operands. Each CTA
 // owns a BM x BN tile of C and one slice of the K range (split-K); slices
