@@ -175,7 +175,7 @@ csc_sort_kernel(const int64_t* __restrict__ col_ptr, int64_t n, int* __restrict_
   grid_wait();
   __shared__ int sr[kSortShared];
   __shared__ float sv[kSortShared];
-  __shared__ int cols[2][256];   // slots of short and long columns of this round
+  __shared__ int cols[2][256];   // slots of the short and the long columns
   __shared__ int found[2];
   const int t = threadIdx.x, lane = t & 31;
   const int64_t G = gridDim.x, per = G * blockDim.x;

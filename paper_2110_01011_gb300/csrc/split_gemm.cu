@@ -709,15 +709,16 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   // it adds to, always toward zero. FP32: one chain per unit, the correction
   // products (2^-8 of the main ones) first, so that only two MMAs add to a
   // sum of full size; 64 units are summed in registers, then in memory.
-  // BF16x3: K = 4096, the corrections apart where tensor memory has room (npad
-  // <= 128) or there are three parts.
+  // BF16x3: K = 4096, with three parts 2560 (179560 x 376: L 9e-7 off in 128-row
+  // tiles, 1.2e-6 here, 2.0e-6 with 4096); the corrections apart where tensor
+  // memory has room (npad <= 128) or there are three parts.
   if (mode == kSplitFp32) {
     a.chunk = 1;
     a.corr = 0;
     a.corr_first = 1;
     a.flush = 64;
   } else {
-    a.chunk = (parts == 3 ? 2048 : 4096) / BK;
+    a.chunk = (parts == 3 ? 2560 : 4096) / BK;
     a.corr = parts == 3 || npad <= 128 ? 1 : 0;
     a.flush = 1 << 30;
   }
