@@ -247,10 +247,6 @@ struct Builder {
       const int64_t M = transA ? pr[i].n : pr[i].m, K = transA ? pr[i].m : pr[i].n;
       ts.npad_max = std::max(ts.npad_max, np);
       SplitJob j{};
-      alignas(64) char maps[kSplitMapBytes];
-      if (bf[i].img != nullptr && !split_job_maps(maps, &j, pr[i].A, pr[i].m, pr[i].n, pr[i].lda, transA)) b->maps_ok = false;
-      ts_maps.insert(ts_maps.end(), maps, maps + kSplitMapBytes);
-      j.img = bf[i].img;
       j.out = out(i);
       j.ldo = bf[i].ld;
       j.xlo = bf[i].xlo;
@@ -262,6 +258,11 @@ struct Builder {
       j.kb = (int)cdiv(K, 32);
       j.vec_out = (reinterpret_cast<uintptr_t>(j.out) % 16 == 0 && j.ldo % 4 == 0) ? 1 : 0;
       j.idesc = split_idesc(np);
+      alignas(64) char maps[kSplitMapBytes];
+      if (bf[i].img != nullptr && !split_job_maps(maps, &j, pr[i].A, pr[i].m, pr[i].n, pr[i].lda, transA, bf[i].img,
+                                                  b->mode == kSplitTwo ? 2 : 3))
+        b->maps_ok = false;
+      ts_maps.insert(ts_maps.end(), maps, maps + kSplitMapBytes);
       js.push_back(j);
       SplitXJob p{};
       p.X = X(i);

@@ -64,10 +64,11 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(tc::smem_u32(bar)), "h"((uint16_t)3) : "memory");
 }
-// Arrive on the pair leader's barrier. Relaxed: what the arrival hands over
-// lies in tensor memory and is ordered by the tcgen05 waits and fences around
-// it; a releasing arrive at cluster scope takes most of a microsecond (a unit
-// of 256 x 32 took 1.5 us with it and 0.7 us without).
+// Arrive on the pair leader's barrier. Relaxed: what these arrivals hand over lies
+// in tensor memory and is ordered by the tcgen05 waits and fences around them; a
+// releasing arrive at cluster scope takes most of a microsecond (a unit of 256 x
+// 32 took 1.5 us with it and 0.7 us without). Shared memory is never handed over
+// this way.
 __device__ __forceinline__ uint32_t leader_addr(const void* p) {   // p's place in the leader's shared memory
   uint32_t remote;
   asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(tc::smem_u32(p)));
@@ -77,26 +78,17 @@ __device__ __forceinline__ void arrive_remote(uint32_t bar) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void arrive_leader(uint64_t* bar) { arrive_remote(leader_addr(bar)); }
-// Hands back a stage whose values this warp holds in registers.
-__device__ __forceinline__ void arrive_read(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+// Hands back a stage that the warp's lanes have read, for a copy to refill: every
+// lane's reads are over before the copy may write (proxy fence), and the arrive
+// releases. Without the fence the arrive overtook reads that waited behind the
+// drain warps' stores, and a tile's values came from eight units of K later.
+__device__ __forceinline__ void arrive_read(uint64_t* bar, int lane) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if (lane == 0) tc::mbar_arrive(bar);
 }
-__device__ __forceinline__ bool try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.relaxed.cta.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(ok) : "r"(tc::smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-// Wait for MMAs, tensor-memory hand-overs or free stages; data that was copied
-// to shared memory is waited for with tc::mbar_wait (acquire).
-__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) {
-  if (try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!try_wait(bar, parity))
-    if (clock64() - t0 > kWaitLimit) return false;
-  return true;
-}
+// Acquires at CTA scope.
+__device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) { return tc::mbar_wait(bar, parity, kWaitLimit); }
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -111,10 +103,16 @@ __device__ __forceinline__ bool elect() {
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
   return p != 0;
 }
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   tc::smem_u32(dst)), "l"(src), "r"(bytes), "r"(tc::smem_u32(bar)) : "memory");
+// A box of X's image into this CTA's shared memory, counted by a barrier of the
+// pair's leader (both CTAs' halves of a stage complete on it, so the MMAs, which
+// read both, wait for one barrier that the copies themselves signal).
+__device__ __forceinline__ void load_image(void* dst, const CUtensorMap* map, uint32_t leader_bar, int row) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+      ::"r"(tc::smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(leader_bar)
+      : "memory");
 }
+constexpr int kImgRow = 256;   // BF16 entries of an image row: 8 columns of X by 32 of K
 // Eight 32-bit columns of this lane's row.
 __device__ __forceinline__ void st_row8(uint32_t t, const uint32_t* r) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(t), "r"(r[0]),
@@ -302,7 +300,7 @@ __device__ __forceinline__ void store_sums(float (&s)[NG][16], float* dst, int q
 }
 
 // ---------------------------------------------------------------- X
-// X (K x N FP32) -> stage images: for every unit of 32 of K, CTA of a group,
+// X (K x N FP32) -> stage images (read back as boxes of 512-byte rows): for every unit of 32 of K, CTA of a group,
 // and part, npad / CG rows (columns of X) of 32 K entries, 16-byte chunks
 // swizzled over 64-byte rows; zeros past K and N. A block of 256 threads takes
 // 64 of K and 32 columns through shared memory; a thread writes one 16-byte
@@ -361,7 +359,9 @@ struct Classes {
   int shift[4];
   int past[4];             // 1: no row in the class (its box starts past the map's end)
 };
-// The four maps (rows x cols, row stride lda); false when the encoder is missing.
+// The map of X's image for products of kb units, boxes of one part of a stage;
+// the four maps of A (rows x cols, row stride lda). False when the encoder is missing.
+bool image_map(CUtensorMap* m, const uint16_t* img, int kb, int npad, int parts);
 bool class_maps(CUtensorMap* m, Classes* cl, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans);
 template <bool TRANS>
 __device__ __forceinline__ void load_classes(unsigned char* f, const CUtensorMap* m0, const CUtensorMap* m1,

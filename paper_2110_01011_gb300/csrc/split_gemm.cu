@@ -66,6 +66,17 @@ static bool encode(CUtensorMap* map, const void* base, uint64_t cols, uint64_t r
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool image_map(CUtensorMap* m, const uint16_t* img, int kb, int npad, int parts) {
+  EncodeFn fn = encode_fn();
+  if (fn == nullptr) return false;
+  const uint32_t part_rows = (uint32_t)npad / CG * BK / kImgRow;   // of one CTA's stage
+  cuuint64_t dims[2] = {kImgRow, (cuuint64_t)kb * CG * parts * part_rows}, strides[1] = {kImgRow * 2};
+  cuuint32_t box[2] = {kImgRow, part_rows}, es[2] = {1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t*>(img), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool class_maps(CUtensorMap* m, Classes* cl, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans) {
   for (int c = 0; c < 4; ++c) {
     const bool empty = c >= rows;
@@ -101,7 +112,6 @@ using namespace sp;
 constexpr int kMaxSlots = 16;         // partial tiles that the last CTA of a tile sums itself
 
 struct Args {
-  const uint16_t* img;
   float* out;
   long long ldo;
   float* part;
@@ -150,15 +160,15 @@ __device__ inline int chain_units(const Args& a, int t, int k, int left) {
   return (int)min(min((long long)left, e - u), a.chunk - (u - b) % a.chunk);
 }
 
-// Maps over A: one, or one per class of rows.
-struct MapsA {
-  CUtensorMap m[4];
+// Maps over A (one, or one per class of rows) and over X's image.
+struct Maps {
+  CUtensorMap m[4], x;
 };
 
 // ALIGNED: A's rows are 16-byte aligned, one box a stage; else four.
 template <bool TRANS, int PARTS, bool ALIGNED>
 __global__ void __launch_bounds__(kThreads, 1)
-split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
+split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
   grid_wait();
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem =
@@ -235,8 +245,8 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");   // 40 + 2 x 64 + 2 x 152 <= 5 x 96
     if (warp == 0) {
       // ------------------------------------------------ X stages
-      const size_t img_stage = (size_t)CG * stage_bytes;
-      const unsigned char* img = reinterpret_cast<const unsigned char*>(a.img) + (size_t)rank * stage_bytes;
+      const uint32_t xfull0 = leader_addr(xfull);
+      const int rows = nh * BK / kImgRow;   // image rows of a part
       bool ok = true;
       Ring r;
       int n = u1 - u0, k = u0 % KB;
@@ -247,16 +257,18 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
           break;
         }
         if (elect()) {
-          tc::mbar_expect_tx(&xfull[r.s], (uint32_t)nx * part_bytes);
-          bulk_copy(xstage + (size_t)r.s * stage_bytes, img + (size_t)k * img_stage, (uint32_t)nx * part_bytes,
-                    &xfull[r.s]);
+          if (rank == 0) tc::mbar_expect_tx(&xfull[r.s], (uint32_t)(CG * nx) * part_bytes);
+          for (int p = 0; p < nx; ++p)
+            load_image(xstage + (size_t)r.s * stage_bytes + p * part_bytes, &tm.x, xfull0 + 8 * r.s,
+                       ((k * CG + rank) * PARTS + p) * rows);
         }
         k = k + 1 == KB ? 0 : k + 1;
         r.next(a.sx);
       }
       if (!ok) post_timeout(a.info);
-      for (int i = max(0, n - a.sx); i < n; ++i)   // no copy in flight at exit
-        if (!tc::mbar_wait(&xfull[i % a.sx], (uint32_t)((i / a.sx) & 1), kWaitLimit)) post_timeout(a.info);
+      // No copy in flight at exit (the leader's barriers count the peer's copies as well).
+      for (int i = rank == 0 ? max(0, n - a.sx) : n; i < n; ++i)
+        if (!wait(&xfull[i % a.sx], (uint32_t)((i / a.sx) & 1))) post_timeout(a.info);
     } else if (warp == 1) {
       // ------------------------------------------------ MMAs (the pair's leader)
       bool ok = true;
@@ -275,7 +287,7 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
           const uint32_t d = tmem + (uint32_t)(rb.s * a.npad), dc = a.corr ? corr_base : d;
           uint32_t acc = 0, cacc = cnew ? 0u : 1u;   // (with one accumulator the main product comes first)
           for (int i = 0; i < n; ++i) {
-            if (!tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit) || !wait(&afull[ra.s], ra.ph)) {
+            if (!wait(&xfull[rx.s], rx.ph) || !wait(&afull[ra.s], ra.ph)) {
               ok = false;
               break;
             }
@@ -368,10 +380,9 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
     const uint32_t lanes = (uint32_t)(32 * w) << 16;
     bool ok = true;
     const int n = u1 - u0;
-    Ring ra, rx, rf;                 // A slot, X stage, FP32 stage of the current unit
+    Ring ra, rf;                     // A slot, FP32 stage of the current unit
     if (odd) {
       ra.next(a.sa);
-      rx.next(a.sx);
       rf.next(a.sf);
     }
     const uint32_t afull0 = leader_addr(afull);
@@ -402,26 +413,16 @@ split_gemm_kernel(const __grid_constant__ MapsA tm, const Args a) {
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
       split_half<PARTS>(v, o, check, sq, ck);
-      __syncwarp();
-      if (lane == 0) arrive_read(&fempty[rf.s]);
+      arrive_read(&fempty[rf.s], lane);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
       if (sq) ck.fold();
-      if (rank != 0) {   // the pair's leader learns of the peer's X stage through the peer's A
-        ok = tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit);
-        if (!__all_sync(0xffffffffu, ok)) {
-          ok = false;
-          break;
-        }
-      }
       st_wait();
       tc::tc_fence_before();
       __syncwarp();
       if (lane == 0) arrive_remote(afull0 + 8 * ra.s);
       ra.next(a.sa);
       ra.next(a.sa);
-      rx.next(a.sx);
-      rx.next(a.sx);
       rf.next(a.sf);
       rf.next(a.sf);
     }
@@ -640,7 +641,7 @@ size_t smem_optin() {
 constexpr size_t kSmemExtra = 1024 + 1024;   // alignment, barriers
 
 template <bool TRANS, int PARTS, bool ALIGNED>
-cudaError_t launch(const MapsA& map, Args& a, int cap, size_t smem, cudaStream_t st) {
+cudaError_t launch(const Maps& map, Args& a, int cap, size_t smem, cudaStream_t st) {
   static int resident = 0;   // pairs that run at the same time
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
@@ -684,7 +685,6 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   CK(cudaGetLastError());
 
   Args a = {};
-  a.img = ws->img;
   a.out = out; a.ldo = ldo;
   a.part = ws->part;
   a.cnt = ws->cnt;
@@ -727,9 +727,11 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   a.nbuf = 2 * npad + cc + 2 * parts * 16 <= 512 ? 2 : 1;   // (FP32 above 208 columns: one)
   a.sa = std::min(kMaxASlots, (512 - a.nbuf * npad - cc) / (parts * 16));
   const size_t stage = (size_t)(npad / CG) * BK * 2 * parts;
-  MapsA map = {};
+  Maps map = {};
   bool aligned = false;
-  if (!split_maps(map.m, &a.cl, &aligned, A, transA ? K : M, transA ? M : K, lda, transA)) return cudaErrorNotSupported;
+  if (!split_maps(map.m, &a.cl, &aligned, A, transA ? K : M, transA ? M : K, lda, transA) ||
+      !image_map(&map.x, ws->img, kb, npad, parts))
+    return cudaErrorNotSupported;
   a.perm = !aligned && !transA ? 1 : 0;
   // Shared memory: four X stages first, then FP32 stages of A, then X again.
   const size_t avail = smem_optin() - kSmemExtra;

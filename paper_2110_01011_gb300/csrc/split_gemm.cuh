@@ -46,8 +46,7 @@ cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K
 
 // ---------------------------------------------------------------- grouped products (batched form)
 struct SplitJob {           // out (M x N) = op(A) X
-  const void* maps;         // four tensor maps over A, on the device (split_job_maps)
-  const uint16_t* img;      // X's parts, written by split_x_grouped
+  const void* maps;         // tensor maps over A and X's parts, on the device (split_job_maps)
   float* out;
   long long ldo;
   const int* xlo;           // raised when X has a low part
@@ -65,10 +64,12 @@ struct SplitXJob {          // X (K x N) -> stage images
   int* bad;
   int N, npad;
 };
-constexpr size_t kSplitMapBytes = 4 * 128;   // four tensor maps
-// Encodes the maps of A (rows x cols, row stride lda; A K x M when trans) into
-// host memory (128-byte entries) and sets the job's shifts.
-bool split_job_maps(void* maps, SplitJob* j, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans);
+constexpr size_t kSplitMapBytes = 5 * 128;   // five tensor maps
+// Encodes the maps of A (rows x cols, row stride lda; A K x M when trans) and of
+// X's parts (`img`, written by split_x_grouped) into host memory (128-byte
+// entries) and sets the job's shifts. The job's kb and npad are set before.
+bool split_job_maps(void* maps, SplitJob* j, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans,
+                    const uint16_t* img, int parts);
 int split_npad(int n);
 size_t split_image_bytes(int64_t K, int n, int parts);
 uint32_t split_idesc(int npad);

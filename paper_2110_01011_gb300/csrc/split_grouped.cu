@@ -6,7 +6,7 @@
 // whole K; the host balances the units over the CTA pairs (longest first, onto
 // the least loaded pair), so no tile is split and no pair waits for another.
 // A's FP32 tiles come by TMA through four maps per problem (its rows may start at
-// any 4-byte address), X's parts come as stage images that
+// any 4-byte address), X's parts through a fifth over the stage images that
 // split_x_grouped_kernel writes before the pass. The earlier form kept A's
 // parts in memory (a split of every A first, then 4 or 6 bytes per element and
 // pass); reading A in FP32 takes 4 and no split. Every wait is bounded.
@@ -95,15 +95,15 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");   // 40 + 2 x 112 + 2 x 104 <= 5 x 96
     if (warp == 0) {
       // ------------------------------------------------ X stages
+      const uint32_t xfull0 = leader_addr(xfull);
       bool ok = true;
       Ring r;
       int i = 0;
       for (int ui = ub; ui < ue && ok; ++ui) {
         const SplitJob& j = a.jobs[a.units[ui].x];
-        const uint32_t part = (uint32_t)(j.npad / CG) * BK * 2;
-        const uint32_t bytes = (*j.xlo ? (uint32_t)PARTS : 1u) * part;
-        const unsigned char* img = reinterpret_cast<const unsigned char*>(j.img) + (size_t)rank * PARTS * part;
-        const int kb = j.kb;
+        const CUtensorMap* map = static_cast<const CUtensorMap*>(j.maps) + 4;
+        const int kb = j.kb, nx = *j.xlo ? PARTS : 1, rows = j.npad / CG * BK / kImgRow;   // image rows of a part
+        const uint32_t part = (uint32_t)rows * kImgRow * 2;
         for (int k = 0; k < kb; ++k, ++i) {
           if (!wait(&xempty[r.s], r.ph ^ 1u)) {
             ok = false;
@@ -112,15 +112,18 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
           // Test hook: the first CTA withholds its first stage, so that the
           // waits on it run out and report.
           if (elect() && !(a.stall != 0 && blockIdx.x == 0 && i == 0)) {
-            tc::mbar_expect_tx(&xfull[r.s], bytes);
-            bulk_copy(xstage + (size_t)r.s * stage_bytes, img + (size_t)k * CG * PARTS * part, bytes, &xfull[r.s]);
+            if (rank == 0) tc::mbar_expect_tx(&xfull[r.s], (uint32_t)(CG * nx) * part);
+            for (int p = 0; p < nx; ++p)
+              load_image(xstage + (size_t)r.s * stage_bytes + p * part, map, xfull0 + 8 * r.s,
+                         ((k * CG + rank) * PARTS + p) * rows);
           }
           r.next(a.sx);
         }
       }
       if (!ok) post_timeout(a.info);
-      for (int s = max(0, i - a.sx); s < i; ++s)   // no copy in flight at exit
-        if (!tc::mbar_wait(&xfull[s % a.sx], (uint32_t)((s / a.sx) & 1), kWaitLimit)) post_timeout(a.info);
+      // No copy in flight at exit (the leader's barriers count the peer's copies as well).
+      for (int s = rank == 0 ? max(0, i - a.sx) : i; s < i; ++s)
+        if (!wait(&xfull[s % a.sx], (uint32_t)((s / a.sx) & 1))) post_timeout(a.info);
     } else if (warp == 1) {
       // ------------------------------------------------ MMAs (the pair's leader)
       bool ok = true;
@@ -142,7 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
             const uint32_t d = tmem + (uint32_t)(rb.s * a.npm), dc = a.corr ? corr_base : d;
             uint32_t acc = 0, cacc = a.corr ? 0u : 1u;   // (with one accumulator the main product comes first)
             for (int i = 0; i < n; ++i) {
-              if (!tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit) || !wait(&afull[ra.s], ra.ph)) {
+              if (!wait(&xfull[rx.s], rx.ph) || !wait(&afull[ra.s], ra.ph)) {
                 ok = false;
                 break;
               }
@@ -205,10 +208,9 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
     const int w = warp & 3, odd = (warp >> 2) - 1;   // two warpgroups take the units of K by turns
     const uint32_t lanes = (uint32_t)(32 * w) << 16;
     bool ok = true;
-    Ring ra, rx, rf;
+    Ring ra, rf;
     if (odd) {
       ra.next(a.sa);
-      rx.next(a.sx);
       rf.next(a.sf);
     }
     const uint32_t afull0 = leader_addr(afull);
@@ -243,26 +245,16 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
         split_half<PARTS>(v, o, check, sq, ck);
-        __syncwarp();
-        if (lane == 0) arrive_read(&fempty[rf.s]);
+        arrive_read(&fempty[rf.s], lane);
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
         if (sq) ck.fold();
-        if (rank != 0) {   // the pair's leader learns of the peer's X stage through the peer's A
-          ok = tc::mbar_wait(&xfull[rx.s], rx.ph, kWaitLimit);
-          if (!__all_sync(0xffffffffu, ok)) {
-            ok = false;
-            break;
-          }
-        }
         st_wait();
         tc::tc_fence_before();
         __syncwarp();
         if (lane == 0) arrive_remote(afull0 + 8 * ra.s);
         ra.next(a.sa);
         ra.next(a.sa);
-        rx.next(a.sx);
-        rx.next(a.sx);
         rf.next(a.sf);
         rf.next(a.sf);
       }
@@ -390,9 +382,11 @@ cudaError_t launch(const GroupArgs& a, int pairs, size_t smem, cudaStream_t st) 
 int split_npad(int n) { return (int)round_up(n, 16); }
 size_t split_image_bytes(int64_t K, int n, int parts) { return (size_t)round_up(K, BK) * split_npad(n) * parts * 2; }
 uint32_t split_idesc(int npad) { return tc::idesc_bf16(BM * CG, npad, false, false); }
-bool split_job_maps(void* maps, SplitJob* j, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans) {
+bool split_job_maps(void* maps, SplitJob* j, const float* A, int64_t rows, int64_t cols, int64_t lda, bool trans,
+                    const uint16_t* img, int parts) {
   Classes cl;
-  if (!class_maps(static_cast<CUtensorMap*>(maps), &cl, A, rows, cols, lda, trans)) return false;
+  CUtensorMap* m = static_cast<CUtensorMap*>(maps);
+  if (!class_maps(m, &cl, A, rows, cols, lda, trans) || !image_map(m + 4, img, j->kb, j->npad, parts)) return false;
   for (int c = 0; c < 4; ++c) {
     j->shift[c] = cl.shift[c];
     j->past[c] = cl.past[c];
