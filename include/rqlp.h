@@ -206,7 +206,10 @@ rqlp_status rqlp_factor_noalloc(const float* A, int64_t m, int64_t n, int64_t ld
  * rqlp_sketch: one pass over A (Algorithm 1 steps 3-4 and each power pass).
  *   trans = 1: Y (n x d, ldy) = A^T X with X m x d (ldx);
  *   trans = 0: Y (m x d, ldy) = A X   with X n x d (ldx).
- *   opts->precision selects FP32 or the BF16x3 tensor-core form. */
+ *   opts->precision selects FP32 or the BF16x3 tensor-core form. There is no
+ *   status word: where a bounded wait runs out (RQLP_ERR_TIMEOUT elsewhere) an
+ *   FP32 pass is redone without waits, and the results of a BF16x3 pass that
+ *   were lost are NaN. */
 size_t rqlp_sketch_workspace_bytes(int trans, int64_t m, int64_t n, int d, const rqlp_opts* opts);
 rqlp_status rqlp_sketch(int trans, const float* A, int64_t m, int64_t n, int64_t lda,
                         const float* X, int64_t ldx, int d, float* Y, int64_t ldy,

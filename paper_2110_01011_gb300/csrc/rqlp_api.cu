@@ -77,6 +77,7 @@ class Ops {
     split32_ = split_bytes > 0 && split_gemm_layout(ar, &sg_, part_, block_bytes, tall, tall, dcap_, 3);
   }
   void bind(cudaStream_t st, int* info) { st_ = st; info_ = info; }
+  void set_stall(bool stall) { sg_.stall = stall ? 1 : 0; }   // tests only (see split_gemm.cuh)
   int64_t ld() const { return ld_; }
   // Current sketch width (<= the capacity the workspace was laid out for).
   void set_d(int d) { d_ = d; }
@@ -805,9 +806,9 @@ size_t rqlp_sketch_workspace_bytes(int trans, int64_t m, int64_t n, int d, const
   return sketch_bytes(m, n, d, o);
 }
 
-rqlp_status rqlp_sketch(int trans, const float* A, int64_t m, int64_t n, int64_t lda, const float* X,
-                        int64_t ldx, int d, float* Y, int64_t ldy, void* workspace, size_t ws_bytes,
-                        const rqlp_opts* opts, void* stream) {
+static rqlp_status sketch(int trans, const float* A, int64_t m, int64_t n, int64_t lda, const float* X, int64_t ldx, int d,
+                          float* Y, int64_t ldy, void* workspace, size_t ws_bytes, const rqlp_opts* opts, void* stream,
+                          bool stall) {
   rqlp_opts o = resolve(opts);
   const size_t need = rqlp_sketch_workspace_bytes(trans, m, n, d, &o);
   if (need == 0 || A == nullptr || X == nullptr || Y == nullptr || lda < n || ldx < d || ldy < d)
@@ -820,9 +821,24 @@ rqlp_status rqlp_sketch(int trans, const float* A, int64_t m, int64_t n, int64_t
   ops.layout(ar, Ops::pass_part_floats(m, n, d), o.precision == RQLP_PREC_BF16X3, m, n,
              o.precision == RQLP_PREC_FP32 && Ops::split_pays(m, n, d) ? SIZE_MAX : 0);
   ops.bind(static_cast<cudaStream_t>(stream), nullptr);
+  ops.set_stall(stall);
   cudaError_t e = ops.begin_products();
   if (e == cudaSuccess) e = ops.pass(trans == 1, A, m, n, lda, X, ldx, Y, ldy, nullptr);
   return e == cudaSuccess ? RQLP_OK : RQLP_ERR_CUDA;
+}
+
+rqlp_status rqlp_sketch(int trans, const float* A, int64_t m, int64_t n, int64_t lda, const float* X,
+                        int64_t ldx, int d, float* Y, int64_t ldy, void* workspace, size_t ws_bytes,
+                        const rqlp_opts* opts, void* stream) {
+  return sketch(trans, A, m, n, lda, X, ldx, d, Y, ldy, workspace, ws_bytes, opts, stream, false);
+}
+
+// For tests, not part of the interface: rqlp_sketch whose tensor-core product
+// withholds a stage, so that its bounded waits run out.
+rqlp_status rqlp_test_sketch_stalled(int trans, const float* A, int64_t m, int64_t n, int64_t lda, const float* X,
+                                     int64_t ldx, int d, float* Y, int64_t ldy, void* workspace, size_t ws_bytes,
+                                     const rqlp_opts* opts, void* stream) {
+  return sketch(trans, A, m, n, lda, X, ldx, d, Y, ldy, workspace, ws_bytes, opts, stream, true);
 }
 
 size_t rqlp_orth_workspace_bytes(int64_t rows, int d, const rqlp_opts* opts) {

@@ -89,6 +89,11 @@ __device__ __forceinline__ void arrive_read(uint64_t* bar, int lane) {
 }
 // Acquires at CTA scope.
 __device__ __forceinline__ bool wait(uint64_t* bar, uint32_t parity) { return tc::mbar_wait(bar, parity, kWaitLimit); }
+// The same by a whole warp, with one answer for all lanes: a limit that runs out
+// in some of them must not part the warp in front of an elect or a barrier.
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, wait(bar, parity));
+}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -234,6 +239,15 @@ __device__ __forceinline__ void clear_sums(float (&s)[NG][16]) {
   for (int g = 0; g < NG; ++g)
 #pragma unroll
     for (int j = 0; j < 16; ++j) s[g][j] = 0.f;
+}
+// Sums that a drain warp could not read (its wait ran out): NaN, which no result
+// hides and which check_sums reports.
+template <int NG>
+__device__ __forceinline__ void lose_sums(float (&s)[NG][16]) {
+#pragma unroll
+  for (int g = 0; g < NG; ++g)
+#pragma unroll
+    for (int j = 0; j < 16; ++j) s[g][j] = __int_as_float(0x7fffffff);
 }
 // s += ng groups of 16 accumulator columns of this lane's row; all lanes.
 template <int NG>

@@ -32,7 +32,8 @@
 // registers and add with round-to-nearest. The (tile, unit) pairs are dealt
 // evenly to the CTAs (stream-K); split tiles are summed by the last CTA to
 // arrive, or by split_fixup_kernel when a tile spans more than kMaxSlots of
-// them. Every wait is bounded; a timeout is reported in the status word.
+// them. Every wait is bounded. Where one runs out, the status word reports it and
+// the sums that were not read become NaN, which raises the range word in FP32.
 #include <algorithm>
 
 #include "split_device.cuh"
@@ -129,6 +130,7 @@ struct Args {
   int flush;                // units whose sums are held in registers before they are added to global memory
   int corr;                 // 0: one accumulator; else main chains per chain of the correction accumulator
   int units;                // tiles x kb
+  int stall;                // fault-injection tests: the first CTA withholds its first stage of X
   uint32_t idesc;
   Classes cl;
 };
@@ -251,12 +253,12 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
       Ring r;
       int n = u1 - u0, k = u0 % KB;
       for (int i = 0; i < n; ++i) {
-        if (!wait(&xempty[r.s], r.ph ^ 1u)) {
+        if (!wait_warp(&xempty[r.s], r.ph ^ 1u)) {
           ok = false;
           n = i;
           break;
         }
-        if (elect()) {
+        if (elect() && !(a.stall != 0 && blockIdx.x == 0 && i == 0)) {
           if (rank == 0) tc::mbar_expect_tx(&xfull[r.s], (uint32_t)(CG * nx) * part_bytes);
           for (int p = 0; p < nx; ++p)
             load_image(xstage + (size_t)r.s * stage_bytes + p * part_bytes, &tm.x, xfull0 + 8 * r.s,
@@ -276,23 +278,19 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
         Ring rx, ra, rb;      // X stages, A slots, main accumulators
         int k = u0 % KB, t = u0 / KB, left = u1 - u0, chain = 0;   // chain: main chains of this tile part
         uint32_t cph = 0;     // parity of the correction chains
-        while (left > 0 && ok) {
+        // A lane whose wait ran out goes on without waiting, and nothing is issued
+        // where it is the one elected: the lanes stay together without a vote on
+        // the path from a drained accumulator to its next chain (1 % at 224 columns).
+        while (left > 0) {
           const int n = chain_units(a, t, k, min(left, KB - k));
           const bool cnew = a.corr != 0 && chain % a.corr == 0;   // a correction chain begins
-          if (!wait(&acce[rb.s], rb.ph ^ 1u) || (cnew && !wait(corre, cph ^ 1u))) {
-            ok = false;
-            break;
-          }
-          tc::tc_fence_after();
+          ok = ok && wait(&acce[rb.s], rb.ph ^ 1u) && (!cnew || wait(corre, cph ^ 1u));
           const uint32_t d = tmem + (uint32_t)(rb.s * a.npad), dc = a.corr ? corr_base : d;
           uint32_t acc = 0, cacc = cnew ? 0u : 1u;   // (with one accumulator the main product comes first)
           for (int i = 0; i < n; ++i) {
-            if (!wait(&xfull[rx.s], rx.ph) || !wait(&afull[ra.s], ra.ph)) {
-              ok = false;
-              break;
-            }
+            ok = ok && wait(&xfull[rx.s], rx.ph) && wait(&afull[ra.s], ra.ph);
             tc::tc_fence_after();
-            if (elect()) {
+            if (elect() && ok) {
               // Descriptors of the stage's parts; 16 of K are 32 bytes on.
               uint64_t x[PARTS];
 #pragma unroll
@@ -307,8 +305,7 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
             rx.next(a.sx);
             ra.next(a.sa);
           }
-          if (!ok) break;
-          if (elect()) commit(&accf[rb.s]);
+          if (elect() && ok) commit(&accf[rb.s]);
           rb.next(a.nbuf);
           ++chain;
           k += n;
@@ -331,7 +328,7 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
       Cursor c(u0, KB);
       int n = u1 - u0;
       for (int i = 0; i < n; ++i) {
-        if (!wait(&fempty[r.s], r.ph ^ 1u)) {
+        if (!wait_warp(&fempty[r.s], r.ph ^ 1u)) {
           ok = false;
           n = i;
           break;
@@ -351,7 +348,7 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
       }
       if (!ok) post_timeout(a.info);
       for (int i = max(0, n - a.sf); i < n; ++i)
-        if (!tc::mbar_wait(&ffull[i % a.sf], (uint32_t)((i / a.sf) & 1), kWaitLimit)) post_timeout(a.info);
+        if (!wait(&ffull[i % a.sf], (uint32_t)((i / a.sf) & 1))) post_timeout(a.info);
     }
   } else if (warp < 12) {
     // -------------------------------------------------- A: load, split, store to tensor memory
@@ -392,20 +389,14 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
         if (ALIGNED) read(f, half, v);
         else read_classes<TRANS>(f, a.cl, w, half, lane, v);
       };
-      ok = tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit);
-      if (!__all_sync(0xffffffffu, ok)) {
-        ok = false;
-        break;
-      }
+      ok = wait_warp(&ffull[rf.s], rf.ph);
+      if (!ok) break;
       float v[16];
       uint32_t o[PARTS][8];
       fetch(0, v);
       // (the slot is waited for while the values are on their way)
-      ok = wait(&aempty[ra.s], ra.ph ^ 1u);
-      if (!__all_sync(0xffffffffu, ok)) {
-        ok = false;
-        break;
-      }
+      ok = wait_warp(&aempty[ra.s], ra.ph ^ 1u);
+      if (!ok) break;
       tc::tc_fence_after();
       split_half<PARTS>(v, o, check, sq, ck);
       fetch(1, v);
@@ -447,11 +438,10 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
     while (left > 0) {
       const int n = chain_units(a, t, k, min(left, KB - k));
       const bool part_end = n == left || k + n == KB;
-      if (ok && !wait(&accf[rb.s], rb.ph)) {
+      if (ok && !wait_warp(&accf[rb.s], rb.ph)) {
         ok = false;
         if (lane == 0) post_timeout(a.info);
       }
-      ok = __all_sync(0xffffffffu, ok);
       if (ok) {
         tc::tc_fence_after();
         const uint32_t lanes = (uint32_t)(32 * (e & 3)) << 16, cols = (uint32_t)(16 * g0);
@@ -486,6 +476,7 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
         qstep = 4 * BM;
         vec = true;
       }
+      if (!ok) lose_sums(s);
       if (PARTS == 3 && a.bad != nullptr) check_sums(s, g0, ng, gm < a.M ? a.N : 0, a.bad);
       store_sums(s, dst, qstep, g0, ng, ncols, vec, flushed);
       if (part_end && !all && !a.fixup) {
@@ -699,6 +690,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   a.tiles = (int)cdiv(M, (int64_t)BM * CG);
   if ((long long)a.tiles * kb > (1LL << 30)) return cudaErrorInvalidValue;
   a.units = a.tiles * kb;
+  a.stall = ws->stall;
   // Short K: a split tile would cost more than it saves; whole tiles per CTA.
   a.whole = kb <= 32 ? 1 : 0;
   // Groups: at most two partial tiles each (none with whole tiles).

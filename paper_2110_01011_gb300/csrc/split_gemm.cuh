@@ -18,6 +18,7 @@ struct SplitGemmWs {
   size_t words_bytes = 0;    // words and counters, one block
   int slots = 0;             // 128-row partial slots that fit in part
   int turn = 0;
+  int stall = 0;             // fault-injection tests: see Args::stall
 };
 // Block that serves every product at full width (16-byte aligned); parts: 2 or
 // 3 (the largest used).
@@ -38,8 +39,9 @@ enum SplitMode { kSplitTwo = 2, kSplitThree = 3, kSplitFp32 = 4 };
 // K x N (N <= 256), all row-major FP32. sumsq (optional) += sum of squares of
 // A. *range_word (optional) receives the device word that a kSplitFp32 product
 // raises when a value of A or X lies outside the range that the parts
-// represent: the result then has to be recomputed in FP32, gated on that word
-// (before the next product but one clears it). Null in the other modes.
+// represent, or a wait ran out: the result then has to be recomputed in FP32,
+// gated on that word. Null in the other modes, where results that a wait lost
+// are NaN.
 cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K, const float* A, int64_t lda,
                        const float* X, int64_t ldx, float* out, int64_t ldo, SplitMode mode, double* sumsq,
                        const int** range_word, int* info, bool profiled, cudaStream_t st);

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         const int kb = j.kb, nx = *j.xlo ? PARTS : 1, rows = j.npad / CG * BK / kImgRow;   // image rows of a part
         const uint32_t part = (uint32_t)rows * kImgRow * 2;
         for (int k = 0; k < kb; ++k, ++i) {
-          if (!wait(&xempty[r.s], r.ph ^ 1u)) {
+          if (!wait_warp(&xempty[r.s], r.ph ^ 1u)) {
             ok = false;
             break;
           }
@@ -129,28 +129,21 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       bool ok = true;
       if (rank == 0) {
         Ring rx, ra, rb;
-        uint32_t cph = 0;
-        for (int ui = ub; ui < ue && ok; ++ui) {
+        uint32_t cph = 0;   // (timeouts: see split_gemm.cu)
+        for (int ui = ub; ui < ue; ++ui) {
           const SplitJob& j = a.jobs[a.units[ui].x];
           const uint32_t part = (uint32_t)(j.npad / CG) * BK * 2, idesc = j.idesc;
           const int nx = *j.xlo ? PARTS : 1;
           int left = j.kb;
-          while (left > 0 && ok) {
+          while (left > 0) {
             const int n = min(left, a.chunk);
-            if (!wait(&acce[rb.s], rb.ph ^ 1u) || (a.corr && !wait(corre, cph ^ 1u))) {
-              ok = false;
-              break;
-            }
-            tc::tc_fence_after();
+            ok = ok && wait(&acce[rb.s], rb.ph ^ 1u) && (!a.corr || wait(corre, cph ^ 1u));
             const uint32_t d = tmem + (uint32_t)(rb.s * a.npm), dc = a.corr ? corr_base : d;
             uint32_t acc = 0, cacc = a.corr ? 0u : 1u;   // (with one accumulator the main product comes first)
             for (int i = 0; i < n; ++i) {
-              if (!wait(&xfull[rx.s], rx.ph) || !wait(&afull[ra.s], ra.ph)) {
-                ok = false;
-                break;
-              }
+              ok = ok && wait(&xfull[rx.s], rx.ph) && wait(&afull[ra.s], ra.ph);
               tc::tc_fence_after();
-              if (elect()) {
+              if (elect() && ok) {
                 uint64_t x[PARTS];
 #pragma unroll
                 for (int p = 0; p < PARTS; ++p)
@@ -164,8 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
               rx.next(a.sx);
               ra.next(a.sa);
             }
-            if (!ok) break;
-            if (elect()) commit(&accf[rb.s]);
+            if (elect() && ok) commit(&accf[rb.s]);
             rb.next(a.nbuf);
             left -= n;
             if (a.corr) cph ^= 1u;   // drained with every chain
@@ -189,7 +181,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         for (int c = 0; c < 4; ++c) cl.past[c] = j.past[c];
         const int n = j.kb, row = (un.y * CG + rank) * BM;
         for (int k = 0; k < n; ++k, ++i) {
-          if (!wait(&fempty[r.s], r.ph ^ 1u)) {
+          if (!wait_warp(&fempty[r.s], r.ph ^ 1u)) {
             ok = false;
             break;
           }
@@ -200,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       }
       if (!ok) post_timeout(a.info);
       for (int s = max(0, i - a.sf); s < i; ++s)
-        if (!tc::mbar_wait(&ffull[s % a.sf], (uint32_t)((s / a.sf) & 1), kWaitLimit)) post_timeout(a.info);
+        if (!wait(&ffull[s % a.sf], (uint32_t)((s / a.sf) & 1))) post_timeout(a.info);
     }
   } else if (warp < 12) {
     // -------------------------------------------------- A: split, store to tensor memory
@@ -225,19 +217,13 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       const int n = j.kb;
       for (int k = turn; k < n; k += 2) {
         const unsigned char* f = fstage + rf.s * kClassBytes;
-        ok = tc::mbar_wait(&ffull[rf.s], rf.ph, kWaitLimit);
-        if (!__all_sync(0xffffffffu, ok)) {
-          ok = false;
-          break;
-        }
+        ok = wait_warp(&ffull[rf.s], rf.ph);
+        if (!ok) break;
         float v[16];
         uint32_t o[PARTS][8];
         read_classes<TRANS>(f, cl, w, 0, lane, v);
-        ok = wait(&aempty[ra.s], ra.ph ^ 1u);
-        if (!__all_sync(0xffffffffu, ok)) {
-          ok = false;
-          break;
-        }
+        ok = wait_warp(&aempty[ra.s], ra.ph ^ 1u);
+        if (!ok) break;
         tc::tc_fence_after();
         split_half<PARTS>(v, o, check, sq, ck);
         read_classes<TRANS>(f, cl, w, 1, lane, v);
@@ -284,11 +270,10 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       int left = j.kb, since = 0;
       while (left > 0) {
         const int n = min(left, a.chunk);
-        if (ok && !wait(&accf[rb.s], rb.ph)) {
+        if (ok && !wait_warp(&accf[rb.s], rb.ph)) {
           ok = false;
           if (lane == 0) post_timeout(a.info);
         }
-        ok = __all_sync(0xffffffffu, ok);
         if (ok) {
           tc::tc_fence_after();
           drain_columns(s, tmem + lanes + (uint32_t)(rb.s * a.npm + 16 * g0), ng);
@@ -302,6 +287,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         left -= n;
         since += n;
         if (left > 0 && since < a.flush) continue;
+        if (!ok) lose_sums(s);
         if (PARTS == 3 && j.bad != nullptr) check_sums(s, g0, ng, ncols, j.bad);
         store_sums(s, dst, 4, g0, ng, ncols, j.vec_out != 0, flushed);
         clear_sums(s);
