@@ -641,10 +641,11 @@ size_t layout(rqlp_batch_s* b, int count, const rqlp_problem* probs, Arena& ar, 
   const int parts = split ? (b->opts.bf16_parts == 2 ? 2 : 3) : 0;
   b->mode = !split ? kSplitFp32 : parts == 2 ? kSplitTwo : kSplitThree;
   // FP32 passes go to the tensor cores where a pass over all problems has
-  // enough multiply-adds to be worth the two launches.
+  // enough multiply-adds to be worth the two launches, and where there is an
+  // encoder for their tensor maps (else FMA products, as for one matrix).
   double work = 0;
   for (int i = 0; i < count; ++i) work += (double)probs[i].m * probs[i].n * (probs[i].k + probs[i].p);
-  b->tc = split || work >= 3e8;
+  b->tc = split || (work >= 3e8 && tc_supported(nullptr, 0, nullptr, 0));
   int* flags = nullptr;
   if (b->tc) flags = ar.take<int>(2 * (size_t)count);
   if (split) ar.take<char>((size_t)count * 12 * 128);   // (tensor maps of the panel layout: see take_bufs)
