@@ -732,19 +732,6 @@ chol_batched_kernel(const CholJob* __restrict__ jobs, int count) {
   chol_body<T, true>(j.d, j.G, j.ldg, j.R, j.Rinv, j.ldr, j.info, j.shift_count, j.gate_out, j.gate_in, nullptr);
 }
 
-size_t smem_optin_chol() {
-  static size_t v = 0;
-  if (v == 0) {
-    int dev = 0, x = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&x, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess && x > 0)
-      v = (size_t)x;
-    else
-      v = 227 * 1024;
-  }
-  return v;
-}
-
 template <typename T>
 size_t square_bytes(int d) { return (size_t)d * lds_of(d) * sizeof(T); }
 template <typename T>
@@ -753,21 +740,15 @@ template <typename T>
 size_t static_bytes() { return (kMaxD + Panel<T>::NB) * sizeof(T) + 96; }
 template <typename T>
 bool square_in_smem(int d) {
-  return square_bytes<T>(d) + panel_bytes<T>() + static_bytes<T>() <= smem_optin_chol();
+  return square_bytes<T>(d) + panel_bytes<T>() + static_bytes<T>() <= smem_optin();
 }
 
 template <typename T>
 cudaError_t launch(int d, const float* G, int64_t ldg, float* R, float* Rinv, int64_t ldr, int* info,
                    double* shift_count, int* gate_out, const int* gate_in, void* gstore, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    const int cap = (int)(smem_optin_chol() - static_bytes<T>());
-    cudaError_t e = cudaFuncSetAttribute(chol_blocked_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(chol_blocked_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice<char> once[2];
+  CK(allow_smem(&once[0], chol_blocked_kernel<T, true>, smem_optin() - static_bytes<T>()));
+  CK(allow_smem(&once[1], chol_blocked_kernel<T, false>, smem_optin() - static_bytes<T>()));
   const bool in_smem = square_in_smem<T>(d);
   if (!in_smem && gstore == nullptr) return cudaErrorInvalidValue;
   const size_t dyn = panel_bytes<T>() + (in_smem ? square_bytes<T>(d) : 0);
@@ -784,12 +765,8 @@ cudaError_t launch(int d, const float* G, int64_t ldg, float* R, float* Rinv, in
 template <int NB>
 cudaError_t launch_cluster(int d, const float* G, int64_t ldg, float* R, float* Rinv, int64_t ldr, int* info,
                            double* shift_count, int* gate_out, const int* gate_in, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    CK(cudaFuncSetAttribute(chol_cluster_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)cluster_smem_bytes<NB>(kMaxD)));
-    configured = true;
-  }
+  static PerDevice<char> once;
+  CK(allow_smem(&once, chol_cluster_kernel<NB>, cluster_smem_bytes<NB>(kMaxD)));
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -812,13 +789,8 @@ cudaError_t launch_cluster(int d, const float* G, int64_t ldg, float* R, float* 
 
 template <typename T>
 cudaError_t launch_batched(const CholJob* jobs, int count, int dmax, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(chol_batched_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(smem_optin_chol() - static_bytes<T>()));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice<char> once;
+  CK(allow_smem(&once, chol_batched_kernel<T>, smem_optin() - static_bytes<T>()));
   if (count <= 0) return cudaSuccess;   // configuration only
   if (!square_in_smem<T>(dmax)) return cudaErrorInvalidValue;
   const size_t dyn = panel_bytes<T>() + square_bytes<T>(dmax);
@@ -842,7 +814,7 @@ cudaError_t chol_inv_batched(const CholJob* jobs, int count, int dmax, bool fp64
 template <typename T>
 size_t global_bytes(int d) {
   const size_t panels = (size_t)32 * round_up(d, 16) * sizeof(T), fixed = (2 * kMaxD + 16) * sizeof(T) + 96;
-  return square_bytes<T>(d) + panels + fixed <= smem_optin_chol() ? 0 : square_bytes<T>(d);
+  return square_bytes<T>(d) + panels + fixed <= smem_optin() ? 0 : square_bytes<T>(d);
 }
 size_t chol_global_bytes(int d, bool fp64) { return fp64 ? global_bytes<double>(d) : global_bytes<float>(d); }
 

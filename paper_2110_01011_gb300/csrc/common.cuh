@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "../../include/rqlp.h"
+#include "per_device.cuh"
 
 // Return the CUDA error of x from the enclosing function.
 #define CK(x)                         \
@@ -45,7 +46,19 @@ struct Arena {
   }
 };
 
+// Of the current device: its number, SMs, and shared memory that a CTA may opt in to.
+int current_device();
 int sm_count();
+size_t smem_optin();
+// Lets `kernel` use that many bytes of dynamic shared memory on the current
+// device; `once` (a static beside the launch) remembers where it was done.
+template <typename K>
+cudaError_t allow_smem(PerDevice<char>* once, K* kernel, size_t bytes) {
+  char done;
+  return (cudaError_t)once->get(current_device(), &done, [&](char*) {
+    return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
+}
 
 // Asynchronous global -> shared copies (cp.async): `bytes` of the copy are
 // read from src, the rest of the 4- or 16-byte destination is zero-filled

@@ -534,19 +534,6 @@ int big_bn(int64_t N, int64_t K) { return K <= 256 && cdiv(N, 32) * 32 < cdiv(N,
 
 }  // namespace
 
-int sm_count() {
-  static int cached = 0;
-  if (cached == 0) {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0)
-      cached = n;
-    else
-      cached = 152;
-  }
-  return cached;
-}
-
 int gemm_f32_splits(int64_t M, int64_t N, int64_t K) {
   const bool wide = use_wide(M, N, K), big = use_big(M, N);
   const int64_t BM = big ? 128 : 32, BN = wide ? wide_bn(N) : big ? big_bn(N, K) : 32;
@@ -594,14 +581,8 @@ static cudaError_t launch_gemm(bool transA, const GemmArgs& g, int splits, cudaS
     dim3 grid((unsigned)cdiv(g.N, bn), (unsigned)cdiv(g.M, kWideBM), (unsigned)splits);
 #define RQLP_WIDE(T, V, W)                                                                              \
   do {                                                                                                  \
-    static bool set_ = false;                                                                           \
-    if (!set_) {                                                                                        \
-      const cudaError_t e_ = cudaFuncSetAttribute(gemm_f32_wide_kernel<T, V, W>,                       \
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,          \
-                                                  (int)wide_tot_bytes<W>());                            \
-      if (e_ != cudaSuccess) return e_;                                                                 \
-      set_ = true;                                                                                      \
-    }                                                                                                   \
+    static PerDevice<char> once_;                                                                       \
+    CK(allow_smem(&once_, gemm_f32_wide_kernel<T, V, W>, wide_tot_bytes<W>()));                         \
     launch_pdl(gemm_f32_wide_kernel<T, V, W>, grid, kWideThreads, wide_tot_bytes<W>(), st, g);                 \
   } while (0)
     if (bn == 112) {
@@ -663,7 +644,7 @@ cudaError_t gemm_f32_ex(bool transA, int64_t M, int64_t N, int64_t K, const floa
 
 // Grouped configurations (BM, BN, BK, TM, TN; threads = (BM/TM) (BN/TN)).
 namespace {
-// Resident CTAs per SM of one configuration (queried once; a launch with
+// Resident CTAs per SM of one configuration (queried once per device; a launch with
 // total <= 0 only primes the query, so that no query runs under capture).
 // persistent: a few CTAs per SM walk the tile list; otherwise one CTA per
 // tile and the hardware scheduler balances them.
@@ -671,16 +652,17 @@ template <int BM, int BN, int TM, int TN>
 cudaError_t launch_grouped_cfg(bool transA, bool persistent, const GroupGemm* jobs, const int* tile_start,
                                int count, int total, cudaStream_t st) {
   constexpr int NT = (BM / TM) * (BN / TN);
-  static int per_sm[2] = {0, 0};
-  int& occ = per_sm[transA ? 1 : 0];
-  if (occ == 0) {
-    cudaError_t e = transA ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                 &occ, gemm_grouped_kernel<BM, BN, 16, TM, TN, true>, NT, 0)
-                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                                 &occ, gemm_grouped_kernel<BM, BN, 16, TM, TN, false>, NT, 0);
-    if (e != cudaSuccess) return e;
-    if (occ < 1) occ = 1;
-  }
+  static PerDevice<int> per_sm[2];
+  int occ = 1;
+  const int e = per_sm[transA ? 1 : 0].get(current_device(), &occ, [&](int* n) {
+    const cudaError_t q = transA ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                       n, gemm_grouped_kernel<BM, BN, 16, TM, TN, true>, NT, 0)
+                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                                       n, gemm_grouped_kernel<BM, BN, 16, TM, TN, false>, NT, 0);
+    *n = std::max(1, *n);
+    return (int)q;
+  });
+  CK((cudaError_t)e);
   if (total <= 0 || count <= 0) return cudaSuccess;
   const int grid = persistent ? std::max(1, std::min(total, sm_count() * occ)) : total;
   if (transA) gemm_grouped_kernel<BM, BN, 16, TM, TN, true><<<grid, NT, 0, st>>>(jobs, tile_start, count);

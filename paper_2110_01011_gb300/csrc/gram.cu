@@ -286,7 +286,7 @@ int gram_threads(int d) { return gram_blocks(d) > kGramThreads ? kGramMaxThreads
 // One cluster per share of the rows, all of them resident at the same time.
 template <int NT>
 cudaError_t launch(const GramJob& j, float* part, size_t part_floats, int* clusters, cudaStream_t st) {
-  static int resident = 0;
+  static PerDevice<int> known;   // clusters that run at the same time
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   cfg.blockDim = dim3(NT);
@@ -300,13 +300,14 @@ cudaError_t launch(const GramJob& j, float* part, size_t part_floats, int* clust
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  if (resident == 0) {
-    CK(cudaFuncSetAttribute(gram_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem(NT)));
+  int resident = 1;
+  CK((cudaError_t)known.get(current_device(), &resident, [&](int* n) {
+    cudaError_t e = cudaFuncSetAttribute(gram_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_smem(NT));
     cfg.gridDim = dim3((unsigned)(sm_count() / kCluster * kCluster));
-    int n = 0;
-    CK(cudaOccupancyMaxActiveClusters(&n, gram_kernel<NT>, &cfg));
-    resident = std::max(1, std::min(n, sm_count() / kCluster));
-  }
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(n, gram_kernel<NT>, &cfg);
+    *n = std::max(1, std::min(*n, sm_count() / kCluster));
+    return (int)e;
+  }));
   const long long slot = gram_slot(j.d);
   *clusters = (int)std::min<long long>(resident, (long long)part_floats / slot);
   cfg.gridDim = dim3((unsigned)(*clusters * kCluster));

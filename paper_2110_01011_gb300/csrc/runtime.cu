@@ -11,6 +11,33 @@
 
 namespace rqlp {
 
+int current_device() {
+  int dev = 0;
+  return cudaGetDevice(&dev) == cudaSuccess ? dev : 0;
+}
+
+namespace {
+int attribute(PerDevice<int>& known, cudaDeviceAttr what, int otherwise) {
+  const int dev = current_device();
+  int v = 0;
+  const int e = known.get(dev, &v, [&](int* x) {
+    const cudaError_t q = cudaDeviceGetAttribute(x, what, dev);
+    return q != cudaSuccess ? (int)q : *x > 0 ? 0 : 1;
+  });
+  return e == 0 ? v : otherwise;
+}
+}  // namespace
+
+int sm_count() {
+  static PerDevice<int> known;
+  return attribute(known, cudaDevAttrMultiProcessorCount, 152);
+}
+
+size_t smem_optin() {
+  static PerDevice<int> known;
+  return (size_t)attribute(known, cudaDevAttrMaxSharedMemoryPerBlockOptin, 227 * 1024);
+}
+
 Range::Range(const char* name) { nvtxRangePushA(name); }
 Range::~Range() { nvtxRangePop(); }
 

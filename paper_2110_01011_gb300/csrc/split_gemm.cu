@@ -617,23 +617,11 @@ split_x_kernel(const float* __restrict__ X, long long K, int N, long long ldx, u
 
 int npad_of(int n) { return (int)round_up(n, 16); }   // N of the MMA; each CTA holds half of it, a multiple of 8
 
-size_t smem_optin() {
-  static size_t v = 0;
-  if (v == 0) {
-    int dev = 0, x = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&x, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess && x > 0)
-      v = (size_t)x;
-    else
-      v = 227 * 1024;
-  }
-  return v;
-}
 constexpr size_t kSmemExtra = 1024 + 1024;   // alignment, barriers
 
 template <bool TRANS, int PARTS, bool ALIGNED>
 cudaError_t launch(const Maps& map, Args& a, int cap, size_t smem, cudaStream_t st) {
-  static int resident = 0;   // pairs that run at the same time
+  static PerDevice<int> known;   // pairs that run at the same time
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[2];
   cfg.blockDim = dim3(kThreads);
@@ -646,15 +634,16 @@ cudaError_t launch(const Maps& map, Args& a, int cap, size_t smem, cudaStream_t 
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  if (resident == 0) {
-    CK(cudaFuncSetAttribute(split_gemm_kernel<TRANS, PARTS, ALIGNED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)smem_optin()));
-    int n = 0;
+  int resident = 1;
+  CK((cudaError_t)known.get(current_device(), &resident, [&](int* n) {
+    cudaError_t e = cudaFuncSetAttribute(split_gemm_kernel<TRANS, PARTS, ALIGNED>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_optin());
     cfg.gridDim = dim3((unsigned)(sm_count() / CG * CG));
     cfg.dynamicSmemBytes = smem_optin();
-    CK(cudaOccupancyMaxActiveClusters(&n, split_gemm_kernel<TRANS, PARTS, ALIGNED>, &cfg));
-    resident = std::max(1, std::min(n, sm_count() / CG));
-  }
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(n, split_gemm_kernel<TRANS, PARTS, ALIGNED>, &cfg);
+    *n = std::max(1, std::min(*n, sm_count() / CG));
+    return (int)e;
+  }));
   a.G = std::min(resident, cap);
   a.fixup = (!a.whole && a.G / a.tiles + 2 > kMaxSlots) ? 1 : 0;
   cfg.gridDim = dim3((unsigned)(a.G * CG));

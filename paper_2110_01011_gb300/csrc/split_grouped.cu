@@ -324,27 +324,10 @@ split_x_grouped_kernel(const SplitXJob* __restrict__ jobs, const int* __restrict
                local / kt * 32, j.xlo, j.bad);
 }
 
-size_t smem_optin_grouped() {
-  static size_t v = 0;
-  if (v == 0) {
-    int dev = 0, x = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&x, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess && x > 0)
-      v = (size_t)x;
-    else
-      v = 227 * 1024;
-  }
-  return v;
-}
-
 template <bool TRANS, int PARTS>
 cudaError_t launch(const GroupArgs& a, int pairs, size_t smem, cudaStream_t st) {
-  static bool configured = false;
-  if (!configured) {
-    CK(cudaFuncSetAttribute(split_grouped_kernel<TRANS, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)smem_optin_grouped()));
-    configured = true;
-  }
+  static PerDevice<char> once;
+  CK(allow_smem(&once, split_grouped_kernel<TRANS, PARTS>, smem_optin()));
   if (pairs <= 0) return cudaSuccess;   // configuration only
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
@@ -407,7 +390,7 @@ cudaError_t split_grouped(bool transA, const SplitJob* jobs, const int2* units, 
   a.nbuf = 2 * a.npm + cc + 2 * parts * 16 <= 512 ? 2 : 1;
   a.sa = std::min(kMaxASlots, (512 - a.nbuf * a.npm - cc) / (parts * 16));
   const size_t stage = (size_t)parts * (a.npm / CG) * BK * 2, extra = 2048;
-  const size_t avail = smem_optin_grouped() - extra;
+  const size_t avail = smem_optin() - extra;
   a.sf = (int)std::min<size_t>(kMaxStages, (avail - 4 * stage) / kClassBytes);
   a.sx = (int)std::min<size_t>(kMaxStages, (avail - a.sf * kClassBytes) / stage);
   if (a.sa < 2) return cudaErrorInvalidValue;

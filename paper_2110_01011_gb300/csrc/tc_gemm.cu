@@ -646,23 +646,10 @@ uint32_t stage_bytes_of(int npad, bool exact, int bkp) {
   return (exact ? 3u : 2u) * (uint32_t)(BM * bkp * 2) + (exact ? 3u : 2u) * (uint32_t)npad * bkp * 2;
 }
 
-size_t smem_optin_tc() {
-  static size_t v = 0;
-  if (v == 0) {
-    int dev = 0, x = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&x, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess && x > 0)
-      v = (size_t)x;
-    else
-      v = 227 * 1024;
-  }
-  return v;
-}
-
 // Pipeline stages of a pass (>= 1; the exact mode's stages at d = 256 hold
 // one at a time, which its short K does not need more than).
 int stages_of(int npad, bool exact, int bkp) {
-  const size_t avail = smem_optin_tc() - 1024 - 512;
+  const size_t avail = smem_optin() - 1024 - 512;
   int s = (int)(avail / stage_bytes_of(npad, exact, bkp));
   return std::max(1, std::min(kMaxStages, s));
 }
@@ -673,13 +660,8 @@ cudaError_t launch_pass(const CUtensorMap& ah, const CUtensorMap& al, const CUte
                         const CUtensorMap& xl, const CUtensorMap& al2, const CUtensorMap& xl2, const TcArgs& a,
                         cudaStream_t st) {
   const size_t smem = (size_t)a.stages * a.stage_bytes + 1024 + 512;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tc_pass_kernel<BKP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(smem_optin_tc()));
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice<char> once;
+  CK(allow_smem(&once, tc_pass_kernel<BKP>, smem_optin()));
   launch_pdl(tc_pass_kernel<BKP>, a.G, kThreads, smem, st, ah, al, xh, xl, al2, xl2, a);
   note_launch();
   return cudaGetLastError();
@@ -816,7 +798,7 @@ cudaError_t TcEngine::gram(float* Gout, int64_t ldg, int* info, cudaStream_t st)
   a.mtiles = mtiles;
   a.nbox = std::max((int)cdiv(npad, 64), 2 * mtiles);
   a.stage_bytes = 2u * (uint32_t)a.nbox * 4096u;
-  a.stages = std::max(2, std::min(kMaxStages, (int)((smem_optin_tc() - 1024 - 512) / a.stage_bytes)));
+  a.stages = std::max(2, std::min(kMaxStages, (int)((smem_optin() - 1024 - 512) / a.stage_bytes)));
   a.part = gpart_;
   a.info = info;
   a.idesc = tc::idesc_bf16(BM, npad, true, true);
@@ -829,13 +811,8 @@ cudaError_t TcEngine::gram(float* Gout, int64_t ldg, int* info, cudaStream_t st)
   if (!make_panel_map(&hi, Ahi_, m_, cdiv(cols, 64), 64, BK, 1, CU_TENSOR_MAP_SWIZZLE_128B) ||
       !make_panel_map(&lo, Alo_, m_, cdiv(cols, 64), 64, BK, 1, CU_TENSOR_MAP_SWIZZLE_128B))
     return cudaErrorInvalidValue;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(tc_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem_optin_tc());
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice<char> once;
+  CK(allow_smem(&once, tc_gram_kernel, smem_optin()));
   const size_t smem = (size_t)a.stages * a.stage_bytes + 1024 + 512;
   launch_pdl(tc_gram_kernel, a.G, kThreads, smem, st, hi, lo, a);
   note_launch();
