@@ -3,8 +3,8 @@
 // rqlp_factor (Algorithm 1 steps 3-5 with q power passes, truncated to
 // d = k + p columns, CholeskyQR orthonormalisations). The passes over A take the
 // grouped split product in BF16x3, and in FP32 where the batch has 3e8
-// multiply-adds (with an FMA product behind it for problems with values that
-// the parts do not represent); everything else is FP32.
+// multiply-adds (with an FMA product behind it for problems whose sums are not
+// finite); everything else is FP32.
 //
 // Every step of the chain is one grouped launch over all problems: the
 // products are persistent grouped GEMMs over a flattened tile list, the
@@ -84,7 +84,7 @@ struct Bufs {
   int64_t ld;
   uint16_t* img = nullptr;   // tensor-core passes: the parts of a pass's X
   int* xlo = nullptr;        // X low part nonzero (per pass)
-  int* bad = nullptr;        // a value outside the parts' range (per pass, FP32)
+  int* bad = nullptr;        // a sum that is not finite (per pass, FP32)
 };
 constexpr int kMaxTcCtas = 1024;
 
@@ -270,7 +270,6 @@ struct Builder {
       p.K = K;
       p.img = bf[i].img;
       p.xlo = bf[i].xlo;
-      p.bad = j.bad;
       p.N = di;
       p.npad = np;
       ps.push_back(p);
@@ -500,7 +499,7 @@ struct Builder {
 
     // A pass over every problem (sumsq: ||A||_F^2 rides along): on the tensor
     // cores where b->tc, else as grouped FP32 products. In FP32 the latter follow
-    // the former for the problems whose values the parts do not represent.
+    // the former for the problems whose sums are not finite.
     auto pass = [&](bool transA, auto X, auto ldx, auto out, bool sumsq) {
       if (b->tc) {
         tc_pass(transA, X, ldx, out, sumsq);

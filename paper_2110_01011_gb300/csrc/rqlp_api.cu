@@ -177,7 +177,7 @@ class Ops {
   static bool split_pays(int64_t M, int64_t K, int d) { return (double)M * K * d >= 2e8; }
   // The same product in FP32. Where it pays it runs on the
   // tensor cores in three parts; an FMA product gated on the range word then
-  // redoes it where a value lies outside what the parts represent.
+  // redoes it where a sum is not finite (values too large for the parts).
   cudaError_t product32(bool transA, int64_t M, int64_t K, const float* A, int64_t lda, const float* X, int64_t ldx,
                         float* out, int64_t ldout, double* sumsq) {
     const int* word = nullptr;

@@ -21,10 +21,15 @@ constexpr int kMaxStages = 8;
 constexpr int kMaxASlots = 8;
 constexpr uint32_t kABytes = BM * BK * 4;        // FP32 stage of A by TMA
 constexpr long long kWaitLimit = 4000000000LL;   // cycles (~2 s)
-// Parts hold a value exactly when its magnitude lies in [2^-96, 2^127) (or is
-// zero): below, the last part would be subnormal; above, the first may round
-// to infinity.
-constexpr uint32_t kRangeHi = 0x7F000000u, kRangeLo = 0x0F800000u;
+// The FP32 form splits 2^24 A and 2^24 X: no FP32 value has a bit below 2^-149, so
+// every nonzero part is then a normal BF16 number and three of them hold the value,
+// however small it is. (Without the factor one nonzero value below 2^-96, of which a
+// kernel matrix or a localised basis has many, sent the whole product to the FMA
+// units: 16384 x 12288, q = 1 with such entries 11.9 ms, now 3.24 as without them.)
+// The drain warps take the sums back by 2^-48 in the multiply-add that was an add,
+// so ordinary results are the same bits. What overflows on the way, values of 2^104 and sums of
+// 2^80 upward, gives sums that are not finite, which the drain warps look for.
+constexpr float kScaleUp = 16777216.f, kScaleDown = 1.f / (kScaleUp * kScaleUp);
 
 __device__ inline void post_timeout(int* info) {
   if (info != nullptr && atomicCAS(info, 0, RQLP_ERR_TIMEOUT) == 0) info[1] = 0;
@@ -190,20 +195,14 @@ __device__ __forceinline__ void issue_products(uint32_t d, uint32_t dc, uint32_t
   }
 }
 
-// What the split warps collect beside the parts: the smallest nonzero |A| and
-// the sum of squares, Kahan-compensated per unit. (Values too large for the
-// parts give sums that are not finite: the drain warps look for those.)
-struct Checks {
-  uint32_t umin = 0xFFFFFFFFu;   // of 2 |bits| - 1: zero wraps to the largest value
+// The split warps' sum of squares of A, Kahan-compensated per unit.
+struct Squares {
   float ss = 0.f, comp = 0.f, part = 0.f;
   __device__ void fold() {
     const float y = part - comp, t = ss + y;
     comp = (t - ss) - y;
     ss = t;
     part = 0.f;
-  }
-  __device__ void report(int* bad, int lane) const {
-    if (__any_sync(0xffffffffu, umin < 2u * kRangeLo - 1u) && lane == 0) atomicOr(bad, 1);
   }
   __device__ void add(double* sumsq, int lane) const {
     double v = (double)ss - (double)comp;
@@ -213,15 +212,14 @@ struct Checks {
 };
 // Sixteen values along K -> eight packed columns per part.
 template <int PARTS>
-__device__ __forceinline__ void split_half(const float* v, uint32_t (&o)[PARTS][8], bool check, bool sq, Checks& ck) {
-  if (check) {
-#pragma unroll
-    for (int j = 0; j < 16; j += 2)
-      ck.umin = __vimin3_u32(ck.umin, 2u * __float_as_uint(v[j]) - 1u, 2u * __float_as_uint(v[j + 1]) - 1u);
-  }
+__device__ __forceinline__ void split_half(float* v, uint32_t (&o)[PARTS][8], bool scaled, bool sq, Squares& sum) {
   if (sq) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) ck.part = fmaf(v[j], v[j], ck.part);
+    for (int j = 0; j < 16; ++j) sum.part = fmaf(v[j], v[j], sum.part);
+  }
+  if (scaled) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] *= kScaleUp;
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -249,9 +247,9 @@ __device__ __forceinline__ void lose_sums(float (&s)[NG][16]) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) s[g][j] = __int_as_float(0x7fffffff);
 }
-// s += ng groups of 16 accumulator columns of this lane's row; all lanes.
+// s += f times ng groups of 16 accumulator columns of this lane's row; all lanes.
 template <int NG>
-__device__ __forceinline__ void drain_columns(float (&s)[NG][16], uint32_t ta, int ng) {
+__device__ __forceinline__ void drain_columns(float (&s)[NG][16], uint32_t ta, int ng, float f) {
 #pragma unroll
   for (int g = 0; g < NG; ++g) {
     if (g < ng) {
@@ -260,7 +258,7 @@ __device__ __forceinline__ void drain_columns(float (&s)[NG][16], uint32_t ta, i
       ld_wait();
       ld_done(v);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) s[g][j] += v[j];
+      for (int j = 0; j < 16; ++j) s[g][j] = fmaf(v[j], f, s[g][j]);
     }
   }
   tc::tc_fence_before();
@@ -321,7 +319,7 @@ __device__ __forceinline__ void store_sums(float (&s)[NG][16], float* dst, int q
 // chunk (8 of K) of each part.
 __device__ __forceinline__ void split_x_tile(const float* __restrict__ X, long long K, int N, long long ldx,
                                              uint16_t* __restrict__ img, int npad, int parts, int kb, long long k0,
-                                             int n0, int* xlo, int* bad) {
+                                             int n0, int* xlo, bool scaled) {
   __shared__ float tile[64][33];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
@@ -333,18 +331,16 @@ __device__ __forceinline__ void split_x_tile(const float* __restrict__ X, long l
   const int nn = threadIdx.x >> 3, ch = threadIdx.x & 7;   // column, chunk of 8 of K
   const int n = n0 + nn;
   const long long unit = (k0 >> 5) + (ch >> 2);
-  bool any = false, out_of_range = false;
+  const float up = scaled ? kScaleUp : 1.f;
+  bool any = false;
   if (n < npad && unit < kb) {
     uint32_t p[3][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       uint32_t q[3];
-      const float x0 = tile[ch * 8 + 2 * j][nn], x1 = tile[ch * 8 + 2 * j + 1][nn];
-      split2<3>(x0, x1, q);
+      split2<3>(up * tile[ch * 8 + 2 * j][nn], up * tile[ch * 8 + 2 * j + 1][nn], q);
       p[0][j] = q[0]; p[1][j] = q[1]; p[2][j] = q[2];
       any |= (q[1] & 0x7FFF7FFFu) != 0;
-      const uint32_t m0 = __float_as_uint(x0) & 0x7FFFFFFFu, m1 = __float_as_uint(x1) & 0x7FFFFFFFu;
-      out_of_range |= max(m0, m1) >= kRangeHi || min(m0 - 1u, m1 - 1u) < kRangeLo - 1u;
     }
     const int nh = npad / CG, r = n % nh;
     const size_t stage = ((size_t)unit * CG + n / nh) * parts * nh * 32;
@@ -353,7 +349,6 @@ __device__ __forceinline__ void split_x_tile(const float* __restrict__ X, long l
       *reinterpret_cast<uint4*>(img + at + (size_t)q * nh * 32) = make_uint4(p[q][0], p[q][1], p[q][2], p[q][3]);
   }
   if (__syncthreads_or(any) && threadIdx.x == 0 && *(volatile int*)xlo == 0) atomicOr(xlo, 1);
-  if (bad != nullptr && __syncthreads_or(out_of_range) && threadIdx.x == 0) atomicOr(bad, 1);
 }
 
 // ---------------------------------------------------------------- A with rows at any 4-byte address

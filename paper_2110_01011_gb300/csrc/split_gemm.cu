@@ -132,6 +132,7 @@ struct Args {
   int units;                // tiles x kb
   int stall;                // fault-injection tests: the first CTA withholds its first stage of X
   uint32_t idesc;
+  float down;               // factor of the sums (FP32: kScaleDown, A and X being scaled up)
   Classes cl;
 };
 
@@ -354,8 +355,8 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
     // -------------------------------------------------- A: load, split, store to tensor memory
     asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
     const int w = warp & 3, odd = (warp >> 2) - 1;   // two warpgroups take the units by turns
-    const bool check = PARTS == 3 && a.bad != nullptr, sq = a.sumsq != nullptr;
-    Checks ck;
+    const bool scaled = PARTS == 3 && a.down != 1.f, sq = a.sumsq != nullptr;
+    Squares sum;
     // A stage holds 128 rows of op(A) by 32 of K. TRANS: as in memory, [K][row];
     // else [row][K] with the 16-byte chunks of a row xored with row % 8 (the
     // 128-byte swizzle). v[j] = op(A)(this lane's row, 16 half + j): both reads
@@ -398,16 +399,16 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
       ok = wait_warp(&aempty[ra.s], ra.ph ^ 1u);
       if (!ok) break;
       tc::tc_fence_after();
-      split_half<PARTS>(v, o, check, sq, ck);
+      split_half<PARTS>(v, o, scaled, sq, sum);
       fetch(1, v);
       const uint32_t ta = a_base + lanes + (uint32_t)(ra.s * PARTS * 16);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
-      split_half<PARTS>(v, o, check, sq, ck);
+      split_half<PARTS>(v, o, scaled, sq, sum);
       arrive_read(&fempty[rf.s], lane);
 #pragma unroll
       for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
-      if (sq) ck.fold();
+      if (sq) sum.fold();
       st_wait();
       tc::tc_fence_before();
       __syncwarp();
@@ -418,8 +419,7 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
       rf.next(a.sf);
     }
     if (!ok && lane == 0) post_timeout(a.info);
-    if (check) ck.report(a.bad, lane);
-    if (sq) ck.add(a.sumsq, lane);
+    if (sq) sum.add(a.sumsq, lane);
   } else {
     // -------------------------------------------------- drain: TMEM -> registers -> global
     asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
@@ -445,10 +445,10 @@ split_gemm_kernel(const __grid_constant__ Maps tm, const Args a) {
       if (ok) {
         tc::tc_fence_after();
         const uint32_t lanes = (uint32_t)(32 * (e & 3)) << 16, cols = (uint32_t)(16 * g0);
-        drain_columns(s, tmem + lanes + (uint32_t)(rb.s * a.npad) + cols, ng);
+        drain_columns(s, tmem + lanes + (uint32_t)(rb.s * a.npad) + cols, ng, a.down);
         if (lane == 0) arrive_leader(&acce[rb.s]);
         if (a.corr && ((chain + 1) % a.corr == 0 || part_end)) {
-          drain_columns(s, corr_base + lanes + cols, ng);
+          drain_columns(s, corr_base + lanes + cols, ng, a.down);
           if (lane == 0) arrive_leader(corre);
         }
       }
@@ -610,9 +610,9 @@ __global__ void split_fixup_kernel(const Args a) {
 
 __global__ void __launch_bounds__(256)
 split_x_kernel(const float* __restrict__ X, long long K, int N, long long ldx, uint16_t* __restrict__ img, int npad,
-               int parts, int kb, int* xlo, int* bad) {
+               int parts, int kb, int* xlo, bool scaled) {
   grid_wait();
-  split_x_tile(X, K, N, ldx, img, npad, parts, kb, (long long)blockIdx.x * 64, blockIdx.y * 32, xlo, bad);
+  split_x_tile(X, K, N, ldx, img, npad, parts, kb, (long long)blockIdx.x * 64, blockIdx.y * 32, xlo, scaled);
 }
 
 int npad_of(int n) { return (int)round_up(n, 16); }   // N of the MMA; each CTA holds half of it, a multiple of 8
@@ -660,7 +660,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   const int npad = npad_of(N), kb = (int)cdiv(K, BK);
   int* w = ws->words;
   launch_pdl(split_x_kernel, dim3((unsigned)cdiv(kb, 2), (unsigned)cdiv(npad, 32)), 256, 0, st, X, K, N, ldx, ws->img,
-             npad, parts, kb, w + turn, bad);
+             npad, parts, kb, w + turn, mode == kSplitFp32);
   note_launch();
   CK(cudaGetLastError());
 
@@ -670,6 +670,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   a.cnt = ws->cnt;
   a.xlo = w + turn;
   a.bad = bad;
+  a.down = mode == kSplitFp32 ? kScaleDown : 1.f;
   a.next0 = w + (turn ^ 1);
   a.next1 = w + 2 + (turn ^ 1);
   a.sumsq = sumsq;

@@ -13,7 +13,7 @@ namespace rqlp {
 struct SplitGemmWs {
   uint16_t* img = nullptr;   // X's parts as shared-memory stage images
   float* part = nullptr;     // partial tiles of split K ranges
-  int* words = nullptr;      // [0..1] X low part nonzero, [2..3] values outside the split's range, by turn
+  int* words = nullptr;      // [0..1] X low part nonzero, [2..3] sums that are not finite, by turn
   int* cnt = nullptr;        // tile arrival counters
   size_t words_bytes = 0;    // words and counters, one block
   int slots = 0;             // 128-row partial slots that fit in part
@@ -38,9 +38,10 @@ enum SplitMode { kSplitTwo = 2, kSplitThree = 3, kSplitFp32 = 4 };
 // transA: out (M x N) = A^T X with A K x M; else out = A X with A M x K; X is
 // K x N (N <= 256), all row-major FP32. sumsq (optional) += sum of squares of
 // A. *range_word (optional) receives the device word that a kSplitFp32 product
-// raises when a value of A or X lies outside the range that the parts
-// represent, or a wait ran out: the result then has to be recomputed in FP32,
-// gated on that word. Null in the other modes, where results that a wait lost
+// raises when a sum is not finite, because of values of A or X that are not or
+// are too large for the form (split_device.cuh), or because a wait ran out: the
+// result then has to be recomputed in FP32, gated on that word, before the next
+// product, which clears it. Null in the other modes, where results that a wait lost
 // are NaN.
 cudaError_t split_gemm(SplitGemmWs* ws, bool transA, int64_t M, int N, int64_t K, const float* A, int64_t lda,
                        const float* X, int64_t ldx, float* out, int64_t ldo, SplitMode mode, double* sumsq,
@@ -52,7 +53,7 @@ struct SplitJob {           // out (M x N) = op(A) X
   float* out;
   long long ldo;
   const int* xlo;           // raised when X has a low part
-  int* bad;                 // raised on values outside the parts' range (FP32; else null)
+  int* bad;                 // raised on sums that are not finite (FP32; else null)
   double* sumsq;            // += sum of squares of A (or null)
   int M, N, npad, kb, vec_out;
   uint32_t idesc;
@@ -63,7 +64,6 @@ struct SplitXJob {          // X (K x N) -> stage images
   long long ldx, K;
   uint16_t* img;
   int* xlo;
-  int* bad;
   int N, npad;
 };
 constexpr size_t kSplitMapBytes = 5 * 128;   // five tensor maps

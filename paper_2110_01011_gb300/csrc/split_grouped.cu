@@ -29,6 +29,7 @@ struct GroupArgs {
   int* info;
   int npm;                  // largest npad: the layout of shared and tensor memory
   int sx, sf, sa, nbuf, corr, corr_first, chunk, flush, stall;
+  float down;               // (see split_gemm.cu)
 };
 
 template <bool TRANS, int PARTS>
@@ -206,11 +207,12 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
       rf.next(a.sf);
     }
     const uint32_t afull0 = leader_addr(afull);
+    const bool scaled = PARTS == 3 && a.down != 1.f;
     int turn = odd;   // this warpgroup's first unit of K within the tile
     for (int ui = ub; ui < ue && ok; ++ui) {
       const SplitJob& j = a.jobs[a.units[ui].x];
-      const bool check = PARTS == 3 && j.bad != nullptr, sq = j.sumsq != nullptr;
-      Checks ck;
+      const bool sq = j.sumsq != nullptr;
+      Squares sum;
       Classes cl;
 #pragma unroll
       for (int c = 0; c < 4; ++c) cl.shift[c] = j.shift[c];
@@ -225,16 +227,16 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         ok = wait_warp(&aempty[ra.s], ra.ph ^ 1u);
         if (!ok) break;
         tc::tc_fence_after();
-        split_half<PARTS>(v, o, check, sq, ck);
+        split_half<PARTS>(v, o, scaled, sq, sum);
         read_classes<TRANS>(f, cl, w, 1, lane, v);
         const uint32_t ta = a_base + lanes + (uint32_t)(ra.s * PARTS * 16);
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16, o[q]);
-        split_half<PARTS>(v, o, check, sq, ck);
+        split_half<PARTS>(v, o, scaled, sq, sum);
         arrive_read(&fempty[rf.s], lane);
 #pragma unroll
         for (int q = 0; q < PARTS; ++q) st_row8(ta + q * 16 + 8, o[q]);
-        if (sq) ck.fold();
+        if (sq) sum.fold();
         st_wait();
         tc::tc_fence_before();
         __syncwarp();
@@ -245,8 +247,7 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         rf.next(a.sf);
       }
       if (n & 1) turn ^= 1;   // the other warpgroup begins the next tile
-      if (check) ck.report(j.bad, lane);
-      if (sq) ck.add(j.sumsq, lane);
+      if (sq) sum.add(j.sumsq, lane);
     }
     if (!ok && lane == 0) post_timeout(a.info);
   } else {
@@ -276,10 +277,10 @@ __global__ void __launch_bounds__(kThreads, 1) split_grouped_kernel(const GroupA
         }
         if (ok) {
           tc::tc_fence_after();
-          drain_columns(s, tmem + lanes + (uint32_t)(rb.s * a.npm + 16 * g0), ng);
+          drain_columns(s, tmem + lanes + (uint32_t)(rb.s * a.npm + 16 * g0), ng, a.down);
           if (lane == 0) arrive_leader(&acce[rb.s]);
           if (a.corr) {
-            drain_columns(s, corr_base + lanes + (uint32_t)(16 * g0), ng);
+            drain_columns(s, corr_base + lanes + (uint32_t)(16 * g0), ng, a.down);
             if (lane == 0) arrive_leader(corre);
           }
         }
@@ -316,12 +317,12 @@ __device__ __forceinline__ int problem_of(const int* __restrict__ start, int cou
 }
 
 __global__ void __launch_bounds__(256)
-split_x_grouped_kernel(const SplitXJob* __restrict__ jobs, const int* __restrict__ start, int count, int parts) {
+split_x_grouped_kernel(const SplitXJob* __restrict__ jobs, const int* __restrict__ start, int count, int parts, bool scaled) {
   const int b = problem_of(start, count, blockIdx.x);
   const SplitXJob j = jobs[b];
   const int local = (int)blockIdx.x - start[b], kt = (int)cdiv(j.K, 64);
   split_x_tile(j.X, j.K, j.N, j.ldx, j.img, j.npad, parts, (int)cdiv(j.K, BK), (long long)(local % kt) * 64,
-               local / kt * 32, j.xlo, j.bad);
+               local / kt * 32, j.xlo, scaled);
 }
 
 template <bool TRANS, int PARTS>
@@ -367,7 +368,7 @@ int split_x_blocks(int64_t K, int npad) { return (int)(cdiv(K, 64) * cdiv(npad, 
 cudaError_t split_x_grouped(const SplitXJob* jobs, const int* start, int count, int total, SplitMode mode,
                             cudaStream_t st) {
   if (total <= 0) return cudaSuccess;
-  split_x_grouped_kernel<<<total, 256, 0, st>>>(jobs, start, count, mode == kSplitTwo ? 2 : 3);
+  split_x_grouped_kernel<<<total, 256, 0, st>>>(jobs, start, count, mode == kSplitTwo ? 2 : 3, mode == kSplitFp32);
   note_launch();
   return cudaGetLastError();
 }
@@ -382,6 +383,7 @@ cudaError_t split_grouped(bool transA, const SplitJob* jobs, const int2* units, 
   a.info = info;
   a.npm = std::max(npad_max, 16);
   a.stall = stall;
+  a.down = mode == kSplitFp32 ? kScaleDown : 1.f;
   a.corr = mode == kSplitFp32 ? 0 : 1;
   a.corr_first = mode == kSplitFp32 ? 1 : 0;
   a.chunk = mode == kSplitFp32 ? 1 : 4096 / BK;   // (see split_gemm.cu)
