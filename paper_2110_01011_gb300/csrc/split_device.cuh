@@ -19,6 +19,14 @@ constexpr int kThreads = 640;         // 4 + 8 + 8 warps
 constexpr int kGroups = 7;            // 16-column groups of a drain warp: N <= 224
 constexpr int kMaxStages = 8;
 constexpr int kMaxASlots = 8;
+// Units per accumulation chain of the BF16x3 form: the loss of a chain grows with
+// its length. Three parts, against 64 bits: K = 4096, 2560, 2048, 1024 leave L of 15
+// factorisations 1.48e-6, 1.28e-6, 1.26e-6, 9.0e-7 off on average (P 5.5e-6, 4.5e-6,
+// 4.4e-6, 2.9e-6); 8192^2, k = 128 took 1204 us at 2048 and 1222 us at 1024, where the
+// single main accumulator waits for every drain. Batches keep 4096 with three parts
+// as well (24 problems: L 2.8e-6 off, 2.3e-6 at 2048): with other chains single entries of
+// ill-conditioned problems move by up to 1.6e-3 of their size.
+constexpr int kChainTwo = 4096 / BK, kChainThree = 2048 / BK, kChainBatch = 4096 / BK;
 constexpr uint32_t kABytes = BM * BK * 4;        // FP32 stage of A by TMA
 constexpr long long kWaitLimit = 4000000000LL;   // cycles (~2 s)
 // The FP32 form splits 2^24 A and 2^24 X: no FP32 value has a bit below 2^-149, so

@@ -150,11 +150,12 @@ __host__ __device__ inline int unit_owner(int u, int units, int G) {
 // to the end of an even share of the 128-row tiles per SM, at most `chunk` from
 // its start. Truncation makes every chain lose a little toward zero, so the
 // lengths and places of the chains are what the result's rounding consists of.
-// They follow from the product's shape alone, not from how its tiles are paired
-// and dealt: a pair's range can be twice a share where one of its CTAs has no
-// rows (156512 x 336: L 8e-6 off with chains as long as the ranges, 2e-6 with
-// shares), and chains cut at the same K in all rows add up to a coherent change
-// of A (P of the 20000^2 learned factorisation 3.8e-5 off, else 2.7e-5).
+// They follow from the product's shape and, where a pair's range ends inside a
+// share, from the number of pairs (`left`), but not from the ranges alone: a range
+// can be twice a share where one CTA of the pair has no rows (156512 x 336: L 8e-6
+// off with chains as long as the ranges, 2e-6 with shares), and chains cut at the
+// same K in all rows add up to a coherent change of A (P of the 20000^2 learned
+// factorisation 3.8e-5 off, else 2.7e-5).
 __device__ inline int chain_units(const Args& a, int t, int k, int left) {
   if (a.shares == 0) return min(left, a.chunk);
   const long long units = (long long)cdiv(a.M, (int64_t)BM) * a.kb, u0 = (long long)CG * t * a.kb, u = u0 + k;
@@ -691,16 +692,15 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   // it adds to, always toward zero. FP32: one chain per unit, the correction
   // products (2^-8 of the main ones) first, so that only two MMAs add to a
   // sum of full size; 64 units are summed in registers, then in memory.
-  // BF16x3: K = 4096, with three parts 2560 (179560 x 376: L 9e-7 off in 128-row
-  // tiles, 1.2e-6 here, 2.0e-6 with 4096); the corrections apart where tensor
-  // memory has room (npad <= 128) or there are three parts.
+  // BF16x3: see kChainTwo; the corrections apart where tensor memory has room (npad
+  // <= 128) or there are three parts.
   if (mode == kSplitFp32) {
     a.chunk = 1;
     a.corr = 0;
     a.corr_first = 1;
     a.flush = 64;
   } else {
-    a.chunk = (parts == 3 ? 2560 : 4096) / BK;
+    a.chunk = parts == 3 ? kChainThree : kChainTwo;
     a.corr = parts == 3 || npad <= 128 ? 1 : 0;
     a.flush = 1 << 30;
   }

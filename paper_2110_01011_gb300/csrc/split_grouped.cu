@@ -386,7 +386,7 @@ cudaError_t split_grouped(bool transA, const SplitJob* jobs, const int2* units, 
   a.down = mode == kSplitFp32 ? kScaleDown : 1.f;
   a.corr = mode == kSplitFp32 ? 0 : 1;
   a.corr_first = mode == kSplitFp32 ? 1 : 0;
-  a.chunk = mode == kSplitFp32 ? 1 : 4096 / BK;   // (see split_gemm.cu)
+  a.chunk = mode == kSplitFp32 ? 1 : kChainBatch;
   a.flush = mode == kSplitFp32 ? 64 : 1 << 30;
   const int cc = a.corr ? a.npm : 0;
   a.nbuf = 2 * a.npm + cc + 2 * parts * 16 <= 512 ? 2 : 1;
