@@ -820,14 +820,9 @@ cudaError_t chol_inv_batched(const CholJob* jobs, int count, int dmax, bool fp64
   return fp64 ? launch_batched<double>(jobs, count, dmax, st) : launch_batched<float>(jobs, count, dmax, st);
 }
 
-// (Workspace sizes that callers see include this: it reserves the buffer from
-// the d on where panel buffers of 2 x 16 columns left no room for the square.)
-template <typename T>
-size_t global_bytes(int d) {
-  const size_t panels = (size_t)32 * round_up(d, 16) * sizeof(T), fixed = (2 * kMaxD + 16) * sizeof(T) + 96;
-  return square_bytes<T>(d) + panels + fixed <= smem_optin() ? 0 : square_bytes<T>(d);
-}
-size_t chol_global_bytes(int d, bool fp64) { return fp64 ? global_bytes<double>(d) : global_bytes<float>(d); }
+// The square of a single FP64 factor that does not fit in shared memory; one in FP32
+// lies in a cluster's.
+size_t chol_global_bytes(int d, bool fp64) { return fp64 && !square_in_smem<double>(d) ? square_bytes<double>(d) : 0; }
 
 cudaError_t chol_inv(int d, const float* G, int64_t ldg, float* R, float* Rinv, int64_t ldr, int* info,
                      double* shift_count, int* gate_out, const int* gate_in, void* gstore, bool fp64,

@@ -349,6 +349,7 @@ struct Dims {
   int64_t m, n, lda, ldo;
   int k, p, q, d;
   bool learned = false;   // d = k + 20 is a capacity; the run picks p in {5, 10, 20}
+  bool sparse = false;    // A in CSR: no dense pass
 };
 
 struct Out {
@@ -413,10 +414,10 @@ class Plan {
   }
 
   // FP32 plans take the tensor-core products where one pass over A is worth
-  // them. Their scratch does not lift a workspace that fits the allocation-free
+  // them (sparse ones have none). Their scratch does not lift a workspace that fits the allocation-free
   // entry's array above it.
   size_t layout(Arena& ar) {
-    if (o_.precision != RQLP_PREC_FP32 || !Ops::split_pays(d_.m, d_.n, d_.d)) return layout(ar, 0);
+    if (o_.precision != RQLP_PREC_FP32 || d_.sparse || !Ops::split_pays(d_.m, d_.n, d_.d)) return layout(ar, 0);
     constexpr size_t kLimit = RQLP_NOALLOC_SCRATCH_BYTES;
     Arena plain;
     plain.dry = true;
@@ -1063,6 +1064,11 @@ rqlp_status rqlp_factor_learned_host(const float* hA, int64_t m, int64_t n, int6
 }
 
 namespace {
+Dims sparse_dims(const rqlp_csr* A, int k, int p, int q, int64_t ldo) {
+  Dims dm = make_dims(A->m, A->n, A->n, k, p, q, ldo);
+  dm.sparse = true;
+  return dm;
+}
 bool valid_csr(const rqlp_csr* A) {
   return A != nullptr && A->m > 0 && A->n > 0 && A->nnz >= 0 && A->row_ptr != nullptr &&
          (A->nnz == 0 || (A->col_idx != nullptr && A->vals != nullptr)) && A->nnz < (int64_t(1) << 31);
@@ -1074,7 +1080,7 @@ size_t rqlp_sparse_workspace_bytes(const rqlp_csr* A, int k, int p, int q, const
   if (!valid_csr(A) || !valid_opts(o) || o.precision != RQLP_PREC_FP32 || o.literal_step5 != 0 ||
       o.fused_power != 0 || !valid_sizes(A->m, A->n, k, p, q))
     return 0;
-  return round_up((int64_t)plan_bytes(make_dims(A->m, A->n, A->n, k, p, q, k + p), o), 256) +
+  return round_up((int64_t)plan_bytes(sparse_dims(A, k, p, q, k + p), o), 256) +
          sparse_csc_bytes(A->n, A->nnz);
 }
 
@@ -1089,7 +1095,7 @@ rqlp_status rqlp_factor_sparse(const rqlp_csr* A, int k, int p, int q, const flo
   if (ldo < d || ldq < d || ldl < d || ldp < d) return RQLP_ERR_ARG;
   const size_t need = rqlp_sparse_workspace_bytes(A, k, p, q, &o);
   if (workspace == nullptr || ws_bytes < need || !aligned(workspace, 256)) return RQLP_ERR_WORKSPACE;
-  Dims dm = make_dims(A->m, A->n, A->n, k, p, q, ldo);
+  const Dims dm = sparse_dims(A, k, p, q, ldo);
   const size_t core = (size_t)round_up((int64_t)plan_bytes(dm, o), 256);
   Arena ar = arena_over(workspace, core);
   Plan pl(dm, o);

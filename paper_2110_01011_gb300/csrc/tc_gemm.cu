@@ -689,16 +689,13 @@ void TcEngine::layout(Arena& ar, int64_t rows_cap, int64_t cols_cap, int d_cap, 
   k_cap_ = k_cap;
   ldb_ = round_up(cols_cap, 64);   // whole 64-column panels
   G_ = sm_count();
-  const int npad = npad_of(d_cap);
   Ahi_ = ar.take<uint16_t>((size_t)(rows_cap * ldb_));
   Alo_ = ar.take<uint16_t>((size_t)(rows_cap * ldb_));
   Alo2_ = three_part ? ar.take<uint16_t>((size_t)(rows_cap * ldb_)) : nullptr;
   Xhi_ = ar.take<uint16_t>((size_t)d_cap * round_up(k_cap, 8));
   Xlo_ = ar.take<uint16_t>((size_t)d_cap * round_up(k_cap, 8));
   Xlo2_ = three_part ? ar.take<uint16_t>((size_t)d_cap * round_up(k_cap, 8)) : nullptr;
-  ar.take<float>((size_t)2 * G_ * BM * npad);   // (partial tiles and their counters once: the reported size stays)
   flag_ = ar.take<int>(4);
-  ar.take<int>((size_t)cdiv(std::max(rows_cap, cols_cap), BM));
   if (gram) {
     const int gp = npad_of((int)cols_cap);
     gpart_ = ar.take<float>((size_t)kGramMaxCtas * cdiv(cols_cap, BM) * BM * gp);
