@@ -606,7 +606,6 @@ chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __re
         // done its diagonal block), j0 .. d - 1 above.
         const bool lower = rank >= J;
         const int cend = lower ? min(d, i0 + NB) : d;
-        const int w0 = rank == J ? warp - 1 : warp, ws = rank == J ? nwarps - 1 : nwarps;
         if (!(rank == J)) {
           for (int e = tid; e < (cend - j0) * (NB / 4); e += kClusterThreads) {
             const int c = j0 + e / (NB / 4), k = 4 * (e % (NB / 4)), o = c / NB;
@@ -614,7 +613,7 @@ chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __re
             *reinterpret_cast<float4*>(&C[(c - j0) * kCLd + k]) = v;
           }
           __syncthreads();
-          for (int t = w0; j0 + 16 * t < cend; t += ws) {
+          for (int t = warp; j0 + 16 * t < cend; t += nwarps) {
             const int r = lane >> 2, c = j0 + 16 * t + (lane & 3);   // rows r + 8 i, columns c + 4 j
             bool va[4], vb[4];
 #pragma unroll

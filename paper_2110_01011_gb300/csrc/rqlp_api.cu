@@ -71,7 +71,7 @@ class Ops {
       ar.off = std::max(ar.off, at + panel_bytes(m, n));
       // Tall d-column operands of CholeskyQR: the Gram (BF16x3) and the
       // products X R^{-1} (exact mode, six products) on the tensor cores.
-      tcs_.layout(ar, std::max(m, n), dcap_, dcap_, dcap_, true, /*three_part=*/true);
+      tcs_.layout(ar, std::max(m, n), dcap_);
     }
     tc_on_ = with_tc;
     split32_ = split_bytes > 0 && split_gemm_layout(ar, &sg_, part_, block_bytes, tall, tall, dcap_, 3);
@@ -97,7 +97,7 @@ class Ops {
   cudaError_t apply_r0(const float* X, int64_t ldx, int64_t rows, float* out, int64_t ldout) {
     if (tc_on_ && rows > (int64_t)d_) {
       tcs_.reset();
-      CK(tcs_.split(X, rows, d_, ldx, nullptr, st_));
+      CK(tcs_.split(X, rows, d_, ldx, st_));
       return tcs_.product(Ri_[0], ld_, d_, out, ldout, info_, st_);
     }
     return trmm(X, ldx, rows, Ri_[0], out, ldout);
@@ -233,7 +233,7 @@ class Ops {
   cudaError_t tc_cqr(const float* X, int64_t ldx, int64_t rows, float* out, int64_t ldout, int slot,
                      int* gate_out, bool want_r) {
     tcs_.reset();
-    CK(tcs_.split(X, rows, d_, ldx, nullptr, st_));
+    CK(tcs_.split(X, rows, d_, ldx, st_));
     CK(tcs_.gram(G_, ld_, info_, st_));
     CK(chol(slot, gate_out, nullptr, want_r));
     return tcs_.product(Ri_[slot], ld_, d_, out, ldout, info_, st_);

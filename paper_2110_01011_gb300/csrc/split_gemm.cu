@@ -38,24 +38,11 @@
 
 #include "split_device.cuh"
 #include "split_gemm.cuh"
+#include "tc_gemm.cuh"
 
 namespace rqlp {
 namespace sp {
 
-using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static EncodeFn encode_fn() {
-  static const EncodeFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return reinterpret_cast<EncodeFn>(p);
-  }();
-  return fn;
-}
 static bool encode(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows, uint64_t stride, uint32_t bc,
                    uint32_t br, CUtensorMapSwizzle sw) {
   EncodeFn fn = encode_fn();
@@ -123,7 +110,7 @@ struct Args {
   int* next1;
   double* sumsq;
   int* info;
-  int M, N, K, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole, perm;   // sx, sf, sa: stages of X, of A in FP32, A slots
+  int M, N, npad, kb, tiles, G, sx, sf, sa, nbuf, vec_out, fixup, whole, perm;   // sx, sf, sa: stages of X, of A in FP32, A slots
   int chunk;                // units per chain of the main accumulator
   int shares;               // SMs whose even shares bound the chains (0: the chunk alone)
   int corr_first;           // chains of one unit, the correction products first
@@ -676,7 +663,7 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   a.next1 = w + 2 + (turn ^ 1);
   a.sumsq = sumsq;
   a.info = info;
-  a.M = (int)M; a.N = N; a.K = (int)K; a.npad = npad;
+  a.M = (int)M; a.N = N; a.npad = npad;
   a.kb = kb;
   a.tiles = (int)cdiv(M, (int64_t)BM * CG);
   if ((long long)a.tiles * kb > (1LL << 30)) return cudaErrorInvalidValue;
