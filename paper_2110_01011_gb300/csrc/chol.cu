@@ -197,12 +197,8 @@ __device__ __forceinline__ bool update_tile(T* S, int LDS, const T* DT, int d, i
 // scaled by 1 / sqrt(pivot) and later columns c take l_it l_ct. On the path
 // from a pivot to the next lie its root, two products and a shuffle; the
 // columns after next take column t from LT a step later, while the next root
-// is on its way. rsqrtf is 5e-8 low on average next to 1, where the pivots of a
-// second CholeskyQR pass lie: every column of the result came out short by that
-// and L with it (30 FP32 factorisations: L off by 2.6e-7, 1.8e-7 with the step).
-// A Newton step per lane on the finished roots takes it out of L's diagonal and
-// of 1 / L_jj, behind the chain. tol: this lane's pivot bound. Returns the first
-// failing column (the block is then left as it was), or -1.
+// is on its way. tol: this lane's pivot bound. Returns the first failing
+// column, or -1 (the block is then left as it was).
 template <typename T, int NB>
 __device__ __forceinline__ int factor_diagonal(T* D, int ld, int jb, T tol, T* LT, T* rdiag, int lane) {
   T a[NB], lc[NB];   // the lane's row; the column before the current one
@@ -235,24 +231,26 @@ __device__ __forceinline__ int factor_diagonal(T* D, int ld, int jb, T tol, T* L
 #pragma unroll
     for (int c = (t + 2) / 4 * 4; c < NB; c += 4) ld4(&LT[t * NB + c], &lc[c]);
   }
-  T diag = 0;
-  if (lane < jb) {
-    const T r = rdiag[lane], l = LT[lane * NB + lane], h = (T)0.5 * fma(-l, r, (T)1);
-    rdiag[lane] = fma(r, h, r);
-    LT[lane * NB + lane] = diag = fma(l, h, l);
-  }
-  __syncwarp();
   if (f < 0 && lane < jb) {
 #pragma unroll
     for (int k = 0; k < NB; k += 4) {
       T o[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) o[u] = k + u < lane ? a[k + u] : (k + u == lane ? diag : (T)0);
+      for (int u = 0; u < 4; ++u) o[u] = k + u <= lane ? a[k + u] : (T)0;
       st4(&D[(size_t)lane * ld + k], o);
     }
   }
   return f;
 }
+
+// What 1 / sqrt(pivot) = r, with l = pivot r on L's diagonal, lacks relative to
+// itself (one Newton step). rsqrtf is 5e-8 low on average next to 1, where the
+// pivots of a second CholeskyQR pass lie: every column of the result came out short by
+// that and L with it (30 FP32 factorisations: L off by 2.6e-7; 1.7e-7 with the
+// step). Column t of L and row t of W carry the factor; both are corrected on their
+// way out (in the chain above, or behind it, the step took 0.3 us per panel).
+template <typename T>
+__device__ __forceinline__ T root_correction(T l, T r) { return (T)0.5 * fma(-l, r, (T)1); }
 
 // v = L_JJ^{-1} v by forward substitution, column by column: an entry is final
 // one product after the one before it.
@@ -289,6 +287,7 @@ __device__ __forceinline__ void chol_body(int d, const float* __restrict__ G, in
   T* S = kShared ? LT + NB * NB : gS;
   __shared__ __align__(32) T gdiag[kMaxD];   // G's diagonal; W's once a panel is done
   __shared__ T rdiag[NB];                    // 1 / L_jj of the current diagonal block
+  __shared__ T corr[kMaxD];                  // root_correction of every column
   __shared__ int s_fail, s_tile;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
@@ -415,6 +414,7 @@ __device__ __forceinline__ void chol_body(int d, const float* __restrict__ G, in
         solve_row<T, NB>(v, LT, rdiag, jb);
         if (own) {
           gdiag[r] = rdiag[cc];
+          corr[r] = root_correction(LT[cc * NB + cc], rdiag[cc]);
 #pragma unroll
           for (int k = 0; k < NB; k += 4) st4(&DT[cc * kDtLd + k], &v[k]);
 #pragma unroll
@@ -481,8 +481,10 @@ __device__ __forceinline__ void chol_body(int d, const float* __restrict__ G, in
 #pragma unroll
     for (int t = 0; t < kMaxD / 32; ++t) {
       const int l = lane + 32 * t;
-      x[t] = l < d && l > i ? (float)S[(size_t)i * LDS + l] : (l == i ? (float)gdiag[i] : 0.f);
-      y[t] = l < d && l >= i && R != nullptr ? (float)S[(size_t)l * LDS + i] : 0.f;
+      const T v = l < d && l >= i ? (l > i ? S[(size_t)i * LDS + l] : gdiag[i]) : (T)0;
+      const T w = l < d && l >= i && R != nullptr ? S[(size_t)l * LDS + i] : (T)0;
+      x[t] = (float)fma(v, l < d ? corr[l] : (T)0, v);
+      y[t] = (float)fma(w, corr[i], w);
     }
 #pragma unroll
     for (int t = 0; t < kMaxD / 32; ++t) {
@@ -554,6 +556,7 @@ chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __re
   float* LT = DT + NB * kCLd;                      // L_JJ by columns: the owner's, or a copy
   float* rdiag = LT + NB * NB;                     // (behind LT: one copy takes both)
   __shared__ float gdiag[NB];                      // G's diagonal; W's once the panel is done
+  __shared__ float corr[kMaxD];                    // root_correction of every column
   __shared__ int s_fail;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = kClusterThreads / 32;
   const int i0 = NB * rank, rows = min(NB, d - i0);
@@ -669,6 +672,8 @@ chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __re
 #pragma unroll
           for (int k = 0; k < NB; k += 4) st4(&row[k], &v[k]);
         }
+      } else if (warp == 1 && lane < jb) {
+        corr[j0 + lane] = root_correction(LT[lane * NB + lane], rdiag[lane]);
       }
       __syncthreads();
       if (J + 1 == P) break;
@@ -723,12 +728,19 @@ chol_cluster_kernel(int d, const float* __restrict__ G, int64_t ldg, float* __re
 #pragma unroll
     for (int t = 0; t < kMaxD / 32; ++t) {
       const int l = lane + 32 * t;
-      if (l < d) ri[l] = l > i0 + i ? S[i * LDS + l] : (l == i0 + i ? gdiag[i] : 0.f);
+      if (32 * t >= d) break;
+      if (l < d) {
+        const float v = l > i0 + i ? S[i * LDS + l] : (l == i0 + i ? gdiag[i] : 0.f);
+        ri[l] = fmaf(v, corr[l], v);
+      }
     }
   }
   if (R != nullptr && lane < rows) {
 #pragma unroll 4
-    for (int i = warp; i < d; i += nwarps) R[(int64_t)i * ldr + i0 + lane] = i <= i0 + lane ? S[lane * LDS + i] : 0.f;
+    for (int i = warp; i < d; i += nwarps) {
+      const float v = i <= i0 + lane ? S[lane * LDS + i] : 0.f;
+      R[(int64_t)i * ldr + i0 + lane] = fmaf(v, corr[i], v);
+    }
   }
 }
 
@@ -747,7 +759,7 @@ size_t square_bytes(int d) { return (size_t)d * lds_of(d) * sizeof(T); }
 template <typename T>
 size_t panel_bytes() { return (size_t)Panel<T>::NB * (2 * Panel<T>::NB + kDtPad) * sizeof(T); }
 template <typename T>
-size_t static_bytes() { return (kMaxD + Panel<T>::NB) * sizeof(T) + 96; }
+size_t static_bytes() { return (2 * kMaxD + Panel<T>::NB) * sizeof(T) + 96; }
 template <typename T>
 bool square_in_smem(int d) {
   return square_bytes<T>(d) + panel_bytes<T>() + static_bytes<T>() <= smem_optin();
