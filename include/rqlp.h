@@ -75,8 +75,9 @@ typedef struct {
                    /* the passes over A. 2: A = A_hi + A_lo, X = X_hi + X_lo, */
                    /* three products, error ~2^-16 |A| |X| per pass; 3: a    */
                    /* third part each (A_lo2 = bf16(A - A_hi - A_lo)), the   */
-                   /* six products above 2^-24, FP32-level error at twice    */
-                   /* the MMA work (A is read in FP32 either way);           */
+                   /* six products above 2^-24, error ~2^-19 (what is left is */
+                   /* the loss of long sums, not of parts) at twice the MMA   */
+                   /* work (A is read in FP32 either way);                    */
                    /* 0: automatic: three parts when p < 5 or m n <= 2^27,  */
                    /* else two (the batched form: three parts)               */
   int literal_step5; /* 0: step 5 on the d x d R, (P^, R^) = qr(R^T),         */

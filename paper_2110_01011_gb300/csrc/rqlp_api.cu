@@ -174,6 +174,12 @@ class Ops {
     return split_gemm(&sg_, transA, M, d_, K, A, lda, X, ldx, out, ldout, three_ ? kSplitThree : kSplitTwo, sumsq,
                       nullptr, info_, true, st_);
   }
+  // From 2e8 multiply-adds on FP32 products go to the tensor cores, which halve their
+  // error. A sketch of 4e8 and more is nearly always faster there, one below often
+  // not: few rows leave most CTA pairs without a tile (us, FMA and split: 1500 x 1000,
+  // d = 200 36, 48; 300 x 3400, d = 200 29, 52; 3000 x 500, d = 140 44, 30; 2000 x 1100,
+  // d = 100 70, 50); in a factorisation the difference is within its launches' (1214 x
+  // 12424, k = 12: 231 us either way).
   static bool split_pays(int64_t M, int64_t K, int d) { return (double)M * K * d >= 2e8; }
   // The same product in FP32. Where it pays it runs on the
   // tensor cores in three parts; an FMA product gated on the range word then

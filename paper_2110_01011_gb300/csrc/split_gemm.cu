@@ -3,37 +3,41 @@
 //
 // A = A_1 + A_2 [+ A_3] and X likewise, each part the BF16 rounding of what
 // the earlier ones leave. Two parts: A_1 X_1 + A_1 X_2 + A_2 X_1 (the BF16x3
-// form, products above 2^-16). Three parts: the six products above 2^-24;
-// three parts hold all 24 bits of an FP32 value, so the sum is as accurate as
-// FP32 arithmetic.
+// form, products above 2^-16). Three parts hold all 24 bits of an FP32 value; of
+// their nine products the six above 2^-24 are taken. In FP32 (chains of one unit)
+// a result is off by 1.5e-7 of its norm on average where FMAs in two levels of
+// sums leave 2.9e-7 (10007 x 6001 and 16384 x 12288); 4.5e-8 of it is a loss
+// toward zero, which FMAs do not have (the adds in tensor memory truncate).
 //
 // What bounds the product: with A's parts in shared memory the MMAs read A (4
 // KB) and X (up to 8 KB) per product and 16 of K, and the copies into shared
 // memory come on top: ~170 bytes per clock against the 128 that shared memory
-// delivers. Here A never passes through shared memory: four warps load it from
-// global memory into registers, split it there and store the parts to tensor
-// memory, from where the MMA takes its A operand. Shared memory then serves X
-// only, and neither a separate pass over A nor a copy of its parts is needed
-// (4 bytes per element of A and pass instead of 4 or 6 and a 8 or 10 byte
-// split).
+// delivers. Here A passes through shared memory once, in FP32: TMA writes a stage
+// of 16 KB, the split warps read it, split it in registers and store the parts to
+// tensor memory, from where the MMAs take their A operand. Two parts at d = 205:
+// 16 + 16 KB of A, 13 KB of X written and 20 KB read by the MMAs per CTA and unit of
+// ~1000 clocks, half of what shared memory delivers. Neither a separate pass over
+// A nor a copy of its parts is needed (4 bytes per element of A and pass instead
+// of 4 or 6 and a 8 or 10 byte split).
 //
 // CG = 2: two CTAs of a cluster share one 256-row tile (cta_group::2): each
 // holds half of X's columns, so X is read from L2 once per 256 rows and each
 // shared memory feeds half of X.
 //
 // X's parts are written by split_x_kernel as the images of the shared-memory
-// stages (32 of K, K-major rows of 64 bytes, 64-byte swizzle), so a stage is
-// one bulk copy.
+// stages (32 of K, K-major rows of 64 bytes, 64-byte swizzle), copied by one TMA
+// box per part.
 //
-// Warps: 0 copies X stages, 1 issues the MMAs, 2 allocates tensor memory; 4-7
-// load and split A; 8-15 drain the accumulators. Chains in tensor memory are
-// cut every `chunk` units of 32 (the accumulation there loses a little of
-// every add in the same direction); the drain warps hold the running sums in
-// registers and add with round-to-nearest. The (tile, unit) pairs are dealt
-// evenly to the CTAs (stream-K); split tiles are summed by the last CTA to
-// arrive, or by split_fixup_kernel when a tile spans more than kMaxSlots of
-// them. Every wait is bounded. Where one runs out, the status word reports it and
-// the sums that were not read become NaN, which raises the range word in FP32.
+// Warps: 0 copies X stages, 1 issues the MMAs, 2 allocates tensor memory, 3 copies
+// stages of A; 4-11 split them, two warpgroups by turns; 12-19 drain the
+// accumulators. Chains in tensor memory are cut every `chunk` units of 32 (the
+// accumulation there loses a little of every add in the same direction); the drain
+// warps hold the running sums in registers and add with round-to-nearest. The
+// (tile, unit) pairs are dealt evenly to the CTA pairs (stream-K; whole tiles for K
+// <= 1024); split tiles are summed by the last pair to arrive, or by
+// split_fixup_kernel when a tile spans more than kMaxSlots of them. Every wait is
+// bounded. Where one runs out, the status word reports it and the sums that were
+// not read become NaN, which raises the range word in FP32.
 #include <algorithm>
 
 #include "split_device.cuh"
@@ -672,7 +676,11 @@ cudaError_t product(SplitGemmWs* ws, int turn, bool transA, int64_t M, int N, in
   if ((long long)a.tiles * kb > (1LL << 30)) return cudaErrorInvalidValue;
   a.units = a.tiles * kb;
   a.stall = ws->stall;
-  // Short K: a split tile would cost more than it saves; whole tiles per CTA.
+  // Short K: whole tiles per pair, also where most pairs then have none. Dealing the
+  // units instead costs more in sums of split tiles than it spares where tiles are few
+  // (FP32, us: 1500 x 1000, d = 200 48 whole and 70 dealt, 4000 x 500, d = 120 30 and 49);
+  // it wins with 79 tiles on 76 pairs or one accumulator (20000 x 1000, d = 60 67 and
+  // 59, 1000 x 1000, d = 210 83 and 42).
   a.whole = kb <= 32 ? 1 : 0;
   // Groups: at most two partial tiles each (none with whole tiles).
   const int cap = a.whole ? a.tiles : std::min(a.units, ws->slots / (2 * CG));
