@@ -247,9 +247,12 @@ def run_reference(a):
 # ------------------------------------------------------------------ our arm
 
 def kernel_sha(prec):
-    """Hash of the source file that holds the dominant kernel (of both precisions)."""
-    p = os.path.join(ROOT, "paper_2110_01011_gb300", "csrc", "split_gemm.cu")
-    return hashlib.sha256(open(p, "rb").read()).hexdigest()[:12]
+    """Hash of the source files that hold the dominant kernel (of both precisions)."""
+    h = hashlib.sha256()
+    for name in ("split_gemm.cu", "split_device.cuh", "tc_ptx.cuh"):
+        with open(os.path.join(ROOT, "paper_2110_01011_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
 
 
 def traffic_for(kernel, sha):
