@@ -70,3 +70,14 @@ def test_batch_keeps_small_entries():
         return [x.clone() for x in b.L]
     for a, b in zip(run(0.0), run(1e-35)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("scale_a,scale_x", [(1e20, 1.0), (1e30, 1.0), (1.0, 1e30), (1e18, 1e18), (1e33, 1e-33)])
+def test_large_values(scale_a, scale_x):
+    """Sums and values that overflow in the scaled form come from the FMA units,
+    the others from the tensor cores; either way they are FP32's."""
+    A, X = _randn(M, N, seed=8) * scale_a, _randn(N, D, seed=9) * scale_x
+    Y, _ = rqlp.sketch(A, X, 0, precision=rqlp.PREC_FP32)
+    ref = A.double() @ X.double()
+    assert bool(Y.isfinite().all())
+    assert bool(((Y.double() - ref).abs() <= 4e-6 * (A.double().abs() @ X.double().abs())).all())
